@@ -44,6 +44,9 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     if debug:  # the shared-memory kernels only; the rest of the launchers answer "unsupported"
         sources = [f for f in sources if not f.startswith(("pvq_big", "pvq_wide"))]
         extra = ["-DPVQ_DEBUG"]
+    newest = max([hdr] + [os.path.getmtime(os.path.join(CSRC, f)) for f in sources])
+    if not force and os.path.exists(lib) and os.path.getmtime(lib) >= newest:
+        return lib  # also where the objects are not at hand
     for src in sources:
         s = os.path.join(CSRC, src)
         o = os.path.join(objdir, src[:-3] + ".o")

@@ -1,4 +1,4 @@
-// Encode kernel (and the fused encode -> decode round trip): templates shared by
+// The general encode kernel (rotation, least-squares amplitude, wide codes): templates shared by
 // the per-group-size translation units.
 //
 // One thread encodes one group; a thread block covers whole rows (the row norm
@@ -228,51 +228,6 @@ __device__ __forceinline__ mp<W> enumerate_v(const float (&mag)[N], int K, uint3
     return c;
 }
 
-// Algorithm 2 as the walk of pvq_walk.cuh run forwards, on the decoder's table: from
-// (0, K), a pulse at the current position adds t (its first) or 2t (a further one) and
-// goes left, the end of a position adds t when y_i < 0 and goes down; t = N(N-1-i, col).
-// N + K steps of the same instructions for every thread.  Used by the fused kernel when
-// the cumulative tables do not fit in shared memory beside the decoder's.  y: the thread's
-// slots holding the signed point (one spare slot is read past the end).
-template <int N, int W, int EB, typename YT>
-__device__ __forceinline__ mp<W> enumerate_walk(const YT* y, uint32_t tab0, int rowlen, int K) {
-    mp<W> c;
-    mp_zero(c);
-    const int D = (rowlen + 1) * EB;
-    uint32_t p = tab0 + K * EB;
-    int yi = y[0];
-    int rem = abs(yi);
-    int v = 0;
-    const int S = N + K;
-#pragma unroll 2
-    for (int s = 0; s < S; ++s) {
-        const mp<W> t = load_entry<W>(p);
-        const bool more = rem > 0;
-        const bool add1 = more || (yi < 0);
-        const bool add2 = more && v > 0;
-        mp<W> a1, a2;
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            a1.w[w] = add1 ? t.w[w] : 0u;
-            a2.w[w] = add2 ? t.w[w] : 0u;
-        }
-        mp_add<W>(c, a1);
-        mp_add<W>(c, a2);
-        if (more) {
-            rem -= 1;
-            v += 1;
-        } else {
-            ++y;
-            yi = *y;
-            rem = abs(yi);
-            v = 0;
-            p += D;
-        }
-        p -= EB;
-    }
-    return c;
-}
-
 // The N values of one group as they sit in memory, fetched with 16-byte loads.
 template <int N, bool BF16>
 __device__ __forceinline__ void load_raw(const void* base, size_t elem_off, uint32_t (&r)[BF16 ? N / 2 : N]) {
@@ -291,12 +246,10 @@ __device__ __forceinline__ void load_raw(const void* base, size_t elem_off, uint
 // Launch-time geometry of the encode kernels' shared memory (bytes from the start).
 struct EncodeSmem {
     uint32_t enc_bytes;   // staged encoder table(s)
-    uint32_t walk_bytes;  // fused: staged walk tables
-    uint32_t ss_off, edges_off, levels_off, idx_off, wbuf_off;
+    uint32_t ss_off, edges_off, idx_off;
     int ss_floats;        // per buffer (there are two)
     int idx_words;        // per buffer (there are two)
-    int enum_mode;        // 2: U and 2V staged, 1: V only, 0: none (fused: the walk table serves)
-    int walk_phases;
+    int enum_mode;        // 2: U and 2V staged, 1: V only
     uint32_t signs_off;   // rotation: rot_block floats
     uint32_t xbuf_off;    // rotation across more than a warp: threads * N floats
 };
@@ -378,8 +331,7 @@ __device__ __forceinline__ TileLoc locate(const BatchArgs& a, unsigned tile) {
     return t;
 }
 
-// Shared memory: [encoder tables][walk tables (fused)][2 x ss per thread slot, padded rows]
-//                [edges][levels (fused)][2 x scale-index words][per-warp slots (fused)]
+// Shared memory: [encoder tables][2 x ss per thread slot, padded rows][edges][2 x scale-index words]
 // The two ss / scale-index buffers alternate between consecutive tiles, and a tile's index
 // words are written out behind the next tile's first barrier, which leaves two block-wide
 // barriers per tile; the input of the next tile is
@@ -389,13 +341,12 @@ __device__ __forceinline__ TileLoc locate(const BatchArgs& a, unsigned tile) {
 // values, whatever type the input has.
 // LS: the least-squares amplitude of Step 4 (a kernel of its own: its extra live values would
 // otherwise cost the common path registers).
-template <int N, int W, bool FUSED, typename YT, bool BF16, bool ROT, bool LS>
+template <int N, int W, bool BF16, bool ROT, bool LS>
 __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ BatchArgs a,
                                                       const __grid_constant__ EncodeSmem sm) {
     extern __shared__ __align__(16) uint8_t smem[];
     constexpr int TW = W <= 2 ? W : (W <= 4 ? 4 : 6);
     constexpr int EB = TW * 4;
-    constexpr int YS = N * static_cast<int>(sizeof(YT)) + 4;
     constexpr int RW = BF16 ? N / 2 : N;      // words of a group as loaded
     constexpr bool WBF16 = BF16 && !ROT;       // the form the kernel works on: packed bf16, or fp32
     constexpr int WW = WBF16 ? N / 2 : N;
@@ -418,7 +369,6 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
     }
     float* s_ss2 = reinterpret_cast<float*>(smem + sm.ss_off);
     float* s_edges = reinterpret_cast<float*>(smem + sm.edges_off);
-    float* s_levels = reinterpret_cast<float*>(smem + sm.levels_off);
     uint32_t* s_idx2 = reinterpret_cast<uint32_t*>(smem + sm.idx_off);
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -429,21 +379,13 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
     const BulkStage stage = bulk_stage_begin(&stage_bar);
     if (threadIdx.x == 0) {
         const uint8_t* blob = reinterpret_cast<const uint8_t*>(a.table);
-        bulk_stage_expect(stage, sm.enc_bytes + (FUSED ? walk_tables_stage_bytes(L, sm.walk_phases) : 0u));
-        if (sm.enc_bytes)
-            bulk_stage_copy(stage, smem, blob + (sm.enum_mode == 2 ? L.enc_off[0] : L.enc_off[2]), sm.enc_bytes);
-        if constexpr (FUSED) walk_tables_stage(stage, smem + sm.enc_bytes, a.table, L, sm.walk_phases);
+        bulk_stage_expect(stage, sm.enc_bytes);
+        bulk_stage_copy(stage, smem, blob + (sm.enum_mode == 2 ? L.enc_off[0] : L.enc_off[2]), sm.enc_bytes);
     }
     for (int i = threadIdx.x; i < 2 * sm.idx_words; i += blockDim.x) s_idx2[i] = 0u;
     const uint32_t tabA = shared_addr(smem);
     const uint32_t tabB = tabA + ((L.enc_bytes + 127u) & ~127u);  // 2V, when two tables are staged
     const int rowbytes = (K + 2) * EB;
-    WalkTables wt;
-    YT* yslots = nullptr;
-    if constexpr (FUSED) {
-        wt = walk_tables(L, tabA + sm.enc_bytes, sm.walk_phases, a);
-        yslots = reinterpret_cast<YT*>(smem + sm.wbuf_off + threadIdx.x * YS);
-    }
     const float* cur_edges = nullptr;
 
     unsigned tile = blockIdx.x;
@@ -462,8 +404,7 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
     }
     __syncthreads();                      // index words cleared
 #ifdef PVQ_DEBUG
-    debug_begin(tabA, tabA + sm.enc_bytes + (FUSED ? sm.walk_bytes : 0u), tabA + sm.wbuf_off, YS,
-                N * static_cast<uint32_t>(sizeof(YT)), a.debug_status);
+    debug_begin(tabA, tabA + sm.enc_bytes, 0u, 0u, 0u, a.debug_status);
 #endif
     struct {
         bool valid;
@@ -516,11 +457,9 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
 
         if (nedges != 0 && cur_edges != m.edges) {  // uniform across the block
             for (int i = threadIdx.x; i < nedges; i += blockDim.x) s_edges[i] = m.edges[i];
-            if constexpr (FUSED)
-                for (int i = threadIdx.x; i <= nedges; i += blockDim.x) s_levels[i] = m.levels[i];
             cur_edges = m.edges;
         }
-        if constexpr (!FUSED) {
+        {
             // The previous tile's index words (the other buffer) are complete: every thread added
             // its bits before it came to barrier (1).  Write them out and clear them for the next tile.
             uint32_t* other = s_idx2 + (buf ^ 1) * sm.idx_words;
@@ -589,20 +528,8 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
         mp<W> c;
         if (sm.enum_mode == 2) {
             c = enumerate_uv<N, W, EB>(mag, K, tabA, tabB, rowbytes);
-        } else if (sm.enum_mode == 1) {
-            c = enumerate_v<N, W, EB>(mag, K, tabA, rowbytes);
         } else {
-            if constexpr (FUSED) {
-#pragma unroll
-                for (int i = 0; i < N; ++i) {
-                    const int mb = __float_as_int(mag[i]);
-                    const int mi2 = (mb & 0x7fffffff) - kMagicBits;
-                    yslots[i] = static_cast<YT>(mb < 0 ? -mi2 : mi2);
-                }
-                c = enumerate_walk<N, W, EB, YT>(yslots, wt.tab0, wt.rowlen, K);
-            } else {
-                mp_zero(c);
-            }
+            c = enumerate_v<N, W, EB>(mag, K, tabA, rowbytes);
         }
 
         __syncthreads();  // (2) row energies are in s_ss[r * gp]
@@ -623,36 +550,26 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
             }
         }
 
-        if constexpr (!FUSED) {
-            if (active) {
-                if (g == 0) m.row_norm[row] = rnorm;
-                uint32_t* cp = m.codes + (static_cast<size_t>(row) * G + g) * W;
-                if (PVQ_DEBUG_INDEX(row * G + g, m.rows * G, PVQ_DEBUG_GLOBAL_STORE)) {
+        if (active) {
+            if (g == 0) m.row_norm[row] = rnorm;
+            uint32_t* cp = m.codes + (static_cast<size_t>(row) * G + g) * W;
+            if (PVQ_DEBUG_INDEX(row * G + g, m.rows * G, PVQ_DEBUG_GLOBAL_STORE)) {
 #pragma unroll
-                    for (int w = 0; w < W; ++w) cp[w] = c.w[w];
-                }
-                const unsigned bit = static_cast<unsigned>(g) * b;
-                const unsigned sh = bit & 31u;
-                atomicOr(&s_idx[rl * idx_words + (bit >> 5)], static_cast<uint32_t>(q) << sh);
-                if (sh + b > 32u)
-                    atomicOr(&s_idx[rl * idx_words + (bit >> 5) + 1], static_cast<uint32_t>(q) >> (32u - sh));
+                for (int w = 0; w < W; ++w) cp[w] = c.w[w];
             }
-            prev.valid = true;  // written out after the next tile's first barrier, or after the loop
-            prev.mi = loc.mi;
-            prev.rpt = rpt;
-            prev.row0 = row0;
-        } else {
-            // decode the code just made (every thread of the warp walks, in lockstep)
-            const float amp = !active ? 0.0f
-                              : b == 16 ? __half2float(__ushort_as_half(static_cast<unsigned short>(q)))
-                                        : __fmul_rn(rnorm, s_levels[q]);
-            if (!active) mp_zero(c);
-            walk_code<N, W, YT>(c, wt, K, yslots);
-            if (active) emit_group<N, YT>(m, yslots, amp, static_cast<unsigned>(row), static_cast<unsigned>(g));
+            const unsigned bit = static_cast<unsigned>(g) * b;
+            const unsigned sh = bit & 31u;
+            atomicOr(&s_idx[rl * idx_words + (bit >> 5)], static_cast<uint32_t>(q) << sh);
+            if (sh + b > 32u)
+                atomicOr(&s_idx[rl * idx_words + (bit >> 5) + 1], static_cast<uint32_t>(q) >> (32u - sh));
         }
+        prev.valid = true;  // written out after the next tile's first barrier, or after the loop
+        prev.mi = loc.mi;
+        prev.rpt = rpt;
+        prev.row0 = row0;
 
         if (!have_next) {
-            if constexpr (!FUSED) {
+            {
                 __syncthreads();  // the last tile's index words are complete
                 for (int i = threadIdx.x; i < rpt * idx_words; i += blockDim.x) {
                     const int r2 = i / idx_words;
@@ -669,9 +586,8 @@ __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ Bat
     }
 }
 
-template <int N, int W, bool FUSED, typename YT, bool BF16, bool ROT, bool LS = false>
+template <int N, int W, bool BF16, bool ROT, bool LS = false>
 static int launch_encode_t(BatchArgs& a, cudaStream_t stream) {
-    constexpr int YS = N * static_cast<int>(sizeof(YT)) + 4;
     // Block size: a multiple of 32 that wastes the fewest thread slots over the batch.
     int best_threads = 0;
     long long best_cost = -1;
@@ -722,46 +638,25 @@ static int launch_encode_t(BatchArgs& a, cudaStream_t stream) {
     // rotation: the signs, and an exchange buffer when a rotation block spans more than a warp
     const size_t rot_signs_b = ROT ? static_cast<size_t>(a.rot_block) * 4u : 0;
     const size_t rot_xbuf_b = ROT && a.rot_block / N > 32 ? static_cast<size_t>(threads) * N * 4u : 0;
-    const size_t small = (2 * static_cast<size_t>(ss_floats) + 256 + (FUSED ? 256 : 0) + 2 * max_idx_words) * 4u + 64u +
+    const size_t small = (2 * static_cast<size_t>(ss_floats) + 256 + 2 * max_idx_words) * 4u + 64u +
                          rot_signs_b + rot_xbuf_b;
-    const size_t wbufs = FUSED ? static_cast<size_t>(threads) * YS : 0;
     const size_t enc_one = (L.enc_bytes + 127u) & ~size_t(127);
     EncodeSmem sm;
-    sm.walk_bytes = 0;
-    sm.walk_phases = 0;
-    size_t walk = 0;
     const size_t cap = static_cast<size_t>(smem_max);
-    if (FUSED) {  // the widest walk table has to fit; then as many encoder tables as still do
-        sm.enum_mode = -1;
-        for (int mode = 2; mode >= 0 && sm.enum_mode < 0; --mode) {
-            const size_t fixed = mode * enc_one + small + wbufs;
-            if (fixed >= cap) continue;
-            const int ph = walk_phases_that_fit(L, cap - fixed);
-            if (ph == 0) continue;
-            sm.enum_mode = mode;
-            sm.walk_phases = ph;
-        }
-        if (sm.enum_mode < 0) return PVQ_ERR_UNSUPPORTED;
-        walk = (walk_tables_bytes(L, sm.walk_phases) + 15u) & ~size_t(15);
-        sm.walk_bytes = static_cast<uint32_t>(walk);
-    } else {
-        sm.enum_mode = 2 * enc_one + small <= cap ? 2 : 1;
-        if (sm.enum_mode == 1 && enc_one + small > cap) return PVQ_ERR_UNSUPPORTED;
-    }
+    sm.enum_mode = 2 * enc_one + small <= cap ? 2 : 1;
+    if (sm.enum_mode == 1 && enc_one + small > cap) return PVQ_ERR_UNSUPPORTED;
     sm.enc_bytes = static_cast<uint32_t>(sm.enum_mode * enc_one);
     sm.ss_floats = ss_floats;
     sm.idx_words = max_idx_words;
-    sm.ss_off = static_cast<uint32_t>(sm.enc_bytes + walk);
+    sm.ss_off = sm.enc_bytes;
     sm.edges_off = sm.ss_off + 2u * ss_floats * 4u;
-    sm.levels_off = sm.edges_off + 256u * 4u;
-    sm.idx_off = sm.levels_off + (FUSED ? 256u * 4u : 0u);
+    sm.idx_off = sm.edges_off + 256u * 4u;
     sm.signs_off = (sm.idx_off + 2u * max_idx_words * 4u + 15u) & ~15u;
     sm.xbuf_off = sm.signs_off + static_cast<uint32_t>(rot_signs_b);
-    sm.wbuf_off = sm.xbuf_off + static_cast<uint32_t>(rot_xbuf_b);
-    const size_t smem = sm.wbuf_off + wbufs;
+    const size_t smem = sm.xbuf_off + rot_xbuf_b;
     if (smem > static_cast<size_t>(smem_max)) return PVQ_ERR_UNSUPPORTED;
 
-    auto kern = encode_kernel<N, W, FUSED, YT, BF16, ROT, LS>;
+    auto kern = encode_kernel<N, W, BF16, ROT, LS>;
     int per_sm = 0;
     if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
@@ -772,25 +667,18 @@ static int launch_encode_t(BatchArgs& a, cudaStream_t stream) {
 }
 
 template <int N, int W, bool BF16>
-static int launch_encode_nwb(BatchArgs& a, bool fused, cudaStream_t s) {
-    if (a.amp_mode == 1) {  // least squares: the plain encoder only
-        if (fused || a.rot_block != 0) return PVQ_ERR_UNSUPPORTED;
-        return launch_encode_t<N, W, false, int8_t, BF16, false, true>(a, s);
+static int launch_encode_nwb(BatchArgs& a, cudaStream_t s) {
+    if (a.amp_mode == 1) {  // least squares: not with a rotation
+        if (a.rot_block != 0) return PVQ_ERR_UNSUPPORTED;
+        return launch_encode_t<N, W, BF16, false, true>(a, s);
     }
-    if (a.rot_block != 0) {  // rotating kernels are built for byte-sized slots only (K <= 127)
-        if (!fused) return launch_encode_t<N, W, false, int8_t, BF16, true>(a, s);
-        if (a.K <= 127) return launch_encode_t<N, W, true, int8_t, BF16, true>(a, s);
-        return PVQ_ERR_UNSUPPORTED;
-    }
-    if (!fused) return launch_encode_t<N, W, false, int8_t, BF16, false>(a, s);
-    if (a.K <= 127) return launch_encode_t<N, W, true, int8_t, BF16, false>(a, s);
-    return launch_encode_t<N, W, true, int16_t, BF16, false>(a, s);
+    if (a.rot_block != 0) return launch_encode_t<N, W, BF16, true>(a, s);
+    return launch_encode_t<N, W, BF16, false>(a, s);
 }
 
 template <int N, int W>
-static int launch_encode_nw(BatchArgs& a, int dtype, bool fused, cudaStream_t s) {
-    return dtype == PVQ_DTYPE_BF16 ? launch_encode_nwb<N, W, true>(a, fused, s)
-                                   : launch_encode_nwb<N, W, false>(a, fused, s);
+static int launch_encode_nw(BatchArgs& a, int dtype, cudaStream_t s) {
+    return dtype == PVQ_DTYPE_BF16 ? launch_encode_nwb<N, W, true>(a, s) : launch_encode_nwb<N, W, false>(a, s);
 }
 
 }  // namespace pvq

@@ -2,7 +2,7 @@
 #include "pvq_encode_fast.cuh"
 
 namespace pvq {
-int launch_encode_n64_w5(BatchArgs& a, int dtype, bool fused, cudaStream_t s) {
-    return launch_encode_any<64, 5>(a, dtype, fused, s);
+int launch_encode_n64_w5(BatchArgs& a, int dtype, cudaStream_t s) {
+    return launch_encode_any<64, 5>(a, dtype, s);
 }
 }  // namespace pvq

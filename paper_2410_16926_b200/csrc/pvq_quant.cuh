@@ -1,0 +1,374 @@
+// Direction of a group (Sec. 2.5 / Algorithm 1 in the floor + greedy reading) for the kernels
+// that spread a group over lanes: the L = 1, 2, 4 or 8 neighbouring lanes of a group hold E = 8,
+// 16 or 32 of its N = E * L consecutive values each.
+//
+//   a_i = |x_i| * (K / l1), f_i = floor(a_i), e_i = a_i - f_i, d = K - sum f_i;
+//   the d largest residuals e_i get one more pulse, lowest index first among equals
+//   (why this is the greedy loop's result: quantize_direction in pvq_encode_impl.cuh).
+//
+// Nothing is sorted.  The residuals' leading 7 bits sit in the bytes of E / 4 words, so that one
+// subtract per word compares four of them with a threshold (bit 7 of a byte of
+// 0x80 + residual - threshold is "not below"), and a few such passes bracket the d-th largest.
+// What is left between the two ends of the bracket, at most a few residuals per lane, is
+// ranked on the exact fp32 values, fetched again from where the group came from.  A sorting
+// network over 32 fp32 residuals is 382 min / max instructions at half rate; this is about
+// five passes of 8 subtracts, 8 ands and 8 byte sums.
+//
+// The result is a point packed in bytes: word j holds |y_i| of positions 4j .. 4j+3, last
+// position lowest, which is the order in which the Fischer index needs the pulses behind
+// a position (a multiplication by 0x01010101 is then the running sum).  K > 127 (WIDE): 16-bit
+// halves, word h holds positions 2h (high) and 2h+1 (low).
+#pragma once
+#include <cuda_bf16.h>
+
+#include "pvq_internal.cuh"
+
+namespace pvq {
+
+constexpr uint32_t kH4 = 0x80808080u, kOne4 = 0x01010101u;
+
+// Two fp32 in a register pair: one instruction for two roundings (same results as two scalar
+// operations; what it saves is issue slots).
+struct f32x2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2_rd(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+// A lane's E values as they sit in memory: E/2 words of two bf16, or E words.
+template <int E, bool BF16>
+constexpr int kRawWords = BF16 ? E / 2 : E;
+
+template <int E, bool BF16>
+__device__ __forceinline__ void load_chunk(const void* base, size_t elem_off, uint32_t (&r)[kRawWords<E, BF16>]) {
+    const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint8_t*>(base) + elem_off * (BF16 ? 2 : 4));
+#pragma unroll
+    for (int v = 0; v < kRawWords<E, BF16> / 4; ++v) {
+        const uint4 q = __ldg(p + v);
+        r[4 * v] = q.x, r[4 * v + 1] = q.y, r[4 * v + 2] = q.z, r[4 * v + 3] = q.w;
+    }
+}
+
+template <int E, bool BF16>
+__device__ __forceinline__ float chunk_abs(const uint32_t (&raw)[kRawWords<E, BF16>], int i) {
+    if constexpr (BF16)
+        return __uint_as_float((i & 1) ? (raw[i / 2] & 0x7fff0000u) : ((raw[i / 2] & 0x7fffu) << 16));
+    else
+        return fabsf(__uint_as_float(raw[i]));
+}
+
+// |x_i| one at a time, from where the lane's values came from (global memory)
+template <bool BF16>
+struct FetchGlobal {
+    const void* p;  // the lane's first value
+    __device__ __forceinline__ float operator()(int i) const {
+        if constexpr (BF16)
+            return __uint_as_float(static_cast<uint32_t>(__ldg(static_cast<const unsigned short*>(p) + i) & 0x7fffu) << 16);
+        else
+            return fabsf(__ldg(static_cast<const float*>(p) + i));
+    }
+};
+
+// all lanes of a group get the sum over its lanes (contiguous halves: the balanced tree's order)
+template <int L>
+__device__ __forceinline__ float group_add(float v) {
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+template <int L>
+__device__ __forceinline__ int group_add(int v) {
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// The group's norms by the balanced tree over contiguous halves, and the lane's |x_i|.
+// Values i and i + E/2 share a register pair: the halves of the tree only meet in its last
+// addition.
+template <int E, int L, bool BF16>
+__device__ __forceinline__ void group_norms(const uint32_t (&raw)[kRawWords<E, BF16>], float (&ax)[E], float& l1, float& ss) {
+    constexpr int H = E / 2, Q = E / 4;
+#pragma unroll
+    for (int i = 0; i < E; ++i) ax[i] = chunk_abs<E, BF16>(raw, i);
+    f32x2 s[Q], q[Q];
+#pragma unroll
+    for (int w = 0; w < Q; ++w) {
+        const f32x2 a = pack2(ax[2 * w], ax[2 * w + H]), b = pack2(ax[2 * w + 1], ax[2 * w + 1 + H]);
+        s[w] = add2(a, b);
+        q[w] = add2(mul2(a, a), mul2(b, b));
+    }
+#pragma unroll
+    for (int st = 1; st < Q; st <<= 1) {
+#pragma unroll
+        for (int w = 0; w < Q; w += 2 * st) {
+            s[w] = add2(s[w], s[w + st]);
+            q[w] = add2(q[w], q[w + st]);
+        }
+    }
+    float lo, hi;
+    unpack2(s[0], lo, hi);
+    l1 = group_add<L>(__fadd_rn(lo, hi));
+    unpack2(q[0], lo, hi);
+    ss = group_add<L>(__fadd_rn(lo, hi));
+}
+
+// prmt with the selectors' top bits in use (the byte's sign, eight times); __byte_perm ignores them
+__device__ __forceinline__ uint32_t perm_sign(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+
+// 0xff in the bytes whose value has its sign bit set, in the packed point's order
+template <int E, bool BF16>
+__device__ __forceinline__ uint32_t chunk_signs4(const uint32_t (&raw)[kRawWords<E, BF16>], int j) {
+    if constexpr (BF16)
+        return perm_sign(raw[2 * j + 1], raw[2 * j], 0xDF9B);
+    else
+        return __byte_perm(perm_sign(raw[4 * j + 3], raw[4 * j + 2], 0x00FB), perm_sign(raw[4 * j + 1], raw[4 * j], 0x00FB), 0x5410);
+}
+
+// A lane's share of the point.
+template <int E, bool WIDE>
+struct LanePoint {
+    static constexpr int J = E / 4;
+    static constexpr int FW = WIDE ? E / 2 : E / 4;
+    uint32_t y[FW];  // |y_i|, packed as said at the top
+    bool has_dir;    // false: the group's point is (K, 0, ..., 0), its first coordinate positive
+};
+
+// bit of the pulse mask that belongs to position i of a lane, and the other way round: words
+// of compare results are folded into one another a bit apart
+template <int E>
+__device__ __forceinline__ int mask_bit_position(int bit) {
+    return 4 * ((bit & 7) - (8 - E / 4)) + 3 - (bit >> 3);
+}
+
+// Bit 8b + 8-J + j: residual of byte b of word j is not below the threshold.
+template <int J>
+__device__ __forceinline__ uint32_t not_below_mask(const uint32_t (&x)[J], uint32_t t4) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int j = 0; j < J; ++j) m = (m >> 1) | ((x[j] - t4) & kH4);
+    return m;
+}
+
+template <int J>
+__device__ __forceinline__ int not_below_count(const uint32_t (&x)[J], uint32_t t4) {
+    unsigned c = 0u;
+#pragma unroll
+    for (int j = 0; j < J; ++j) c = __dp4a((x[j] - t4) & kH4, kOne4, c);
+    return static_cast<int>(c >> 7);
+}
+
+// The residuals of the candidates (bits of `cand`), exactly, and which of the group's candidates
+// are the r largest, lowest index first among equals.  Returns the chosen bits.  Called by
+// all lanes of a warp; a group with nothing to choose comes with cand = 0.
+//   Usual: no lane has more than C candidates; every candidate counts the better ones.
+//   Otherwise (many equal or nearly equal residuals): one value class after the other, from the
+//   largest down, until r are chosen.
+template <int E, int L, class Fetch>
+__device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, float gsc, const Fetch& fetch) {
+    constexpr int C = L == 1 ? 4 : 2;
+    constexpr float magic = 8388608.0f;  // 2^23
+    auto residual = [&](int i) {
+        const float a = __fmul_rn(fetch(i), gsc);
+        return __fsub_rn(a, __fsub_rn(__fadd_rd(a, magic), magic));
+    };
+    const int sub = static_cast<int>(threadIdx.x) & (L - 1);
+    uint32_t chosen = 0u;
+    if (__all_sync(0xffffffffu, __popc(cand) <= C)) {
+        float e[C];
+        int pos[C];
+        uint32_t bit[C];
+        uint32_t left = cand;
+#pragma unroll
+        for (int s = 0; s < C; ++s) {
+            const int b = 31 - __clz(static_cast<int>(left));
+            bit[s] = left ? 1u << b : 0u;
+            left ^= bit[s];
+            pos[s] = bit[s] ? mask_bit_position<E>(b) : 0;
+            e[s] = -1.0f;
+            if (bit[s]) e[s] = residual(pos[s]);
+        }
+        int better[C];
+#pragma unroll
+        for (int s = 0; s < C; ++s) {
+            better[s] = 0;
+#pragma unroll
+            for (int u = 0; u < C; ++u)
+                if (u != s) better[s] += (e[u] > e[s] || (e[u] == e[s] && pos[u] < pos[s])) ? 1 : 0;
+        }
+#pragma unroll
+        for (int o = 1; o < L; ++o) {
+            const bool lower = (sub ^ o) < sub;  // that lane holds lower positions: it wins ties
+#pragma unroll
+            for (int u = 0; u < C; ++u) {
+                const float eo = __shfl_xor_sync(0xffffffffu, e[u], o);
+#pragma unroll
+                for (int s = 0; s < C; ++s) better[s] += (eo > e[s] || (lower && eo == e[s])) ? 1 : 0;
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < C; ++s)
+            if (better[s] < r) chosen |= bit[s];
+        return chosen;
+    }
+    for (int round = 0; round < E * L; ++round) {
+        if (!__any_sync(0xffffffffu, cand != 0u && r > 0)) break;
+        float top = -1.0f;  // the group's largest residual left
+        for (uint32_t left = cand; left; left &= left - 1u) top = fmaxf(top, residual(mask_bit_position<E>(__ffs(left) - 1)));
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        uint32_t equal = 0u;
+        for (uint32_t left = cand; left; left &= left - 1u)
+            if (residual(mask_bit_position<E>(__ffs(left) - 1)) == top) equal |= left & (0u - left);
+        const int mine = __popc(equal);
+        int before = 0, all = 0;  // of the class: in lower lanes, in the group
+#pragma unroll
+        for (int o = 0; o < L; ++o) {
+            const int n = L == 1 ? mine : __shfl_xor_sync(0xffffffffu, mine, o);
+            all += n;
+            if ((sub ^ o) < sub) before += n;
+        }
+        if (all <= r) {
+            chosen |= equal;
+        } else {  // the lowest positions of the class
+            int take = min(max(r - before, 0), mine);
+            for (int i = 0; i < E && take > 0; ++i) {
+                const uint32_t b = 1u << (8 * (3 - (i & 3)) + 8 - E / 4 + (i >> 2));
+                if (equal & b) chosen |= b, --take;
+            }
+        }
+        r -= min(all, r);
+        cand &= ~equal;
+        if (r == 0) cand = 0u;
+    }
+    return chosen;
+}
+
+// ax: |x_i| of the lane's values; l1: of the whole group.
+template <int E, int L, bool WIDE, class Fetch>
+__device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, int K, const Fetch& fetch,
+                                               LanePoint<E, WIDE>& pt) {
+    constexpr int N = E * L, J = E / 4, H = E / 2;
+    constexpr int CMAX = L == 1 ? 4 : 2;           // candidates that may be left for the exact comparison
+    const float gsc = __fdiv_rn(static_cast<float>(K), l1);
+    // no direction: l1 zero or not finite, or a scale that overflows
+    bool has_dir = (l1 > 0.0f) && (l1 <= 3.4028234e38f) && (gsc <= 3.4028234e38f);
+    // a + 2^16 rounded down is 2^16 + floor(128 a) / 128: the floor and 7 bits of the residual
+    // sit in the low mantissa bits
+    uint32_t t[E];
+    {
+        const f32x2 g2 = pack2(gsc, gsc), m2 = pack2(65536.0f, 65536.0f);
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            float lo, hi;
+            unpack2(add2_rd(mul2(pack2(ax[i], ax[i + H]), g2), m2), lo, hi);
+            t[i] = __float_as_uint(lo);
+            t[i + H] = __float_as_uint(hi);
+        }
+    }
+    uint32_t x[J];  // 0x80 + leading 7 bits of the residual, a byte each
+    int fsum;
+    if constexpr (!WIDE) {
+        uint32_t sum4 = 0u;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t u = __byte_perm(t[4 * j + 3], t[4 * j + 2], 0x5410), v = __byte_perm(t[4 * j + 1], t[4 * j], 0x5410);
+            x[j] = __byte_perm(u, v, 0x6420) | kH4;
+            pt.y[j] = __byte_perm(u + u, v + v, 0x7531);  // floors, below 128
+            sum4 += pt.y[j];                              // no byte passes K
+        }
+        fsum = static_cast<int>(__dp4a(sum4, kOne4, 0u));
+    } else {
+        uint32_t sum2 = 0u;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t u = __byte_perm(t[4 * j + 3], t[4 * j + 2], 0x0040), v = __byte_perm(t[4 * j + 1], t[4 * j], 0x0040);
+            x[j] = __byte_perm(u, v, 0x5410) | kH4;
+            pt.y[2 * j] = __byte_perm(t[4 * j + 1] << 1, t[4 * j] << 1, 0x6521);
+            pt.y[2 * j + 1] = __byte_perm(t[4 * j + 3] << 1, t[4 * j + 2] << 1, 0x6521);
+            sum2 += pt.y[2 * j] + pt.y[2 * j + 1];
+        }
+        fsum = static_cast<int>((sum2 & 0xffffu) + (sum2 >> 16));
+    }
+    int d = K - group_add<L>(fsum);
+    // 0 <= d <= N for finite input (sum floor(a_i) <= sum a_i < K + 1); anything else is treated
+    // as "no direction"
+    has_dir = has_dir && d >= 0 && d <= N;
+    if (!has_dir) d = 0;
+
+    // bracket [lo, hi) of thresholds with count(lo) >= d >= count(hi)
+    int lo = d == N ? 0 : 128, hi = lo, clo = d, chi = d;
+    bool open = d > 0 && d < N;
+    if (open) lo = 0, hi = 128, clo = N, chi = 0;
+    int T = 128 - (N > 128 ? d / (N / 128) : d * (128 / (N > 128 ? 128 : N)));  // residuals are close to uniform
+    T = min(max(T, 1), 127);
+    for (int it = 0; it < 12; ++it) {
+        const int c = group_add<L>(not_below_count<J>(x, static_cast<uint32_t>(T) * kOne4));
+        if (open) {
+            if (c >= d) lo = T, clo = c;
+            if (c <= d) hi = T, chi = c;
+            open = clo - chi > CMAX && hi - lo > 1;
+        }
+        if (!__any_sync(0xffffffffu, open)) break;
+        // a step by the density of the residuals and half a residual further, then bisection
+        int next = (lo + hi) >> 1;
+        if (it < 2 && (lo == 0 || hi == 128)) {
+            const int over = 2 * (c - d) + (c > d ? 1 : -1);  // in half residuals, 64 / N steps each
+            next = T + (N <= 64 ? over * (64 / (N <= 64 ? N : 64)) : over / (N / 64));
+        }
+        T = open ? min(max(next, lo + 1), hi - 1) : T;
+    }
+    uint32_t sel = not_below_mask<J>(x, static_cast<uint32_t>(hi) * kOne4);
+    uint32_t cand = not_below_mask<J>(x, static_cast<uint32_t>(lo) * kOne4) & ~sel;
+    if (__any_sync(0xffffffffu, cand != 0u)) sel |= choose_candidates<E, L>(cand, d - chi, gsc, fetch);
+
+    if constexpr (!WIDE) {
+#pragma unroll
+        for (int j = 0; j < J; ++j) pt.y[j] += (sel >> (8 - J + j)) & kOne4;
+    } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t b4 = (sel >> (8 - J + j)) & kOne4;
+            pt.y[2 * j] += __byte_perm(b4, 0u, 0x4342);      // positions 4j+1 (low half), 4j
+            pt.y[2 * j + 1] += __byte_perm(b4, 0u, 0x4140);  // positions 4j+3, 4j+2
+        }
+    }
+    if (!has_dir) {  // (K, 0, ..., 0)
+#pragma unroll
+        for (int w = 0; w < LanePoint<E, WIDE>::FW; ++w) pt.y[w] = 0u;
+        if ((threadIdx.x & (L - 1)) == 0) pt.y[0] = static_cast<uint32_t>(K) << (WIDE ? 16 : 24);
+    }
+    pt.has_dir = has_dir;
+}
+
+}  // namespace pvq
