@@ -472,7 +472,7 @@ int run_batch(const pvq_matrix_desc* descs, int count, int need, int dtype, int 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // codes the shared-memory kernels are built for, by group size
     const int fast_words = c.N == 8 ? 2 : (c.N == 16 ? 3 : (c.N == 32 ? 4 : (c.N == 64 ? 6 : 0)));
-    if (kind == 2) return launch_roundtrip(a.m[0], dtype, c.N, K, scale_bits, rot_block, d_signs, a.debug_status, s);
+    if (kind == 2) return launch_roundtrip(a.m[0], dtype, c.N, K, scale_bits, rot_block, d_signs, a.status, a.debug_status, s);
     if (c.W > fast_words) {  // large groups, wide codes
         return launch_big(a, dtype, c.N, c.W, kind == 1, s);
     }

@@ -275,7 +275,7 @@ int launch_big(const BatchArgs& args, int dtype, int N, int W, bool decode, cuda
 int launch_encode(const BatchArgs& args, int dtype, int N, int W, cudaStream_t stream);  // rotates when args.rot_block != 0
 // encode -> decode of one matrix, rotated first when rot_block != 0 (every group size and code width)
 int launch_roundtrip(const MatrixArgs& m, int dtype, int N, int K, int scale_bits, int rot_block, const float* signs,
-                     uint32_t* debug_status, cudaStream_t stream);
+                     uint32_t* status, uint32_t* debug_status, cudaStream_t stream);
 
 // ---------------------------------------------------------------- device bits
 

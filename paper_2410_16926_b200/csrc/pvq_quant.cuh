@@ -50,16 +50,21 @@ __device__ __forceinline__ f32x2 add2_rd(f32x2 a, f32x2 b) {
     asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     f32x2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return r;
 }
+// A product on its own.  Where an addition follows, the rounding of the product has to stay: the
+// assembler was seen to merge a mul.rn.f32x2 into a following add.rn.f32x2 (a group's energy then
+// came out an ulp off).  mul2_rounded is a multiply-add of a -0 that it cannot see (a kernel
+// argument), which changes no result and leaves nothing to merge.
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2_rounded(f32x2 a, f32x2 b, float minus_zero) { return fma2(a, b, pack2(minus_zero, minus_zero)); }
 
 // A lane's E values as they sit in memory: E/2 words of two bf16, or E words.
 template <int E, bool BF16>
@@ -83,6 +88,14 @@ __device__ __forceinline__ float chunk_abs(const uint32_t (&raw)[kRawWords<E, BF
         return fabsf(__uint_as_float(raw[i]));
 }
 
+// A tile of bf16 values lies in shared memory as it does in global memory, E values (E / 8 pieces of 16
+// bytes) a lane.  For the lanes' 16-byte accesses to hit different banks, lane l starts with
+// piece lane_rotation(l) and goes round.
+template <int E>
+__device__ __forceinline__ int lane_rotation(int lane) {
+    return (lane * (E / 8) >> 3) & (E / 8 - 1);
+}
+
 // |x_i| one at a time, from where the lane's values came from (global memory)
 template <bool BF16>
 struct FetchGlobal {
@@ -93,6 +106,12 @@ struct FetchGlobal {
         else
             return fabsf(__ldg(static_cast<const float*>(p) + i));
     }
+};
+
+// |x_i| of a lane whose values sit in shared memory
+struct FetchShared {
+    const unsigned short* p;
+    __device__ __forceinline__ float operator()(int i) const { return __uint_as_float(static_cast<uint32_t>(p[i] & 0x7fffu) << 16); }
 };
 
 // all lanes of a group get the sum over its lanes (contiguous halves: the balanced tree's order)
@@ -111,9 +130,11 @@ __device__ __forceinline__ int group_add(int v) {
 
 // The group's norms by the balanced tree over contiguous halves, and the lane's |x_i|.
 // Values i and i + E/2 share a register pair: the halves of the tree only meet in its last
-// addition.
+// addition.  A lane may hold its values rotated by a number of runs of 8 (see lane_rotation):
+// all that changes is which quarters belong together when that number is odd.
 template <int E, int L, bool BF16>
-__device__ __forceinline__ void group_norms(const uint32_t (&raw)[kRawWords<E, BF16>], float (&ax)[E], float& l1, float& ss) {
+__device__ __forceinline__ void group_norms(const uint32_t (&raw)[kRawWords<E, BF16>], float (&ax)[E], float& l1, float& ss,
+                                            float minus_zero, int rotation = 0) {
     constexpr int H = E / 2, Q = E / 4;
 #pragma unroll
     for (int i = 0; i < E; ++i) ax[i] = chunk_abs<E, BF16>(raw, i);
@@ -122,10 +143,18 @@ __device__ __forceinline__ void group_norms(const uint32_t (&raw)[kRawWords<E, B
     for (int w = 0; w < Q; ++w) {
         const f32x2 a = pack2(ax[2 * w], ax[2 * w + H]), b = pack2(ax[2 * w + 1], ax[2 * w + 1 + H]);
         s[w] = add2(a, b);
-        q[w] = add2(mul2(a, a), mul2(b, b));
+        // (squares of bf16 are exact)
+        q[w] = BF16 ? add2(mul2(a, a), mul2(b, b)) : add2(mul2_rounded(a, a, minus_zero), mul2_rounded(b, b, minus_zero));
     }
 #pragma unroll
     for (int st = 1; st < Q; st <<= 1) {
+        if (E == 32 && 2 * st == Q) {  // quarters 0 | 2 in s[0], 1 | 3 in s[st]
+            float a, b;
+            unpack2(s[st], a, b);
+            s[st] = (rotation & 1) ? pack2(b, a) : pack2(a, b);
+            unpack2(q[st], a, b);
+            q[st] = (rotation & 1) ? pack2(b, a) : pack2(a, b);
+        }
 #pragma unroll
         for (int w = 0; w < Q; w += 2 * st) {
             s[w] = add2(s[w], s[w + st]);
@@ -194,8 +223,9 @@ __device__ __forceinline__ int not_below_count(const uint32_t (&x)[J], uint32_t 
 //   Usual: no lane has more than C candidates; every candidate counts the better ones.
 //   Otherwise (many equal or nearly equal residuals): one value class after the other, from the
 //   largest down, until r are chosen.
+// rotation: position i of the lane is held as position i - 8 * rotation (modulo E).
 template <int E, int L, class Fetch>
-__device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, float gsc, const Fetch& fetch) {
+__device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, float gsc, const Fetch& fetch, int rotation) {
     constexpr int C = L == 1 ? 4 : 2;
     constexpr float magic = 8388608.0f;  // 2^23
     auto residual = [&](int i) {
@@ -206,25 +236,33 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
     uint32_t chosen = 0u;
     if (__all_sync(0xffffffffu, __popc(cand) <= C)) {
         float e[C];
-        int pos[C];
+        int pos[C], better[C];
         uint32_t bit[C];
         uint32_t left = cand;
 #pragma unroll
         for (int s = 0; s < C; ++s) {
-            const int b = 31 - __clz(static_cast<int>(left));
-            bit[s] = left ? 1u << b : 0u;
+            const int b = 31 - __clz(static_cast<int>(left));  // -1: no candidate left
+            bit[s] = left & (1u << (b & 31));
             left ^= bit[s];
-            pos[s] = bit[s] ? mask_bit_position<E>(b) : 0;
-            e[s] = -1.0f;
-            if (bit[s]) e[s] = residual(pos[s]);
+            pos[s] = bit[s] ? (mask_bit_position<E>(b) + 8 * rotation) & (E - 1) : 0;
         }
-        int better[C];
+#pragma unroll
+        for (int s = 0; s < C; ++s) e[s] = fetch(pos[s]);
 #pragma unroll
         for (int s = 0; s < C; ++s) {
+            const float a = __fmul_rn(e[s], gsc);
+            e[s] = __fsub_rn(a, __fsub_rn(__fadd_rd(a, magic), magic));
+            if (!bit[s]) e[s] = -1.0f;
             better[s] = 0;
+        }
 #pragma unroll
-            for (int u = 0; u < C; ++u)
-                if (u != s) better[s] += (e[u] > e[s] || (e[u] == e[s] && pos[u] < pos[s])) ? 1 : 0;
+        for (int s = 0; s < C; ++s) {
+#pragma unroll
+            for (int u = s + 1; u < C; ++u) {
+                const bool second = e[u] > e[s] || (e[u] == e[s] && pos[u] < pos[s]);
+                better[s] += second ? 1 : 0;
+                better[u] += second ? 0 : 1;
+            }
         }
 #pragma unroll
         for (int o = 1; o < L; ++o) {
@@ -244,12 +282,12 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
     for (int round = 0; round < E * L; ++round) {
         if (!__any_sync(0xffffffffu, cand != 0u && r > 0)) break;
         float top = -1.0f;  // the group's largest residual left
-        for (uint32_t left = cand; left; left &= left - 1u) top = fmaxf(top, residual(mask_bit_position<E>(__ffs(left) - 1)));
+        for (uint32_t left = cand; left; left &= left - 1u) top = fmaxf(top, residual((mask_bit_position<E>(__ffs(left) - 1) + 8 * rotation) & (E - 1)));
 #pragma unroll
         for (int o = 1; o < L; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
         uint32_t equal = 0u;
         for (uint32_t left = cand; left; left &= left - 1u)
-            if (residual(mask_bit_position<E>(__ffs(left) - 1)) == top) equal |= left & (0u - left);
+            if (residual((mask_bit_position<E>(__ffs(left) - 1) + 8 * rotation) & (E - 1)) == top) equal |= left & (0u - left);
         const int mine = __popc(equal);
         int before = 0, all = 0;  // of the class: in lower lanes, in the group
 #pragma unroll
@@ -263,7 +301,8 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
         } else {  // the lowest positions of the class
             int take = min(max(r - before, 0), mine);
             for (int i = 0; i < E && take > 0; ++i) {
-                const uint32_t b = 1u << (8 * (3 - (i & 3)) + 8 - E / 4 + (i >> 2));
+                const int held = (i - 8 * rotation) & (E - 1);
+                const uint32_t b = 1u << (8 * (3 - (held & 3)) + 8 - E / 4 + (held >> 2));
                 if (equal & b) chosen |= b, --take;
             }
         }
@@ -277,7 +316,7 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
 // ax: |x_i| of the lane's values; l1: of the whole group.
 template <int E, int L, bool WIDE, class Fetch>
 __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, int K, const Fetch& fetch,
-                                               LanePoint<E, WIDE>& pt) {
+                                               LanePoint<E, WIDE>& pt, float minus_zero, int rotation = 0) {
     constexpr int N = E * L, J = E / 4, H = E / 2;
     constexpr int CMAX = L == 1 ? 4 : 2;           // candidates that may be left for the exact comparison
     const float gsc = __fdiv_rn(static_cast<float>(K), l1);
@@ -291,7 +330,7 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
 #pragma unroll
         for (int i = 0; i < H; ++i) {
             float lo, hi;
-            unpack2(add2_rd(mul2(pack2(ax[i], ax[i + H]), g2), m2), lo, hi);
+            unpack2(add2_rd(mul2_rounded(pack2(ax[i], ax[i + H]), g2, minus_zero), m2), lo, hi);
             t[i] = __float_as_uint(lo);
             t[i + H] = __float_as_uint(hi);
         }
@@ -326,31 +365,32 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
     has_dir = has_dir && d >= 0 && d <= N;
     if (!has_dir) d = 0;
 
-    // bracket [lo, hi) of thresholds with count(lo) >= d >= count(hi)
-    int lo = d == N ? 0 : 128, hi = lo, clo = d, chi = d;
-    bool open = d > 0 && d < N;
-    if (open) lo = 0, hi = 128, clo = N, chi = 0;
+    // Bracket [lo, hi) of thresholds with count(lo) >= d >= count(hi), kept as count * 256 +
+    // threshold: the difference of the two ends then says in one comparison whether few enough
+    // residuals are left between them.  A group that is done goes on halving: its bracket stays
+    // one.  (d = 0 and d = N start and stay with both ends at the threshold that selects none / all.)
+    int lo = N << 8, hi = 128;
+    if (d == 0) lo = 128;
+    if (d == N) hi = lo;
     int T = 128 - (N > 128 ? d / (N / 128) : d * (128 / (N > 128 ? 128 : N)));  // residuals are close to uniform
-    T = min(max(T, 1), 127);
     for (int it = 0; it < 12; ++it) {
         const int c = group_add<L>(not_below_count<J>(x, static_cast<uint32_t>(T) * kOne4));
-        if (open) {
-            if (c >= d) lo = T, clo = c;
-            if (c <= d) hi = T, chi = c;
-            open = clo - chi > CMAX && hi - lo > 1;
+        const int at = (c << 8) + T;
+        if (c >= d) lo = at;
+        if (c <= d) hi = at;
+        const int lo_t = lo & 255, hi_t = hi & 255;
+        if (it > 0 && !__any_sync(0xffffffffu, lo - hi > (CMAX << 8) && hi_t - lo_t > 1)) break;
+        T = (lo_t + hi_t) >> 1;
+        if (it < 2 && (lo_t == 0 || hi_t == 128)) {
+            // one end not met yet: a step by the density of the residuals and half a residual further
+            const int over = 2 * (c - d) + (c > d ? 1 : -1);  // in half residuals, 64 / N thresholds each
+            const int step = N <= 64 ? over * (64 / (N <= 64 ? N : 64)) : over / (N / 64);
+            T = min(max((at & 255) + step, lo_t), hi_t);
         }
-        if (!__any_sync(0xffffffffu, open)) break;
-        // a step by the density of the residuals and half a residual further, then bisection
-        int next = (lo + hi) >> 1;
-        if (it < 2 && (lo == 0 || hi == 128)) {
-            const int over = 2 * (c - d) + (c > d ? 1 : -1);  // in half residuals, 64 / N steps each
-            next = T + (N <= 64 ? over * (64 / (N <= 64 ? N : 64)) : over / (N / 64));
-        }
-        T = open ? min(max(next, lo + 1), hi - 1) : T;
     }
-    uint32_t sel = not_below_mask<J>(x, static_cast<uint32_t>(hi) * kOne4);
-    uint32_t cand = not_below_mask<J>(x, static_cast<uint32_t>(lo) * kOne4) & ~sel;
-    if (__any_sync(0xffffffffu, cand != 0u)) sel |= choose_candidates<E, L>(cand, d - chi, gsc, fetch);
+    uint32_t sel = not_below_mask<J>(x, static_cast<uint32_t>(hi & 255) * kOne4);
+    uint32_t cand = not_below_mask<J>(x, static_cast<uint32_t>(lo & 255) * kOne4) & ~sel;
+    if (__any_sync(0xffffffffu, cand != 0u)) sel |= choose_candidates<E, L>(cand, d - (hi >> 8), gsc, fetch, rotation);
 
     if constexpr (!WIDE) {
 #pragma unroll
@@ -363,10 +403,13 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
             pt.y[2 * j + 1] += __byte_perm(b4, 0u, 0x4140);  // positions 4j+3, 4j+2
         }
     }
-    if (!has_dir) {  // (K, 0, ..., 0)
+    if (__any_sync(0xffffffffu, !has_dir)) {
+        if (!has_dir) {  // (K, 0, ..., 0)
+            const int first = (threadIdx.x & (L - 1)) == 0 ? (-8 * rotation) & (E - 1) : -1;  // where position 0 is held
 #pragma unroll
-        for (int w = 0; w < LanePoint<E, WIDE>::FW; ++w) pt.y[w] = 0u;
-        if ((threadIdx.x & (L - 1)) == 0) pt.y[0] = static_cast<uint32_t>(K) << (WIDE ? 16 : 24);
+            for (int w = 0; w < LanePoint<E, WIDE>::FW; ++w)
+                pt.y[w] = (WIDE ? 2 * w : 4 * w) == first ? static_cast<uint32_t>(K) << (WIDE ? 16 : 24) : 0u;
+        }
     }
     pt.has_dir = has_dir;
 }

@@ -30,7 +30,8 @@ __device__ __forceinline__ void pack_signs(uint32_t* s_signs, const float* signs
 // c: the lane's index in its row.  xbuf: E * blockDim.x floats, used when a block spans more than a warp,
 // and for the copy of the rotated values that is left there ([i][thread]).
 template <int E>
-__device__ __forceinline__ void rotate_lanes(float (&x)[E], const uint32_t* s_signs, int block, float scale, int c, float* xbuf) {
+__device__ __forceinline__ void rotate_lanes(float (&x)[E], const uint32_t* s_signs, int block, float scale, int c, float* xbuf,
+                                             float minus_zero) {
     constexpr int H = E / 2;
     const int tid = threadIdx.x, T = blockDim.x, T0 = block / E;
     const uint32_t sb = s_signs[c & (T0 - 1)];
@@ -90,7 +91,7 @@ __device__ __forceinline__ void rotate_lanes(float (&x)[E], const uint32_t* s_si
     const f32x2 k2 = pack2(scale, scale);
 #pragma unroll
     for (int i = 0; i < H; ++i) {
-        unpack2(mul2(v[i], k2), x[i], x[i + H]);
+        unpack2(mul2_rounded(v[i], k2, minus_zero), x[i], x[i + H]);
         xbuf[i * T + tid] = x[i];
         xbuf[(i + H) * T + tid] = x[i + H];
     }

@@ -7,18 +7,16 @@
 // quantile level, or binary16), so the kernel quantises both and scales the point; the index
 // and its inverse cancel.  No count table is read.
 //
-// A group lies on L = N / 32 neighbouring lanes (pvq_quant.cuh), so every size loads 64 bytes of bf16 a
-// lane and the work per lane is the same from group size 32 up.  A thread block takes whole
-// rows, or one row in chunks when it is longer than the block (then the energies are summed in a
-// pass of their own, since every group's amplitude needs its row's).
-// What bounds it: issue slots and the integer pipe (about 40 instructions a value-quad; see
-// profiles/), not the 4 bytes a value moves.
+// A group lies on L = N / 32 neighbouring lanes (pvq_quant.cuh): the work and the bytes per lane are the
+// same from group size 32 up.  What bounds it: issue slots and the half-rate integer pipe (about
+// 1300 warp instructions per 1024 values), not the 4 bytes a value moves.
 #include <algorithm>
 
 #include <cuda_fp16.h>
 
 #include "pvq_rotate.cuh"
 #include "pvq_rows.cuh"
+#include "pvq_stage.cuh"
 
 namespace pvq {
 
@@ -35,48 +33,41 @@ struct RoundArgs {
     long long rows, cols, ld, ld_out;
     int G, gp;        // groups per row, and that rounded up to a power of two
     int C;            // lanes per row
-    int rpt, chunks;  // rows per block; pieces a row longer than the block is taken in
+    int rpt, chunks;  // rows per tile; pieces a row longer than the block is taken in
+    unsigned tiles;
     int K, b;
     int rot_block;
-    uint32_t ss_off, levels_off, signs_off, xbuf_off;  // in shared memory, behind the bin edges
+    float minus_zero;  // -0 (see mul2_rounded)
+    uint32_t levels_off, ss_off, signs_off, xbuf_off;  // in shared memory, behind the bin edges
+    uint32_t ring_off, tile_bytes;                     // three buffers for input and output tiles
+    uint32_t* status;
     uint32_t* debug_status;
 };
 
-// One lane's values of the point, scaled and rounded to bf16.
-template <int E, bool BF16, bool WIDE>
-__device__ __forceinline__ void emit_lane(const LanePoint<E, WIDE>& pt, const uint32_t (&raw)[kRawWords<E, BF16>], float sc,
-                                          __nv_bfloat16* dst) {
-    const f32x2 sc2 = pack2(sc, sc);
+// Four values of the point (word j of its packing, or two words when WIDE), scaled and rounded to
+// bf16.  neg: 0xff in the bytes of negative values.
+template <int E, bool WIDE>
+__device__ __forceinline__ uint2 scaled_values(const LanePoint<E, WIDE>& pt, int j, uint32_t neg, f32x2 sc2) {
     const f32x2 off = WIDE ? pack2(-8421376.0f, -8421376.0f) : pack2(-8388736.0f, -8388736.0f);  // -(2^23 + the bias)
-    uint32_t o[E / 2];
+    float f[4];
+    if constexpr (!WIDE) {
+        // 128 + y_i in a byte; as the low mantissa bits of 2^23 it becomes a float by one subtraction
+        const uint32_t biased = ((kH4 + pt.y[j]) & ~neg) | ((kH4 - pt.y[j]) & neg);
 #pragma unroll
-    for (int j = 0; j < E / 4; ++j) {
-        const uint32_t neg = pt.has_dir ? chunk_signs4<E, BF16>(raw, j) : 0u;
-        float f[4];
-        if constexpr (!WIDE) {
-            // 128 + y_i in a byte; as the low mantissa bits of 2^23 it becomes a float by one subtraction
-            const uint32_t biased = ((kH4 + pt.y[j]) & ~neg) | ((kH4 - pt.y[j]) & neg);
+        for (int e = 0; e < 4; ++e) f[e] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540u + 3 - e));
+    } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) f[e] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540u + 3 - e));
-        } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {  // positions 4j + 2h (high half), 4j + 2h + 1
-                const uint32_t y = pt.y[2 * j + h], n2 = __byte_perm(neg, 0u, h == 0 ? 0x3322 : 0x1100);
-                const uint32_t biased = ((0x80008000u + y) & ~n2) | ((0x80008000u - y) & n2);
-                f[2 * h] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7532u));
-                f[2 * h + 1] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7510u));
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float lo, hi;
-            unpack2(mul2(add2(pack2(f[2 * h], f[2 * h + 1]), off), sc2), lo, hi);
-            o[2 * j + h] = pack_bf16x2(lo, hi);
+        for (int h = 0; h < 2; ++h) {  // positions 4j + 2h (high half), 4j + 2h + 1
+            const uint32_t y = pt.y[2 * j + h], n2 = __byte_perm(neg, 0u, h == 0 ? 0x3322 : 0x1100);
+            const uint32_t biased = ((0x80008000u + y) & ~n2) | ((0x80008000u - y) & n2);
+            f[2 * h] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7532u));
+            f[2 * h + 1] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7510u));
         }
     }
-#pragma unroll
-    for (int q = 0; q < E / 8; ++q)
-        reinterpret_cast<uint4*>(dst)[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+    float a, b, c, d;
+    unpack2(mul2(add2(pack2(f[0], f[1]), off), sc2), a, b);
+    unpack2(mul2(add2(pack2(f[2], f[3]), off), sc2), c, d);
+    return make_uint2(pack_bf16x2(a, b), pack_bf16x2(c, d));
 }
 
 template <int E, bool WIDE>
@@ -95,9 +86,189 @@ __device__ __forceinline__ int lane_squares(const LanePoint<E, WIDE>& pt) {
     return static_cast<int>(s);
 }
 
+// The group's dequantised amplitude.
+__device__ __forceinline__ float amplitude(float ss, float ss_row, int b, const float* s_edges, const float* s_levels) {
+    if (b == 16) return __half2float(__float2half_rn(__fsqrt_rn(ss)));  // the amplitude as binary16
+    // Step 5: q = floor(CDF(u) 2^b) as the number of bin edges <= u, then the bin's level
+    const float u = ss_row > 0.0f ? __fdiv_rn(ss, ss_row) : 0.0f;
+    int q = 0;
+    for (int step = 1 << (b - 1); step >= 1; step >>= 1)
+        if (s_edges[q + step - 1] <= u) q += step;
+    return __fmul_rn(__fsqrt_rn(ss_row), s_levels[q]);
+}
+
+// For bf16 input in rows of up to 512 lanes.  A block stays and takes tile after tile of whole rows.
+// Input tiles arrive in shared memory by bulk copy, a tile ahead; the results are written over
+// the input in place and leave by bulk copy: no thread waits for global memory, and the copies
+// are whole lines whatever the lanes' access pattern (64 bytes a lane, 16 at a time).  Three
+// buffers: one worked on, one arriving, one leaving.  One block-wide barrier per tile.
+template <int E, int L, bool WIDE, bool ROT>
+__global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __grid_constant__ RoundArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t full[3];
+    constexpr int P = E / 8;  // 16-byte pieces a lane
+    float* s_edges = reinterpret_cast<float*>(smem);
+    float* s_levels = reinterpret_cast<float*>(smem + a.levels_off);
+    uint32_t* s_signs = reinterpret_cast<uint32_t*>(smem + a.signs_off);
+    float* s_xbuf = reinterpret_cast<float*>(smem + a.xbuf_off);
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+    const int b = a.b;
+    const uint32_t row_bytes = static_cast<uint32_t>(a.cols) * 2u;
+    auto tile_rows = [&](unsigned tile) {
+        return static_cast<int>(min(static_cast<long long>(a.rpt), a.rows - static_cast<long long>(tile) * a.rpt));
+    };
+    auto request = [&](unsigned tile, int buf) {  // thread 0
+        const int nr = tile_rows(tile);
+        const BulkStage st{shared_addr(full + buf)};
+        bulk_stage_expect(st, nr * row_bytes);
+        uint8_t* dst = smem + a.ring_off + buf * a.tile_bytes;
+        const uint8_t* src = static_cast<const uint8_t*>(a.x) + static_cast<size_t>(tile) * a.rpt * a.ld * 2;
+        if (a.ld == a.cols)
+            bulk_stage_copy(st, dst, src, nr * row_bytes);
+        else
+            for (int r = 0; r < nr; ++r) bulk_stage_copy(st, dst + r * row_bytes, src + static_cast<size_t>(r) * a.ld * 2, row_bytes);
+    };
+    auto deliver = [&](unsigned tile, int buf) {  // thread 0
+        const int nr = tile_rows(tile);
+        const uint8_t* src = smem + a.ring_off + buf * a.tile_bytes;
+        uint8_t* dst = static_cast<uint8_t*>(a.out) + static_cast<size_t>(tile) * a.rpt * a.ld_out * 2;
+        if (a.ld_out == a.cols)
+            bulk_store(dst, src, nr * row_bytes);
+        else
+            for (int r = 0; r < nr; ++r) bulk_store(dst + static_cast<size_t>(r) * a.ld_out * 2, src + r * row_bytes, row_bytes);
+        bulk_store_commit();
+    };
+
+    unsigned tile = blockIdx.x;
+    if (tid == 0) {
+        for (int i = 0; i < 3; ++i) mbarrier_init_one(full + i);
+        mbarrier_init_fence();
+        request(tile, 0);
+    }
+    float rot_scale = 1.0f;
+    if constexpr (ROT) {
+        pack_signs<E>(s_signs, a.signs, a.rot_block);
+        rot_scale = static_cast<float>(1.0 / sqrt(static_cast<double>(a.rot_block)));
+    }
+    const int nlevels = b <= 8 ? 1 << b : 0;  // 16 bits: the amplitude itself, no codebook
+    for (int i = tid; i < nlevels; i += T) {
+        if (i + 1 < nlevels) s_edges[i] = a.edges[i];
+        s_levels[i] = a.levels[i];
+    }
+#ifdef PVQ_DEBUG
+    debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
+#endif
+    __syncthreads();  // barriers, codebook, signs
+
+    const int rl = tid / a.C, c = tid - rl * a.C;
+    const int rot8 = ROT ? 0 : lane_rotation<E>(lane);
+    // a row inside a warp: its energy is a sum over lanes, no shared memory
+    const bool in_warp = a.C <= 32 && (a.C & (a.C - 1)) == 0;
+    const uint32_t lane_off = a.ring_off + static_cast<uint32_t>(tid) * (E * 2);  // rows of a tile follow one another
+    int buf = 0, parity = 0;
+    for (int i = 0;; ++i) {
+        uint8_t* mine = smem + lane_off + buf * a.tile_bytes;
+        const bool active = rl < a.rpt && static_cast<long long>(tile) * a.rpt + rl < a.rows;
+        float* s_ss = reinterpret_cast<float*>(smem + a.ss_off) + (i & 1) * a.rpt * a.gp;
+        if (!mbarrier_wait(shared_addr(full + buf), parity)) {  // the copy never arrived: report and leave rather than spin
+            if (a.status) atomicOr(a.status, PVQ_STATUS_STAGING_TIMEOUT);
+            return;
+        }
+        float ss;
+        uint32_t neg[E / 4];
+        LanePoint<E, WIDE> pt;
+        {
+            float ax[E], l1;
+            uint32_t raw[E / 2];
+#pragma unroll
+            for (int v = 0; v < P; ++v) {
+                uint4 q = make_uint4(0u, 0u, 0u, 0u);
+                if (active) q = reinterpret_cast<const uint4*>(mine)[(v + rot8) & (P - 1)];
+                raw[4 * v] = q.x, raw[4 * v + 1] = q.y, raw[4 * v + 2] = q.z, raw[4 * v + 3] = q.w;
+            }
+            if constexpr (ROT) {
+                float x[E];
+                uint32_t w[E];
+#pragma unroll
+                for (int k = 0; k < E; ++k) x[k] = __uint_as_float((k & 1) ? (raw[k / 2] & 0xffff0000u) : (raw[k / 2] << 16));
+                rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf, a.minus_zero);
+#pragma unroll
+                for (int k = 0; k < E; ++k) w[k] = __float_as_uint(x[k]);
+#pragma unroll
+                for (int j = 0; j < E / 4; ++j) neg[j] = chunk_signs4<E, false>(w, j);
+                group_norms<E, L, false>(w, ax, l1, ss, a.minus_zero);
+                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated{s_xbuf + tid, T}, pt, a.minus_zero);
+            } else {
+#pragma unroll
+                for (int j = 0; j < E / 4; ++j) neg[j] = chunk_signs4<E, true>(raw, j);
+                group_norms<E, L, true>(raw, ax, l1, ss, a.minus_zero, rot8);
+                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, a.minus_zero, rot8);
+            }
+        }
+        if (!in_warp) {
+            if (active && (c & (L - 1)) == 0 && PVQ_DEBUG_INDEX(rl * a.gp + c / L, a.rpt * a.gp, PVQ_DEBUG_SHARED_INDEX))
+                s_ss[rl * a.gp + c / L] = ss;
+            if (a.gp != a.G)  // zero padding of the rows' trees
+                for (int j = tid; j < a.rpt * a.gp; j += T)
+                    if ((j & (a.gp - 1)) >= a.G) s_ss[j] = 0.0f;
+        }
+        // energies are in place, and the tile before this one is complete in its buffer
+        bulk_store_fence();
+        __syncthreads();
+        const unsigned next = tile + gridDim.x;
+        const bool have_next = next < a.tiles;
+        const int nbuf = buf == 2 ? 0 : buf + 1;
+        if (tid == 0) {
+            if (i > 0) deliver(tile - gridDim.x, buf == 0 ? 2 : buf - 1);
+            if (have_next) {
+                bulk_store_wait_read<1>();  // what was in the buffer has left it
+                request(next, nbuf);
+            }
+        }
+        float ss_row;
+        if (in_warp) {
+            ss_row = ss;
+            for (int o = L; o < a.C; o <<= 1) ss_row = __fadd_rn(ss_row, __shfl_xor_sync(0xffffffffu, ss_row, o));
+        } else {
+            ss_row = row_energy(s_ss, a.gp, rl, a.rpt, lane);
+        }
+        const float amp = amplitude(ss, ss_row, b, s_edges, s_levels);
+        const int ssy = group_add<L>(lane_squares<E, WIDE>(pt));
+        const float sc = __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(ssy)));
+        const f32x2 sc2 = pack2(sc, sc);
+        if (active) {
+            if (!pt.has_dir) {  // (K, 0, ..., 0), positive
+#pragma unroll
+                for (int j = 0; j < E / 4; ++j) neg[j] = 0u;
+            }
+#pragma unroll
+            for (int v = 0; v < P; ++v) {
+                const uint2 lo = scaled_values<E, WIDE>(pt, 2 * v, neg[2 * v], sc2);
+                const uint2 hi = scaled_values<E, WIDE>(pt, 2 * v + 1, neg[2 * v + 1], sc2);
+                const int piece = (v + rot8) & (P - 1);
+                if (PVQ_DEBUG_INDEX(tid * P + piece, a.tile_bytes / 16, PVQ_DEBUG_SHARED_INDEX))
+                    reinterpret_cast<uint4*>(mine)[piece] = make_uint4(lo.x, lo.y, hi.x, hi.y);
+            }
+        }
+        if (!have_next) break;
+        tile = next;
+        buf = nbuf;
+        if (buf == 0) parity ^= 1;
+    }
+    bulk_store_fence();
+    __syncthreads();
+    if (tid == 0) {
+        deliver(tile, buf);
+        bulk_store_wait_read<0>();
+    }
+}
+
+// For fp32 input and for rows longer than a thread block: one tile of whole rows per block, or one row in
+// chunks (then the energies are summed in a pass of their own, since every group's amplitude needs
+// its row's), loads and stores straight from and to global memory.
 template <int E, int L, bool BF16, bool WIDE, bool ROT>
-__global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __grid_constant__ RoundArgs a) {
-    extern __shared__ __align__(16) uint8_t smem[];
+__global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_rows_kernel(const __grid_constant__ RoundArgs a) {
+    extern __shared__ __align__(128) uint8_t smem[];
     constexpr bool WBF16 = BF16 && !ROT;  // the form the kernel works on: packed bf16, or fp32
     float* s_edges = reinterpret_cast<float*>(smem);
     float* s_levels = reinterpret_cast<float*>(smem + a.levels_off);
@@ -106,7 +277,6 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __gri
     float* s_xbuf = reinterpret_cast<float*>(smem + a.xbuf_off);
     const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
     const int b = a.b;
-    const int nedges = b <= 8 ? (1 << b) - 1 : 0;  // 16 bits: the amplitude itself, no codebook
     float rot_scale = 1.0f;
 #ifdef PVQ_DEBUG
     debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
@@ -115,8 +285,11 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __gri
         pack_signs<E>(s_signs, a.signs, a.rot_block);
         rot_scale = static_cast<float>(1.0 / sqrt(static_cast<double>(a.rot_block)));
     }
-    for (int i = tid; i < nedges; i += T) s_edges[i] = a.edges[i];
-    for (int i = tid; i <= nedges && nedges > 0; i += T) s_levels[i] = a.levels[i];
+    const int nlevels = b <= 8 ? 1 << b : 0;  // 16 bits: the amplitude itself, no codebook
+    for (int i = tid; i < nlevels; i += T) {
+        if (i + 1 < nlevels) s_edges[i] = a.edges[i];
+        s_levels[i] = a.levels[i];
+    }
     if (ROT) __syncthreads();
 
     const int rl = a.chunks == 1 ? tid / a.C : 0;
@@ -126,22 +299,22 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __gri
     // a row inside a warp: its energy is a sum over lanes, no shared memory
     const bool in_warp = a.C <= 32 && (a.C & (a.C - 1)) == 0;
 
+    auto at = [&](int c) { return static_cast<size_t>(row) * a.ld + static_cast<size_t>(c) * E; };  // of a lane's first value
     auto load = [&](int c, bool active, uint32_t (&w)[kRawWords<E, WBF16>]) {
-        const size_t at = static_cast<size_t>(row) * a.ld + static_cast<size_t>(c) * E;
         if constexpr (!ROT) {
 #pragma unroll
             for (int i = 0; i < kRawWords<E, WBF16>; ++i) w[i] = 0u;
-            if (active) load_chunk<E, BF16>(a.x, at, w);
+            if (active) load_chunk<E, BF16>(a.x, at(c), w);
         } else {
             uint32_t r[kRawWords<E, BF16>];
             float x[E];
 #pragma unroll
             for (int i = 0; i < kRawWords<E, BF16>; ++i) r[i] = 0u;
-            if (active) load_chunk<E, BF16>(a.x, at, r);
+            if (active) load_chunk<E, BF16>(a.x, at(c), r);
 #pragma unroll
             for (int i = 0; i < E; ++i)
                 x[i] = BF16 ? __uint_as_float((i & 1) ? (r[i / 2] & 0xffff0000u) : (r[i / 2] << 16)) : __uint_as_float(r[BF16 ? i / 2 : i]);
-            rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf);
+            rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf, a.minus_zero);
 #pragma unroll
             for (int i = 0; i < E; ++i) w[i] = __float_as_uint(x[i]);
         }
@@ -154,7 +327,7 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __gri
             uint32_t raw[kRawWords<E, WBF16>];
             float ax[E], l1, ss;
             load(c, active, raw);
-            group_norms<E, L, WBF16>(raw, ax, l1, ss);
+            group_norms<E, L, WBF16>(raw, ax, l1, ss, a.minus_zero);
             if (active && (c & (L - 1)) == 0) s_ss[c / L] = ss;
         }
         for (int g = a.G + tid; g < a.gp; g += T) s_ss[g] = 0.0f;
@@ -170,14 +343,12 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __gri
         load(c, active, raw);
         {
             float ax[E], l1;
-            group_norms<E, L, WBF16>(raw, ax, l1, ss);
+            group_norms<E, L, WBF16>(raw, ax, l1, ss, a.minus_zero);
             if constexpr (ROT)
-                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated{s_xbuf + tid, T}, pt);
+                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated{s_xbuf + tid, T}, pt, a.minus_zero);
             else
-                quantize_group<E, L, WIDE>(ax, l1, a.K,
-                                           FetchGlobal<BF16>{static_cast<const uint8_t*>(a.x) +
-                                                             (static_cast<size_t>(row) * a.ld + static_cast<size_t>(c) * E) * (BF16 ? 2 : 4)},
-                                           pt);
+                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchGlobal<BF16>{static_cast<const uint8_t*>(a.x) + (active ? at(c) : 0) * (BF16 ? 2 : 4)}, pt,
+                                           a.minus_zero);
         }
         if (in_warp) {
             ss_row = ss;
@@ -194,23 +365,22 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_kernel(const __gri
             }
             ss_row = row_energy(s_ss, a.gp, rl, a.rpt, lane);
         }
-        float amp;
-        if (b == 16) {  // the amplitude as binary16
-            amp = __half2float(__float2half_rn(__fsqrt_rn(ss)));
-        } else {
-            // Step 5: q = floor(CDF(u) 2^b) as the number of bin edges <= u, then the bin's level
-            const float u = ss_row > 0.0f ? __fdiv_rn(ss, ss_row) : 0.0f;
-            int q = 0;
-            for (int step = 1 << (b - 1); step >= 1; step >>= 1)
-                if (s_edges[q + step - 1] <= u) q += step;
-            amp = __fmul_rn(__fsqrt_rn(ss_row), s_levels[q]);
-        }
+        const float amp = amplitude(ss, ss_row, b, s_edges, s_levels);
         const int ssy = group_add<L>(lane_squares<E, WIDE>(pt));
         const float sc = __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(ssy)));
+        const f32x2 sc2 = pack2(sc, sc);
         if (active && PVQ_DEBUG_INDEX(row, a.rows, PVQ_DEBUG_GLOBAL_STORE) &&
-            PVQ_DEBUG_INDEX(static_cast<long long>(c + 1) * E - 1, a.cols, PVQ_DEBUG_GLOBAL_STORE))
-            emit_lane<E, WBF16, WIDE>(pt, raw, sc,
-                                      static_cast<__nv_bfloat16*>(a.out) + static_cast<size_t>(row) * a.ld_out + static_cast<size_t>(c) * E);
+            PVQ_DEBUG_INDEX(static_cast<long long>(c + 1) * E - 1, a.cols, PVQ_DEBUG_GLOBAL_STORE)) {
+            uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.out) + static_cast<size_t>(row) * a.ld_out +
+                                                  static_cast<size_t>(c) * E);
+#pragma unroll
+            for (int q = 0; q < E / 8; ++q) {
+                // a group without direction: (K, 0, ..., 0), positive (the sign of a zero does not matter)
+                const uint2 lo = scaled_values<E, WIDE>(pt, 2 * q, q > 0 || pt.has_dir ? chunk_signs4<E, WBF16>(raw, 2 * q) : 0u, sc2);
+                const uint2 hi = scaled_values<E, WIDE>(pt, 2 * q + 1, chunk_signs4<E, WBF16>(raw, 2 * q + 1), sc2);
+                dst[q] = make_uint4(lo.x, lo.y, hi.x, hi.y);
+            }
+        }
     }
 }
 
@@ -235,12 +405,12 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
         // fewest lanes idle; among equals the largest, or the smallest when the launch would
         // not fill the SMs anyway.
         a.chunks = 1;
+        const int need = (a.C + 31) / 32 * 32;
         long long best = -1;
-        for (int t = std::max(64, (a.C + 31) / 32 * 32); t <= std::max(256, (a.C + 31) / 32 * 32); t += 32) {
+        for (int t = std::max(64, need); t <= std::max(256, need); t += 32) {
             const int rpt = t / a.C;
             const long long tiles = (a.rows + rpt - 1) / rpt, cost = tiles * t;
-            const bool few = tiles < 2 * di.sms;
-            if (best < 0 || cost < best || (cost == best && !few)) {
+            if (best < 0 || cost < best || (cost == best && tiles >= 2 * di.sms)) {
                 best = cost;
                 threads = t;
             }
@@ -249,19 +419,30 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
     }
     const long long tiles = (a.rows + a.rpt - 1) / a.rpt;
     if (tiles > 0x7fffffffLL) return PVQ_ERR_UNSUPPORTED;
+    a.tiles = static_cast<unsigned>(tiles);
     a.levels_off = a.b <= 8 ? 4u << a.b : 0u;
-    a.ss_off = 2u * a.levels_off;
-    a.ss_off = (a.ss_off + 15u) & ~15u;
-    a.signs_off = (a.ss_off + static_cast<uint32_t>(a.rpt * a.gp) * 4u + 15u) & ~15u;
+    a.ss_off = (2u * a.levels_off + 15u) & ~15u;
+    a.signs_off = (a.ss_off + 2u * static_cast<uint32_t>(a.rpt * a.gp) * 4u + 15u) & ~15u;
     a.xbuf_off = a.signs_off + (ROT ? (static_cast<uint32_t>(a.rot_block / E) * 4u + 15u) & ~15u : 0u);
-    const size_t smem = a.xbuf_off + (ROT ? static_cast<size_t>(threads) * E * 4u : 0u);
+    a.ring_off = (a.xbuf_off + (ROT ? static_cast<uint32_t>(threads) * E * 4u : 0u) + 127u) & ~127u;
+    a.tile_bytes = static_cast<uint32_t>(threads) * E * 2u;
+    size_t smem = a.ring_off;
+    const void* kern = reinterpret_cast<const void*>(roundtrip_rows_kernel<E, L, BF16, WIDE, ROT>);
+    bool stays = false;  // the block stays and takes tile after tile
+    if constexpr (BF16) {
+        if (a.chunks == 1 && smem + 3u * a.tile_bytes <= static_cast<size_t>(di.smem_max)) {
+            stays = true;
+            smem += 3u * a.tile_bytes;
+            kern = reinterpret_cast<const void*>(roundtrip_kernel<E, L, WIDE, ROT>);
+        }
+    }
     if (smem > static_cast<size_t>(di.smem_max)) return PVQ_ERR_UNSUPPORTED;
-    auto kern = roundtrip_kernel<E, L, BF16, WIDE, ROT>;
     int per_sm = 0;
-    if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
+    if ((st = prepare_kernel(kern, threads, smem, &per_sm)) != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
-    kern<<<static_cast<unsigned>(tiles), threads, smem, stream>>>(a);
-    const cudaError_t e = cudaGetLastError();
+    const unsigned grid = stays ? std::min(a.tiles, static_cast<unsigned>(di.sms * per_sm)) : a.tiles;
+    void* params[] = {&a};
+    const cudaError_t e = cudaLaunchKernel(kern, dim3(grid), dim3(threads), params, smem, stream);
     return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
 }
 
@@ -279,7 +460,7 @@ int launch_round_n(RoundArgs& a, bool bf16, cudaStream_t s) {
 }  // namespace
 
 int launch_roundtrip(const MatrixArgs& m, int dtype, int N, int K, int scale_bits, int rot_block, const float* signs,
-                     uint32_t* debug_status, cudaStream_t stream) {
+                     uint32_t* status, uint32_t* debug_status, cudaStream_t stream) {
     RoundArgs a;
     a.x = m.x;
     a.out = m.out;
@@ -294,6 +475,8 @@ int launch_roundtrip(const MatrixArgs& m, int dtype, int N, int K, int scale_bit
     a.K = K;
     a.b = scale_bits;
     a.rot_block = rot_block;
+    a.minus_zero = -0.0f;
+    a.status = status;
     a.debug_status = debug_status;
     const bool bf16 = dtype == PVQ_DTYPE_BF16;
     switch (N) {
