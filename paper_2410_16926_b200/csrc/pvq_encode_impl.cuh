@@ -344,7 +344,7 @@ __device__ __forceinline__ TileLoc locate(const BatchArgs& a, unsigned tile) {
 template <int N, int W, bool BF16, bool ROT, bool LS>
 __global__ void __launch_bounds__(512) encode_kernel(const __grid_constant__ BatchArgs a,
                                                       const __grid_constant__ EncodeSmem sm) {
-    extern __shared__ __align__(16) uint8_t smem[];
+    extern __shared__ __align__(128) uint8_t smem[];
     constexpr int TW = W <= 2 ? W : (W <= 4 ? 4 : 6);
     constexpr int EB = TW * 4;
     constexpr int RW = BF16 ? N / 2 : N;      // words of a group as loaded

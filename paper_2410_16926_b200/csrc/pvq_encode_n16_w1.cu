@@ -1,5 +1,6 @@
 // Encode kernels for group size 16, 1-word codes.
-#include "pvq_encode_fast.cuh"
+#include "pvq_encode_impl.cuh"
+#include "pvq_encode_lanes.cuh"
 
 namespace pvq {
 int launch_encode_n16_w1(BatchArgs& a, int dtype, cudaStream_t s) {
