@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "pvq_encode_impl.cuh"
+#include "pvq_encode_lanes.cuh"
 
 namespace pvq {
 
@@ -681,7 +682,7 @@ int launch_big_w(BatchArgs& a, int dtype, bool decode, cudaStream_t s) {
     const bool bf16 = dtype == PVQ_DTYPE_BF16;
     if (a.rot_block != 0)
         return bf16 ? launch_encode_big_t<N, W, EXACT, true, true>(a, s) : launch_encode_big_t<N, W, EXACT, false, true>(a, s);
-    return bf16 ? launch_encode_big_t<N, W, EXACT, true, false>(a, s) : launch_encode_big_t<N, W, EXACT, false, false>(a, s);
+    return launch_encode_lanes_global<N, W>(a, dtype, s);
 }
 
 }  // namespace

@@ -666,19 +666,10 @@ static int launch_encode_t(BatchArgs& a, cudaStream_t stream) {
     return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
 }
 
-template <int N, int W, bool BF16>
-static int launch_encode_nwb(BatchArgs& a, cudaStream_t s) {
-    if (a.amp_mode == 1) {  // least squares: not with a rotation
-        if (a.rot_block != 0) return PVQ_ERR_UNSUPPORTED;
-        return launch_encode_t<N, W, BF16, false, true>(a, s);
-    }
-    if (a.rot_block != 0) return launch_encode_t<N, W, BF16, true>(a, s);
-    return launch_encode_t<N, W, BF16, false>(a, s);
-}
-
 template <int N, int W>
 static int launch_encode_nw(BatchArgs& a, int dtype, cudaStream_t s) {
-    return dtype == PVQ_DTYPE_BF16 ? launch_encode_nwb<N, W, true>(a, s) : launch_encode_nwb<N, W, false>(a, s);
+    if (a.amp_mode == 1) return PVQ_ERR_UNSUPPORTED;  // least squares: not with a rotation
+    return dtype == PVQ_DTYPE_BF16 ? launch_encode_t<N, W, true, true>(a, s) : launch_encode_t<N, W, false, true>(a, s);
 }
 
 }  // namespace pvq

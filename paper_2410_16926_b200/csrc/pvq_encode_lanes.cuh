@@ -13,6 +13,9 @@
 //     else uses, without carries; positions whose M stays below 2^48 have no upper half to read;
 //   - the input arrives in shared memory by asynchronous copies of whole lines, a chunk ahead, each
 //     lane's run padded by 16 bytes so that the lanes' 16-byte reads hit different banks.
+// Larger groups and wider codes (any group size, up to 32 words, any K): the same kernel with a group on up
+// to 8 lanes, the point in 16-bit halves, and Algorithm 2's two terms per position read from the cumulative
+// tables in global memory (L1, L2), only as many words as the position's counts have.
 // One block per SM shares one copy of the tables; within it, teams of threads take whole rows, in chunks
 // of a lane per 32 values, each at its own pace.  A team of one warp needs no barrier and spreads the
 // work per row over most chunks; larger teams make more tiles of few rows (LaneGeom's choice in the launcher).
@@ -27,7 +30,9 @@
 
 namespace pvq {
 
-constexpr int kLaneThreadsMax = 768;
+// threads per block: the wide kernels' accumulators need more registers
+template <int W>
+constexpr int kLaneThreads = W <= 16 ? 768 : 512;
 constexpr int kSplitBit = 48;
 
 struct LaneGeom {
@@ -210,15 +215,96 @@ __device__ __forceinline__ mp<W> lanes_index(const LanePoint<E, false>& pt, cons
     return c;
 }
 
+// Words [0, W) of a table entry of TW words in global memory, no more than `words` of them (the rest zero).
+template <int W>
+__device__ __forceinline__ mp<W> global_entry(const uint32_t* p, int TW, int words) {
+    mp<W> t;
+    if ((TW & 3) == 0) {
+#pragma unroll
+        for (int v = 0; v < (W + 3) / 4; ++v) {
+            uint4 q = make_uint4(0u, 0u, 0u, 0u);
+            if (4 * v < words) q = __ldg(reinterpret_cast<const uint4*>(p) + v);
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (4 * v + u < W) t.w[4 * v + u] = w[u];
+        }
+    } else if ((TW & 1) == 0) {
+#pragma unroll
+        for (int v = 0; v < (W + 1) / 2; ++v) {
+            uint2 q = make_uint2(0u, 0u);
+            if (2 * v < words) q = __ldg(reinterpret_cast<const uint2*>(p) + v);
+            t.w[2 * v] = q.x;
+            if (2 * v + 1 < W) t.w[2 * v + 1] = q.y;
+        }
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) t.w[w] = w < words ? __ldg(p + w) : 0u;
+    }
+    return t;
+}
+
+// The index of the group's point from the cumulative tables (Algorithm 2, App. C.2): with k pulses before a
+// position and k' behind it, U(n,k) - U(n,k') for y < 0, U(n,k) - 2 V(n,k') for y > 0, nothing
+// for y = 0.  s_words: words of the counts at every position.  All lanes of a group get the sum.
+template <int E, int L, int W>
+__device__ __forceinline__ mp<W> lanes_index_global(const LanePoint<E, true>& pt, const uint32_t (&neg)[E / 4], int K, const uint32_t* tab_u,
+                                                    const uint32_t* tab_2v, int TW, const uint8_t* s_words) {
+    const int sub = static_cast<int>(threadIdx.x) & (L - 1);
+    int behind = 0;  // pulses behind the lane's positions
+    if constexpr (L > 1) {
+        uint32_t own2 = 0u;
+#pragma unroll
+        for (int h = 0; h < E / 2; ++h) own2 += pt.y[h];
+        const int own = static_cast<int>((own2 & 0xffffu) + (own2 >> 16));
+#pragma unroll
+        for (int o = 1; o < L; ++o) {
+            const int other = __shfl_xor_sync(kFull, own, o);
+            if ((sub ^ o) > sub) behind += other;
+        }
+    }
+    mp<W> c;
+    mp_zero(c);
+    const uint32_t rowlen = static_cast<uint32_t>(K + 2) * TW;
+#pragma unroll
+    for (int h = E / 2 - 1; h >= 0; --h) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {  // position 2h + 1 (low half), then 2h
+            const int pos = 2 * h + 1 - half;
+            const int y = static_cast<int>(half ? pt.y[h] >> 16 : pt.y[h] & 0xffffu);
+            const bool negative = (neg[pos / 4] >> (8 * (3 - (pos & 3)))) & 1u;
+            if (y != 0) {
+                const int i = sub * E + pos;
+                const int words = s_words[i];
+                const uint32_t row = static_cast<uint32_t>(i) * rowlen;
+                const mp<W> u = global_entry<W>(tab_u + row + static_cast<uint32_t>(behind + y + 1) * TW, TW, words);
+                const mp<W> x = global_entry<W>((negative ? tab_u : tab_2v) + row + static_cast<uint32_t>(behind + 1) * TW, TW, words);
+                mp_add<W>(c, u);
+                mp<W> d;
+                mp_sub_borrow<W>(d, c, x);
+                c = d;
+                behind += y;
+            }
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) {
+        mp<W> other;
+#pragma unroll
+        for (int w = 0; w < W; ++w) other.w[w] = __shfl_xor_sync(kFull, c.w[w], o);
+        mp_add<W>(c, other);
+    }
+    return c;
+}
+
 // Step 4 as least squares: a = (sum |y_i| |x_i|) / sqrt(sum y_i^2), the rounded products summed by
 // the balanced tree.
-template <int E, int L, bool BF16>
-__device__ __forceinline__ float least_squares_amplitude(const LanePoint<E, false>& pt, const uint8_t* mine) {
+template <int E, int L, bool BF16, bool WIDE>
+__device__ __forceinline__ float least_squares_amplitude(const LanePoint<E, WIDE>& pt, const uint8_t* mine) {
     float t[E];
     unsigned sq = 0u;
 #pragma unroll
     for (int j = 0; j < E / 4; ++j) {
-        sq = __dp4a(pt.y[j], pt.y[j], sq);
         float x[4];
         if constexpr (BF16) {
             const uint2 q = reinterpret_cast<const uint2*>(mine)[j];
@@ -229,7 +315,15 @@ __device__ __forceinline__ float least_squares_amplitude(const LanePoint<E, fals
             x[0] = fabsf(q.x), x[1] = fabsf(q.y), x[2] = fabsf(q.z), x[3] = fabsf(q.w);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) t[4 * j + e] = __fmul_rn(static_cast<float>((pt.y[j] >> (8 * (3 - e))) & 0xffu), x[e]);
+        for (int e = 0; e < 4; ++e) {
+            unsigned y;
+            if constexpr (WIDE)
+                y = (e & 1) ? pt.y[2 * j + e / 2] & 0xffffu : pt.y[2 * j + e / 2] >> 16;
+            else
+                y = (pt.y[j] >> (8 * (3 - e))) & 0xffu;
+            sq += y * y;
+            t[4 * j + e] = __fmul_rn(static_cast<float>(y), x[e]);
+        }
     }
     const float dot = group_add<L>(tree_sum<E>(t));
     const int ssy = group_add<L>(static_cast<int>(sq));
@@ -286,15 +380,20 @@ __device__ __forceinline__ void flush_index_words(const MatrixArgs& m, unsigned 
     }
 }
 
+// RE: entries per row of the staged table (codes of exactly W words); 0: the tables stay in global memory,
+// codes of up to W words.
 template <int E, int L, int W, int RE, bool BF16, bool LS>
-__global__ void __launch_bounds__(kLaneThreadsMax, 1) encode_lanes_kernel(const __grid_constant__ BatchArgs a,
+__global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const __grid_constant__ BatchArgs a,
                                                                            const __grid_constant__ LaneGeom g) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_wide_blocks;
+    __shared__ uint8_t s_words[RE == 0 ? E * L : 1];
     constexpr int N = E * L;
+    constexpr bool GLOBAL = RE == 0;
     constexpr int P = E * (BF16 ? 2 : 4) / 16, RUN = kLaneRun<E, BF16>;
     const int K = a.K, b = a.scale_bits;
-    const TableLayout TL = table_layout(N, K, W);
+    const int Wc = GLOBAL ? a.code_words : W;  // words of a code in memory
+    const TableLayout TL = table_layout(N, K, Wc);
     const int T = g.team, team = threadIdx.x / T, tid = threadIdx.x - team * T, lane = threadIdx.x & 31;
     uint8_t* area = smem + g.team_off + team * g.team_bytes;
 
@@ -309,20 +408,34 @@ __global__ void __launch_bounds__(kLaneThreadsMax, 1) encode_lanes_kernel(const 
         uint32_t* s_idx2 = reinterpret_cast<uint32_t*>(area + g.idx_off);
         for (int i = tid; i < 2 * g.idx_words; i += T) s_idx2[i] = 0u;
     }
-    if (W == 2 || W == 3) {
-        if (threadIdx.x == 0) s_wide_blocks = 0;
-        __syncthreads();
-    }
-    stage_lane_table<N, W, RE>(smem, a.table, TL, K, &s_wide_blocks);
-    mp<W> start;
-#pragma unroll
-    for (int w = 0; w < W; ++w) start.w[w] = a.table[TL.start_off / 4 + w];
+    mp<GLOBAL ? 1 : W> start;
+    if constexpr (GLOBAL) {
+        // words of N(n+1,K) = U(n,K), which no term of the position exceeds (N(N,K) may be a power of two
+        // beyond the entry: all words)
+        for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            const uint32_t* u = a.table + TL.enc_off[0] / 4 + (static_cast<size_t>(i) * (K + 2) + K + 1) * TL.top_words;
+            int words = Wc;
+            while (i > 0 && words > 1 && __ldg(u + words - 1) == 0u) --words;
+            s_words[i] = static_cast<uint8_t>(words);
+        }
 #ifdef PVQ_DEBUG
-    debug_begin(shared_addr(smem), shared_addr(smem) + kLaneTableBytes<N, W, RE>, 0u, 0u, 0u, a.debug_status);
+        debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
 #endif
+    } else {
+        if (W == 2 || W == 3) {
+            if (threadIdx.x == 0) s_wide_blocks = 0;
+            __syncthreads();
+        }
+        stage_lane_table<N, W, GLOBAL ? 64 : RE>(smem, a.table, TL, K, &s_wide_blocks);
+#pragma unroll
+        for (int w = 0; w < W; ++w) start.w[GLOBAL ? 0 : w] = a.table[TL.start_off / 4 + w];
+#ifdef PVQ_DEBUG
+        debug_begin(shared_addr(smem), shared_addr(smem) + kLaneTableBytes<N, W, RE>, 0u, 0u, 0u, a.debug_status);
+#endif
+    }
     __syncthreads();  // the tables; from here on the teams go their own way
     if (!works) return;
-    const int wide_blocks = W == 2 || W == 3 ? s_wide_blocks : 0;
+    const int wide_blocks = !GLOBAL && (W == 2 || W == 3) ? s_wide_blocks : 0;
 
     int in_buf = 0, buf = 0;
     int done_mi = -1;  // matrix of the tile before, whose index words are still to be written out
@@ -357,7 +470,7 @@ __global__ void __launch_bounds__(kLaneThreadsMax, 1) encode_lanes_kernel(const 
             const int c = cur.c0 + cur.ch * T;
             const uint8_t* mine = area + in_buf * g.in_bytes + tid * RUN;
             uint32_t neg[E / 4];
-            LanePoint<E, false> pt;
+            LanePoint<E, GLOBAL> pt;
             float ss;
             {
                 // (a lane beyond the values works on whatever is there: any bits are safe)
@@ -372,27 +485,51 @@ __global__ void __launch_bounds__(kLaneThreadsMax, 1) encode_lanes_kernel(const 
                 for (int j = 0; j < E / 4; ++j) neg[j] = chunk_signs4<E, BF16>(raw, j);
                 group_norms<E, L, BF16>(raw, ax, l1, ss, g.minus_zero);
                 if constexpr (BF16)
-                    quantize_group<E, L, false>(ax, l1, K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, g.minus_zero);
+                    quantize_group<E, L, GLOBAL>(ax, l1, K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, g.minus_zero);
                 else
-                    quantize_group<E, L, false>(ax, l1, K, FetchSharedF32{reinterpret_cast<const float*>(mine)}, pt, g.minus_zero);
+                    quantize_group<E, L, GLOBAL>(ax, l1, K, FetchSharedF32{reinterpret_cast<const float*>(mine)}, pt, g.minus_zero);
             }
             const bool leader = row_ok && c < C && (c & (L - 1)) == 0;
             const int slot = cur.rl * gp + c / L;
             if (leader && PVQ_DEBUG_INDEX(slot, g.ss_floats, PVQ_DEBUG_SHARED_INDEX)) s_ss[slot] = ss;
             if constexpr (LS) {
-                const float ls = least_squares_amplitude<E, L, BF16>(pt, mine);
+                const float ls = least_squares_amplitude<E, L, BF16, GLOBAL>(pt, mine);
                 if (leader) s_amp[slot] = ls;
             }
             if (!pt.has_dir) {  // (K, 0, ..., 0), positive
 #pragma unroll
                 for (int j = 0; j < E / 4; ++j) neg[j] = 0u;
             }
-            const mp<W> code = lanes_index<E, L, W, RE>(pt, neg, K, smem, wide_blocks, start);
             const long long group = row * G + c / L;
-            if (leader && PVQ_DEBUG_INDEX(group, m.rows * G, PVQ_DEBUG_GLOBAL_STORE)) {
-                uint32_t* cp = m.codes + static_cast<size_t>(group) * W;
+            if constexpr (GLOBAL) {
+                const mp<W> code = lanes_index_global<E, L, W>(pt, neg, K, a.table + TL.enc_off[0] / 4, a.table + TL.enc_off[1] / 4, TL.top_words, s_words);
+                // the lanes of the group share the stores
+                if (row_ok && c < C) {
+                    uint32_t* cp = m.codes + static_cast<size_t>(group) * Wc;
+                    const bool quads = ((Wc & 3) | (reinterpret_cast<uintptr_t>(m.codes) & 15u)) == 0;
 #pragma unroll
-                for (int w = 0; w < W; ++w) cp[w] = code.w[w];
+                    for (int v = 0; v < (W + 3) / 4; ++v) {
+                        if ((v & (L - 1)) != (c & (L - 1)) || 4 * v >= Wc) continue;
+                        uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (4 * v + u < W) w[u] = code.w[4 * v + u < W ? 4 * v + u : 0];
+                        if (quads) {
+                            reinterpret_cast<uint4*>(cp)[v] = make_uint4(w[0], w[1], w[2], w[3]);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (4 * v + u < Wc) cp[4 * v + u] = w[u];
+                        }
+                    }
+                }
+            } else {
+                const mp<W> code = lanes_index<E, L, W, GLOBAL ? 64 : RE>(pt, neg, K, smem, wide_blocks, start);
+                if (leader && PVQ_DEBUG_INDEX(group, m.rows * G, PVQ_DEBUG_GLOBAL_STORE)) {
+                    uint32_t* cp = m.codes + static_cast<size_t>(group) * W;
+#pragma unroll
+                    for (int w = 0; w < W; ++w) cp[w] = code.w[w];
+                }
             }
         }
         if (!last_chunk) continue;
@@ -448,7 +585,7 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
     if (st != PVQ_OK) return st;
     LaneGeom g;
     g.minus_zero = -0.0f;
-    g.team_off = (static_cast<uint32_t>(kLaneTableBytes<N, W, RE>) + 127u) & ~127u;
+    g.team_off = RE == 0 ? 0u : (static_cast<uint32_t>(kLaneTableBytes<N, W, RE>) + 127u) & ~127u;
 
     // Team size: the one whose rounds of tiles cost least.  A chunk costs about as much as six times
     // what a tile adds (energies, amplitude indices), eight with a barrier between warps; what
@@ -480,14 +617,14 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
         c.idx_off = c.amp_off + (LS ? 2u * static_cast<uint32_t>(c.ss_floats) * 4u : 0u);
         c.team_bytes = (c.idx_off + 2u * static_cast<uint32_t>(idx_words) * 4u + 127u) & ~127u;
         // as many teams as the threads, the shared memory and (larger than a warp) the named barriers hold
-        long long teams = std::min(kLaneThreadsMax / t, t == 32 ? 24 : 15);
+        long long teams = std::min(kLaneThreads<W> / t, t == 32 ? 32 : 15);
         teams = std::min(teams, (static_cast<long long>(di.smem_max) - c.team_off) / c.team_bytes);
         if (teams < 1) continue;
         const double per_tile = static_cast<double>(chunks_all) / tiles + (t == 32 ? 0.16 : 0.25);
         const double rounds = std::ceil(static_cast<double>(tiles) / (static_cast<double>(teams) * di.sms));
         // an SM with fewer warps than it holds runs them faster, down to about a quarter of the time
-        const double load = std::max(0.25, std::min(1.0, static_cast<double>(teams) * t / kLaneThreadsMax));
-        const double few = rounds > 1.0 ? 1.0 : std::max(0.25, std::min(1.0, static_cast<double>(tiles) * t / (static_cast<double>(di.sms) * kLaneThreadsMax)));
+        const double load = std::max(0.25, std::min(1.0, static_cast<double>(teams) * t / kLaneThreads<W>));
+        const double few = rounds > 1.0 ? 1.0 : std::max(0.25, std::min(1.0, static_cast<double>(tiles) * t / (static_cast<double>(di.sms) * kLaneThreads<W>)));
         const double cost = rounds * per_tile * load * few;
         if (best < 0.0 || cost < best) {
             best = cost;
@@ -535,17 +672,30 @@ static int launch_encode_lanes(BatchArgs& a, cudaStream_t s) {
     }
 }
 
-// Entry of the per-(N, W) translation units: everything but the rotation goes to the kernel above when
-// the tables fit it, the rest (5- and 6-word codes, K > 127) to the general one.
+// The kernel with the tables in global memory, computing in W words: W and up to the code's width.
+template <int N, int W>
+static int launch_encode_lanes_global(BatchArgs& a, int dtype, cudaStream_t s) {
+    constexpr int E = N <= 32 ? N : 32, L = N / E;
+    const bool bf16 = dtype == PVQ_DTYPE_BF16;
+    if (a.amp_mode == 1)
+        return bf16 ? launch_encode_lanes_t<E, L, W, 0, true, true>(a, s) : launch_encode_lanes_t<E, L, W, 0, false, true>(a, s);
+    return bf16 ? launch_encode_lanes_t<E, L, W, 0, true, false>(a, s) : launch_encode_lanes_t<E, L, W, 0, false, false>(a, s);
+}
+
+// Entry of the per-(N, W) translation units of the codes the shared-memory kernels are built for:
+// everything but the rotation goes to the kernels above, with the tables in shared memory where
+// they fit; the rotation to the general one.
 template <int N, int W>
 static int launch_encode_any(BatchArgs& a, int dtype, cudaStream_t s) {
-    if constexpr (W <= 4) {
-        constexpr int E = N <= 32 ? N : 32, L = N / E;
-        if (a.rot_block == 0) {
-            BatchArgs b = a;
+    if (a.rot_block == 0) {
+        BatchArgs b = a;
+        if constexpr (W <= 4) {
+            constexpr int E = N <= 32 ? N : 32, L = N / E;
             const int st = dtype == PVQ_DTYPE_BF16 ? launch_encode_lanes<E, L, W, true>(b, s) : launch_encode_lanes<E, L, W, false>(b, s);
             if (st != PVQ_ERR_UNSUPPORTED) return st;
         }
+        b = a;
+        return launch_encode_lanes_global<N, (W <= 4 ? 4 : W)>(b, dtype, s);
     }
     return launch_encode_nw<N, W>(a, dtype, s);
 }
