@@ -4,9 +4,12 @@ Argument marshalling only: every function checks tensor device / dtype /
 contiguity, passes raw device pointers and the current CUDA stream to the
 library call of the same name, and raises on a non-zero status.  No arithmetic
 of the codec happens here, and there is no fallback: a missing library is an
-error.
+error.  The set-up calls go through ctypes; the hot calls do the same work in a
+CPython extension (csrc/bind/pvq_bind.cpp), handed the library's entry points.
 """
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
@@ -15,6 +18,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 # PVQ_B200_LIB selects another build of the same library, e.g. the bounds-checked one
 # (libpvq_b200_debug.so, see pvq_debug_status in include/pvq.h).
 LIB_PATH = os.environ.get("PVQ_B200_LIB") or os.path.join(_HERE, "libpvq_b200.so")
+BIND_PATH = os.path.join(_HERE, "_bind.so")
 
 DTYPE_F32 = 0
 DTYPE_BF16 = 1
@@ -23,6 +27,7 @@ STATUS_STAGING_TIMEOUT = 2
 STATUS_TABLE_MISMATCH = 4
 
 _lib = None
+_native = None
 
 
 class PvqError(RuntimeError):
@@ -91,6 +96,26 @@ def _check(status, where):
         raise PvqError(status, where)
 
 
+def _raise(status, where):
+    raise PvqError(status, where)
+
+
+def _load_native():
+    """The extension with the hot calls, holding the entry points of lib(); raises if it has not been built."""
+    global _native
+    L = lib()
+    if not os.path.exists(BIND_PATH):
+        raise RuntimeError("PVQ binding not built: %s is missing (run `python -m paper_2410_16926_b200.build`)" % BIND_PATH)
+    loader = importlib.machinery.ExtensionFileLoader("_bind", BIND_PATH)
+    m = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_bind", BIND_PATH, loader=loader))
+    loader.exec_module(m)
+    names = ("encode", "encode_amp", "decode", "roundtrip", "rotate_encode", "rotate_roundtrip", "encode_batched",
+             "decode_batched", "code_words", "scale_row_stride")
+    m.init(_raise, *(C.cast(getattr(L, "pvq_" + n), C.c_void_p).value for n in names))
+    _native = m
+    return m
+
+
 def _stream():
     return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
@@ -105,14 +130,6 @@ def _ptr(t, dtype=None):
     if not t.is_contiguous() and not (t.dim() == 2 and t.stride(1) == 1):
         raise ValueError("expected a row-major tensor")
     return C.c_void_p(t.data_ptr())
-
-
-def _dtype_code(x):
-    if x.dtype == torch.float32:
-        return DTYPE_F32
-    if x.dtype == torch.bfloat16:
-        return DTYPE_BF16
-    raise TypeError("input must be float32 or bfloat16")
 
 
 def encode_status(word):
@@ -194,34 +211,12 @@ def encode(x, N, K, scale_bits, table, edges, out=None, amp_mode=None):
     """x [rows][cols] float32 / bfloat16 on the GPU -> (codes int32 [rows][G][W],
     scale_idx uint8 [rows][stride], row_norm float32 [rows]).  amp_mode (0 / 1) goes through
     pvq_encode_amp; scale_bits 16 takes no edges."""
-    rows, cols = x.shape
-    G = cols // N
-    if out is None:
-        out = alloc_encoded(rows, G, code_words(N, K), scale_bits, x.device)
-    codes, sidx, rnorm = out
-    if amp_mode is not None:
-        _check(lib().pvq_encode_amp(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), N, K, scale_bits, amp_mode,
-                                    _ptr(table, torch.int32), _ptr(edges, torch.float32),
-                                    _ptr(codes, torch.int32), _ptr(sidx, torch.uint8),
-                                    _ptr(rnorm, torch.float32), _stream()), "pvq_encode_amp")
-        return codes, sidx, rnorm
-    _check(lib().pvq_encode(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), N, K, scale_bits,
-                            _ptr(table, torch.int32), _ptr(edges, torch.float32), _ptr(codes, torch.int32),
-                            _ptr(sidx, torch.uint8), _ptr(rnorm, torch.float32), _stream()), "pvq_encode")
-    return codes, sidx, rnorm
+    return (_native or _load_native()).encode(x, N, K, scale_bits, table, edges, out, amp_mode)
 
 
 def decode(codes, sidx, rnorm, N, K, scale_bits, table, levels, out=None, status=None):
     """-> bfloat16 [rows][G*N].  `status`: optional int32 device tensor of one element."""
-    rows, G, _ = codes.shape
-    cols = G * N
-    if out is None:
-        out = torch.empty((rows, cols), dtype=torch.bfloat16, device=codes.device)
-    _check(lib().pvq_decode(_ptr(codes, torch.int32), _ptr(sidx, torch.uint8), _ptr(rnorm, torch.float32),
-                            rows, cols, N, K, scale_bits, _ptr(table, torch.int32),
-                            _ptr(levels, torch.float32), _ptr(out, torch.bfloat16), out.stride(0),
-                            _ptr(status, torch.int32), _stream()), "pvq_decode")
-    return out
+    return (_native or _load_native()).decode(codes, sidx, rnorm, N, K, scale_bits, table, levels, out, status)
 
 
 def decode_static_table(codes, sidx, rnorm, N, K, scale_bits, levels, out=None, status=None):
@@ -242,72 +237,26 @@ def decode_static_table(codes, sidx, rnorm, N, K, scale_bits, levels, out=None, 
 
 def roundtrip(x, N, K, scale_bits, table, edges, levels, out=None):
     """Fused encode -> decode: bfloat16 [rows][cols]."""
-    rows, cols = x.shape
-    if out is None:
-        out = torch.empty((rows, cols), dtype=torch.bfloat16, device=x.device)
-    _check(lib().pvq_roundtrip(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), N, K, scale_bits,
-                               _ptr(table, torch.int32), _ptr(edges, torch.float32),
-                               _ptr(levels, torch.float32), _ptr(out, torch.bfloat16), out.stride(0),
-                               _stream()), "pvq_roundtrip")
-    return out
+    return (_native or _load_native()).roundtrip(x, N, K, scale_bits, table, edges, levels, out)
 
 
 def rotate_encode(x, block, signs, N, K, scale_bits, table, edges, out=None):
     """encode() of the rows of x rotated on the fly by the random-sign Hadamard of size `block`
     (signs: float32 +-1, `block` of them)."""
-    rows, cols = x.shape
-    G = cols // N
-    if out is None:
-        out = alloc_encoded(rows, G, code_words(N, K), scale_bits, x.device)
-    codes, sidx, rnorm = out
-    _check(lib().pvq_rotate_encode(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), block,
-                                   _ptr(signs, torch.float32), N, K, scale_bits, _ptr(table, torch.int32),
-                                   _ptr(edges, torch.float32), _ptr(codes, torch.int32),
-                                   _ptr(sidx, torch.uint8), _ptr(rnorm, torch.float32), _stream()),
-           "pvq_rotate_encode")
-    return codes, sidx, rnorm
+    return (_native or _load_native()).rotate_encode(x, block, signs, N, K, scale_bits, table, edges, out)
 
 
 def rotate_roundtrip(x, block, signs, N, K, scale_bits, table, edges, levels, out=None):
     """roundtrip() of the rows of x rotated on the fly: bfloat16 [rows][cols] in the rotated basis."""
-    rows, cols = x.shape
-    if out is None:
-        out = torch.empty((rows, cols), dtype=torch.bfloat16, device=x.device)
-    _check(lib().pvq_rotate_roundtrip(_ptr(x), _dtype_code(x), rows, cols, x.stride(0), block,
-                                      _ptr(signs, torch.float32), N, K, scale_bits,
-                                      _ptr(table, torch.int32), _ptr(edges, torch.float32),
-                                      _ptr(levels, torch.float32), _ptr(out, torch.bfloat16), out.stride(0),
-                                      _stream()), "pvq_rotate_roundtrip")
-    return out
-
-
-def _descs(items):
-    arr = (MatrixDesc * len(items))()
-    for d, it in zip(arr, items):
-        x, outp = it.get("x"), it.get("out")
-        codes, sidx, rnorm = it["codes"], it["scale_idx"], it["row_norm"]
-        rows, G, _ = codes.shape
-        d.d_x = x.data_ptr() if x is not None else None
-        d.d_out = outp.data_ptr() if outp is not None else None
-        d.d_codes, d.d_scale_idx, d.d_row_norm = codes.data_ptr(), sidx.data_ptr(), rnorm.data_ptr()
-        d.d_edges = it["edges"].data_ptr() if it.get("edges") is not None else None
-        d.d_levels = it["levels"].data_ptr() if it.get("levels") is not None else None
-        d.rows, d.cols = rows, it["cols"]
-        d.ld = x.stride(0) if x is not None else it["cols"]
-        d.ld_out = outp.stride(0) if outp is not None else it["cols"]
-    return arr
+    return (_native or _load_native()).rotate_roundtrip(x, block, signs, N, K, scale_bits, table, edges, levels, out)
 
 
 def encode_batched(items, dtype, N, K, scale_bits, table):
     """items: dicts with x, codes, scale_idx, row_norm, edges, cols.  One launch."""
-    arr = _descs(items)
     code = DTYPE_BF16 if dtype == torch.bfloat16 else DTYPE_F32
-    _check(lib().pvq_encode_batched(arr, len(items), code, N, K, scale_bits, _ptr(table, torch.int32),
-                                    _stream()), "pvq_encode_batched")
+    (_native or _load_native()).encode_batched(items, code, N, K, scale_bits, table)
 
 
 def decode_batched(items, N, K, scale_bits, table, status=None):
     """items: dicts with out, codes, scale_idx, row_norm, levels, cols.  One launch."""
-    arr = _descs(items)
-    _check(lib().pvq_decode_batched(arr, len(items), N, K, scale_bits, _ptr(table, torch.int32),
-                                    _ptr(status, torch.int32), _stream()), "pvq_decode_batched")
+    (_native or _load_native()).decode_batched(items, N, K, scale_bits, table, status)
