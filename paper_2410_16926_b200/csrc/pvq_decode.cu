@@ -27,7 +27,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
 
     // stage the walk tables with the bulk-copy engine; waited for below
     __shared__ uint64_t stage_bar;
+    grid_launch_dependents();
     const BulkStage stage = bulk_stage_begin(&stage_bar);
+    grid_dependency_wait();
     if (threadIdx.x == 0) {
         bulk_stage_expect(stage, walk_tables_stage_bytes(L, a.walk_phases));
         walk_tables_stage(stage, smem, a.table, L, a.walk_phases);
@@ -166,9 +168,7 @@ int launch_decode_t(BatchArgs& a, cudaStream_t stream) {
     const unsigned warps_per_block = threads / 32;
     const unsigned blocks_needed = (tiles + warps_per_block - 1) / warps_per_block;
     const unsigned grid = std::max(1u, std::min<unsigned>(blocks_needed, static_cast<unsigned>(sms * per_sm)));
-    kern<<<grid, threads, smem, stream>>>(a);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
+    return launch_hot(kern, grid, threads, smem, stream, a);
 }
 
 template <int N, int W>

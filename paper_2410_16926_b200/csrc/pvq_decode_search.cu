@@ -42,7 +42,9 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
 
     // stage the search section with the bulk-copy engine; waited for below
     __shared__ uint64_t stage_bar;
+    grid_launch_dependents();
     const BulkStage stage = bulk_stage_begin(&stage_bar);
+    grid_dependency_wait();
     // (records and bucket tables, then the increments E where the blob has the thresholds T)
     const uint8_t* section = reinterpret_cast<const uint8_t*>(a.table) + a.srch_off;
     const uint32_t staged = a.srch_bytes - a.srch_t_before_e;
@@ -213,9 +215,7 @@ int launch_search_t(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
     const unsigned warps_per_block = threads / 32;
     const unsigned blocks_needed = (tiles + warps_per_block * GP - 1) / (warps_per_block * GP);
     const unsigned grid = std::max(1u, std::min<unsigned>(blocks_needed, static_cast<unsigned>(di.sms * per_sm)));
-    kern<<<grid, threads, smem, stream>>>(a);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
+    return launch_hot(kern, grid, threads, smem, stream, a);
 }
 
 // Two groups per thread: enough independent chains to cover the latency of the dependent

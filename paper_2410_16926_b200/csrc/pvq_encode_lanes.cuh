@@ -89,34 +89,38 @@ __device__ __forceinline__ T lane_entry(const uint8_t* p) {
 template <int N, int W, int RE>
 __device__ __forceinline__ void stage_lane_table(uint8_t* tab, const uint32_t* blob, const TableLayout& L, int K, int* wide_blocks) {
     constexpr int TW = W <= 2 ? W : 4;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int i = warp; i < N; i += nwarps) {
-        bool wide = false;
-        for (int m = lane; m < 2 * K + 2; m += 32) {
-            const uint32_t* src = blob + ((m & 1) ? L.cenc_off[1] : L.cenc_off[0]) / 4 + static_cast<size_t>(i) * TW * L.crow + (m >> 1);
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
+    // entry by entry, several loads in flight: a small launch consists mostly of this
+    int wide = 0;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < N * RE; e += blockDim.x) {
+        const int i = e / RE, m = e & (RE - 1);
+        if (m >= 2 * K + 2) continue;
+        const uint32_t* src = blob + ((m & 1) ? L.cenc_off[1] : L.cenc_off[0]) / 4 + static_cast<size_t>(i) * TW * L.crow + (m >> 1);
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-            for (int j = 0; j < W; ++j) w[j] = __ldg(src + j * L.crow);
-            uint8_t* dst = tab + (i * RE + m) * kLaneEntry<W>;
-            if constexpr (W == 1) {
-                *reinterpret_cast<uint32_t*>(dst) = w[0];
-            } else if constexpr (W <= 3) {
-                // E is never positive: M = -E in 32 W bits, split
-                mp<W> zero, e, neg;
-                mp_zero(zero);
+        for (int j = 0; j < W; ++j) w[j] = __ldg(src + j * L.crow);
+        uint8_t* dst = tab + e * kLaneEntry<W>;
+        if constexpr (W == 1) {
+            *reinterpret_cast<uint32_t*>(dst) = w[0];
+        } else if constexpr (W <= 3) {
+            // E is never positive: M = -E in 32 W bits, split
+            mp<W> zero, v, neg;
+            mp_zero(zero);
 #pragma unroll
-                for (int j = 0; j < W; ++j) e.w[j] = w[j];
-                mp_sub_borrow<W>(neg, zero, e);
-                const unsigned long long low = static_cast<unsigned long long>(neg.w[0]) | (static_cast<unsigned long long>(neg.w[1]) << 32);
-                const unsigned long long up = (low >> kSplitBit) | (static_cast<unsigned long long>(W == 3 ? neg.w[W - 1] : 0u) << (64 - kSplitBit));
-                *reinterpret_cast<double*>(dst) = static_cast<double>(low & ((1ull << kSplitBit) - 1ull));
-                *reinterpret_cast<double*>(dst + N * RE * 8) = static_cast<double>(up);
-                wide = wide || up != 0;
-            } else {
-                *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+            for (int j = 0; j < W; ++j) v.w[j] = w[j];
+            mp_sub_borrow<W>(neg, zero, v);
+            const unsigned long long low = static_cast<unsigned long long>(neg.w[0]) | (static_cast<unsigned long long>(neg.w[1]) << 32);
+            const unsigned long long up = (low >> kSplitBit) | (static_cast<unsigned long long>(W == 3 ? neg.w[W - 1] : 0u) << (64 - kSplitBit));
+            *reinterpret_cast<double*>(dst) = static_cast<double>(low & ((1ull << kSplitBit) - 1ull));
+            *reinterpret_cast<double*>(dst + N * RE * 8) = static_cast<double>(up);
+            if (up != 0) wide = max(wide, i / 4 + 1);
+        } else {
+            *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        if ((W == 2 || W == 3) && __any_sync(kFull, wide) && lane == 0) atomicMax(wide_blocks, i / 4 + 1);
+    }
+    if constexpr (W == 2 || W == 3) {
+        const unsigned all = __reduce_max_sync(kFull, static_cast<unsigned>(wide));
+        if ((threadIdx.x & 31) == 0) atomicMax(wide_blocks, static_cast<int>(all));
     }
 }
 
@@ -394,6 +398,7 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
     const int K = a.K, b = a.scale_bits;
     const int Wc = GLOBAL ? a.code_words : W;  // words of a code in memory
     const TableLayout TL = table_layout(N, K, Wc);
+    grid_launch_dependents();
     const int T = g.team, team = threadIdx.x / T, tid = threadIdx.x - team * T, lane = threadIdx.x & 31;
     uint8_t* area = smem + g.team_off + team * g.team_bytes;
 
@@ -402,12 +407,15 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
     at.ch = 0;
     const unsigned stride = gridDim.x * static_cast<unsigned>(g.teams);
     const bool works = team < g.teams && at.tile < a.total_tiles;
+    if (!GLOBAL && threadIdx.x == 0) s_wide_blocks = 0;
     if (works) {
         enter_matrix(a, at, find_matrix(a, at.tile), tid, L);
-        request_input<E, L, BF16>(a, at, shared_addr(area), T, tid);
         uint32_t* s_idx2 = reinterpret_cast<uint32_t*>(area + g.idx_off);
         for (int i = tid; i < 2 * g.idx_words; i += T) s_idx2[i] = 0u;
     }
+    __syncthreads();  // s_wide_blocks
+    grid_dependency_wait();
+    if (works) request_input<E, L, BF16>(a, at, shared_addr(area), T, tid);
     mp<GLOBAL ? 1 : W> start;
     if constexpr (GLOBAL) {
         // words of N(n+1,K) = U(n,K), which no term of the position exceeds (N(N,K) may be a power of two
@@ -422,10 +430,6 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
         debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
 #endif
     } else {
-        if (W == 2 || W == 3) {
-            if (threadIdx.x == 0) s_wide_blocks = 0;
-            __syncthreads();
-        }
         stage_lane_table<N, W, GLOBAL ? 64 : RE>(smem, a.table, TL, K, &s_wide_blocks);
 #pragma unroll
         for (int w = 0; w < W; ++w) start.w[GLOBAL ? 0 : w] = a.table[TL.start_off / 4 + w];
@@ -646,17 +650,15 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
     a.total_tiles = tiles;
 
     const size_t smem = g.team_off + static_cast<size_t>(g.teams) * g.team_bytes;
-    // at least eight warps, which share the staging of the tables
-    const int threads = std::max(g.team * g.teams, 256);
+    // at least sixteen warps to share the staging of the tables
+    const int threads = std::max(g.team * g.teams, RE == 0 ? 64 : 512);
     auto kern = encode_lanes_kernel<E, L, W, RE, BF16, LS>;
     int per_sm = 0;
     if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
     const unsigned blocks = (tiles + g.teams - 1) / g.teams;
     const unsigned grid = std::min<unsigned>(blocks, static_cast<unsigned>(di.sms * per_sm));
-    kern<<<grid, threads, smem, stream>>>(a, g);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
+    return launch_hot(kern, grid, threads, smem, stream, a, g);
 }
 
 template <int E, int L, int W, bool BF16>

@@ -6,6 +6,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 
 #include "pvq.h"
 
@@ -280,6 +281,31 @@ int launch_roundtrip(const MatrixArgs& m, int dtype, int N, int K, int scale_bit
 // ---------------------------------------------------------------- device bits
 
 #ifdef __CUDACC__
+
+// Launch of a hot-path kernel so that it may be set up while the kernel before it in the stream still runs
+// (programmatic dependent launch): between two small calls that hides most of the launch.  Such a
+// kernel calls grid_dependency_wait() in every thread before it touches global memory - it returns when
+// everything before in the stream is complete and visible - and, so that the next one can come
+// early in turn, grid_launch_dependents() at its start (the next kernel's blocks are only placed once
+// all blocks of this one have said so, hence take no place from them).  Tables and inputs are not read before
+// the wait: the kernel before may have written them.
+template <typename... Params, typename... Args>
+inline int launch_hot(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+    return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
+}
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // balanced tree over contiguous halves, each addition rounded to fp32
 template <int N>

@@ -143,8 +143,10 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
     if (tid == 0) {
         for (int i = 0; i < 3; ++i) mbarrier_init_one(full + i);
         mbarrier_init_fence();
-        request(tile, 0);
     }
+    grid_launch_dependents();
+    grid_dependency_wait();
+    if (tid == 0) request(tile, 0);
     float rot_scale = 1.0f;
     if constexpr (ROT) {
         pack_signs<E>(s_signs, a.signs, a.rot_block);
@@ -277,6 +279,8 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_rows_kernel(const 
     float* s_xbuf = reinterpret_cast<float*>(smem + a.xbuf_off);
     const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
     const int b = a.b;
+    grid_launch_dependents();
+    grid_dependency_wait();
     float rot_scale = 1.0f;
 #ifdef PVQ_DEBUG
     debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
@@ -427,23 +431,21 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
     a.ring_off = (a.xbuf_off + (ROT ? static_cast<uint32_t>(threads) * E * 4u : 0u) + 127u) & ~127u;
     a.tile_bytes = static_cast<uint32_t>(threads) * E * 2u;
     size_t smem = a.ring_off;
-    const void* kern = reinterpret_cast<const void*>(roundtrip_rows_kernel<E, L, BF16, WIDE, ROT>);
+    void (*kern)(RoundArgs) = roundtrip_rows_kernel<E, L, BF16, WIDE, ROT>;
     bool stays = false;  // the block stays and takes tile after tile
     if constexpr (BF16) {
         if (a.chunks == 1 && smem + 3u * a.tile_bytes <= static_cast<size_t>(di.smem_max)) {
             stays = true;
             smem += 3u * a.tile_bytes;
-            kern = reinterpret_cast<const void*>(roundtrip_kernel<E, L, WIDE, ROT>);
+            kern = roundtrip_kernel<E, L, WIDE, ROT>;
         }
     }
     if (smem > static_cast<size_t>(di.smem_max)) return PVQ_ERR_UNSUPPORTED;
     int per_sm = 0;
-    if ((st = prepare_kernel(kern, threads, smem, &per_sm)) != PVQ_OK) return st;
+    if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
     const unsigned grid = stays ? std::min(a.tiles, static_cast<unsigned>(di.sms * per_sm)) : a.tiles;
-    void* params[] = {&a};
-    const cudaError_t e = cudaLaunchKernel(kern, dim3(grid), dim3(threads), params, smem, stream);
-    return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
+    return launch_hot(kern, grid, threads, smem, stream, a);
 }
 
 template <int E, int L>
