@@ -8,7 +8,9 @@
 #include <utility>
 #include <vector>
 
+#include "pvq_bigint.h"
 #include "pvq_internal.cuh"
+#include "pvq_window.cuh"
 
 namespace pvq {
 
@@ -20,64 +22,6 @@ int set_cuda_error(cudaError_t e) {
 }
 
 bool is_aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
-
-// ------------------------------------------------------------------ big ints
-// Unsigned integers of up to kLimbs 32-bit limbs; only what choosing K needs.
-namespace {
-
-constexpr int kLimbs = 48;
-
-struct BigU {
-    uint32_t w[kLimbs];
-    BigU() { std::memset(w, 0, sizeof w); }
-    explicit BigU(uint32_t v) {
-        std::memset(w, 0, sizeof w);
-        w[0] = v;
-    }
-    // *this += o; false when the sum overflows kLimbs
-    bool add(const BigU& o) {
-        uint64_t c = 0;
-        for (int i = 0; i < kLimbs; ++i) {
-            uint64_t s = static_cast<uint64_t>(w[i]) + o.w[i] + c;
-            w[i] = static_cast<uint32_t>(s);
-            c = s >> 32;
-        }
-        return c == 0;
-    }
-    int bit_length() const {
-        for (int i = kLimbs - 1; i >= 0; --i)
-            if (w[i]) return 32 * i + (32 - __builtin_clz(w[i]));
-        return 0;
-    }
-    bool is_pow2() const {
-        int ones = 0;
-        for (int i = 0; i < kLimbs; ++i) ones += __builtin_popcount(w[i]);
-        return ones == 1;
-    }
-    // ceil(log2 v) for v >= 1
-    int ceil_log2() const { return is_pow2() ? bit_length() - 1 : bit_length(); }
-};
-
-// col[n] = N(n,k) for n = 0..N, advanced from k to k+1 with
-// N(n,k+1) = N(n-1,k+1) + N(n,k) + N(n-1,k)   (Sec. 2.4).
-struct CountColumn {
-    std::vector<BigU> col;
-    int k = 0;
-    explicit CountColumn(int N) : col(static_cast<size_t>(N) + 1, BigU(1u)) {}  // N(n,0) = 1
-    bool advance() {
-        std::vector<BigU> nxt(col.size());
-        nxt[0] = BigU(0u);  // N(0,k>=1) = 0
-        for (size_t n = 1; n < col.size(); ++n) {
-            nxt[n] = nxt[n - 1];
-            if (!nxt[n].add(col[n]) || !nxt[n].add(col[n - 1])) return false;
-        }
-        col.swap(nxt);
-        ++k;
-        return true;
-    }
-};
-
-}  // namespace
 
 static int index_bits_exact(int N, int K) {
     if (N < 1 || N > 4096 || K < 0 || K > 65535) return -1;
@@ -473,6 +417,10 @@ int run_batch(const pvq_matrix_desc* descs, int count, int need, int dtype, int 
     // codes the shared-memory kernels are built for, by group size
     const int fast_words = c.N == 8 ? 2 : (c.N == 16 ? 3 : (c.N == 32 ? 4 : (c.N == 64 ? 6 : 0)));
     if (kind == 2) return launch_roundtrip(a.m[0], dtype, c.N, K, scale_bits, rot_block, d_signs, a.status, a.debug_status, s);
+    if (kind == 1) {  // wide codes whose windowed tables are at hand
+        st = launch_decode_window(a, c.N, c.W, s);
+        if (st != PVQ_ERR_UNSUPPORTED) return st;
+    }
     if (c.W > fast_words) {  // large groups, wide codes
         return launch_big(a, dtype, c.N, c.W, kind == 1, s);
     }

@@ -4,6 +4,7 @@
 #include "mp_uint.cuh"
 #include "pvq_internal.cuh"
 #include "pvq_search.cuh"
+#include "pvq_window.cuh"
 
 namespace pvq {
 
@@ -567,6 +568,7 @@ extern "C" int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t byt
     if (!is_aligned(d_table, 16)) return PVQ_ERR_ALIGNMENT;
     if (bytes < pvq_count_table_bytes(N, K)) return PVQ_ERR_TABLE_TOO_SMALL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    build_window_tables(N, K, s);
     // more pulses than threads of a block, or rows of 32 KB and more: the multi-block builder, in 8, 16 or 32 words
     if (K > 1023 || static_cast<long long>(K + 1) * W >= 8192) {
         if (W <= 8) return launch_count_table_chunked<8>(N, K, W, d_table, s);

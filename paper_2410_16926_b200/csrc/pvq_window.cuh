@@ -1,0 +1,72 @@
+// Windowed search tables of the decoder for wide codes (pvq_decode_window.cu): layout and host interface.
+//
+// As in SearchLayout, with q = N(n+1,k) - r the coordinate of a position (n dimensions behind it) follows
+// from where q falls among the thresholds T_n[2k'] = N(n+1,k'), T_n[2k'+1] = N(n+1,k') + N(n,k'), and the next
+// position's q is q + E_n[m], E_n[m] = N(n,k') - T_n[m].  A table of all thresholds of all rows is too large for
+// shared memory when codes are wide.  But the pulses k' left after a position hardly ever stray far
+// from their mean: a row keeps only the window klo..khi outside of which no more than a share eps of all
+// codes lies on either side.  A group whose path leaves the window somewhere is found out (see `last`
+// below) and walked by Algorithm 3 instead.
+//
+// Rows are taken in blocks of four positions.  A block's numbers are kept left-aligned: multiplied by the power
+// of two that brings the largest q of the block to the top of its `words` 32-bit words.  The top two words
+// (three at N = 128, whose windows span more than 56 bits) then hold the leading bits of q whatever the row;
+// as an fp32, truncated, they are the key that numbers a bucket.  From one block to the next q is shifted left by `delta` bits.
+//
+// Block b in memory (block_off[b], a multiple of 16 bytes):
+//     E        four rows, each `words` planes of `plane` 32-bit words: word w (lowest first) of
+//              entry m - 2 klo of the row, modulo 2^(32 words)
+//     buckets  four tables, 4 bytes a bucket: in the low byte m0, the local index of the first threshold
+//              that a q of the bucket can be at or below, above it the complement of the low 24 key bits of
+//              that threshold if it lies in the bucket (else zeros): the sum with a q's 24 key bits carries
+//              iff q's are larger, and leaves all ones iff they are the same.  The last entry
+//              of a table (index `last`) catches every key outside the window: m0 = 255, which makes the
+//              pulses left grow, and that is seen.
+#pragma once
+#include <memory>
+
+#include "pvq_internal.cuh"
+
+namespace pvq {
+
+constexpr int kWinRows = 128, kWinBlocks = kWinRows / 4;
+constexpr uint32_t kWinPad = 1024;  // bytes behind the last block that an out-of-window read may touch
+
+__host__ __device__ constexpr int win_key_words(int N) { return N > 64 ? 3 : 2; }
+
+struct WinRow {
+    uint32_t buckets;  // byte offset of the row's bucket table in its block
+    uint32_t first;    // number of its first bucket
+    uint32_t last;     // index of the entry for keys outside the window
+    uint32_t shift;    // key >> shift is the bucket number
+};
+
+struct WinArgs {
+    const uint8_t* data;
+    const uint8_t* thr;                  // thresholds (aligned), laid out like E; read when key bits are the same
+    uint32_t block_off[kWinBlocks + 1];  // the last one: bytes in all
+    uint32_t thr_off[kWinBlocks];
+    uint32_t dlo4[kWinBlocks];           // klo of the position before minus klo of the position, a byte each
+    uint8_t delta[kWinBlocks];           // bits q is shifted left by when the block begins
+    uint8_t blocks_of[33];               // blocks_of[w]: blocks done in w words or more
+    WinRow row[kWinRows];
+};
+
+struct WinTables {
+    WinArgs args;
+    int plane;           // 96, 128, 160 or 192
+    uint32_t max_block;  // bytes of the largest block
+};
+
+// The tables for (N,K) on the current device, or null (never built here, or no such kernel).  The holder keeps them
+// from being freed until its launch is enqueued; freeing waits for the kernels that read them.
+std::shared_ptr<const WinTables> window_tables(int N, int K);
+// Builds them, once per device and (N,K): called when a count table is built, off the hot path.  The tables of at most
+// kWinKept (N,K) are kept per device, the oldest are freed.  Failing to build is not an error: decoding walks.
+constexpr int kWinKept = 8;
+void build_window_tables(int N, int K, cudaStream_t stream);
+
+// PVQ_ERR_UNSUPPORTED: no tables or no kernel for it; the caller walks
+int launch_decode_window(const BatchArgs& args, int N, int W, cudaStream_t stream);
+
+}  // namespace pvq
