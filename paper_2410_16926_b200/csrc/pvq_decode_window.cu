@@ -62,45 +62,120 @@ __device__ __forceinline__ uint32_t win_key(const mp<PW>& v) {
     return __float_as_uint(x);
 }
 
-// The four positions once more, comparing in full where the key bits were the same.
+// What the repeated search of a block works on: q (`over`: the word above the block's, for paths above the windows), the
+// local pulses left, and what it hands back.
+template <int PW>
+struct WinExact {
+    mp<PW> v;
+    uint32_t over;
+    int h;
+    uint32_t y4, ssy;
+    bool lost;
+};
+
+// Word w of an entry of one of the blob's tables: zero from Wc on.
+__device__ __forceinline__ uint32_t win_count_word(const uint32_t* t, int w, int Wc) { return w < Wc ? __ldg(t + w) : 0u; }
+
+// t < q ?  (t: an entry of Wc words; q: PW + 1 words)
+template <int PW>
+__device__ __forceinline__ bool win_less(const uint32_t* t, int Wc, const uint32_t (&q)[PW + 1]) {
+    long long c = 0;
+#pragma unroll
+    for (int w = 0; w <= PW; ++w) c = (c + static_cast<long long>(win_count_word(t, w, Wc)) - q[w]) >> 32;
+    uint32_t rest = 0u;
+    for (int w = PW + 1; w < Wc; ++w) rest |= __ldg(t + w);
+    return c < 0 && rest == 0u;
+}
+
+// The four positions of block b once more, for the paths that the fast pass cannot decide: key bits the same as a
+// threshold's (compared in full), positions outside the window (searched in the whole row, in global memory).
 template <int PW, int PLANE, int KW>
-__device__ __noinline__ uint32_t win_exact4(mp<PW>& v, uint32_t acc, uint32_t stage, const WinRow* rows, const uint32_t* thr) {
+__device__ __noinline__ void win_exact4(WinExact<PW>& st, uint32_t acc, uint32_t stage, const WinArgs& t, int b, const uint32_t* blob, int N,
+                                        int K, int Wc) {
+    const WinRow* rows = t.row + 4 * b;
 #pragma unroll 1
     for (int s = 3; s >= 0; --s) {  // back to where the block began
         mp<PW> e, d;
         win_entry<PW, PLANE, 0>(e, stage + static_cast<uint32_t>(s) * (PW * PLANE * 4) + ((acc >> (8 * s)) & 0xffu) * 4u);
-        mp_sub_borrow<PW>(d, v, e);
-        v = d;
+        mp_sub_borrow<PW>(d, st.v, e);
+        st.v = d;
     }
-    acc = 0u;
+    const TableLayout L = table_layout(N, K, Wc);
+    const int up = t.up[b];
+    int k = (b > 0 ? t.klo[4 * b - 1] : K) + st.h;  // pulses left before the position
+    st.y4 = 0u;
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
-        const uint32_t key = win_key<PW, KW>(v);
+        const int i = 4 * b + s, n = N - 1 - i;
+        const uint32_t key = win_key<PW, KW>(st.v);
         const uint32_t x = min((key >> rows[s].shift) - rows[s].first, rows[s].last);
         const uint32_t entry = win_load(stage + rows[s].buckets + x * 4u);
         const uint32_t m0 = entry & 0xffu, sum = (key << 8) + entry;
-        uint32_t m = m0 + (sum < entry ? 1u : 0u);
-        if (sum >= 0xffffff00u && m0 < PLANE) {
-            mp<PW> t, d;
+        int left;
+        bool odd;
+        if (st.over == 0u && x < rows[s].last) {
+            uint32_t m = m0 + (sum < entry ? 1u : 0u);
+            if (sum >= 0xffffff00u) {
+                const uint32_t* thr = reinterpret_cast<const uint32_t*>(t.thr + t.thr_off[b]) + s * PW * PLANE + m0;
+                mp<PW> th, d;
 #pragma unroll
-            for (int w = 0; w < PW; ++w) t.w[w] = __ldg(thr + (s * PW + w) * PLANE + m0);
-            m = m0 + (mp_sub_borrow<PW>(d, t, v) ? 1u : 0u);
+                for (int w = 0; w < PW; ++w) th.w[w] = __ldg(thr + w * PLANE);
+                m = m0 + (mp_sub_borrow<PW>(d, th, st.v) ? 1u : 0u);
+            }
+            mp<PW> e;
+            win_entry<PW, PLANE, 0>(e, stage + static_cast<uint32_t>(s) * (PW * PLANE * 4) + m * 4u);
+            mp_add<PW>(st.v, e);
+            left = t.klo[i] + static_cast<int>(m >> 1);
+            odd = (m & 1u) != 0u;
+        } else {
+            uint32_t q[PW + 1];
+#pragma unroll
+            for (int w = 0; w <= PW; ++w) {
+                const uint32_t lo = w < PW ? st.v.w[w < PW ? w : 0] : st.over;
+                const uint32_t hi = w + 1 < PW ? st.v.w[w + 1 < PW ? w + 1 : 0] : (w + 1 == PW ? st.over : 0u);
+                q[w] = __funnelshift_r(lo, hi, up);
+            }
+            const uint32_t* row_u = blob + L.enc_off[0] / 4 + static_cast<size_t>(i) * (K + 2) * L.top_words;
+            const uint32_t* row_v = blob + L.enc_off[1] / 4 + static_cast<size_t>(i) * (K + 2) * L.top_words;
+            left = max(min(k, K), 0);
+            // 2 V(n, left - 1) < q <= 2 V(n, left)
+            while (left > 0 && !win_less<PW>(row_v + static_cast<size_t>(left) * L.top_words, Wc, q)) --left;
+            const uint32_t* u = row_u + static_cast<size_t>(left + 1) * L.top_words;
+            odd = win_less<PW>(u, Wc, q);
+            if (odd) u = row_v + static_cast<size_t>(left + 1) * L.top_words;
+            // q -= T - N(n, left)
+            const uint32_t* c0 = blob + (static_cast<size_t>(n) * (K + 1) + left) * Wc;
+            long long c = 0;
+#pragma unroll
+            for (int w = 0; w <= PW; ++w) {
+                c += static_cast<long long>(q[w]) - win_count_word(u, w, Wc) + win_count_word(c0, w, Wc);
+                q[w] = static_cast<uint32_t>(c);
+                c >>= 32;
+            }
+            st.over = __funnelshift_l(q[PW - 1], q[PW], up);
+            st.lost = st.lost || (up > 0 && (q[PW] >> (32 - up)) != 0u);
+#pragma unroll
+            for (int w = PW - 1; w >= 0; --w) st.v.w[w] = __funnelshift_l(w > 0 ? q[w > 0 ? w - 1 : 0] : 0u, q[w], up);
         }
-        mp<PW> e;
-        win_entry<PW, PLANE, 0>(e, stage + static_cast<uint32_t>(s) * (PW * PLANE * 4) + m * 4u);
-        mp_add<PW>(v, e);
-        acc |= m << (8 * s);
+        const int mag = k - left;
+        st.lost = st.lost || mag < 0 || mag > 127;
+        st.y4 |= (static_cast<uint32_t>(128 + (odd ? mag : -mag)) & 0xffu) << (8 * s);
+        st.ssy += static_cast<uint32_t>(mag * mag);
+        k = left;
     }
-    return acc;
+    st.h = k - t.klo[4 * b + 3];
+    if (st.over >= 0x10000u) st.lost = true;  // the next block's shift (16 bits at most) would push bits out
+    if (st.lost) st.over = 0u, st.h = 0;
 }
 
 // State of one thread's search.  a[0] is the leading word; the words a block does not work on are zero.
 template <int W>
 struct WinState {
     uint32_t a[W + 1];
-    uint32_t h;     // local index >> 1 of the position before
-    uint32_t flag;  // bit 7 of a byte set: some |y| was out of range, the path left the window
+    uint32_t over;  // the word above a[0]: zero but for paths above the windows
+    int h;          // pulses left after the position before, minus its klo
     uint32_t ssy;   // sum of y^2
+    bool lost;      // some |y| has no byte, or q no room: the group is walked
 };
 
 template <int PW, int PLANE, int KW, int S>
@@ -120,11 +195,12 @@ __device__ __forceinline__ void win_position(mp<PW>& v, uint32_t& acc, uint32_t&
     acc = __funnelshift_r(acc, m, 8);
 }
 
-template <int PW, int PLANE, int KW, int W>
-__device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, const WinArgs& t, int b, uint32_t y) {
+template <int N, int PW, int PLANE, int KW, int W>
+__device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, const BatchArgs& a, const WinArgs& t, int b, uint32_t y) {
     mp<PW> v;
     {
         const uint32_t delta = t.delta[b];
+        st.over = __funnelshift_l(st.a[0], st.over, delta);
 #pragma unroll
         for (int j = 0; j < PW; ++j) v.w[PW - 1 - j] = __funnelshift_l(st.a[j + 1], st.a[j], delta);
         st.a[PW] = 0u;
@@ -134,37 +210,47 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
     win_position<PW, PLANE, KW, 1>(v, acc, top, stage, t.row[4 * b + 1]);
     win_position<PW, PLANE, KW, 2>(v, acc, top, stage, t.row[4 * b + 2]);
     win_position<PW, PLANE, KW, 3>(v, acc, top, stage, t.row[4 * b + 3]);
-    if (__any_sync(kFull, top >= 0xffffff00u)) {
-        mp<PW> u = v;
-        acc = win_exact4<PW, PLANE, KW>(u, acc, stage, t.row + 4 * b, reinterpret_cast<const uint32_t*>(t.thr + t.thr_off[b]));
-        v = u;
-    }
-    // |y|: pulses left before the position minus those left after it, a byte each (a byte that runs below
-    // zero shows in its bit 7); y > 0 where the index is odd
+    // |y|: pulses left before the position minus those left after it, a byte each: one sum, whose bytes do not
+    // touch each other while all of them are 0..127 (else some bit 7 shows, unless the position before was out of the
+    // window too, and then h shows it); y > 0 where the index is odd
     const uint32_t after = (acc >> 1) & 0x7f7f7f7fu;
-    const uint32_t mag = ((after << 8) | st.h) + t.dlo4[b] - after;
-    st.h = after >> 24;
-    st.flag |= mag;
-    st.ssy = __dp4a(mag, mag, st.ssy);
+    const uint32_t mag = (after << 8) + t.dlo4[b] - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;
-    asm volatile("st.shared.u32 [%0], %1;" ::"r"(y), "r"(((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos)) : "memory");
+    uint32_t y4 = ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos);
+    if (__any_sync(kFull, top >= 0xffffff00u || (((mag | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
+        WinExact<PW> x;
+        x.v = v;
+        x.over = st.over, x.h = st.h, x.ssy = st.ssy, x.lost = st.lost;
+        win_exact4<PW, PLANE, KW>(x, acc, stage, t, b, a.table, N, a.K, W);
+        v = x.v;
+        st.over = x.over, st.h = x.h, st.ssy = x.ssy, st.lost = x.lost;
+        y4 = x.y4;
+    } else {
+        st.h = static_cast<int>(after >> 24);
+        st.ssy = __dp4a(mag, mag, st.ssy);
+    }
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(y), "r"(y4) : "memory");
 #pragma unroll
     for (int j = 0; j < PW; ++j) st.a[j] = v.w[PW - 1 - j];
 }
 
 // All blocks from the one that PW words are first enough for: the widest first.
-template <int PW, int PLANE, int KW, int W, typename Enter, typename Leave>
-__device__ __forceinline__ void win_blocks(WinState<W>& st, const WinArgs& t, int& b, uint32_t y, Enter&& enter, Leave&& leave) {
+template <int N, int PW, int PLANE, int KW, int W, typename Enter, typename Leave>
+__device__ __forceinline__ void win_blocks(WinState<W>& st, const BatchArgs& a, const WinArgs& t, int& b, uint32_t y, Enter&& enter, Leave&& leave) {
 #pragma unroll 1
     for (; b < t.blocks_of[PW]; ++b) {
-        win_block4<PW, PLANE, KW, W>(st, enter(b), t, b, y + static_cast<uint32_t>(b) * 4u);
+        const uint32_t stage = enter(b), yb = y + static_cast<uint32_t>(b) * 4u;
+        if (t.narrow[b])
+            win_block4<N, PW, 64, KW, W>(st, stage, a, t, b, yb);
+        else
+            win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
         leave(b);
     }
-    if constexpr (PW > 1) win_blocks<PW - 1, PLANE, KW, W>(st, t, b, y, enter, leave);
+    if constexpr (PW > 1) win_blocks<N, PW - 1, PLANE, KW, W>(st, a, t, b, y, enter, leave);
 }
 
-// Algorithm 3 step by step for the group at hand, from the count table in global memory: for the few groups whose
-// path leaves the windows.  Its point goes to the thread's slot if all |y| < 128; else its values are
+// Algorithm 3 step by step for the group at hand, from the count table in global memory: for points with a |y| of 128 or
+// more, or with a path far above the windows.  Its point goes to the thread's slot if all |y| < 128; else its values are
 // written to `out` right away (the walk done twice), and the result is true.
 __device__ __noinline__ bool win_walk(const uint32_t* count, int N, int K, int W, const uint32_t* code, uint8_t* slot, float amp,
                                       __nv_bfloat16* out, uint32_t* ssy_out) {
@@ -261,24 +347,29 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
         bad = bad || !valid;
     }
     WinState<W> st;
-    bool alone;  // the point (K, 0, ..., 0), which a group of zeros has: q = 2
-    {
+    bool alone = false;  // the point (K, 0, ..., 0), which a group of zeros has: q = 2
+    if (valid) {
         mp<W> q;
-        mp_sub_borrow<W>(q, bound, c);  // 1 <= q <= N(N,K) (an invalid code: whatever, it is not used)
+        mp_sub_borrow<W>(q, bound, c);  // 1 <= q <= N(N,K)
         uint32_t rest = q.w[0] ^ 2u;
 #pragma unroll
         for (int w = 1; w < W; ++w) rest |= q.w[w];
         alone = rest == 0u;
-        // to the top of the words: the first block's delta is the shift
+        // (the first block's delta brings it to the top of the words)
 #pragma unroll
         for (int j = 0; j < W; ++j) st.a[j] = q.w[W - 1 - j];
-        st.a[W] = 0u;
     }
-    st.h = 0u;
-    st.flag = 0u;
+    if (!valid || alone) {  // not searched: a path that costs nothing extra in its place
+#pragma unroll
+        for (int j = 0; j < W; ++j) st.a[j] = t.typical[W - 1 - j];
+    }
+    st.a[W] = 0u;
+    st.over = 0u;
+    st.h = 0;
     st.ssy = 0u;
+    st.lost = false;
     int blk = 0;
-    win_blocks<W, PLANE, win_key_words(N), W>(st, t, blk, y, enter, leave);
+    win_blocks<N, W, PLANE, win_key_words(N), W>(st, a, t, blk, y, enter, leave);
 
     float amp = 0.0f;
     __nv_bfloat16* out = static_cast<__nv_bfloat16*>(m.out) + static_cast<size_t>(row) * m.ld_out + static_cast<size_t>(g) * N;
@@ -295,7 +386,7 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
         for (int i = 0; i < N / 4; ++i) reinterpret_cast<uint32_t*>(slot)[i] = 0x80808080u;
         if (single) slot[0] = static_cast<uint8_t>(128 + a.K);
         st.ssy = single ? static_cast<uint32_t>(a.K * a.K) : 1u;
-    } else if (valid && (st.flag & 0x80808080u) != 0u) {
+    } else if (valid && (st.lost || alone)) {
         uint32_t ssy;
         done = win_walk(a.table, N, a.K, W, code, slot, amp, out, &ssy);
         st.ssy = ssy;
@@ -354,7 +445,7 @@ __global__ void __launch_bounds__(1024, 1)
     const uint32_t base = shared_addr(smem);
     uint8_t* slot = smem + g.slots_off + threadIdx.x * (N + 4);
     const uint32_t y = shared_addr(slot), slots = y - (threadIdx.x & 31) * (N + 4);
-    const unsigned warp = threadIdx.x >> 5, total = gridDim.x * g.warps;
+    const unsigned warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), total = gridDim.x * g.warps;
     bool bad = false;
     int mi = 0;
     for (unsigned tile = warp * gridDim.x + blockIdx.x; tile < a.total_tiles; tile += total)
@@ -390,7 +481,7 @@ __global__ void __launch_bounds__(928, 1)
     }
     __syncthreads();
     grid_dependency_wait();
-    const unsigned warp = threadIdx.x >> 5, step = gridDim.x * g.warps, first = blockIdx.x;
+    const unsigned warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), step = gridDim.x * g.warps, first = blockIdx.x;
     const int passes = first < a.total_tiles ? static_cast<int>((a.total_tiles - first + step - 1) / step) : 0;
     if (warp == static_cast<unsigned>(g.warps)) {  // feeds the ring
         if ((threadIdx.x & 31) == 0) {
@@ -450,7 +541,7 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
     std::memset(&g, 0, sizeof g);
     const uint32_t all = t.args.block_off[N / 4], ys = N + 4;
     const uint32_t limit = static_cast<uint32_t>(di.smem_max);
-    const bool resident = N <= 64 && all + kWinPad + 512u * ys <= limit;
+    const bool resident = N <= 64 && all + 512u * ys <= limit;
     const int most = resident ? 32 : 28;
     int warps = 0;
     double best = -1.0;
@@ -458,9 +549,9 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
         g.bufs = 0;
         uint32_t smem;
         if (resident) {
-            smem = all + kWinPad + w * 32u * ys;
+            smem = all + w * 32u * ys;
         } else {
-            smem = 3u * t.max_block + kWinPad + w * 32u * ys;
+            smem = 3u * t.max_block + w * 32u * ys;
         }
         if (smem > limit) continue;
         // every tile costs the same: rounds of one tile per warp, the fullest last round wins, with a preference for
@@ -475,12 +566,12 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
     const uint32_t slot_bytes = warps * 32u * ys;
     uint32_t tables;
     if (resident) {
-        tables = (all + kWinPad + 127u) & ~127u;
+        tables = (all + 127u) & ~127u;
     } else {
         g.buf_bytes = (t.max_block + 127u) & ~127u;
-        g.bufs = static_cast<int>(std::min<uint32_t>(kWinBufs, (limit - slot_bytes - kWinPad - 128u) / g.buf_bytes));
+        g.bufs = static_cast<int>(std::min<uint32_t>(kWinBufs, (limit - slot_bytes - 128u) / g.buf_bytes));
         if (g.bufs < 2) return PVQ_ERR_UNSUPPORTED;
-        tables = (g.bufs * g.buf_bytes + kWinPad + 127u) & ~127u;
+        tables = (g.bufs * g.buf_bytes + 127u) & ~127u;
     }
     g.slots_off = tables;
     const size_t smem = tables + slot_bytes;
@@ -501,6 +592,7 @@ template <int N, int W>
 int launch_window_w(BatchArgs& a, const WinTables& t, cudaStream_t s) {
     switch (t.plane) {
         case 96: return launch_window_t<N, W, 96>(a, t, s);
+        case 112: return launch_window_t<N, W, 112>(a, t, s);
         case 128: return launch_window_t<N, W, 128>(a, t, s);
         case 160: return launch_window_t<N, W, 160>(a, t, s);
         case 192: if constexpr (N == 64) return launch_window_t<N, W, 192>(a, t, s);

@@ -98,24 +98,24 @@ struct Builder {
     int before(int i) const { return i > 0 ? hi[i - 1] : K; }
 
     // Fills t, data and thr for the current windows; false: cannot be done.
-    bool layout(int plane) {
+    bool layout(const int wide_plane) {
         const int blocks = N / 4;
         bits.assign(blocks, 0);
         words.assign(blocks, 0);
         std::memset(&t, 0, sizeof t);
-        t.plane = plane;
+        t.plane = wide_plane;
         data.clear();
         thr.clear();
         std::vector<int> last_m(N);
         std::vector<char> closed(N);  // no q of the row is beyond its last threshold
         for (int i = 0; i < N; ++i) {
             const int n = N - 1 - i;
-            last_m[i] = hi[i] == before(i) ? 2 * hi[i] : 2 * hi[i] + 1;
+            last_m[i] = hi[i] == K ? 2 * K : 2 * hi[i] + 1;
             const BigU top = threshold(n, last_m[i]);
-            closed[i] = !top.less(count(n + 1, before(i)));
+            closed[i] = !top.less(count(n + 1, K));
             bits[i / 4] = std::max({bits[i / 4], top.bit_length(), count(n + 1, before(i)).bit_length()});
         }
-        for (int b = 1; b < blocks; ++b) bits[b] = std::min(bits[b - 1], std::max(bits[b], bits[b - 1] - 31));
+        for (int b = 1; b < blocks; ++b) bits[b] = std::min(bits[b - 1], std::max(bits[b], bits[b - 1] - 16));
         for (int b = 0; b < blocks; ++b) {
             words[b] = (bits[b] + 31) / 32;
             if (words[b] > 32) return false;
@@ -123,6 +123,11 @@ struct Builder {
             const int delta = (b > 0 ? bits[b - 1] : 32 * words[0]) - bits[b];
             t.args.delta[b] = static_cast<uint8_t>(delta);
             const int W = words[b], up = 32 * W - bits[b], kw = std::min(W, win_key_words(N));
+            bool narrow = true;
+            for (int i = 4 * b; i < 4 * b + 4; ++i) narrow = narrow && last_m[i] - 2 * lo[i] + 1 <= 64;
+            const int plane = narrow ? 64 : wide_plane;
+            t.args.narrow[b] = narrow;
+            t.args.up[b] = static_cast<uint8_t>(up);
             const size_t at = data.size(), planes = static_cast<size_t>(4) * W * plane;
             t.args.block_off[b] = static_cast<uint32_t>(at * 4);
             t.args.thr_off[b] = static_cast<uint32_t>(thr.size() * 4);
@@ -134,6 +139,7 @@ struct Builder {
                 const int dlo = (i > 0 ? lo[i - 1] : K) - lo[i];
                 // |y| and the sums of the packed arithmetic stay below 256, and an out-of-window index always shows
                 if (dlo < 0 || dlo > 127 || before(i) - lo[i] >= 127 || last_m[i] - 2 * lo[i] + 1 > plane) return false;
+                t.args.klo[i] = static_cast<int16_t>(lo[i]);
                 t.args.dlo4[b] |= static_cast<uint32_t>(dlo) << (8 * s);
                 std::vector<uint32_t> key;
                 const bool below = lo[i] > 0;
@@ -179,28 +185,35 @@ struct Builder {
                 }
                 data.push_back(0xffu);
             }
-            while (data.size() & 3u) data.push_back(0u);
+            // (an out-of-window index reads up to 256 entries from the start of a plane)
+            while ((data.size() & 3u) || data.size() < at + planes + 256 - plane) data.push_back(0u);
             t.max_block = std::max(t.max_block, static_cast<uint32_t>((data.size() - at) * 4));
         }
         t.args.block_off[blocks] = static_cast<uint32_t>(data.size() * 4);
-        return true;
+        BigU q(1u);
+        for (int i = 0, k = K; i < N; ++i) {
+            const int n = N - 1 - i, left = std::min(k, (lo[i] + hi[i]) / 2), m = 2 * left + (left < k ? 1 : 0);
+            q.add(threshold(n, m));
+            q.sub(count(n, left));
+            k = left;
+        }
+        for (int w = 0; w < 12; ++w) t.args.typical[w] = q.w[w];
+        return words[0] <= 12;
     }
 
-    // The widest windows whose tables fit beside the output slots of 1024 threads (group size 64); where none
-    // does, the tables are streamed, and the widest that 160 (or 192) entries a row hold are taken.
+    // The widest windows (the smallest share outside) whose tables fit beside the output slots of 30 warps (group size
+    // 64); where none does, the tables are streamed, and the widest that 160 (or 192) entries a row hold are taken.
     bool choose(uint32_t smem_max) {
-        const auto plane_of = [](int entries) { return entries <= 96 ? 96 : (entries <= 128 ? 128 : (entries <= 160 ? 160 : 192)); };
-        const double shares[] = {1e-8, 1e-7, 1e-6, 1e-5, 3e-5, 1e-4, 3e-4, 1e-3};
-        const uint32_t room = smem_max - kWinPad - 1024u * (N + 4);
-        for (double eps : shares) {
-            if (N > 64) break;
-            const int entries = windows(eps);
-            if (entries <= 192 && layout(plane_of(entries)) && t.args.block_off[N / 4] <= room) return true;
-        }
-        for (double eps : shares) {
-            const int entries = windows(eps);
-            if (entries <= (N == 64 ? 192 : 160) && layout(plane_of(entries))) return true;
-        }
+        const uint32_t room = smem_max - 128u - 30u * 32u * (N + 4);
+        for (int streamed = N > 64 ? 1 : 0; streamed < 2; ++streamed)
+            for (double eps : {1e-9, 3e-9, 1e-8, 3e-8, 1e-7, 3e-7, 1e-6, 3e-6, 1e-5, 3e-5, 1e-4, 3e-4, 1e-3}) {
+                const int entries = windows(eps);
+                for (int plane : {96, 112, 128, 160, 192})
+                    if (entries <= plane) {
+                        if ((plane < 192 || N == 64) && layout(plane) && (streamed || t.args.block_off[N / 4] <= room)) return true;
+                        break;
+                    }
+            }
         return false;
     }
 };

@@ -5,8 +5,8 @@
 // position's q is q + E_n[m], E_n[m] = N(n,k') - T_n[m].  A table of all thresholds of all rows is too large for
 // shared memory when codes are wide.  But the pulses k' left after a position hardly ever stray far
 // from their mean: a row keeps only the window klo..khi outside of which no more than a share eps of all
-// codes lies on either side.  A group whose path leaves the window somewhere is found out (see `last`
-// below) and walked by Algorithm 3 instead.
+// codes lies on either side.  A path that leaves the window somewhere is found out (see `last` below); those
+// positions are searched in the count table's sections in global memory.
 //
 // Rows are taken in blocks of four positions.  A block's numbers are kept left-aligned: multiplied by the power
 // of two that brings the largest q of the block to the top of its `words` 32-bit words.  The top two words
@@ -14,14 +14,14 @@
 // as an fp32, truncated, they are the key that numbers a bucket.  From one block to the next q is shifted left by `delta` bits.
 //
 // Block b in memory (block_off[b], a multiple of 16 bytes):
-//     E        four rows, each `words` planes of `plane` 32-bit words: word w (lowest first) of
+//     E        four rows, each `words` planes of 64 (if its rows' windows allow) or `plane` 32-bit words: word w (lowest first) of
 //              entry m - 2 klo of the row, modulo 2^(32 words)
 //     buckets  four tables, 4 bytes a bucket: in the low byte m0, the local index of the first threshold
 //              that a q of the bucket can be at or below, above it the complement of the low 24 key bits of
 //              that threshold if it lies in the bucket (else zeros): the sum with a q's 24 key bits carries
 //              iff q's are larger, and leaves all ones iff they are the same.  The last entry
 //              of a table (index `last`) catches every key outside the window: m0 = 255, which makes the
-//              pulses left grow, and that is seen.
+//              pulses left grow, and that is seen.  (The read of E at 255 stays within the block.)
 #pragma once
 #include <memory>
 
@@ -30,7 +30,6 @@
 namespace pvq {
 
 constexpr int kWinRows = 128, kWinBlocks = kWinRows / 4;
-constexpr uint32_t kWinPad = 1024;  // bytes behind the last block that an out-of-window read may touch
 
 __host__ __device__ constexpr int win_key_words(int N) { return N > 64 ? 3 : 2; }
 
@@ -47,14 +46,18 @@ struct WinArgs {
     uint32_t block_off[kWinBlocks + 1];  // the last one: bytes in all
     uint32_t thr_off[kWinBlocks];
     uint32_t dlo4[kWinBlocks];           // klo of the position before minus klo of the position, a byte each
+    uint8_t narrow[kWinBlocks];          // planes of 64
     uint8_t delta[kWinBlocks];           // bits q is shifted left by when the block begins
+    uint8_t up[kWinBlocks];              // bits by which its numbers are multiplied
     uint8_t blocks_of[33];               // blocks_of[w]: blocks done in w words or more
+    int16_t klo[kWinRows];
+    uint32_t typical[12];                // q of a code whose path stays in the middle of the windows
     WinRow row[kWinRows];
 };
 
 struct WinTables {
     WinArgs args;
-    int plane;           // 96, 128, 160 or 192
+    int plane;           // 96, 112, 128, 160 or 192
     uint32_t max_block;  // bytes of the largest block
 };
 
