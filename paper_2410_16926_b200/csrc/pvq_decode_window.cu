@@ -53,6 +53,13 @@ __device__ __forceinline__ void win_entry(mp<PW>& e, uint32_t addr) {
     }
 }
 
+// A row's record (WinRow): x base, y last, z shift, w buckets.
+__device__ __forceinline__ uint4 win_record(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+
 // The key of q: its KW leading words as an fp32, every step rounded towards zero.
 template <int PW, int KW>
 __device__ __forceinline__ uint32_t win_key(const mp<PW>& v) {
@@ -92,11 +99,10 @@ __device__ __forceinline__ bool win_less(const uint32_t* t, int Wc, const uint32
 template <int PW, int PLANE, int KW>
 __device__ __noinline__ void win_exact4(WinExact<PW>& st, uint32_t acc, uint32_t stage, const WinArgs& t, int b, const uint32_t* blob, int N,
                                         int K, int Wc) {
-    const WinRow* rows = t.row + 4 * b;
 #pragma unroll 1
     for (int s = 3; s >= 0; --s) {  // back to where the block began
         mp<PW> e, d;
-        win_entry<PW, PLANE, 0>(e, stage + static_cast<uint32_t>(s) * (PW * PLANE * 4) + ((acc >> (8 * s)) & 0xffu) * 4u);
+        win_entry<PW, PLANE, 0>(e, stage + kWinHead + static_cast<uint32_t>(s) * (PW * PLANE * 4) + ((acc >> (8 * s)) & 0xffu) * 4u);
         mp_sub_borrow<PW>(d, st.v, e);
         st.v = d;
     }
@@ -107,23 +113,22 @@ __device__ __noinline__ void win_exact4(WinExact<PW>& st, uint32_t acc, uint32_t
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
         const int i = 4 * b + s, n = N - 1 - i;
-        const uint32_t key = win_key<PW, KW>(st.v);
-        const uint32_t x = min((key >> rows[s].shift) - rows[s].first, rows[s].last);
-        const uint32_t entry = win_load(stage + rows[s].buckets + x * 4u);
-        const uint32_t m0 = entry & 0xffu, sum = (key << 8) + entry;
+        const uint4 r = win_record(stage + 16u * static_cast<uint32_t>(s));
+        const uint32_t key = min(win_key<PW, KW>(st.v) - r.x, r.y);
+        const uint32_t sum = key + win_load(stage + r.w + ((key >> r.z) << 2));
         int left;
         bool odd;
-        if (st.over == 0u && x < rows[s].last) {
-            uint32_t m = m0 + (sum < entry ? 1u : 0u);
-            if (sum >= 0xffffff00u) {
-                const uint32_t* thr = reinterpret_cast<const uint32_t*>(t.thr + t.thr_off[b]) + s * PW * PLANE + m0;
+        if (st.over == 0u && key < r.y) {
+            uint32_t m = sum >> 24;
+            if ((sum | 0xff000000u) == 0xffffffffu) {
+                const uint32_t* thr = reinterpret_cast<const uint32_t*>(t.thr + t.thr_off[b]) + s * PW * PLANE + m;
                 mp<PW> th, d;
 #pragma unroll
                 for (int w = 0; w < PW; ++w) th.w[w] = __ldg(thr + w * PLANE);
-                m = m0 + (mp_sub_borrow<PW>(d, th, st.v) ? 1u : 0u);
+                m += mp_sub_borrow<PW>(d, th, st.v) ? 1u : 0u;
             }
             mp<PW> e;
-            win_entry<PW, PLANE, 0>(e, stage + static_cast<uint32_t>(s) * (PW * PLANE * 4) + m * 4u);
+            win_entry<PW, PLANE, 0>(e, stage + kWinHead + static_cast<uint32_t>(s) * (PW * PLANE * 4) + m * 4u);
             mp_add<PW>(st.v, e);
             left = t.klo[i] + static_cast<int>(m >> 1);
             odd = (m & 1u) != 0u;
@@ -179,45 +184,40 @@ struct WinState {
 };
 
 template <int PW, int PLANE, int KW, int S>
-__device__ __forceinline__ void win_position(mp<PW>& v, uint32_t& acc, uint32_t& top, uint32_t stage, const WinRow& r) {
-    const uint32_t key = win_key<PW, KW>(v);
-    const uint32_t x = min((key >> r.shift) - r.first, r.last);
-    const uint32_t entry = win_load(stage + r.buckets + (x << 2));
-    uint32_t sum, m;
-    asm("add.cc.u32 %0, %2, %3;\n\t"
-        "addc.u32 %1, %4, 0;"
-        : "=&r"(sum), "=r"(m)
-        : "r"(key << 8), "r"(entry), "r"(entry & 0xffu));
-    top = max(top, sum);
+__device__ __forceinline__ void win_position(mp<PW>& v, uint32_t& acc, uint32_t& top, uint32_t stage) {
+    const uint4 r = win_record(stage + 16u * S);
+    const uint32_t key = min(win_key<PW, KW>(v) - r.x, r.y);
+    const uint32_t sum = key + win_load(stage + r.w + ((key >> r.z) << 2));
+    top = max(top, sum | 0xff000000u);
+    acc = __byte_perm(acc, sum, 0x7321);
     mp<PW> e;
-    win_entry<PW, PLANE, S * PW>(e, stage + (m << 2));
+    win_entry<PW, PLANE, S * PW>(e, stage + kWinHead + ((sum >> 24) << 2));
     mp_add<PW>(v, e);
-    acc = __funnelshift_r(acc, m, 8);
 }
 
 template <int N, int PW, int PLANE, int KW, int W>
 __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, const BatchArgs& a, const WinArgs& t, int b, uint32_t y) {
     mp<PW> v;
     {
-        const uint32_t delta = t.delta[b];
+        const uint32_t delta = win_load_at<kWinDelta>(stage);
         st.over = __funnelshift_l(st.a[0], st.over, delta);
 #pragma unroll
         for (int j = 0; j < PW; ++j) v.w[PW - 1 - j] = __funnelshift_l(st.a[j + 1], st.a[j], delta);
         st.a[PW] = 0u;
     }
     uint32_t acc = 0u, top = 0u;
-    win_position<PW, PLANE, KW, 0>(v, acc, top, stage, t.row[4 * b]);
-    win_position<PW, PLANE, KW, 1>(v, acc, top, stage, t.row[4 * b + 1]);
-    win_position<PW, PLANE, KW, 2>(v, acc, top, stage, t.row[4 * b + 2]);
-    win_position<PW, PLANE, KW, 3>(v, acc, top, stage, t.row[4 * b + 3]);
+    win_position<PW, PLANE, KW, 0>(v, acc, top, stage);
+    win_position<PW, PLANE, KW, 1>(v, acc, top, stage);
+    win_position<PW, PLANE, KW, 2>(v, acc, top, stage);
+    win_position<PW, PLANE, KW, 3>(v, acc, top, stage);
     // |y|: pulses left before the position minus those left after it, a byte each: one sum, whose bytes do not
     // touch each other while all of them are 0..127 (else some bit 7 shows, unless the position before was out of the
     // window too, and then h shows it); y > 0 where the index is odd
     const uint32_t after = (acc >> 1) & 0x7f7f7f7fu;
-    const uint32_t mag = (after << 8) + t.dlo4[b] - after + static_cast<uint32_t>(st.h);
+    const uint32_t mag = (after << 8) + win_load_at<kWinDlo4>(stage) - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;
     uint32_t y4 = ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos);
-    if (__any_sync(kFull, top >= 0xffffff00u || (((mag | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
+    if (__any_sync(kFull, top == 0xffffffffu || (((mag | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
         WinExact<PW> x;
         x.v = v;
         x.over = st.over, x.h = st.h, x.ssy = st.ssy, x.lost = st.lost;
@@ -240,10 +240,7 @@ __device__ __forceinline__ void win_blocks(WinState<W>& st, const BatchArgs& a, 
 #pragma unroll 1
     for (; b < t.blocks_of[PW]; ++b) {
         const uint32_t stage = enter(b), yb = y + static_cast<uint32_t>(b) * 4u;
-        if (t.narrow[b])
-            win_block4<N, PW, 64, KW, W>(st, stage, a, t, b, yb);
-        else
-            win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
+        win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
         leave(b);
     }
     if constexpr (PW > 1) win_blocks<N, PW - 1, PLANE, KW, W>(st, a, t, b, y, enter, leave);
@@ -393,14 +390,16 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
     }
     const float sc = zeros ? 0.0f : __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(static_cast<int>(st.ssy))));
     // The warp writes the groups one after the other, 16 bytes a lane: whole lines.
-    const unsigned long long at = done ? 0ull : reinterpret_cast<unsigned long long>(out);
+    const uint32_t at = done ? 0xffffffffu : static_cast<uint32_t>((static_cast<size_t>(row) * m.ld_out + static_cast<size_t>(g) * N) >> 3);
+    uint4* base = static_cast<uint4*>(m.out);
     __syncwarp();
-#pragma unroll 1
-    for (int p = 0; p < N / 8; ++p) {
-        const int piece = p * 32 + lane, from = piece / (N / 8), sub = piece % (N / 8);
+    constexpr int PIECES = N / 8;  // lanes that share a group
+    const uint32_t sub = static_cast<uint32_t>(lane) % PIECES;
+    uint32_t src = slots + static_cast<uint32_t>(lane / PIECES) * YS + sub * 8u;
+#pragma unroll 2
+    for (int from = lane / PIECES; from < 32; from += 32 / PIECES, src += 32 / PIECES * YS) {
         const float s = __shfl_sync(kFull, sc, from);
-        const unsigned long long dst = __shfl_sync(kFull, at, from);
-        const uint32_t src = slots + static_cast<uint32_t>(from) * YS + static_cast<uint32_t>(sub) * 8u;
+        const uint32_t dst = __shfl_sync(kFull, at, from);
         const uint32_t lo = win_load(src), hi = win_load_at<4>(src);
         float f[8];
 #pragma unroll
@@ -408,9 +407,8 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
             f[e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
             f[4 + e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
         }
-        if (dst != 0ull)
-            reinterpret_cast<uint4*>(dst)[sub] =
-                make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+        if (dst != 0xffffffffu)
+            base[dst + sub] = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
     }
     __syncwarp();  // the slots are free
 }
@@ -541,7 +539,7 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
     std::memset(&g, 0, sizeof g);
     const uint32_t all = t.args.block_off[N / 4], ys = N + 4;
     const uint32_t limit = static_cast<uint32_t>(di.smem_max);
-    const bool resident = N <= 64 && all + 512u * ys <= limit;
+    const bool resident = N == 64 && PLANE == 96 && all + 512u * ys <= limit;
     const int most = resident ? 32 : 28;
     int warps = 0;
     double best = -1.0;
@@ -578,7 +576,7 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
     if (smem > limit) return PVQ_ERR_UNSUPPORTED;
     const int threads = warps * 32 + (resident ? 0 : 32);
     auto kern = decode_window_stream_kernel<N, W, PLANE>;
-    if constexpr (N <= 64) {
+    if constexpr (N == 64 && PLANE == 96) {
         if (resident) kern = decode_window_kernel<N, W, PLANE>;
     }
     int per_sm = 0;
@@ -590,14 +588,8 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
 
 template <int N, int W>
 int launch_window_w(BatchArgs& a, const WinTables& t, cudaStream_t s) {
-    switch (t.plane) {
-        case 96: return launch_window_t<N, W, 96>(a, t, s);
-        case 112: return launch_window_t<N, W, 112>(a, t, s);
-        case 128: return launch_window_t<N, W, 128>(a, t, s);
-        case 160: return launch_window_t<N, W, 160>(a, t, s);
-        case 192: if constexpr (N == 64) return launch_window_t<N, W, 192>(a, t, s);
-        default: return PVQ_ERR_UNSUPPORTED;
-    }
+    if constexpr (N == 64) return t.plane == 96 ? launch_window_t<N, W, 96>(a, t, s) : launch_window_t<N, W, 192>(a, t, s);
+    return launch_window_t<N, W, N == 64 ? 192 : 160>(a, t, s);
 }
 
 #endif
@@ -613,6 +605,7 @@ int launch_decode_window(const BatchArgs& args, int N, int W, cudaStream_t strea
     for (int i = 0; i < a.count; ++i) {
         a.m[i].tile_begin = tiles;
         tiles += static_cast<unsigned>((a.m[i].rows * a.m[i].G + 31) / 32);
+        if (a.m[i].rows * a.m[i].ld_out >= (1ll << 35) - 8) return PVQ_ERR_UNSUPPORTED;  // 32 bits number its 16-byte pieces
     }
     a.total_tiles = tiles;
     switch (N * 16 + W) {

@@ -421,6 +421,10 @@ int run_batch(const pvq_matrix_desc* descs, int count, int need, int dtype, int 
         st = launch_decode_window(a, c.N, c.W, s);
         if (st != PVQ_ERR_UNSUPPORTED) return st;
     }
+    if (kind == 0 && rot_block == 0) {
+        st = launch_encode_window(a, dtype, c.N, c.W, s);
+        if (st != PVQ_ERR_UNSUPPORTED) return st;
+    }
     if (c.W > fast_words) {  // large groups, wide codes
         return launch_big(a, dtype, c.N, c.W, kind == 1, s);
     }

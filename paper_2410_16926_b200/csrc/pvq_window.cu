@@ -98,12 +98,12 @@ struct Builder {
     int before(int i) const { return i > 0 ? hi[i - 1] : K; }
 
     // Fills t, data and thr for the current windows; false: cannot be done.
-    bool layout(const int wide_plane) {
+    bool layout(const int plane) {
         const int blocks = N / 4;
         bits.assign(blocks, 0);
         words.assign(blocks, 0);
         std::memset(&t, 0, sizeof t);
-        t.plane = wide_plane;
+        t.plane = plane;
         data.clear();
         thr.clear();
         std::vector<int> last_m(N);
@@ -121,17 +121,14 @@ struct Builder {
             if (words[b] > 32) return false;
             for (int w = 0; w <= words[b]; ++w) ++t.args.blocks_of[w];
             const int delta = (b > 0 ? bits[b - 1] : 32 * words[0]) - bits[b];
-            t.args.delta[b] = static_cast<uint8_t>(delta);
             const int W = words[b], up = 32 * W - bits[b], kw = std::min(W, win_key_words(N));
-            bool narrow = true;
-            for (int i = 4 * b; i < 4 * b + 4; ++i) narrow = narrow && last_m[i] - 2 * lo[i] + 1 <= 64;
-            const int plane = narrow ? 64 : wide_plane;
-            t.args.narrow[b] = narrow;
             t.args.up[b] = static_cast<uint8_t>(up);
             const size_t at = data.size(), planes = static_cast<size_t>(4) * W * plane;
             t.args.block_off[b] = static_cast<uint32_t>(at * 4);
             t.args.thr_off[b] = static_cast<uint32_t>(thr.size() * 4);
-            data.resize(at + planes, 0u);
+            const size_t e_at = at + kWinHead / 4;
+            data.resize(e_at + planes, 0u);
+            uint32_t dlo4 = 0, klo4 = 0, width4 = 0;
             const size_t tat = thr.size();
             thr.resize(tat + planes, 0u);
             for (int s = 0; s < 4; ++s) {
@@ -140,7 +137,9 @@ struct Builder {
                 // |y| and the sums of the packed arithmetic stay below 256, and an out-of-window index always shows
                 if (dlo < 0 || dlo > 127 || before(i) - lo[i] >= 127 || last_m[i] - 2 * lo[i] + 1 > plane) return false;
                 t.args.klo[i] = static_cast<int16_t>(lo[i]);
-                t.args.dlo4[b] |= static_cast<uint32_t>(dlo) << (8 * s);
+                klo4 |= static_cast<uint32_t>(lo[i]) << (8 * (3 - s));
+                width4 |= static_cast<uint32_t>(hi[i] - lo[i]) << (8 * (3 - s));
+                dlo4 |= static_cast<uint32_t>(dlo) << (8 * s);
                 std::vector<uint32_t> key;
                 const bool below = lo[i] > 0;
                 if (below) key.push_back(aligned_key(threshold(n, 2 * lo[i] - 1), bits[b], kw));
@@ -152,7 +151,7 @@ struct Builder {
                     for (int w = 0; w < W; ++w) {
                         const size_t o = (static_cast<size_t>(s) * W + w) * plane + (m - 2 * lo[i]);
                         carry += static_cast<uint32_t>(~word_at(M, 32 * w - up));
-                        data[at + o] = static_cast<uint32_t>(carry);
+                        data[e_at + o] = static_cast<uint32_t>(carry);
                         carry >>= 32;
                         thr[tat + o] = word_at(T, 32 * w - up);
                     }
@@ -166,27 +165,32 @@ struct Builder {
                     if (distinct) shift = 23 - f;
                 }
                 if (shift < 0) return false;
-                WinRow& r = t.args.row[i];
-                r.buckets = static_cast<uint32_t>((data.size() - at) * 4);
-                r.shift = static_cast<uint32_t>(shift);
-                r.first = (key[0] >> shift) + (below ? 1u : 0u);
-                r.last = (key.back() >> shift) - r.first + (closed[i] ? 1u : 0u);
+                const uint32_t first = (key[0] >> shift) + (below ? 1u : 0u);
+                const uint32_t many = (key.back() >> shift) - first + (closed[i] ? 1u : 0u);
+                const WinRow r = {first << shift, many << shift, static_cast<uint32_t>(shift), static_cast<uint32_t>((data.size() - at) * 4)};
+                std::memcpy(&data[at + 4 * s], &r, sizeof r);
                 uint32_t m0 = 0;
-                for (uint32_t x = 0; x < r.last; ++x) {
+                for (uint32_t x = 0; x < many; ++x) {
                     const uint32_t k = key[m0 + (below ? 1 : 0)];
-                    uint32_t e = m0;
-                    if ((k >> shift) == r.first + x) {
+                    uint32_t e = (m0 - ((x << shift) >> 24)) << 24;
+                    if ((k >> shift) == first + x) {
                         // an integer below 2^23 is its key: half a step more, and equal keys need no further look
                         const bool exact = bits[b] <= 32 * kw && threshold(n, 2 * lo[i] + static_cast<int>(m0)).bit_length() < 23;
-                        e |= ~((k + (exact ? 1u : 0u)) & 0xffffffu) << 8;
+                        e |= ~(k + (exact ? 1u : 0u) - r.base) & 0xffffffu;
                         ++m0;
                     }
                     data.push_back(e);
                 }
-                data.push_back(0xffu);
+                data.push_back((255u - (r.last >> 24)) << 24);
             }
+            data[at + kWinDlo4 / 4] = dlo4;
+            data[at + kWinDelta / 4] = static_cast<uint32_t>(delta);
+            data[at + kWinKlo4 / 4] = klo4;
+            data[at + kWinWidth4 / 4] = width4;
+            t.args.words[b] = static_cast<uint8_t>(W);
+            t.max_rows = std::max(t.max_rows, win_rows_bytes(W, plane));
             // (an out-of-window index reads up to 256 entries from the start of a plane)
-            while ((data.size() & 3u) || data.size() < at + planes + 256 - plane) data.push_back(0u);
+            while ((data.size() & 3u) || data.size() < e_at + planes + 256 - plane) data.push_back(0u);
             t.max_block = std::max(t.max_block, static_cast<uint32_t>((data.size() - at) * 4));
         }
         t.args.block_off[blocks] = static_cast<uint32_t>(data.size() * 4);
@@ -201,18 +205,14 @@ struct Builder {
         return words[0] <= 12;
     }
 
-    // The widest windows (the smallest share outside) whose tables fit beside the output slots of 30 warps (group size
-    // 64); where none does, the tables are streamed, and the widest that 160 (or 192) entries a row hold are taken.
+    // The widest windows (the smallest share outside) whose tables fit beside the output slots of 32 warps (N = 64); where
+    // none does, the tables are streamed, and the widest are taken that 160 (192 at N = 64) entries a row hold.
     bool choose(uint32_t smem_max) {
-        const uint32_t room = smem_max - 128u - 30u * 32u * (N + 4);
-        for (int streamed = N > 64 ? 1 : 0; streamed < 2; ++streamed)
-            for (double eps : {1e-9, 3e-9, 1e-8, 3e-8, 1e-7, 3e-7, 1e-6, 3e-6, 1e-5, 3e-5, 1e-4, 3e-4, 1e-3}) {
-                const int entries = windows(eps);
-                for (int plane : {96, 112, 128, 160, 192})
-                    if (entries <= plane) {
-                        if ((plane < 192 || N == 64) && layout(plane) && (streamed || t.args.block_off[N / 4] <= room)) return true;
-                        break;
-                    }
+        const uint32_t room = smem_max - 128u - 32u * 32u * (N + 4);
+        for (int plane : {96, N == 64 ? 192 : 160})
+            for (double eps : {1e-8, 3e-8, 1e-7, 3e-7, 1e-6, 3e-6, 1e-5, 3e-5, 1e-4, 3e-4, 1e-3}) {
+                if (plane == 96 && N > 64) break;
+                if (windows(eps) <= plane && layout(plane) && (plane != 96 || t.args.block_off[N / 4] <= room)) return true;
             }
         return false;
     }
@@ -247,8 +247,8 @@ std::shared_ptr<const WinTables> window_tables(int N, int K) {
 
 void build_window_tables(int N, int K, cudaStream_t stream) {
     const int W = code_words_for(N, K);
-    // the settings with a kernel: group sizes 64 and 128, codes of up to 8 and 12 words
-    if (!((N == 64 && W >= 5 && W <= 8) || (N == 128 && W >= 9 && W <= 12)) || count_fills_its_words(N, K)) return;
+    // the settings with a kernel: codes of 5 to 8 words at group size 64, 9 to 12 at 128
+    if (!((N == 64 && W >= 5 && W <= 8) || (N == 128 && W >= 9 && W <= 12)) || K > 255 || count_fills_its_words(N, K)) return;
     int dev = 0;
     DeviceInfo di;
     if (cudaGetDevice(&dev) != cudaSuccess || device_info(&di) != PVQ_OK) return;

@@ -1,4 +1,4 @@
-// Windowed search tables of the decoder for wide codes (pvq_decode_window.cu): layout and host interface.
+// Windowed tables for wide codes (pvq_decode_window.cu, pvq_encode_window.cu): layout and host interface.
 //
 // As in SearchLayout, with q = N(n+1,k) - r the coordinate of a position (n dimensions behind it) follows
 // from where q falls among the thresholds T_n[2k'] = N(n+1,k'), T_n[2k'+1] = N(n+1,k') + N(n,k'), and the next
@@ -14,14 +14,18 @@
 // as an fp32, truncated, they are the key that numbers a bucket.  From one block to the next q is shifted left by `delta` bits.
 //
 // Block b in memory (block_off[b], a multiple of 16 bytes):
-//     E        four rows, each `words` planes of 64 (if its rows' windows allow) or `plane` 32-bit words: word w (lowest first) of
+//     head     four 16-byte records (WinRow), one a row; then four words: klo of the position before minus klo of the
+//              position, a byte each (first position lowest); delta; klo and khi - klo, a byte each (first
+//              position highest, as the encoder's points are packed)
+//     E        four rows, each `words` planes of `plane` 32-bit words: word w (lowest first) of
 //              entry m - 2 klo of the row, modulo 2^(32 words)
-//     buckets  four tables, 4 bytes a bucket: in the low byte m0, the local index of the first threshold
-//              that a q of the bucket can be at or below, above it the complement of the low 24 key bits of
-//              that threshold if it lies in the bucket (else zeros): the sum with a q's 24 key bits carries
-//              iff q's are larger, and leaves all ones iff they are the same.  The last entry
-//              of a table (index `last`) catches every key outside the window: m0 = 255, which makes the
-//              pulses left grow, and that is seen.  (The read of E at 255 stays within the block.)
+//     buckets  four tables, 4 bytes a bucket, indexed by the key relative to `base` (its low 24 bits are c, the rest
+//              is the same for the whole bucket).  With m0 the local index of the first threshold that a q of the bucket
+//              can be at or below, and c0 that threshold's c if it lies in the bucket (else all ones): the entry is what added
+//              to the relative key leaves m0 in the top byte, plus one iff c > c0, and all ones in the other
+//              three iff c = c0.  The last entry of a table catches every key outside the window (relative
+//              keys are cut off at `last`): it leaves 255, which makes the pulses left grow, and that is
+//              seen.  (The read of E at 255 stays within the block.)
 #pragma once
 #include <memory>
 
@@ -34,32 +38,35 @@ constexpr int kWinRows = 128, kWinBlocks = kWinRows / 4;
 __host__ __device__ constexpr int win_key_words(int N) { return N > 64 ? 3 : 2; }
 
 struct WinRow {
+    uint32_t base;     // key of the first bucket's start
+    uint32_t last;     // relative key of the entry for keys outside the window
+    uint32_t shift;    // relative key >> shift is the bucket
     uint32_t buckets;  // byte offset of the row's bucket table in its block
-    uint32_t first;    // number of its first bucket
-    uint32_t last;     // index of the entry for keys outside the window
-    uint32_t shift;    // key >> shift is the bucket number
 };
+constexpr uint32_t kWinHead = 96;  // bytes of a block's head
+constexpr uint32_t kWinDlo4 = 64, kWinDelta = 68, kWinKlo4 = 72, kWinWidth4 = 76;
 
 struct WinArgs {
     const uint8_t* data;
     const uint8_t* thr;                  // thresholds (aligned), laid out like E; read when key bits are the same
     uint32_t block_off[kWinBlocks + 1];  // the last one: bytes in all
     uint32_t thr_off[kWinBlocks];
-    uint32_t dlo4[kWinBlocks];           // klo of the position before minus klo of the position, a byte each
-    uint8_t narrow[kWinBlocks];          // planes of 64
-    uint8_t delta[kWinBlocks];           // bits q is shifted left by when the block begins
     uint8_t up[kWinBlocks];              // bits by which its numbers are multiplied
+    uint8_t words[kWinBlocks];
     uint8_t blocks_of[33];               // blocks_of[w]: blocks done in w words or more
     int16_t klo[kWinRows];
     uint32_t typical[12];                // q of a code whose path stays in the middle of the windows
-    WinRow row[kWinRows];
 };
 
 struct WinTables {
     WinArgs args;
-    int plane;           // 96, 112, 128, 160 or 192
+    int plane;           // entries of a plane: 96 (N = 64, tables that fit shared memory) or 192 (others), 160 (N = 128)
     uint32_t max_block;  // bytes of the largest block
+    uint32_t max_rows;   // ... of its head and its four rows of E
 };
+
+// Bytes of a block's head and E, which is all that the encoder reads.
+__host__ __device__ constexpr uint32_t win_rows_bytes(int words, int plane) { return kWinHead + 16u * words * plane; }
 
 // The tables for (N,K) on the current device, or null (never built here, or no such kernel).  The holder keeps them
 // from being freed until its launch is enqueued; freeing waits for the kernels that read them.
@@ -71,5 +78,6 @@ void build_window_tables(int N, int K, cudaStream_t stream);
 
 // PVQ_ERR_UNSUPPORTED: no tables or no kernel for it; the caller walks
 int launch_decode_window(const BatchArgs& args, int N, int W, cudaStream_t stream);
+int launch_encode_window(const BatchArgs& args, int dtype, int N, int W, cudaStream_t stream);
 
 }  // namespace pvq
