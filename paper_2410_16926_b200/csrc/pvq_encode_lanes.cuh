@@ -30,26 +30,35 @@
 
 namespace pvq {
 
-// threads per block: the wide kernels' accumulators need more registers
+// threads per block: the wide kernels' accumulators need more registers.  (4096 x 4096, N = 32, 96 bits: 768 threads
+// 41.8 us, 896 threads 37.6 us.)
 template <int W>
-constexpr int kLaneThreads = W <= 16 ? 768 : 512;
+constexpr int kLaneThreads = W <= 4 ? 896 : (W <= 16 ? 768 : 512);
 constexpr int kSplitBit = 48;
 
 struct LaneGeom {
     int team, teams;                // threads per team, teams per block
-    uint32_t team_off, team_bytes;  // the teams' areas: [2 input buffers][2 x energies][2 x LS amplitudes][2 x index words]
+    uint32_t team_off, team_bytes;  // the teams' areas: [2 input buffers], then one (a team of one warp) or two each of [energies][LS amplitudes][index words]
     uint32_t in_bytes;              // of one input buffer
     uint32_t ss_off, amp_off, idx_off;  // inside a team's area
     int ss_floats, idx_words;       // per buffer
+    int wide_blocks;                // blocks of four positions with entries of 2^48 and more (two and three words)
     float minus_zero;
 };
 
-// The staged table: rows by position, RE entries (a power of two that holds 2 K + 2) of 4, 8 or 16 bytes;
-// two and three words: a plane of lower halves, then one of upper halves (the first `wide` positions).
+// The staged table: rows by position, RE entries (64, 112, 128 or 256, the first that holds 2 K + 2) of 4, 8 or 16 bytes;
+// two and three words: a plane of lower halves, then one of upper halves for the first wide_blocks * 4 positions
+// (for all positions where a group has two lanes, both of which run through as many blocks).
 template <int W>
 constexpr int kLaneEntry = W == 1 ? 4 : (W <= 3 ? 8 : 16);
+template <int N>
+__host__ __device__ constexpr int lane_upper_rows(int wide_blocks) {
+    return N <= 32 ? wide_blocks * 4 : N;
+}
 template <int N, int W, int RE>
-constexpr int kLaneTableBytes = N * RE * kLaneEntry<W> * (W == 2 || W == 3 ? 2 : 1);
+__host__ __device__ constexpr int lane_table_bytes(int wide_blocks) {
+    return N * RE * kLaneEntry<W> + (W == 2 || W == 3 ? lane_upper_rows<N>(wide_blocks) * RE * 8 : 0);
+}
 
 // bytes from one lane's values in an input buffer to the next lane's
 template <int E, bool BF16>
@@ -84,16 +93,14 @@ __device__ __forceinline__ T lane_entry(const uint8_t* p) {
     return *reinterpret_cast<const T*>(p);
 }
 
-// Stages the tables: entry (i, m) from the blob's telescoped word planes.  wide_blocks: how many blocks
-// of four positions (from the first) have entries of 2^48 and more.  A barrier has to follow.
+// Stages the tables: entry (i, m) from the blob's telescoped word planes.  A barrier has to follow.
 template <int N, int W, int RE>
-__device__ __forceinline__ void stage_lane_table(uint8_t* tab, const uint32_t* blob, const TableLayout& L, int K, int* wide_blocks) {
+__device__ __forceinline__ void stage_lane_table(uint8_t* tab, const uint32_t* blob, const TableLayout& L, int K, int wide_blocks) {
     constexpr int TW = W <= 2 ? W : 4;
     // entry by entry, several loads in flight: a small launch consists mostly of this
-    int wide = 0;
 #pragma unroll 4
     for (int e = threadIdx.x; e < N * RE; e += blockDim.x) {
-        const int i = e / RE, m = e & (RE - 1);
+        const int i = e / RE, m = e - i * RE;
         if (m >= 2 * K + 2) continue;
         const uint32_t* src = blob + ((m & 1) ? L.cenc_off[1] : L.cenc_off[0]) / 4 + static_cast<size_t>(i) * TW * L.crow + (m >> 1);
         uint32_t w[4] = {0u, 0u, 0u, 0u};
@@ -112,15 +119,10 @@ __device__ __forceinline__ void stage_lane_table(uint8_t* tab, const uint32_t* b
             const unsigned long long low = static_cast<unsigned long long>(neg.w[0]) | (static_cast<unsigned long long>(neg.w[1]) << 32);
             const unsigned long long up = (low >> kSplitBit) | (static_cast<unsigned long long>(W == 3 ? neg.w[W - 1] : 0u) << (64 - kSplitBit));
             *reinterpret_cast<double*>(dst) = static_cast<double>(low & ((1ull << kSplitBit) - 1ull));
-            *reinterpret_cast<double*>(dst + N * RE * 8) = static_cast<double>(up);
-            if (up != 0) wide = max(wide, i / 4 + 1);
+            if (i < lane_upper_rows<N>(wide_blocks)) *reinterpret_cast<double*>(dst + N * RE * 8) = static_cast<double>(up);
         } else {
             *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         }
-    }
-    if constexpr (W == 2 || W == 3) {
-        const unsigned all = __reduce_max_sync(kFull, static_cast<unsigned>(wide));
-        if ((threadIdx.x & 31) == 0) atomicMax(wide_blocks, static_cast<int>(all));
     }
 }
 
@@ -390,7 +392,6 @@ template <int E, int L, int W, int RE, bool BF16, bool LS>
 __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const __grid_constant__ BatchArgs a,
                                                                            const __grid_constant__ LaneGeom g) {
     extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ int s_wide_blocks;
     __shared__ uint8_t s_words[RE == 0 ? E * L : 1];
     constexpr int N = E * L;
     constexpr bool GLOBAL = RE == 0;
@@ -407,13 +408,11 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
     at.ch = 0;
     const unsigned stride = gridDim.x * static_cast<unsigned>(g.teams);
     const bool works = team < g.teams && at.tile < a.total_tiles;
-    if (!GLOBAL && threadIdx.x == 0) s_wide_blocks = 0;
     if (works) {
         enter_matrix(a, at, find_matrix(a, at.tile), tid, L);
         uint32_t* s_idx2 = reinterpret_cast<uint32_t*>(area + g.idx_off);
-        for (int i = tid; i < 2 * g.idx_words; i += T) s_idx2[i] = 0u;
+        for (int i = tid; i < (T == 32 ? 1 : 2) * g.idx_words; i += T) s_idx2[i] = 0u;
     }
-    __syncthreads();  // s_wide_blocks
     grid_dependency_wait();
     if (works) request_input<E, L, BF16>(a, at, shared_addr(area), T, tid);
     mp<GLOBAL ? 1 : W> start;
@@ -430,16 +429,16 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
         debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
 #endif
     } else {
-        stage_lane_table<N, W, GLOBAL ? 64 : RE>(smem, a.table, TL, K, &s_wide_blocks);
+        stage_lane_table<N, W, GLOBAL ? 64 : RE>(smem, a.table, TL, K, g.wide_blocks);
 #pragma unroll
         for (int w = 0; w < W; ++w) start.w[GLOBAL ? 0 : w] = a.table[TL.start_off / 4 + w];
 #ifdef PVQ_DEBUG
-        debug_begin(shared_addr(smem), shared_addr(smem) + kLaneTableBytes<N, W, RE>, 0u, 0u, 0u, a.debug_status);
+        debug_begin(shared_addr(smem), shared_addr(smem) + lane_table_bytes<N, W, GLOBAL ? 64 : RE>(g.wide_blocks), 0u, 0u, 0u, a.debug_status);
 #endif
     }
     __syncthreads();  // the tables; from here on the teams go their own way
     if (!works) return;
-    const int wide_blocks = !GLOBAL && (W == 2 || W == 3) ? s_wide_blocks : 0;
+    const int wide_blocks = g.wide_blocks;
 
     int in_buf = 0, buf = 0;
     int done_mi = -1;  // matrix of the tile before, whose index words are still to be written out
@@ -569,6 +568,13 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
             atomicOr(s_idx + word, static_cast<uint32_t>(q) << sh);
             if (sh + b > 32u) atomicOr(s_idx + word + 1, static_cast<uint32_t>(q) >> (32u - sh));
         }
+        if (T == 32) {  // no other warp to wait for: out with the index words, and the same buffers again
+            __syncwarp();
+            flush_index_words(m, cur.tile, s_idx, T, tid);
+            __syncwarp();
+            if (!more) break;
+            continue;
+        }
         done_mi = cur.mi;
         if (!more) {
             team_barrier(team, T);  // the last tile's index words are complete
@@ -589,7 +595,8 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
     if (st != PVQ_OK) return st;
     LaneGeom g;
     g.minus_zero = -0.0f;
-    g.team_off = RE == 0 ? 0u : (static_cast<uint32_t>(kLaneTableBytes<N, W, RE>) + 127u) & ~127u;
+    g.wide_blocks = RE != 0 && (W == 2 || W == 3) ? (positions_from(N, a.K, kSplitBit) + 3) / 4 : 0;
+    g.team_off = RE == 0 ? 0u : (static_cast<uint32_t>(lane_table_bytes<N, W, RE == 0 ? 64 : RE>(g.wide_blocks)) + 127u) & ~127u;
 
     // Team size: the one whose rounds of tiles cost least.  A chunk costs about as much as six times
     // what a tile adds (energies, amplitude indices), eight with a barrier between warps; what
@@ -616,10 +623,11 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
         c.in_bytes = (static_cast<uint32_t>(t) * kLaneRun<E, BF16> + 15u) & ~15u;
         c.ss_floats = (ss_floats + 3) & ~3;
         c.idx_words = idx_words;
+        const uint32_t bufs = t == 32 ? 1u : 2u;
         c.ss_off = 2u * c.in_bytes;
-        c.amp_off = c.ss_off + 2u * static_cast<uint32_t>(c.ss_floats) * 4u;
-        c.idx_off = c.amp_off + (LS ? 2u * static_cast<uint32_t>(c.ss_floats) * 4u : 0u);
-        c.team_bytes = (c.idx_off + 2u * static_cast<uint32_t>(idx_words) * 4u + 127u) & ~127u;
+        c.amp_off = c.ss_off + bufs * static_cast<uint32_t>(c.ss_floats) * 4u;
+        c.idx_off = c.amp_off + (LS ? bufs * static_cast<uint32_t>(c.ss_floats) * 4u : 0u);
+        c.team_bytes = (c.idx_off + bufs * static_cast<uint32_t>(idx_words) * 4u + 127u) & ~127u;
         // as many teams as the threads, the shared memory and (larger than a warp) the named barriers hold
         long long teams = std::min(kLaneThreads<W> / t, t == 32 ? 32 : 15);
         teams = std::min(teams, (static_cast<long long>(di.smem_max) - c.team_off) / c.team_bytes);
@@ -668,7 +676,10 @@ static int launch_encode_lanes(BatchArgs& a, cudaStream_t s) {
     const bool ls = a.amp_mode == 1;
     switch (L0.crow) {
         case 32: return ls ? launch_encode_lanes_t<E, L, W, 64, BF16, true>(a, s) : launch_encode_lanes_t<E, L, W, 64, BF16, false>(a, s);
-        case 64: return ls ? launch_encode_lanes_t<E, L, W, 128, BF16, true>(a, s) : launch_encode_lanes_t<E, L, W, 128, BF16, false>(a, s);
+        case 64:
+            if (2 * a.K + 2 <= 112)
+                return ls ? launch_encode_lanes_t<E, L, W, 112, BF16, true>(a, s) : launch_encode_lanes_t<E, L, W, 112, BF16, false>(a, s);
+            return ls ? launch_encode_lanes_t<E, L, W, 128, BF16, true>(a, s) : launch_encode_lanes_t<E, L, W, 128, BF16, false>(a, s);
         case 128: return ls ? launch_encode_lanes_t<E, L, W, 256, BF16, true>(a, s) : launch_encode_lanes_t<E, L, W, 256, BF16, false>(a, s);
         default: return PVQ_ERR_UNSUPPORTED;
     }

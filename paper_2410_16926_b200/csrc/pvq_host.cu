@@ -99,6 +99,20 @@ int code_words_for(int N, int K) {
     return W;
 }
 
+int positions_from(int N, int K, int bits) {  // memoised like code_words_for
+    static std::mutex mu;
+    static std::map<std::tuple<int, int, int>, int> memo;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = memo.find({N, K, bits});
+    if (it != memo.end()) return it->second;
+    CountColumn c(N);
+    bool ok = true;
+    for (int k = 0; k < K && ok; ++k) ok = c.advance();
+    int n = 0;  // dimensions that stay below
+    while (ok && n < N && c.col[static_cast<size_t>(n + 1)].bit_length() <= bits) ++n;
+    return memo[{N, K, bits}] = ok ? N - n : N;
+}
+
 bool count_fills_its_words(int N, int K) {  // memoised like code_words_for: the count takes a while for large (N,K)
     static std::mutex mu;
     static std::map<std::pair<int, int>, bool> memo;
