@@ -143,7 +143,7 @@ __device__ __forceinline__ void store_y4(uint32_t addr, uint32_t val) {
 // `rec` is the shared address of the record of the first of the four rows (the rows of the
 // following positions have the records before it); a record is read once for all chains.
 // `t_rows` plus the shared address of a row of E is the global address of the same row of T.
-// The four y_i + 128 of chain j go to the word at y + j * ychain.
+// The four y_i + 128 of chain j go to the word at y + j * ychain, their squares to ssy[j].
 //
 // Per position: the key of q selects a bucket; its entry is m0 and the low key bits of the
 // threshold T[m0]; q's own low key bits being larger means q > T[m0], smaller means q <= T[m0]
@@ -151,7 +151,7 @@ __device__ __forceinline__ void store_y4(uint32_t addr, uint32_t val) {
 // that is rare, the threads of the warp whose bits were equal compare q with T[m0] in full.
 template <int W, int PW, int GP, int PLANE>
 __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, const uint8_t* t_rows,
-                                              uint32_t y, uint32_t ychain) {
+                                              uint32_t y, uint32_t ychain, uint32_t (&ssy)[GP]) {
     uint32_t acc[GP];  // the four threshold indices m, a byte each, first position lowest
     mp<PW> v[GP];      // the low PW words of q: the rest is zero by now
 #pragma unroll
@@ -208,6 +208,7 @@ __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP],
         const uint32_t after = (acc[j] >> 1) & 0x7f7f7f7fu;
         const uint32_t before = (after << 8) | k[j];
         const uint32_t mag = before - after;
+        ssy[j] = __dp4a(mag, mag, ssy[j]);
         const uint32_t odd = acc[j] & 0x01010101u;
         const uint32_t pos = (odd << 8) - odd;  // 0xff in the bytes with y > 0
         store_y4(y + static_cast<uint32_t>(j) * ychain,
@@ -222,25 +223,25 @@ __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP],
 // row records (absolute shared addresses by now), cnt[w] the number of rows done in w words.
 template <int N, int W, int GP, int PLANE>
 __device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t recs, const uint8_t* t_rows,
-                                             const int (&cnt)[5], uint32_t y, uint32_t ychain) {
+                                             const int (&cnt)[5], uint32_t y, uint32_t ychain, uint32_t (&ssy)[GP]) {
     uint32_t k[GP];
 #pragma unroll
     for (int j = 0; j < GP; ++j) k[j] = static_cast<uint32_t>(K);
     uint32_t rec = recs + static_cast<uint32_t>(N - 1) * 16u;
     if constexpr (W >= 4) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4<W, 4, GP, PLANE>(q, k, rec, t_rows, y, ychain);
+        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4<W, 4, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
     }
     if constexpr (W >= 3) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4<W, 3, GP, PLANE>(q, k, rec, t_rows, y, ychain);
+        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4<W, 3, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
     }
     if constexpr (W >= 2) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4<W, 2, GP, PLANE>(q, k, rec, t_rows, y, ychain);
+        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4<W, 2, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
     }
 #pragma unroll 1
-    for (int b = 0; b < cnt[1]; b += 4, rec -= 64u, y += 4u) search_block4<W, 1, GP, PLANE>(q, k, rec, t_rows, y, ychain);
+    for (int b = 0; b < cnt[1]; b += 4, rec -= 64u, y += 4u) search_block4<W, 1, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
 }
 
 }  // namespace pvq

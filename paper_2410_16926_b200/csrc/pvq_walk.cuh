@@ -1065,29 +1065,10 @@ __device__ __forceinline__ void walk_code(mp<W>& c, const WalkTables& t, int K, 
     }
 }
 
-// After walk_code: scale this thread's point to the unit sphere times `amp` and write its N
-// values as bf16 with 16-byte stores (row `row`, group `g` of matrix m).  Each thread writes
-// its own N*2 contiguous bytes; the threads of a warp hold consecutive groups, so a warp
-// fills a contiguous stretch of the row.
+// This thread's point times `sc`, as bf16, with 16-byte stores (row `row`, group `g` of matrix m).
 template <int N, typename YT>
-__device__ __forceinline__ void emit_group(const MatrixArgs& m, const YT* yslots, float amp, unsigned row,
-                                           unsigned g) {
+__device__ __forceinline__ void emit_scaled(const MatrixArgs& m, const YT* yslots, float sc, unsigned row, unsigned g) {
     const uint32_t* y4 = reinterpret_cast<const uint32_t*>(yslots);
-    int ssy = 0;
-    if constexpr (sizeof(YT) == 1) {
-        // slots hold b = y + 128:  sum y^2 = sum b^2 - 256 sum b + 128^2 N
-        unsigned sq = 0, su = 0;
-#pragma unroll
-        for (int v = 0; v < N / 4; ++v) {
-            sq = __dp4a(y4[v], y4[v], sq);
-            su = __dp4a(y4[v], 0x01010101u, su);
-        }
-        ssy = static_cast<int>(sq) - 256 * static_cast<int>(su) + 16384 * N;
-    } else {
-#pragma unroll 8
-        for (int v = 0; v < N; ++v) ssy += static_cast<int>(yslots[v]) * static_cast<int>(yslots[v]);
-    }
-    const float sc = __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(ssy)));
     if (!PVQ_DEBUG_INDEX(static_cast<long long>(row), m.rows, PVQ_DEBUG_GLOBAL_STORE) ||
         !PVQ_DEBUG_INDEX(static_cast<long long>(g + 1) * N - 1, m.cols, PVQ_DEBUG_GLOBAL_STORE))
         return;
@@ -1114,6 +1095,63 @@ __device__ __forceinline__ void emit_group(const MatrixArgs& m, const YT* yslots
         o.z = pack_bf16x2(__fmul_rn(f[4], sc), __fmul_rn(f[5], sc));
         o.w = pack_bf16x2(__fmul_rn(f[6], sc), __fmul_rn(f[7], sc));
         dst[q] = o;
+    }
+}
+
+// After walk_code: scale this thread's point to the unit sphere times `amp` and write its N
+// values as bf16 with 16-byte stores (row `row`, group `g` of matrix m).  Each thread writes
+// its own N*2 contiguous bytes; the threads of a warp hold consecutive groups, so a warp
+// fills a contiguous stretch of the row.
+template <int N, typename YT>
+__device__ __forceinline__ void emit_group(const MatrixArgs& m, const YT* yslots, float amp, unsigned row,
+                                           unsigned g) {
+    const uint32_t* y4 = reinterpret_cast<const uint32_t*>(yslots);
+    int ssy = 0;
+    if constexpr (sizeof(YT) == 1) {
+        // slots hold b = y + 128:  sum y^2 = sum b^2 - 256 sum b + 128^2 N
+        unsigned sq = 0, su = 0;
+#pragma unroll
+        for (int v = 0; v < N / 4; ++v) {
+            sq = __dp4a(y4[v], y4[v], sq);
+            su = __dp4a(y4[v], 0x01010101u, su);
+        }
+        ssy = static_cast<int>(sq) - 256 * static_cast<int>(su) + 16384 * N;
+    } else {
+#pragma unroll 8
+        for (int v = 0; v < N; ++v) ssy += static_cast<int>(yslots[v]) * static_cast<int>(yslots[v]);
+    }
+    emit_scaled<N, YT>(m, yslots, __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(ssy))), row, g);
+}
+
+// The groups of a warp, slot l (N bytes y_i + 128, N + 4 apart) being lane l's: scaled by that lane's `sc` and written
+// one after the other, 16 bytes a lane, so that a store fills whole lines.
+template <int N>
+__device__ __forceinline__ void emit_warp(const MatrixArgs& m, const uint8_t* slots, float sc, bool active, unsigned row, unsigned g) {
+    constexpr int PIECES = N / 8;  // lanes that share a group
+    const int lane = threadIdx.x & 31;
+    if (active && (!PVQ_DEBUG_INDEX(static_cast<long long>(row), m.rows, PVQ_DEBUG_GLOBAL_STORE) ||
+                   !PVQ_DEBUG_INDEX(static_cast<long long>(g + 1) * N - 1, m.cols, PVQ_DEBUG_GLOBAL_STORE)))
+        active = false;
+    const unsigned long long at =
+        active ? reinterpret_cast<unsigned long long>(static_cast<__nv_bfloat16*>(m.out) + static_cast<size_t>(row) * m.ld_out + static_cast<size_t>(g) * N)
+               : 0ull;
+    const int sub = lane % PIECES;
+    const uint8_t* src = slots + (lane / PIECES) * (N + 4) + sub * 8;
+#pragma unroll
+    for (int p = 0; p < PIECES; ++p, src += 32 / PIECES * (N + 4)) {
+        const int from = p * (32 / PIECES) + lane / PIECES;
+        const float s = __shfl_sync(kFull, sc, from);
+        const unsigned long long dst = __shfl_sync(kFull, at, from);
+        const uint32_t lo = reinterpret_cast<const uint32_t*>(src)[0], hi = reinterpret_cast<const uint32_t*>(src)[1];
+        float f[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {  // byte b into the low mantissa bits of 2^23: the float 2^23 + b, then minus 2^23 + 128
+            f[e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
+            f[4 + e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
+        }
+        if (dst != 0ull)
+            reinterpret_cast<uint4*>(dst)[sub] =
+                make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
     }
 }
 
