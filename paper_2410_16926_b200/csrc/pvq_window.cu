@@ -30,8 +30,8 @@ uint32_t aligned_key(const BigU& v, int bits, int words) {
     unsigned __int128 f = 0;
     for (int w = 1; w <= words; ++w) f = f << 32 | word_at(v, bits - 32 * w);
     if (f == 0) return 0u;
-    int e = 0;
-    while (f >> (e + 1)) ++e;
+    const uint64_t high = static_cast<uint64_t>(f >> 64), low = static_cast<uint64_t>(f);
+    const int e = high ? 127 - __builtin_clzll(high) : 63 - __builtin_clzll(low);
     const uint32_t mant = static_cast<uint32_t>(e >= 23 ? f >> (e - 23) : f << (23 - e));
     return (static_cast<uint32_t>(e + 127) << 23) | (mant & 0x7fffffu);
 }
@@ -137,7 +137,7 @@ struct Builder {
                 // |y| and the sums of the packed arithmetic stay below 256, and an out-of-window index always shows
                 if (dlo < 0 || dlo > 127 || before(i) - lo[i] >= 127 || last_m[i] - 2 * lo[i] + 1 > plane) return false;
                 t.args.klo[i] = static_cast<int16_t>(lo[i]);
-                klo4 |= static_cast<uint32_t>(lo[i]) << (8 * (3 - s));
+                klo4 |= static_cast<uint32_t>(lo[i] & 255) << (8 * (3 - s));  // (read where K <= 255)
                 width4 |= static_cast<uint32_t>(hi[i] - lo[i]) << (8 * (3 - s));
                 dlo4 |= static_cast<uint32_t>(dlo) << (8 * s);
                 std::vector<uint32_t> key;
@@ -201,8 +201,8 @@ struct Builder {
             q.sub(count(n, left));
             k = left;
         }
-        for (int w = 0; w < 12; ++w) t.args.typical[w] = q.w[w];
-        return words[0] <= 12;
+        for (int w = 0; w < kWinWords; ++w) t.args.typical[w] = q.w[w];
+        return words[0] <= kWinWords;
     }
 
     // The widest windows (the smallest share outside) whose tables fit beside the output slots of 32 warps (N = 64); where
@@ -247,8 +247,10 @@ std::shared_ptr<const WinTables> window_tables(int N, int K) {
 
 void build_window_tables(int N, int K, cudaStream_t stream) {
     const int W = code_words_for(N, K);
-    // the settings with a kernel: codes of 5 to 8 words at group size 64, 9 to 12 at 128
-    if (!((N == 64 && W >= 5 && W <= 8) || (N == 128 && W >= 9 && W <= 12)) || K > 255 || count_fills_its_words(N, K)) return;
+    // the settings with a kernel: codes of 5 to 8 words at group size 64, 9 to 12 at 128, 24 at 256 (decoding only)
+    if (!((N == 64 && W >= 5 && W <= 8 && K <= 255) || (N == 128 && W >= 9 && W <= 12 && K <= 255) || (N == 256 && W == 24)) ||
+        count_fills_its_words(N, K))
+        return;
     int dev = 0;
     DeviceInfo di;
     if (cudaGetDevice(&dev) != cudaSuccess || device_info(&di) != PVQ_OK) return;

@@ -10,7 +10,7 @@
 //
 // Rows are taken in blocks of four positions.  A block's numbers are kept left-aligned: multiplied by the power
 // of two that brings the largest q of the block to the top of its `words` 32-bit words.  The top two words
-// (three at N = 128, whose windows span more than 56 bits) then hold the leading bits of q whatever the row;
+// (three from N = 128 on, whose windows span more than 56 bits) then hold the leading bits of q whatever the row;
 // as an fp32, truncated, they are the key that numbers a bucket.  From one block to the next q is shifted left by `delta` bits.
 //
 // Block b in memory (block_off[b], a multiple of 16 bytes):
@@ -33,7 +33,7 @@
 
 namespace pvq {
 
-constexpr int kWinRows = 128, kWinBlocks = kWinRows / 4;
+constexpr int kWinRows = 256, kWinBlocks = kWinRows / 4, kWinWords = 24;
 
 __host__ __device__ constexpr int win_key_words(int N) { return N > 64 ? 3 : 2; }
 
@@ -55,12 +55,12 @@ struct WinArgs {
     uint8_t words[kWinBlocks];
     uint8_t blocks_of[33];               // blocks_of[w]: blocks done in w words or more
     int16_t klo[kWinRows];
-    uint32_t typical[12];                // q of a code whose path stays in the middle of the windows
+    uint32_t typical[kWinWords];                // q of a code whose path stays in the middle of the windows
 };
 
 struct WinTables {
     WinArgs args;
-    int plane;           // entries of a plane: 96 (N = 64, tables that fit shared memory) or 192 (others), 160 (N = 128)
+    int plane;           // entries of a plane: 96 (N = 64, tables that fit shared memory) or 192 (others), 160 (N = 128, 256)
     uint32_t max_block;  // bytes of the largest block
     uint32_t max_rows;   // ... of its head and its four rows of E
 };
