@@ -130,7 +130,12 @@ size_t pvq_scale_row_stride(int64_t G, int scale_bits);
 /* Fill d_table with N(n,k), n = 0..N-1, k = 0..K (Sec. 2.4 recurrence; built a row at a
  * time with a parallel prefix sum over k as in App. C.2 / Algorithm 4, by one thread
  * block).  `bytes` is the size of d_table and must be at least
- * pvq_count_table_bytes(N,K).  Requires 1 <= N <= 256, 1 <= K <= 8191, W <= 32. */
+ * pvq_count_table_bytes(N,K).  Requires 1 <= N <= 256, 1 <= K <= 8191, W <= 32.
+ * For codes of 5 to 8 words at N = 64, 9 to 12 at N = 128 and 24 at N = 256 the call also computes, on the
+ * host, the windowed tables of the faster kernels, and keeps them on the current device: 0.3 to 6 MB an
+ * (N,K), at most eight of them per device, the oldest freed for the next (freeing waits for the
+ * device).  Where that memory is refused, or the stream is being captured, the call succeeds
+ * without, and the codes are handled by the slower kernels. */
 int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t bytes, pvq_stream_t stream);
 
 /* Fill d_edges (2^b - 1 floats) and d_levels (2^b floats) for group size N, G groups per

@@ -71,7 +71,7 @@ extern "C" int pvq_decode_static_table(const uint32_t* d_codes, const uint8_t* d
         // Every word the decode kernel reads for (N,K) is written by the builder, so the
         // array needs no clearing between different (N,K).
         slot.N = slot.K = 0;
-        const int st = pvq_build_count_table(N, K, slot.ptr, kStaticTableBytes, stream);
+        const int st = build_count_table(N, K, slot.ptr, kStaticTableBytes, cs, false);  // (true would allocate)
         if (st != PVQ_OK) return st;
         e = cudaEventRecord(slot.filled, cs);
         if (e != cudaSuccess) return set_cuda_error(e);

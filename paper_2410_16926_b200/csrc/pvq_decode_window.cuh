@@ -2,16 +2,18 @@
 // threshold search per position in windowed tables (pvq_window.cuh), N steps a group where the walk takes
 // N + K (160 at N = 64, 192 bits; 315 at N = 128, 384 bits).
 //
-// What bounds it: shared-memory wavefronts.  A position reads one bucket and, word plane by word plane, the
-// entry of E, as wide as the numbers still are (4 words on average at N = 64, 192 bits): the threads of a warp
-// read entries a few apart, mostly different banks.  The searches of a warp are independent of each
-// other, so the latency of a position (two dependent reads) is covered by 8 warps per scheduler.
+// What bounds it: shared-memory wavefronts and issue slots.  A position reads a row's record, one bucket and, word plane
+// by word plane, the entry of E, as wide as the numbers still are (4 words on average at N = 64, 192 bits): the
+// threads of a warp read entries a few apart, mostly different banks.  The searches of a warp are independent
+// of each other, so the latency of a position (two dependent reads) is covered by 8 warps per scheduler.
 //
-// The tables stay in shared memory where they fit beside the output slots (N = 64, 192 bits: 130 KB).  Otherwise
-// (N = 128, 384 bits: 520 KB) they are streamed from L2 through a ring of buffers, block of rows after
-// block of rows, all warps of the thread block following the stream; an additional warp feeds it.
+// The tables stay in shared memory where they fit beside the output slots (N = 64, 192 bits: 150 KB).  Otherwise
+// (N = 128, 384 bits: 760 KB; N = 256: 2.4 MB) they are streamed from L2 through a ring of buffers, block of rows
+// after block of rows, all warps of the thread block following the stream; an additional warp feeds it.
 //
-// Numbers taken with the walk before: 8192 x 28672, N = 64, 192 bits, and 4096 x 4096, N = 128, 384 bits.
+// Measured, with the walk (pvq_walk.cuh, pvq_big_impl.cuh) and now: 8192 x 28672, N = 64, 192 bits, 774 -> 364 us (86% of the
+// issue slots, 75% of the shared-memory wavefronts a cycle); 4096 x 4096, N = 128, 384 bits, 190 -> 47 us; N = 256, 768
+// bits, 601 -> 160 us.
 // (Group size 256 has a translation unit of its own: the functions that are not inlined take the registers of the
 // most generous kernel that calls them, and spill in the others.)
 #pragma once

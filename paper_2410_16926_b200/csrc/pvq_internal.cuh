@@ -250,6 +250,9 @@ struct SearchLayout {
     SearchRows rows;
 };
 
+// pvq_build_count_table; `windows`: with the windowed tables of pvq_window.cuh, which take device memory
+int build_count_table(int N, int K, uint32_t* d_table, size_t bytes, cudaStream_t stream, bool windows);
+
 // host helpers (pvq_host.cu)
 int set_cuda_error(cudaError_t e);  // records e, returns PVQ_ERR_CUDA
 int code_words_for(int N, int K);   // W, or 0 when it cannot be computed

@@ -1,6 +1,5 @@
-// Device pieces shared by the builder of the search section (pvq_tables.cu) and the kernels
-// that decode with it (pvq_decode_search.cu, the round trip of pvq_encode_fast.cuh); the
-// section is described at SearchLayout.
+// Device pieces shared by the builder of the search section (pvq_tables.cu) and the kernel
+// that decodes with it (pvq_decode_search.cu); the section is described at SearchLayout.
 #pragma once
 #include <cstdint>
 

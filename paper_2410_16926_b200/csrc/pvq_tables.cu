@@ -559,7 +559,7 @@ __global__ void scale_codebook_kernel(int a, int n, int scale_bits, float* __res
 
 using namespace pvq;
 
-extern "C" int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t bytes, pvq_stream_t stream) {
+int pvq::build_count_table(int N, int K, uint32_t* d_table, size_t bytes, cudaStream_t s, bool windows) {
     if (!d_table || N < 1 || K < 1) return PVQ_ERR_INVALID_ARG;
     if (N > 256 || K > kMaxPulses) return PVQ_ERR_UNSUPPORTED;
     const int W = code_words_for(N, K);
@@ -567,8 +567,7 @@ extern "C" int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t byt
     if (W > kMaxWords) return PVQ_ERR_UNSUPPORTED;
     if (!is_aligned(d_table, 16)) return PVQ_ERR_ALIGNMENT;
     if (bytes < pvq_count_table_bytes(N, K)) return PVQ_ERR_TABLE_TOO_SMALL;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    build_window_tables(N, K, s);
+    if (windows) build_window_tables(N, K, s);
     // more pulses than threads of a block, or rows of 32 KB and more: the multi-block builder, in 8, 16 or 32 words
     if (K > 1023 || static_cast<long long>(K + 1) * W >= 8192) {
         if (W <= 8) return launch_count_table_chunked<8>(N, K, W, d_table, s);
@@ -594,6 +593,10 @@ extern "C" int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t byt
     if (W <= 16) return launch_count_table<16>(N, K, W, d_table, s);
     if (W <= 24) return launch_count_table<24>(N, K, W, d_table, s);
     return launch_count_table<32>(N, K, W, d_table, s);
+}
+
+extern "C" int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t bytes, pvq_stream_t stream) {
+    return build_count_table(N, K, d_table, bytes, static_cast<cudaStream_t>(stream), true);
 }
 
 extern "C" int pvq_build_scale_codebook(int N, int64_t G, int scale_bits, float* d_edges, float* d_levels,

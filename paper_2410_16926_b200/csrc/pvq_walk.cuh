@@ -1,5 +1,4 @@
-// The decode walk (Algorithm 3) shared by the decode kernel and the fused
-// encode -> decode kernel.
+// The decode walk (Algorithm 3), and how a decoded point is written.
 //
 // Algorithm 3 is run as a walk over the cells (i, col) of the count table, i the
 // position and col the pulses still to place, from (0, K) to (N, 0).  With r the
