@@ -38,21 +38,20 @@ FALLBACK_HBM_GBS = 6650.0
 # workload and launch configuration as this bench): DRAM bytes read + written, and warp
 # instructions executed.  They hold for the CUDA sources they were captured from, whose hash
 # is recorded with them; with any other sources the line reports them as null.
-NCU_SOURCES = "348419117bfdfb77"
+NCU_SOURCES = "bdf19d7d3e6e68b2"
 NCU_COUNTERS = {
-    ("c3_llama3_8b_layer", "encode"): {"dram_bytes": 436_685_056 + 75_231_744, "warp_inst": 415_329_152,
-                                       "kernel": "encode_fast_kernel<32,3,bf16>", "profile": "profiles/encode_fast_kernel_c3.md"},
-    ("c3_llama3_8b_layer", "decode"): {"dram_bytes": 88_923_904 + 377_352_448, "warp_inst": 255_617_296,
-                                       "kernel": "decode_search_kernel<32,3>", "profile": "profiles/decode_search_kernel_c3.md"},
-    ("c2_bf16_q_proj", "encode"): {"dram_bytes": 33_675_520 + 0, "warp_inst": 31_428_752,
-                                   "kernel": "encode_fast_kernel<32,3,bf16>", "profile": "profiles/encode_fast_kernel_c2.md"},
-    ("c2_bf16_q_proj", "decode"): {"dram_bytes": 6_712_064 + 9_216, "warp_inst": 19_980_032,
-                                   "kernel": "decode_search_kernel<32,3>", "profile": "profiles/decode_search_kernel_c2.md"},
-    ("c4_bf16_down_proj_70b", "decode"): {"dram_bytes": 91_192_832 + 424_887_552, "warp_inst": 648_495_454,
-                                          "kernel": "decode_kernel<64,6,int8>", "profile": "profiles/decode_kernel_c4.md"},
-    ("c5_bf16_activations", "roundtrip"): {"dram_bytes": 134_330_368 + 91_422_976, "warp_inst": 210_351_000,
-                                           "kernel": "encode_fast_kernel<32,2,bf16,FUSED>",
-                                           "profile": "profiles/roundtrip_kernel_c5.md"},
+    ("c3_llama3_8b_layer", "encode"): {"dram_bytes": 436327936 + 75406080, "warp_inst": 313809359,
+        "kernel": "encode_lanes_kernel", "profile": "profiles/kernels.md"},
+    ("c3_llama3_8b_layer", "decode"): {"dram_bytes": 88959232 + 377378048, "warp_inst": 265743296,
+        "kernel": "decode_search_kernel", "profile": "profiles/kernels.md"},
+    ("c2_bf16_q_proj", "encode"): {"dram_bytes": 33665536 + 0, "warp_inst": 25004153,
+        "kernel": "encode_lanes_kernel", "profile": "profiles/kernels.md"},
+    ("c2_bf16_q_proj", "decode"): {"dram_bytes": 6711808 + 18432, "warp_inst": 20766560,
+        "kernel": "decode_search_kernel", "profile": "profiles/kernels.md"},
+    ("c4_bf16_down_proj_70b", "decode"): {"dram_bytes": 91169792 + 409931520, "warp_inst": 314173366,
+        "kernel": "decode_window_kernel", "profile": "profiles/kernels.md"},
+    ("c5_bf16_activations", "roundtrip"): {"dram_bytes": 134265088 + 83834112, "warp_inst": 81882380,
+        "kernel": "roundtrip_kernel", "profile": "profiles/kernels.md"},
 }
 for _c in NCU_COUNTERS.values():
     _c["kernel_sha"] = NCU_SOURCES
@@ -533,7 +532,7 @@ def kernel_table(wl, per, peak, peak_kind):
 
 def issue_table(wl, kernels, clocks, sha):
     """The limit that binds in practice: instruction issue (every kernel here is integer work on
-    a table walk or a sorting network).  achieved = warp instructions per launch (from the ncu
+    table entries and packed residuals).  achieved = warp instructions per launch (from the ncu
     capture under profiles/, valid while the sources are unchanged) / the time measured in this
     run; peak = issue slots per second at the SM clock sampled during the run."""
     issue = {}
