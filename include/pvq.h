@@ -134,8 +134,10 @@ size_t pvq_scale_row_stride(int64_t G, int scale_bits);
  * For codes of 5 to 8 words at N = 64, 9 to 12 at N = 128 and 24 at N = 256 the call also computes, on the
  * host, the windowed tables of the faster kernels, and keeps them on the current device: 0.3 to 6 MB an
  * (N,K), at most eight of them per device, the oldest freed for the next (freeing waits for the
- * device).  Where that memory is refused, or the stream is being captured, the call succeeds
- * without, and the codes are handled by the slower kernels. */
+ * device).  Tables that a captured call has used are never freed, since a graph replays it with
+ * their addresses.  Where there is no room (eight in captures), the memory is refused, or the
+ * stream is being captured, the call succeeds without, and the codes are handled by the slower
+ * kernels. */
 int pvq_build_count_table(int N, int K, uint32_t* d_table, size_t bytes, pvq_stream_t stream);
 
 /* Fill d_edges (2^b - 1 floats) and d_levels (2^b floats) for group size N, G groups per

@@ -221,11 +221,15 @@ struct Builder {
 struct Kept : WinTables {
     int dev, N, K;
     uint8_t* mem = nullptr;
-    ~Kept() { cudaFree(mem); }  // waits for the kernels that may be reading it
+    bool captured = false;  // a stream capture has recorded a launch with these addresses: kept for good
 };
 
 std::mutex g_mu;
 std::list<std::shared_ptr<Kept>>& kept() {  // oldest first; lives as long as the process
+    static auto* l = new std::list<std::shared_ptr<Kept>>;
+    return *l;
+}
+std::list<std::shared_ptr<Kept>>& retired() {  // no longer found; freed when no launch holds them any more
     static auto* l = new std::list<std::shared_ptr<Kept>>;
     return *l;
 }
@@ -236,13 +240,41 @@ std::shared_ptr<Kept> find_kept(int dev, int N, int K) {
     return nullptr;
 }
 
+// Room for one more table on the device: the oldest one that no capture holds goes.  False where there is none.
+bool make_room(int dev) {
+    auto& l = kept();
+    const auto mine = [dev](const std::shared_ptr<Kept>& o) { return o->dev == dev; };
+    if (std::count_if(l.begin(), l.end(), mine) < kWinKept) return true;
+    const auto it = std::find_if(l.begin(), l.end(), [dev](const std::shared_ptr<Kept>& o) { return o->dev == dev && !o->captured; });
+    if (it == l.end()) return false;
+    retired().splice(retired().end(), l, it);
+    return true;
+}
+
+// Frees what has been retired and is in no launching thread's hands (nobody can get hold of it any more; cudaFree waits
+// for the kernels that may be reading it).
+void free_retired(int dev) {
+    retired().remove_if([dev](const std::shared_ptr<Kept>& o) {
+        if (o->dev != dev || o.use_count() > 1) return false;
+        cudaFree(o->mem);
+        return true;
+    });
+}
+
 }  // namespace
 
-std::shared_ptr<const WinTables> window_tables(int N, int K) {
+std::shared_ptr<const WinTables> window_tables(int N, int K, cudaStream_t stream) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lock(g_mu);
-    return find_kept(dev, N, K);
+    auto k = find_kept(dev, N, K);
+    if (k && !k->captured) {
+        // a graph replays the launch with these addresses, whatever has been built in between
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return nullptr;
+        k->captured = capturing != cudaStreamCaptureStatusNone;
+    }
+    return k;
 }
 
 void build_window_tables(int N, int K, cudaStream_t stream) {
@@ -265,25 +297,25 @@ void build_window_tables(int N, int K, cudaStream_t stream) {
     if (!b.counts()) return;
     if (!b.choose(static_cast<uint32_t>(di.smem_max))) return;
 
-    auto k = std::make_shared<Kept>();
-    static_cast<WinTables&>(*k) = b.t;
-    k->dev = dev, k->N = N, k->K = K;
-    const size_t data_bytes = (b.data.size() * 4 + 255) & ~size_t(255), thr_bytes = b.thr.size() * 4;
     // (these calls concern nobody's capture: the memory is this function's own)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
+    const bool room = make_room(dev);
+    free_retired(dev);
+    const size_t data_bytes = (b.data.size() * 4 + 255) & ~size_t(255), thr_bytes = b.thr.size() * 4;
     void* mem = nullptr;
-    if (cudaMalloc(&mem, data_bytes + thr_bytes) == cudaSuccess) {
+    if (room && cudaMalloc(&mem, data_bytes + thr_bytes) == cudaSuccess) {
+        auto k = std::make_shared<Kept>();
+        static_cast<WinTables&>(*k) = b.t;
+        k->dev = dev, k->N = N, k->K = K;
         k->mem = static_cast<uint8_t*>(mem);
         k->args.data = k->mem;
         k->args.thr = k->mem + data_bytes;
         if (cudaMemcpy(k->mem, b.data.data(), b.data.size() * 4, cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(k->mem + data_bytes, b.thr.data(), thr_bytes, cudaMemcpyHostToDevice) == cudaSuccess) {
-            auto& l = kept();
-            const auto mine = [dev](const std::shared_ptr<Kept>& o) { return o->dev == dev; };
-            if (std::count_if(l.begin(), l.end(), mine) >= kWinKept) l.erase(std::find_if(l.begin(), l.end(), mine));
-            l.push_back(k);
-        }
+            cudaMemcpy(k->mem + data_bytes, b.thr.data(), thr_bytes, cudaMemcpyHostToDevice) == cudaSuccess)
+            kept().push_back(k);
+        else
+            cudaFree(mem);
     }
     cudaGetLastError();
     cudaThreadExchangeStreamCaptureMode(&mode);

@@ -68,11 +68,13 @@ struct WinTables {
 // Bytes of a block's head and E, which is all that the encoder reads.
 __host__ __device__ constexpr uint32_t win_rows_bytes(int words, int plane) { return kWinHead + 16u * words * plane; }
 
-// The tables for (N,K) on the current device, or null (never built here, or no such kernel).  The holder keeps them
-// from being freed until its launch is enqueued; freeing waits for the kernels that read them.
-std::shared_ptr<const WinTables> window_tables(int N, int K);
+// The tables for (N,K) on the current device for a launch on `stream`, or null (never built here, or no such kernel).
+// They stay while the holder is held (until the launch is enqueued: freeing waits for the kernels that read them), and
+// for good once they have been handed out for a launch that a stream capture records.
+std::shared_ptr<const WinTables> window_tables(int N, int K, cudaStream_t stream);
 // Builds them, once per device and (N,K): called when a count table is built, off the hot path.  The tables of at most
-// kWinKept (N,K) are kept per device, the oldest are freed.  Failing to build is not an error: decoding walks.
+// kWinKept (N,K) are kept per device; for one more the oldest that no capture has used are freed, by the thread that builds.
+// Failing to build (all are in captures, no memory) is not an error: the calls take the kernels without.
 constexpr int kWinKept = 8;
 void build_window_tables(int N, int K, cudaStream_t stream);
 

@@ -1,0 +1,128 @@
+"""The library's host code on a CUDA runtime without a GPU (tests/fake_cudart.cpp): who owns the memory that launches are
+given, what is waited for, who waits for whom."""
+import ctypes as C
+import glob
+import os
+import shutil
+import subprocess
+import threading
+
+import pytest
+
+from paper_2410_16926_b200 import build as lib_build
+from paper_2410_16926_b200 import pvq
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+P = 1 << 20  # an address, aligned; nothing is read there
+CAPTURED, PLAIN = C.c_void_p(0x100), C.c_void_p(0x200)
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    """The library's objects linked with the fake runtime."""
+    objs = sorted(glob.glob(os.path.join(lib_build.OBJDIR, "*.o")))
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    want = {f[:-3] for f in os.listdir(lib_build.CSRC) if f.endswith(".cu")}
+    objs = [o for o in objs if os.path.basename(o)[:-2] in want]
+    if len(objs) != len(want) or shutil.which("g++") is None:
+        pytest.skip("needs the library's objects (python -m paper_2410_16926_b200.build) and g++")
+    tmp = tmp_path_factory.mktemp("fake")
+    out = str(tmp / "libpvq_fake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-pthread", "-Wl,-Bsymbolic", "-Wl,-s", "-I", os.path.join(cuda, "include"),
+                    os.path.join(ROOT, "tests", "fake_cudart.cpp")] + objs + ["-o", out], check=True)
+    return out
+
+
+@pytest.fixture()
+def fake(fake_lib, tmp_path):
+    """A fresh instance for every test (the library's caches live as long as the process)."""
+    copy = str(tmp_path / "lib.so")
+    shutil.copyfile(fake_lib, copy)
+    L = C.CDLL(copy)
+    os.unlink(copy)
+    i32, i64, vp = C.c_int, C.c_int64, C.c_void_p
+    L.pvq_build_count_table.argtypes = [i32, i32, vp, C.c_size_t, vp]
+    L.pvq_encode.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, vp, vp, vp, vp, vp, vp]
+    L.pvq_decode.argtypes = [vp, vp, vp, i64, i64, i32, i32, i32, vp, vp, vp, i64, vp, vp]
+    L.fake_capture.argtypes = [vp, i32]
+    L.fake_launch_name.restype = C.c_char_p
+    L.fake_launch_table.restype = C.c_uint64
+    L.fake_live.argtypes = [C.c_uint64]
+    return L
+
+
+def build(L, N, K, stream=PLAIN):
+    return L.pvq_build_count_table(N, K, P, 1 << 40, stream)
+
+
+def encode(L, N, K, stream=PLAIN, rows=8, G=4):
+    return L.pvq_encode(P, 1, rows, G * N, G * N, N, K, 16, P, None, P, P, P, stream)
+
+
+def decode(L, N, K, stream=PLAIN, rows=8, G=4):
+    return L.pvq_decode(P, P, P, rows, G * N, N, K, 16, P, None, P, G * N, None, stream)
+
+
+def last_tables(L):
+    """Name and tables of the last launch: ('', ...) unless it was a windowed kernel."""
+    i = L.fake_launches() - 1
+    name = L.fake_launch_name(i).decode()
+    return name, [L.fake_launch_table(i, w) for w in (0, 1)]
+
+
+@pytest.mark.parametrize("call", [encode, decode])
+@pytest.mark.parametrize("N,bits", [(64, 192), (128, 384)])
+def test_tables_of_a_captured_call_stay(fake, call, N, bits):
+    """A graph replays a captured launch with the addresses it was given: they are not freed for other tables."""
+    K = pvq.max_pulses(N, bits)
+    assert build(fake, N, K) == 0
+    fake.fake_capture(CAPTURED, 1)
+    assert call(fake, N, K, CAPTURED) == 0
+    fake.fake_capture(CAPTURED, 0)
+    name, tables = last_tables(fake)
+    assert "window" in name and all(fake.fake_live(t) for t in tables)
+    for k in range(K - 12, K):
+        assert build(fake, N, k) == 0
+    assert all(fake.fake_live(t) for t in tables)
+    # and the number kept stays bounded, also when every one of them has been captured
+    assert fake.fake_allocations() <= 8
+    for k in range(K - 30, K + 1):
+        assert build(fake, N, k) == 0
+        fake.fake_capture(CAPTURED, 1)
+        assert call(fake, N, k, CAPTURED) == 0
+        fake.fake_capture(CAPTURED, 0)
+    assert fake.fake_allocations() <= 8 and all(fake.fake_live(t) for t in tables)
+    assert call(fake, N, K) == 0 and last_tables(fake)[1] == tables
+
+
+def test_tables_that_no_capture_holds_make_room(fake):
+    K = pvq.max_pulses(64, 192)
+    for k in range(K - 12, K + 1):
+        assert build(fake, 64, k) == 0 and decode(fake, 64, k) == 0
+        name, tables = last_tables(fake)
+        assert "window" in name and all(fake.fake_live(t) for t in tables)
+    assert fake.fake_allocations() == 8
+
+
+def test_a_hot_call_never_frees(fake):
+    """Tables that make room while another thread is launching with them stay until it is through, and that
+    thread does not free them (cudaFree waits for the device and ends a capture)."""
+    K = pvq.max_pulses(64, 192)
+    assert build(fake, 64, K) == 0
+    fake.fake_forget_frees()
+    fake.fake_hold(1, 0)
+    status = []
+    launching = threading.Thread(target=lambda: status.append(decode(fake, 64, K)))
+    launching.start()
+    assert fake.fake_wait_until_held(20)
+    for k in range(K - 9, K):
+        assert build(fake, 64, k) == 0
+    fake.fake_hold(0, 0)
+    launching.join()
+    assert status == [0]
+    name, tables = last_tables(fake)
+    assert "window" in name and all(fake.fake_live(t) for t in tables)
+    assert fake.fake_frees_by_others() == 0
+    for k in range(K - 20, K - 9):
+        assert build(fake, 64, k) == 0
+    assert fake.fake_allocations() == 8 and fake.fake_frees() == 1 + 9 + 11 - 8 and fake.fake_frees_by_others() == 0
