@@ -261,6 +261,17 @@ void free_retired(int dev) {
     });
 }
 
+// Copies to the device and waits until the copy is there: launches on any stream may follow.  (A plain cudaMemcpy from
+// pageable memory returns when the data is staged, and orders only the legacy stream behind it.)
+bool upload(uint8_t* dst, const std::vector<uint32_t>& src) {
+    cudaStream_t s = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
+    const bool ok = cudaMemcpyAsync(dst, src.data(), src.size() * 4, cudaMemcpyHostToDevice, s) == cudaSuccess;
+    const bool there = cudaStreamSynchronize(s) == cudaSuccess;
+    cudaStreamDestroy(s);
+    return ok && there;
+}
+
 }  // namespace
 
 std::shared_ptr<const WinTables> window_tables(int N, int K, cudaStream_t stream) {
@@ -311,8 +322,7 @@ void build_window_tables(int N, int K, cudaStream_t stream) {
         k->mem = static_cast<uint8_t*>(mem);
         k->args.data = k->mem;
         k->args.thr = k->mem + data_bytes;
-        if (cudaMemcpy(k->mem, b.data.data(), b.data.size() * 4, cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(k->mem + data_bytes, b.thr.data(), thr_bytes, cudaMemcpyHostToDevice) == cudaSuccess)
+        if (upload(k->mem, b.data) && upload(k->mem + data_bytes, b.thr))
             kept().push_back(k);
         else
             cudaFree(mem);

@@ -39,3 +39,23 @@ def test_replay_after_other_tables(N, bits):
         o = po.encode(x_np, N, K, 16, None, W=W)
         assert np.array_equal(enc[0].cpu().numpy().view(np.uint32), o[0])
         assert np.array_equal(out.view(torch.int16).cpu().numpy().view(np.uint16), po.decode(*o, N, K, 16, None)[0])
+
+
+@pytest.mark.parametrize("N,bits", [(64, 168), (128, 360), (256, 768)])
+def test_tables_built_and_used_on_a_side_stream(N, bits):
+    """No synchronisation between building a count table and the calls that use it, on a stream that does not wait for the
+    legacy stream.  (Pulse counts that nothing else builds: the tables are made here.)"""
+    rows, G = 64, 8
+    K = pvq.max_pulses(N, bits)
+    W = pvq.code_words(N, K)
+    x = (np.random.default_rng(bits).standard_normal((rows, G * N)) * 0.02).astype(np.float32)
+    x_dev = torch.from_numpy(x).cuda()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        table = pvq.build_count_table(N, K)
+        enc = pvq.encode(x_dev, N, K, 16, table, None)
+        out = pvq.decode(*enc, N, K, 16, table, None)
+    torch.cuda.synchronize()
+    o = po.encode(x, N, K, 16, None, W=W)
+    assert np.array_equal(enc[0].cpu().numpy().view(np.uint32), o[0])
+    assert np.array_equal(out.view(torch.int16).cpu().numpy().view(np.uint16), po.decode(*o, N, K, 16, None)[0])

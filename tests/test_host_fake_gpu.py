@@ -126,3 +126,12 @@ def test_a_hot_call_never_frees(fake):
     for k in range(K - 20, K - 9):
         assert build(fake, 64, k) == 0
     assert fake.fake_allocations() == 8 and fake.fake_frees() == 1 + 9 + 11 - 8 and fake.fake_frees_by_others() == 0
+
+
+@pytest.mark.parametrize("N,bits", [(64, 192), (128, 384), (256, 768)])
+def test_tables_are_on_the_device_before_a_launch_can_find_them(fake, N, bits):
+    """Streams that do not wait for the legacy stream follow: nothing may still be on its way when the build returns."""
+    K = pvq.max_pulses(N, bits)
+    assert build(fake, N, K) == 0
+    assert fake.fake_uploads_pending() == 0
+    assert decode(fake, N, K) == 0 and "window" in last_tables(fake)[0]
