@@ -5,6 +5,7 @@
 #include <list>
 #include <memory>
 #include <mutex>
+#include <new>
 
 #include "pvq_bigint.h"
 #include "pvq_window.cuh"
@@ -272,6 +273,33 @@ bool upload(uint8_t* dst, const std::vector<uint32_t>& src) {
     return ok && there;
 }
 
+struct FreeOnDevice {
+    void operator()(uint8_t* p) const { cudaFree(p); }
+};
+
+// (std::bad_alloc leaves everything as it was)
+void compute_and_keep(int dev, int N, int K, uint32_t smem_max) {
+    Builder b;
+    b.N = N;
+    b.K = K;
+    if (!b.counts() || !b.choose(smem_max)) return;
+    auto k = std::make_shared<Kept>();
+    static_cast<WinTables&>(*k) = b.t;
+    k->dev = dev, k->N = N, k->K = K;
+    std::list<std::shared_ptr<Kept>> entry(1, k);
+    const bool room = make_room(dev);
+    free_retired(dev);
+    const size_t data_bytes = (b.data.size() * 4 + 255) & ~size_t(255), thr_bytes = b.thr.size() * 4;
+    void* mem = nullptr;
+    if (!room || cudaMalloc(&mem, data_bytes + thr_bytes) != cudaSuccess) return;
+    std::unique_ptr<uint8_t, FreeOnDevice> held(static_cast<uint8_t*>(mem));
+    if (!upload(held.get(), b.data) || !upload(held.get() + data_bytes, b.thr)) return;
+    k->args.data = held.get();
+    k->args.thr = held.get() + data_bytes;
+    k->mem = held.release();
+    kept().splice(kept().end(), entry);
+}
+
 }  // namespace
 
 std::shared_ptr<const WinTables> window_tables(int N, int K, cudaStream_t stream) {
@@ -301,31 +329,12 @@ void build_window_tables(int N, int K, cudaStream_t stream) {
     if (find_kept(dev, N, K)) return;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) return;
-
-    Builder b;
-    b.N = N;
-    b.K = K;
-    if (!b.counts()) return;
-    if (!b.choose(static_cast<uint32_t>(di.smem_max))) return;
-
     // (these calls concern nobody's capture: the memory is this function's own)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
-    const bool room = make_room(dev);
-    free_retired(dev);
-    const size_t data_bytes = (b.data.size() * 4 + 255) & ~size_t(255), thr_bytes = b.thr.size() * 4;
-    void* mem = nullptr;
-    if (room && cudaMalloc(&mem, data_bytes + thr_bytes) == cudaSuccess) {
-        auto k = std::make_shared<Kept>();
-        static_cast<WinTables&>(*k) = b.t;
-        k->dev = dev, k->N = N, k->K = K;
-        k->mem = static_cast<uint8_t*>(mem);
-        k->args.data = k->mem;
-        k->args.thr = k->mem + data_bytes;
-        if (upload(k->mem, b.data) && upload(k->mem + data_bytes, b.thr))
-            kept().push_back(k);
-        else
-            cudaFree(mem);
+    try {
+        compute_and_keep(dev, N, K, static_cast<uint32_t>(di.smem_max));
+    } catch (const std::bad_alloc&) {  // a few MB to 50 MB of host memory are not there: done without, as said above
     }
     cudaGetLastError();
     cudaThreadExchangeStreamCaptureMode(&mode);

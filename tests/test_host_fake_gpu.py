@@ -5,6 +5,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sys
 import threading
 
 import pytest
@@ -38,8 +39,13 @@ def fake(fake_lib, tmp_path):
     """A fresh instance for every test (the library's caches live as long as the process)."""
     copy = str(tmp_path / "lib.so")
     shutil.copyfile(fake_lib, copy)
-    L = C.CDLL(copy)
+    L = load(copy)
     os.unlink(copy)
+    return L
+
+
+def load(path):
+    L = C.CDLL(path)
     i32, i64, vp = C.c_int, C.c_int64, C.c_void_p
     L.pvq_build_count_table.argtypes = [i32, i32, vp, C.c_size_t, vp]
     L.pvq_encode.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, vp, vp, vp, vp, vp, vp]
@@ -135,3 +141,25 @@ def test_tables_are_on_the_device_before_a_launch_can_find_them(fake, N, bits):
     assert build(fake, N, K) == 0
     assert fake.fake_uploads_pending() == 0
     assert decode(fake, N, K) == 0 and "window" in last_tables(fake)[0]
+
+
+OUT_OF_HOST_MEMORY = """
+import resource, sys
+sys.path.insert(0, sys.argv[2])
+import test_host_fake_gpu as t
+L = t.load(sys.argv[1])
+K = t.pvq.max_pulses(256, 768)
+assert t.build(L, 256, 8) == 0  # (the library's first call, with what it allocates once)
+now = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (now + (8 << 20), resource.RLIM_INFINITY))
+assert t.build(L, 256, K) == 0
+resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+assert t.decode(L, 256, K) == 0 and "big" in t.last_tables(L)[0]
+assert t.build(L, 256, K) == 0 and t.decode(L, 256, K) == 0 and "window" in t.last_tables(L)[0]
+"""
+
+
+def test_no_exception_leaves_a_build_without_host_memory(fake_lib):
+    r = subprocess.run([sys.executable, "-c", OUT_OF_HOST_MEMORY, fake_lib, os.path.dirname(os.path.abspath(__file__))], cwd=ROOT,
+                       env=dict(os.environ, PYTHONPATH=ROOT), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
