@@ -21,6 +21,7 @@ int launch_window_w(BatchArgs& a, const WinTables& t, cudaStream_t s) {
 
 int launch_decode_window(const BatchArgs& args, int N, int W, cudaStream_t stream) {
 #ifndef PVQ_DEBUG
+    if (!has_window_tables(N, W, args.K)) return PVQ_ERR_UNSUPPORTED;
     const auto t = window_tables(N, args.K, stream);
     if (!t || t->args.blocks_of[W] < 1) return PVQ_ERR_UNSUPPORTED;
     BatchArgs a = args;

@@ -440,7 +440,7 @@ int launch_ew(BatchArgs& a, int dtype, const WinTables& t, cudaStream_t s) {
 
 int launch_encode_window(const BatchArgs& args, int dtype, int N, int W, cudaStream_t stream) {
 #ifndef PVQ_DEBUG
-    if (!(N == 64 && W >= 5 && W <= 8) && !(N == 128 && W >= 9 && W <= 12)) return PVQ_ERR_UNSUPPORTED;
+    if (N == 256 || !has_window_tables(N, W, args.K)) return PVQ_ERR_UNSUPPORTED;
     const auto t = window_tables(N, args.K, stream);
     if (!t || t->args.words[N / 4 - 1] != 1) return PVQ_ERR_UNSUPPORTED;
     BatchArgs a = args;

@@ -225,7 +225,8 @@ struct Kept : WinTables {
     bool captured = false;  // a stream capture has recorded a launch with these addresses: kept for good
 };
 
-std::mutex g_mu;
+std::mutex g_build_mu;  // one thread builds at a time
+std::mutex g_mu;        // the lists; held for a look, never while something is computed, allocated, copied or freed
 std::list<std::shared_ptr<Kept>>& kept() {  // oldest first; lives as long as the process
     static auto* l = new std::list<std::shared_ptr<Kept>>;
     return *l;
@@ -243,6 +244,7 @@ std::shared_ptr<Kept> find_kept(int dev, int N, int K) {
 
 // Room for one more table on the device: the oldest one that no capture holds goes.  False where there is none.
 bool make_room(int dev) {
+    std::lock_guard<std::mutex> lock(g_mu);
     auto& l = kept();
     const auto mine = [dev](const std::shared_ptr<Kept>& o) { return o->dev == dev; };
     if (std::count_if(l.begin(), l.end(), mine) < kWinKept) return true;
@@ -255,11 +257,15 @@ bool make_room(int dev) {
 // Frees what has been retired and is in no launching thread's hands (nobody can get hold of it any more; cudaFree waits
 // for the kernels that may be reading it).
 void free_retired(int dev) {
-    retired().remove_if([dev](const std::shared_ptr<Kept>& o) {
-        if (o->dev != dev || o.use_count() > 1) return false;
-        cudaFree(o->mem);
-        return true;
-    });
+    std::list<std::shared_ptr<Kept>> gone;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        for (auto it = retired().begin(); it != retired().end();) {
+            const auto o = it++;
+            if ((*o)->dev == dev && o->use_count() == 1) gone.splice(gone.end(), retired(), o);
+        }
+    }
+    for (const auto& o : gone) cudaFree(o->mem);
 }
 
 // Copies to the device and waits until the copy is there: launches on any stream may follow.  (A plain cudaMemcpy from
@@ -297,6 +303,7 @@ void compute_and_keep(int dev, int N, int K, uint32_t smem_max) {
     k->args.data = held.get();
     k->args.thr = held.get() + data_bytes;
     k->mem = held.release();
+    std::lock_guard<std::mutex> lock(g_mu);
     kept().splice(kept().end(), entry);
 }
 
@@ -317,16 +324,15 @@ std::shared_ptr<const WinTables> window_tables(int N, int K, cudaStream_t stream
 }
 
 void build_window_tables(int N, int K, cudaStream_t stream) {
-    const int W = code_words_for(N, K);
-    // the settings with a kernel: codes of 5 to 8 words at group size 64, 9 to 12 at 128, 24 at 256 (decoding only)
-    if (!((N == 64 && W >= 5 && W <= 8 && K <= 255) || (N == 128 && W >= 9 && W <= 12 && K <= 255) || (N == 256 && W == 24)) ||
-        count_fills_its_words(N, K))
-        return;
+    if (!has_window_tables(N, code_words_for(N, K), K) || count_fills_its_words(N, K)) return;
     int dev = 0;
     DeviceInfo di;
     if (cudaGetDevice(&dev) != cudaSuccess || device_info(&di) != PVQ_OK) return;
-    std::lock_guard<std::mutex> lock(g_mu);
-    if (find_kept(dev, N, K)) return;
+    std::lock_guard<std::mutex> building(g_build_mu);
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (find_kept(dev, N, K)) return;
+    }
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) return;
     // (these calls concern nobody's capture: the memory is this function's own)

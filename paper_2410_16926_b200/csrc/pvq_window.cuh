@@ -68,6 +68,11 @@ struct WinTables {
 // Bytes of a block's head and E, which is all that the encoder reads.
 __host__ __device__ constexpr uint32_t win_rows_bytes(int words, int plane) { return kWinHead + 16u * words * plane; }
 
+// The settings with windowed kernels: codes of 5 to 8 words at group size 64, 9 to 12 at 128, 24 at 256 (decoding only).
+constexpr bool has_window_tables(int N, int W, int K) {
+    return (N == 64 && W >= 5 && W <= 8 && K <= 255) || (N == 128 && W >= 9 && W <= 12 && K <= 255) || (N == 256 && W == 24);
+}
+
 // The tables for (N,K) on the current device for a launch on `stream`, or null (never built here, or no such kernel).
 // They stay while the holder is held (until the launch is enqueued: freeing waits for the kernels that read them), and
 // for good once they have been handed out for a launch that a stream capture records.

@@ -143,6 +143,26 @@ def test_tables_are_on_the_device_before_a_launch_can_find_them(fake, N, bits):
     assert decode(fake, N, K) == 0 and "window" in last_tables(fake)[0]
 
 
+def test_a_hot_call_does_not_wait_for_another_threads_build(fake):
+    """Tables are computed, allocated, copied and freed (which waits for the device) beside the calls of other threads."""
+    K = pvq.max_pulses(64, 192)
+    assert build(fake, 64, K) == 0
+    fake.fake_hold(0, 1)
+    builder = threading.Thread(target=build, args=(fake, 64, K - 1))
+    builder.start()
+    assert fake.fake_wait_until_held(20)
+    done = []
+    calls = [threading.Thread(target=lambda n=n, k=k: done.append(decode(fake, n, k)), daemon=True) for n, k in ((64, K), (64, K - 1), (32, 50))]
+    for c in calls:
+        c.start()
+    for c in calls:
+        c.join(20)
+    finished = len(done)
+    fake.fake_hold(0, 0)
+    builder.join()
+    assert finished == 3 and done == [0, 0, 0]
+
+
 OUT_OF_HOST_MEMORY = """
 import resource, sys
 sys.path.insert(0, sys.argv[2])
