@@ -7,20 +7,15 @@ int launch_decode_window_256(BatchArgs& a, const WinTables& t, cudaStream_t stre
 
 namespace {
 
-#ifndef PVQ_DEBUG
-
 template <int N, int W>
 int launch_window_w(BatchArgs& a, const WinTables& t, cudaStream_t s) {
     if constexpr (N == 64) return t.plane == 96 ? launch_window_t<N, W, 96>(a, t, s) : launch_window_t<N, W, 192>(a, t, s);
     return launch_window_t<N, W, N == 64 ? 192 : 160>(a, t, s);
 }
 
-#endif
-
 }  // namespace
 
 int launch_decode_window(const BatchArgs& args, int N, int W, cudaStream_t stream) {
-#ifndef PVQ_DEBUG
     if (!has_window_tables(N, W, args.K)) return PVQ_ERR_UNSUPPORTED;
     const auto t = window_tables(N, args.K, stream);
     if (!t || t->args.blocks_of[W] < 1) return PVQ_ERR_UNSUPPORTED;
@@ -44,7 +39,6 @@ int launch_decode_window(const BatchArgs& args, int N, int W, cudaStream_t strea
         case 256 * 16 + 24: return launch_decode_window_256(a, *t, stream);
         default: break;
     }
-#endif
     return PVQ_ERR_UNSUPPORTED;
 }
 

@@ -30,8 +30,6 @@ namespace pvq {
 
 namespace {
 
-#ifndef PVQ_DEBUG
-
 struct WinGeom {
     uint32_t slots_off;  // of the output slots in shared memory
     uint32_t buf_bytes;  // streamed: bytes of a buffer
@@ -39,21 +37,24 @@ struct WinGeom {
     int warps;           // that decode
 };
 
-__device__ __forceinline__ uint32_t win_load(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-    return v;
-}
-template <int OFF>
-__device__ __forceinline__ uint32_t win_load_at(uint32_t addr) {
+// A word of the tables in shared memory; win_slot_word: of the output slots.
+template <int OFF = 0>
+__device__ __forceinline__ uint32_t win_slot_word(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
     return v;
 }
+template <int OFF = 0>
+__device__ __forceinline__ uint32_t win_load(uint32_t addr) {
+#ifdef PVQ_DEBUG
+    if (!debug_table_ok(addr + OFF, 4u)) return 0u;
+#endif
+    return win_slot_word<OFF>(addr);
+}
 template <int PW, int PLANE, int FROM, int W = 0>
 __device__ __forceinline__ void win_entry(mp<PW>& e, uint32_t addr) {
     if constexpr (W < PW) {
-        e.w[W] = win_load_at<(FROM + W) * PLANE * 4>(addr);
+        e.w[W] = win_load<(FROM + W) * PLANE * 4>(addr);
         win_entry<PW, PLANE, FROM, W + 1>(e, addr);
     }
 }
@@ -61,6 +62,9 @@ __device__ __forceinline__ void win_entry(mp<PW>& e, uint32_t addr) {
 // A row's record (WinRow): x base, y last, z shift, w buckets.
 __device__ __forceinline__ uint4 win_record(uint32_t addr) {
     uint4 v;
+#ifdef PVQ_DEBUG
+    if ((addr & 15u) != 0u || !debug_table_ok(addr, 16u)) return make_uint4(0u, 0u, 0u, 0u);
+#endif
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
     return v;
 }
@@ -204,7 +208,7 @@ template <int N, int PW, int PLANE, int KW, int W>
 __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, const BatchArgs& a, const WinArgs& t, int b, uint32_t y) {
     mp<PW> v;
     {
-        const uint32_t delta = win_load_at<kWinDelta>(stage);
+        const uint32_t delta = win_load<kWinDelta>(stage);
         st.over = __funnelshift_l(st.a[0], st.over, delta);
 #pragma unroll
         for (int j = 0; j < PW; ++j) v.w[PW - 1 - j] = __funnelshift_l(st.a[j + 1], st.a[j], delta);
@@ -219,7 +223,7 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
     // touch each other while all of them are 0..127 (else some bit 7 shows, unless the position before was out of the
     // window too, and then h shows it); y > 0 where the index is odd
     const uint32_t after = (acc >> 1) & 0x7f7f7f7fu;
-    const uint32_t mag = (after << 8) + win_load_at<kWinDlo4>(stage) - after + static_cast<uint32_t>(st.h);
+    const uint32_t mag = (after << 8) + win_load<kWinDlo4>(stage) - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;
     uint32_t y4 = ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos);
     if (__any_sync(kFull, top == 0xffffffffu || (((mag | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
@@ -234,7 +238,10 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
         st.h = static_cast<int>(after >> 24);
         st.ssy = __dp4a(mag, mag, st.ssy);
     }
-    asm volatile("st.shared.u32 [%0], %1;" ::"r"(y), "r"(y4) : "memory");
+#ifdef PVQ_DEBUG
+    if (debug_slot_ok(y, 4u))
+#endif
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(y), "r"(y4) : "memory");
 #pragma unroll
     for (int j = 0; j < PW; ++j) st.a[j] = v.w[PW - 1 - j];
 }
@@ -396,6 +403,8 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
     }
     const float sc = zeros ? 0.0f : __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(static_cast<int>(st.ssy))));
     // The warp writes the groups one after the other, 16 bytes a lane: whole lines.
+    done = done || !PVQ_DEBUG_INDEX(row, m.rows, PVQ_DEBUG_GLOBAL_STORE) ||
+           !PVQ_DEBUG_INDEX(static_cast<long long>(g + 1) * N - 1, m.cols, PVQ_DEBUG_GLOBAL_STORE);
     const uint32_t at = done ? 0xffffffffu : static_cast<uint32_t>((static_cast<size_t>(row) * m.ld_out + static_cast<size_t>(g) * N) >> 3);
     uint4* base = static_cast<uint4*>(m.out);
     __syncwarp();
@@ -406,7 +415,7 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
     for (int from = lane / PIECES; from < 32; from += 32 / PIECES, src += 32 / PIECES * YS) {
         const float s = __shfl_sync(kFull, sc, from);
         const uint32_t dst = __shfl_sync(kFull, at, from);
-        const uint32_t lo = win_load(src), hi = win_load_at<4>(src);
+        const uint32_t lo = win_slot_word(src), hi = win_slot_word<4>(src);
         float f[8];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {  // byte v into the low mantissa bits of 2^23: the float 2^23 + v, then minus 2^23 + 128
@@ -449,6 +458,9 @@ __global__ void __launch_bounds__(1024, 1)
     const uint32_t base = shared_addr(smem);
     uint8_t* slot = smem + g.slots_off + threadIdx.x * (N + 4);
     const uint32_t y = shared_addr(slot), slots = y - (threadIdx.x & 31) * (N + 4);
+#ifdef PVQ_DEBUG
+    debug_begin(base, base + t.block_off[N / 4], shared_addr(smem) + g.slots_off, N + 4, N, a.debug_status);
+#endif
     const unsigned warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), total = gridDim.x * g.warps;
     bool bad = false;
     int mi = 0;
@@ -485,6 +497,9 @@ __global__ void __launch_bounds__(N == 256 ? 384 : 928, 1)
     }
     __syncthreads();
     grid_dependency_wait();
+#ifdef PVQ_DEBUG
+    debug_begin(shared_addr(smem), shared_addr(smem) + g.bufs * g.buf_bytes, shared_addr(smem) + g.slots_off, N + 4, N, a.debug_status);
+#endif
     const unsigned warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), step = gridDim.x * g.warps, first = blockIdx.x;
     const int passes = first < a.total_tiles ? static_cast<int>((a.total_tiles - first + step - 1) / step) : 0;
     if (warp == static_cast<unsigned>(g.warps)) {  // feeds the ring
@@ -591,8 +606,6 @@ int launch_window_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
     const unsigned grid = std::max(1u, std::min<unsigned>(tiles, static_cast<unsigned>(di.sms)));
     return launch_hot(kern, grid, threads, smem, stream, a, t.args, g);
 }
-
-#endif
 
 }  // namespace
 

@@ -4,11 +4,7 @@
 namespace pvq {
 
 int launch_decode_window_256(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
-#ifndef PVQ_DEBUG
     return launch_window_t<256, 24, 160>(a, t, stream);
-#else
-    return PVQ_ERR_UNSUPPORTED;
-#endif
 }
 
 }  // namespace pvq

@@ -20,8 +20,6 @@ namespace pvq {
 
 namespace {
 
-#ifndef PVQ_DEBUG
-
 constexpr int kEwWarps = 28, kEwBufs = 6;
 
 struct EwGeom {
@@ -36,15 +34,24 @@ struct EwGeom {
 
 __device__ __forceinline__ void ew_barrier(int threads) { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); }
 
-__device__ __forceinline__ uint32_t ew_load(uint32_t addr) {
+// A word of the tables in shared memory; ew_slot_word: of the points.
+template <int OFF = 0>
+__device__ __forceinline__ uint32_t ew_slot_word(uint32_t addr) {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(OFF));
     return v;
+}
+template <int OFF = 0>
+__device__ __forceinline__ uint32_t ew_load(uint32_t addr) {
+#ifdef PVQ_DEBUG
+    if (!debug_table_ok(addr + OFF, 4u)) return 0u;
+#endif
+    return ew_slot_word<OFF>(addr);
 }
 template <int PW, int PLANE, int FROM, int W = 0>
 __device__ __forceinline__ void ew_entry(mp<PW>& e, uint32_t addr) {
     if constexpr (W < PW) {
-        asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(e.w[W]) : "r"(addr), "n"((FROM + W) * PLANE * 4));
+        e.w[W] = ew_load<(FROM + W) * PLANE * 4>(addr);
         ew_entry<PW, PLANE, FROM, W + 1>(e, addr);
     }
 }
@@ -91,7 +98,7 @@ __device__ __forceinline__ void ew_blocks(EwState<W>& st, const WinArgs& t, int&
 #pragma unroll 1
     for (const int end = PW < W ? t.blocks_of[PW + 1] : 0; b >= end; --b) {
         const uint32_t stage = enter();
-        ew_block4<PW, PLANE, W>(st, stage, ew_load(slot + static_cast<uint32_t>(b) * 4u));
+        ew_block4<PW, PLANE, W>(st, stage, ew_slot_word(slot + static_cast<uint32_t>(b) * 4u));
         leave();
     }
     if constexpr (PW < W) ew_blocks<PW + 1, PLANE, W>(st, t, b, slot, enter, leave);
@@ -145,6 +152,9 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
     }
     __syncthreads();
     grid_dependency_wait();
+#ifdef PVQ_DEBUG
+    debug_begin(shared_addr(smem), shared_addr(smem) + g.bufs * g.buf_bytes + (256 - PLANE) * 4, 0u, 0u, 0u, a.debug_status);
+#endif
     const int warp = __shfl_sync(kFull, static_cast<int>(threadIdx.x) >> 5, 0), lane = threadIdx.x & 31;
     const int passes = blockIdx.x < a.total_tiles ? static_cast<int>((a.total_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
     if (warp == g.warps) {  // feeds the ring; the points' input lies there while a tile is quantised
@@ -240,7 +250,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
             const int gi = g0 + lane / L, sub = lane % L;
             const bool ok = gi < groups, leader = ok && sub == 0;
             const int r = gi / G, gr = gi - r * G;
-            if (leader) s_ss[r * gp + gr] = ss;
+            if (leader && PVQ_DEBUG_INDEX(r * gp + gr, (g.amp_off - g.ss_off) / 4, PVQ_DEBUG_SHARED_INDEX)) s_ss[r * gp + gr] = ss;
             if (ls_mode) {
                 const float ls = least_squares_amplitude<E, L, BF16, WIDE>(pt, mine);
                 if (leader) s_amp[r * gp + gr] = ls;
@@ -262,7 +272,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
                     }
                 }
             }
-            if (ok) {
+            if (ok && PVQ_DEBUG_INDEX(gi, T, PVQ_DEBUG_SLOT_WRITE)) {
                 uint32_t* slot = reinterpret_cast<uint32_t*>(smem + g.slots_off + gi * YS) + sub * (E / 4);
 #pragma unroll
                 for (int i = 0; i < E / 4; ++i) {
@@ -301,9 +311,11 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
             }
             if (gr == 0) m.row_norm[row] = __fsqrt_rn(ss_row);
             const unsigned bit = static_cast<unsigned>(gr) * b, sh = bit & 31u;
-            uint32_t* word = s_idx + rl * idx_words + (bit >> 5);
-            atomicOr(word, static_cast<uint32_t>(q) << sh);
-            if (sh + b > 32u) atomicOr(word + 1, static_cast<uint32_t>(q) >> (32u - sh));
+            const int word = rl * idx_words + static_cast<int>(bit >> 5);
+            if (PVQ_DEBUG_INDEX(word + (sh + b > 32u ? 1 : 0), g.idx_words, PVQ_DEBUG_SHARED_INDEX)) {
+                atomicOr(s_idx + word, static_cast<uint32_t>(q) << sh);
+                if (sh + b > 32u) atomicOr(s_idx + word + 1, static_cast<uint32_t>(q) >> (32u - sh));
+            }
         }
 
         // the indices
@@ -327,7 +339,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(shared_addr(&empty[j])) : "memory");
                 if (++j == g.bufs) j = 0, parity ^= 1;
             });
-        if (active) {
+        if (active && PVQ_DEBUG_INDEX(row, m.rows, PVQ_DEBUG_GLOBAL_STORE)) {
             const uint32_t kind = reinterpret_cast<const uint32_t*>(my_slot)[N / 4];
             uint32_t* cp = m.codes + (static_cast<size_t>(row) * G + gr) * W;
             if (kind == kEwPoint && (st.flag & kH4) != 0u) {
@@ -389,11 +401,13 @@ int launch_ew_t(BatchArgs& a, const WinTables& t, cudaStream_t stream) {
         g.warps = w;
         g.idx_words = static_cast<int>(idx);
         g.buf_bytes = (t.max_rows + 127u) & ~127u;
-        const uint32_t slots = static_cast<uint32_t>(T) * (N + 4), rest = (2u * ss + idx) * 4u + 1024u;
+        // (an index outside its window reads as far as 256 entries from the start of a plane: that much behind the last
+        // buffer is not used otherwise; 256 bytes for the alignment of what follows)
+        constexpr uint32_t behind = (256u - PLANE) * 4u;
+        const uint32_t slots = static_cast<uint32_t>(T) * (N + 4), rest = (2u * ss + idx) * 4u + behind + 256u;
         if (slots + rest + 2u * g.buf_bytes > limit) continue;
         g.bufs = static_cast<int>(std::min<uint32_t>(kEwBufs, (limit - slots - rest) / g.buf_bytes));
-        // (an index outside the window reads up to 256 entries from the start of a plane: 1 KB behind the last buffer)
-        uint32_t ring = g.bufs * g.buf_bytes + 1024u - 512u;
+        uint32_t ring = g.bufs * g.buf_bytes + behind;
         ring = std::max(ring, std::min(w * 32u * RUN, (limit - slots - rest) & ~127u));
         g.quant_warps = static_cast<int>(std::min<uint32_t>(w, ring / (32u * RUN)));
         g.slots_off = (ring + 127u) & ~127u;
@@ -434,12 +448,9 @@ int launch_ew(BatchArgs& a, int dtype, const WinTables& t, cudaStream_t s) {
     return bf16 ? launch_ew_t<N, W, N == 64 ? 192 : 160, true>(a, t, s) : launch_ew_t<N, W, N == 64 ? 192 : 160, false>(a, t, s);
 }
 
-#endif
-
 }  // namespace
 
 int launch_encode_window(const BatchArgs& args, int dtype, int N, int W, cudaStream_t stream) {
-#ifndef PVQ_DEBUG
     if (N == 256 || !has_window_tables(N, W, args.K)) return PVQ_ERR_UNSUPPORTED;
     const auto t = window_tables(N, args.K, stream);
     if (!t || t->args.words[N / 4 - 1] != 1) return PVQ_ERR_UNSUPPORTED;
@@ -455,7 +466,6 @@ int launch_encode_window(const BatchArgs& args, int dtype, int N, int W, cudaStr
         case 128 * 16 + 12: return launch_ew<128, 12>(a, dtype, *t, stream);
         default: break;
     }
-#endif
     return PVQ_ERR_UNSUPPORTED;
 }
 

@@ -45,7 +45,11 @@ int device_info(DeviceInfo* out) {
             return set_cuda_error(e);
         if ((e = cudaDeviceGetAttribute(&d.smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
             return set_cuda_error(e);
-        d.smem_max -= 256;  // room for the kernels' few bytes of static shared memory (an mbarrier)
+#ifdef PVQ_DEBUG
+        d.smem_max -= 512;  // ... and the checks' own
+#else
+        d.smem_max -= 256;  // room for the kernels' few bytes of static shared memory (mbarriers)
+#endif
         it = memo.emplace(dev, d).first;
     }
     *out = it->second;

@@ -33,3 +33,17 @@ def test_parity_suite_on_the_bounds_checked_build():
     import re
     m = re.search(r"(\d+) passed", r.stdout)
     assert m and int(m.group(1)) >= 80, tail      # the shared-memory kernels' cases all ran
+
+
+def test_wide_codes_on_the_bounds_checked_build():
+    """The kernels with windowed tables, resident and streamed: tables, output slots, the encoder's shared arrays, stores."""
+    from paper_2410_16926_b200 import build
+    lib = build.build(debug=True)
+    env = dict(os.environ, PVQ_B200_LIB=lib, PVQ_B200_DEBUG_STATUS="1")
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(ROOT, "tests", "test_gpu_wide_codes.py"), "-x", "-q", "-m", "gpu", "-rs"],
+                       cwd=ROOT, env=env, capture_output=True, text=True)
+    tail = (r.stdout + r.stderr)[-3000:]
+    assert r.returncode == 0, tail
+    import re
+    m = re.search(r"(\d+) passed", r.stdout)
+    assert m and int(m.group(1)) >= 60, tail      # (256, 768) is encoded by a global-table kernel: skipped
