@@ -246,13 +246,15 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
     for (int j = 0; j < PW; ++j) st.a[j] = v.w[PW - 1 - j];
 }
 
+constexpr uint32_t kNoStage = 0xffffffffu;  // no block of tables has arrived: nothing is read
+
 // All blocks from the one that PW words are first enough for: the widest first.
 template <int N, int PW, int PLANE, int KW, int W, typename Enter, typename Leave>
 __device__ __forceinline__ void win_blocks(WinState<W>& st, const BatchArgs& a, const WinArgs& t, int& b, uint32_t y, Enter&& enter, Leave&& leave) {
 #pragma unroll 1
     for (; b < t.blocks_of[PW]; ++b) {
         const uint32_t stage = enter(b), yb = y + static_cast<uint32_t>(b) * 4u;
-        win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
+        if (stage != kNoStage) win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
         leave(b);
     }
     if constexpr (PW > 1) win_blocks<N, PW - 1, PLANE, KW, W>(st, a, t, b, y, enter, leave);
@@ -324,10 +326,11 @@ __device__ __noinline__ bool win_walk(const uint32_t* count, int N, int K, const
     return !fits;
 }
 
-// One tile: the 32 groups of a warp, from the code to the stored values.
+// One tile: the 32 groups of a warp, from the code to the stored values.  enter(b) gives the shared address of block b,
+// or kNoStage, to all lanes alike; from then on `failed` is set, and the tile is not written.
 template <int N, int W, int PLANE, typename Enter, typename Leave>
 __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, const mp<W>& bound, unsigned tile, int& mi, uint32_t slots,
-                                         uint32_t y, uint8_t* slot, bool& bad, Enter&& enter, Leave&& leave) {
+                                         uint32_t y, uint8_t* slot, bool& bad, const bool& failed, Enter&& enter, Leave&& leave) {
     constexpr int YS = N + 4;
     const int lane = threadIdx.x & 31;
     const unsigned b = a.scale_bits;
@@ -380,6 +383,7 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
     st.lost = false;
     int blk = 0;
     win_blocks<N, W, PLANE, win_key_words(N), W>(st, a, t, blk, y, enter, leave);
+    if (failed) return;
 
     float amp = 0.0f;
     __nv_bfloat16* out = static_cast<__nv_bfloat16*>(m.out) + static_cast<size_t>(row) * m.ld_out + static_cast<size_t>(g) * N;
@@ -451,7 +455,7 @@ __global__ void __launch_bounds__(1024, 1)
         bulk_stage_copy(stage, smem, t.data, bytes);
     }
     const mp<W> bound = win_bound<W>(a, N);
-    if (!bulk_stage_wait(stage)) {  // the tables never arrived: report and leave
+    if (!__syncthreads_and(bulk_stage_wait(stage))) {  // the tables never arrived: report and leave, all threads
         if (a.status && threadIdx.x == 0) atomicOr(a.status, PVQ_STATUS_STAGING_TIMEOUT);
         return;
     }
@@ -465,7 +469,7 @@ __global__ void __launch_bounds__(1024, 1)
     bool bad = false;
     int mi = 0;
     for (unsigned tile = warp * gridDim.x + blockIdx.x; tile < a.total_tiles; tile += total)
-        win_tile<N, W, PLANE>(a, t, bound, tile, mi, slots, y, slot, bad, [&](int b) { return base + t.block_off[b]; }, [](int) {});
+        win_tile<N, W, PLANE>(a, t, bound, tile, mi, slots, y, slot, bad, false, [&](int b) { return base + t.block_off[b]; }, [](int) {});
     if (bad && a.status) atomicOr(a.status, PVQ_STATUS_INVALID_CODE);
 }
 
@@ -477,8 +481,8 @@ __device__ __forceinline__ void win_arrive(uint32_t bar) {
 
 // Streamed tables.  Buffer j holds the blocks n with n % bufs == j, n counted over all passes; full[j] completes when
 // a block has arrived, empty[j] when every decoding warp is through with it.  A wait that runs out sets the
-// status bit; the block then goes through the remaining motions without waiting and leaves (no copy is
-// issued into a buffer that was not given back, and the feeding warp waits for what it has issued).
+// status bit; the warp then goes through the remaining motions without waiting, reading or writing, and leaves (no copy
+// is issued into a buffer that was not given back, and the feeding warp waits for what it has issued).
 template <int N, int W, int PLANE>
 __global__ void __launch_bounds__(N == 256 ? 384 : 928, 1)
     decode_window_stream_kernel(const __grid_constant__ BatchArgs a, const __grid_constant__ WinArgs t, const __grid_constant__ WinGeom g) {
@@ -501,21 +505,24 @@ __global__ void __launch_bounds__(N == 256 ? 384 : 928, 1)
     debug_begin(shared_addr(smem), shared_addr(smem) + g.bufs * g.buf_bytes, shared_addr(smem) + g.slots_off, N + 4, N, a.debug_status);
 #endif
     const unsigned warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), step = gridDim.x * g.warps, first = blockIdx.x;
+    const bool withheld = debug_withhold(a.debug_status);
     const int passes = first < a.total_tiles ? static_cast<int>((a.total_tiles - first + step - 1) / step) : 0;
     if (warp == static_cast<unsigned>(g.warps)) {  // feeds the ring
         if ((threadIdx.x & 31) == 0) {
             const int n_all = passes * BLOCKS;
             int j = 0, round = 0, issued = 0;
             for (int n = 0, b = 0; n < n_all; ++n) {
-                if (round > 0 && !mbarrier_wait(shared_addr(&empty[j]), (round - 1) & 1)) {
+                if (round > 0 && !mbarrier_wait(shared_addr(&empty[j]), (round - 1) & 1, stream_polls(withheld))) {
                     atomicExch(&s_failed, 1);
                     break;
                 }
-                const BulkStage st{shared_addr(&full[j])};
-                const uint32_t bytes = t.block_off[b + 1] - t.block_off[b];
-                bulk_stage_expect(st, bytes);
-                bulk_stage_copy(st, smem + j * g.buf_bytes, t.data + t.block_off[b], bytes);
-                issued = n + 1;
+                if (!withheld) {
+                    const BulkStage st{shared_addr(&full[j])};
+                    const uint32_t bytes = t.block_off[b + 1] - t.block_off[b];
+                    bulk_stage_expect(st, bytes);
+                    bulk_stage_copy(st, smem + j * g.buf_bytes, t.data + t.block_off[b], bytes);
+                    issued = n + 1;
+                }
                 if (++b == BLOCKS) b = 0;
                 if (++j == g.bufs) j = 0, ++round;
             }
@@ -533,10 +540,11 @@ __global__ void __launch_bounds__(N == 256 ? 384 : 928, 1)
     for (int pass = 0; pass < passes; ++pass) {
         const unsigned tile = pass * step + warp * gridDim.x + blockIdx.x;  // the first tiles go to different SMs
         win_tile<N, W, PLANE>(
-            a, t, bound, tile, mi, slots, y, slot, bad,
+            a, t, bound, tile, mi, slots, y, slot, bad, failed,
             [&](int) {
-                if (!failed && !mbarrier_wait(shared_addr(&full[j]), parity)) failed = true;
-                return base + j * g.buf_bytes;
+                // (the warp as one: its lanes vote with each other further on)
+                if (!failed) failed = !__all_sync(kFull, mbarrier_wait(shared_addr(&full[j]), parity, stream_polls(withheld)));
+                return failed ? kNoStage : base + j * g.buf_bytes;
             },
             [&](int) {
                 __syncwarp();

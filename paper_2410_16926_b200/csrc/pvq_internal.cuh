@@ -397,9 +397,17 @@ __device__ __forceinline__ bool debug_index_ok(long long idx, long long limit, u
     return ok;
 }
 #define PVQ_DEBUG_INDEX(idx, limit, bit) debug_index_ok((idx), (limit), (bit))
+// Streamed tables that never arrive (PVQ_DEBUG_WITHHOLD in the caller's word, read before the block's first barrier):
+// the feeding warp leaves the copies out, and every wait gives up soon.
+__device__ __forceinline__ bool debug_withhold(const uint32_t* status) {
+    return status && (*const_cast<const volatile uint32_t*>(status) & PVQ_DEBUG_WITHHOLD) != 0u;
+}
 #else
 #define PVQ_DEBUG_INDEX(idx, limit, bit) true
+__device__ __forceinline__ constexpr bool debug_withhold(const uint32_t*) { return false; }
 #endif
+// polls of a wait for streamed tables
+__device__ __forceinline__ int stream_polls(bool withheld) { return withheld ? 1 << 6 : 1 << 22; }
 
 #endif  // __CUDACC__
 

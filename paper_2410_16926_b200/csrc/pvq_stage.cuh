@@ -15,9 +15,9 @@ __device__ __forceinline__ void mbarrier_init_fence() { asm volatile("fence.mbar
 
 // Waits for the phase `parity` of the barrier; false when it has not completed after a bounded
 // number of polls (the caller then leaves the kernel instead of spinning).
-__device__ __forceinline__ bool mbarrier_wait(uint32_t bar, int parity) {
+__device__ __forceinline__ bool mbarrier_wait(uint32_t bar, int parity, int polls = 1 << 22) {
     uint32_t done = 0;
-    for (int it = 0; it < (1 << 22) && !done; ++it) {
+    for (int it = 0; it < polls && !done; ++it) {
         asm volatile(
             "{\n\t"
             ".reg .pred p;\n\t"
