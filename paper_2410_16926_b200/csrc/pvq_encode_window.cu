@@ -135,14 +135,14 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
     encode_window_kernel(const __grid_constant__ BatchArgs a, const __grid_constant__ WinArgs t, const __grid_constant__ EwGeom g) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint64_t full[kEwBufs], empty[kEwBufs], go;
-    __shared__ int s_failed;
+    __shared__ int s_failed, s_gave_up;  // s_gave_up: written and read between the working warps' barriers only
     __shared__ uint8_t s_words[N];
     constexpr int E = 32, L = N / E, BLOCKS = N / 4, YS = N + 4, GW = 32 / L;
     constexpr bool WIDE = N == 64 ? W >= 7 : W >= 10;  // K may pass 127
     constexpr int P = E * (BF16 ? 2 : 4) / 16, RUN = kLaneRun<E, BF16>;
     grid_launch_dependents();
     if (threadIdx.x == 0) {
-        s_failed = 0;
+        s_failed = s_gave_up = 0;
         for (int j = 0; j < g.bufs; ++j) {
             mbarrier_init_one(&full[j]);
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(shared_addr(&empty[j])), "r"(g.warps) : "memory");
@@ -157,22 +157,25 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
 #endif
     const int warp = __shfl_sync(kFull, static_cast<int>(threadIdx.x) >> 5, 0), lane = threadIdx.x & 31;
     const int passes = blockIdx.x < a.total_tiles ? static_cast<int>((a.total_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+    const bool withheld = debug_withhold(a.debug_status);
     if (warp == g.warps) {  // feeds the ring; the points' input lies there while a tile is quantised
         if (lane == 0) {
             int j = 0, round = 0, n = 0;
             bool ok = true;
             for (int pass = 0; pass < passes && ok; ++pass) {
-                ok = mbarrier_wait(shared_addr(&go), pass & 1);
+                ok = mbarrier_wait(shared_addr(&go), pass & 1, stream_polls(withheld));
                 for (int b = BLOCKS - 1; b >= 0 && ok; --b) {
-                    if (round > 0 && !mbarrier_wait(shared_addr(&empty[j]), (round - 1) & 1)) {
+                    if (round > 0 && !mbarrier_wait(shared_addr(&empty[j]), (round - 1) & 1, stream_polls(withheld))) {
                         ok = false;
                         break;
                     }
-                    const BulkStage st{shared_addr(&full[j])};
-                    const uint32_t bytes = win_rows_bytes(t.words[b], PLANE);
-                    bulk_stage_expect(st, bytes);
-                    bulk_stage_copy(st, smem + j * g.buf_bytes, t.data + t.block_off[b], bytes);
-                    ++n;
+                    if (!withheld) {
+                        const BulkStage st{shared_addr(&full[j])};
+                        const uint32_t bytes = win_rows_bytes(t.words[b], PLANE);
+                        bulk_stage_expect(st, bytes);
+                        bulk_stage_copy(st, smem + j * g.buf_bytes, t.data + t.block_off[b], bytes);
+                        ++n;
+                    }
                     if (++j == g.bufs) j = 0, ++round;
                 }
             }
@@ -331,7 +334,8 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
         ew_blocks<1, PLANE, W>(
             st, t, blk, slot,
             [&]() {
-                if (!failed && !mbarrier_wait(shared_addr(&full[j]), parity)) failed = true;
+                // (a lane that gives up goes on with what is there, inside the buffer, and writes nothing)
+                if (!failed && !mbarrier_wait(shared_addr(&full[j]), parity, stream_polls(withheld))) failed = true;
                 return shared_addr(smem) + j * g.buf_bytes;
             },
             [&]() {
@@ -339,7 +343,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(shared_addr(&empty[j])) : "memory");
                 if (++j == g.bufs) j = 0, parity ^= 1;
             });
-        if (active && PVQ_DEBUG_INDEX(row, m.rows, PVQ_DEBUG_GLOBAL_STORE)) {
+        if (active && !failed && PVQ_DEBUG_INDEX(row, m.rows, PVQ_DEBUG_GLOBAL_STORE)) {
             const uint32_t kind = reinterpret_cast<const uint32_t*>(my_slot)[N / 4];
             uint32_t* cp = m.codes + (static_cast<size_t>(row) * G + gr) * W;
             if (kind == kEwPoint && (st.flag & kH4) != 0u) {
@@ -358,12 +362,14 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
                 for (int w = 0; w < W; ++w) cp[w] = code.w[w];
             }
         }
+        if (failed) s_gave_up = 1;
         ew_barrier(T);  // the amplitude indices are complete
         for (int i = threadIdx.x; i < nr * idx_words; i += T) {
             const int r = i / idx_words;
             reinterpret_cast<uint32_t*>(m.scale_idx + static_cast<size_t>(row0 + r) * m.sstride)[i - r * idx_words] = s_idx[i];
         }
         ew_barrier(T);
+        if (s_gave_up != 0) break;  // (a copy that comes late would land in the next tile's input)
     }
     if (a.status && (failed || s_failed != 0)) atomicOr(a.status, PVQ_STATUS_STAGING_TIMEOUT);
 }

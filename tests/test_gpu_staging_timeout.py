@@ -65,3 +65,8 @@ def run_child(N, bits, what):
 @pytest.mark.parametrize("N,bits", [(64, 256), (128, 384), (256, 768)])
 def test_decode_without_its_tables(N, bits):
     run_child(N, bits, "decode")
+
+
+@pytest.mark.parametrize("N,bits", [(64, 192), (64, 256), (128, 384)])
+def test_encode_without_its_tables(N, bits):
+    run_child(N, bits, "encode")
