@@ -311,8 +311,8 @@ int pvq_decode_static_table(const uint32_t* d_codes, const uint8_t* d_scale_idx,
 #define PVQ_DEBUG_SLOT_WRITE 2u   /* a write outside the thread's output slots */
 #define PVQ_DEBUG_SHARED_INDEX 4u /* an index outside one of the encoders' shared arrays */
 #define PVQ_DEBUG_GLOBAL_STORE 8u /* a store outside an output buffer */
-/* Set by the caller: the streamed tables of the kernels for wide codes are withheld, so that their
- * bounded waits run out (sooner than otherwise). */
+/* Set by the caller: the streamed tables of the kernels for wide codes and the round trip's input tiles
+ * are withheld, so that the bounded waits for them run out (sooner than otherwise). */
 #define PVQ_DEBUG_WITHHOLD 0x80000000u
 
 /* The library built with -DPVQ_DEBUG (`python -m paper_2410_16926_b200.build --debug`,

@@ -117,7 +117,9 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
     auto tile_rows = [&](unsigned tile) {
         return static_cast<int>(min(static_cast<long long>(a.rpt), a.rows - static_cast<long long>(tile) * a.rpt));
     };
+    const bool withheld = debug_withhold(a.debug_status);
     auto request = [&](unsigned tile, int buf) {  // thread 0
+        if (withheld) return;
         const int nr = tile_rows(tile);
         const BulkStage st{shared_addr(full + buf)};
         bulk_stage_expect(st, nr * row_bytes);
@@ -172,10 +174,8 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         uint8_t* mine = smem + lane_off + buf * a.tile_bytes;
         const bool active = rl < a.rpt && static_cast<long long>(tile) * a.rpt + rl < a.rows;
         float* s_ss = reinterpret_cast<float*>(smem + a.ss_off) + (i & 1) * a.rpt * a.gp;
-        if (!mbarrier_wait(shared_addr(full + buf), parity)) {  // the copy never arrived: report and leave rather than spin
-            if (a.status) atomicOr(a.status, PVQ_STATUS_STAGING_TIMEOUT);
-            return;
-        }
+        // (a thread that gives up works on whatever the buffer holds, as far as the next barrier)
+        const bool failed = !mbarrier_wait(shared_addr(full + buf), parity, stream_polls(withheld));
         float ss;
         uint32_t neg[E / 4];
         LanePoint<E, WIDE> pt;
@@ -216,7 +216,14 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         }
         // energies are in place, and the tile before this one is complete in its buffer
         bulk_store_fence();
-        __syncthreads();
+        if (__syncthreads_or(failed)) {  // the copy never arrived: report and leave rather than spin, all threads
+            if (a.status && failed) atomicOr(a.status, PVQ_STATUS_STAGING_TIMEOUT);
+            if (tid == 0) {
+                if (i > 0) deliver(tile - gridDim.x, buf == 0 ? 2 : buf - 1);
+                bulk_store_wait_read<0>();
+            }
+            return;
+        }
         const unsigned next = tile + gridDim.x;
         const bool have_next = next < a.tiles;
         const int nbuf = buf == 2 ? 0 : buf + 1;

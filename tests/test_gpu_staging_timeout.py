@@ -1,4 +1,4 @@
-"""Streamed tables that never arrive: every wait is bounded, the call ends, its status word says so, and nothing is read or
+"""Streamed tables (and the round trip's input tiles) that never arrive: every wait is bounded, the call ends, its status word says so, and nothing is read or
 written that depends on the tables.  On the bounds-checked build (in a child process), which can withhold the copies and then
 waits for a short while only; afterwards the same calls go through."""
 import os
@@ -15,7 +15,7 @@ CHILD = """
 import sys
 import numpy as np, torch
 from oracle import pvq_oracle as po
-from paper_2410_16926_b200 import pvq
+from paper_2410_16926_b200 import inputs, pvq
 N, bits, what = int(sys.argv[1]), int(sys.argv[2]), sys.argv[3]
 WITHHOLD = -2 ** 31
 K = pvq.max_pulses(N, bits)
@@ -34,7 +34,14 @@ pvq.encode_status(status)
 for withheld in (True, False):
     word.fill_(WITHHOLD if withheld else 0)
     status.zero_()
-    if what == "decode":
+    if what == "roundtrip":
+        out = torch.full((rows, G * N), 77.0, dtype=torch.bfloat16, device="cuda")
+        pvq.roundtrip(x_dev.to(torch.bfloat16), N, K, 16, table, None, None, out=out)
+        torch.cuda.synchronize()
+        got, canary = out.view(torch.int16).cpu().numpy().view(np.uint16), np.uint16(0x429a)
+        b = po.encode(inputs.f32_to_bf16_bits(x), N, K, 16, None, W=W)
+        want = po.decode(*b, N, K, 16, None)[0]
+    elif what == "decode":
         out = torch.full((rows, G * N), 77.0, dtype=torch.bfloat16, device="cuda")
         pvq.decode(*enc, N, K, 16, table, None, out=out, status=status)
         torch.cuda.synchronize()
@@ -70,3 +77,8 @@ def test_decode_without_its_tables(N, bits):
 @pytest.mark.parametrize("N,bits", [(64, 192), (64, 256), (128, 384)])
 def test_encode_without_its_tables(N, bits):
     run_child(N, bits, "encode")
+
+
+@pytest.mark.parametrize("N,bits", [(32, 64), (128, 384)])
+def test_round_trip_without_its_input(N, bits):
+    run_child(N, bits, "roundtrip")
