@@ -207,7 +207,6 @@ template <int N, int W, bool EXACT, typename YT>
 __global__ void __launch_bounds__(kBigThreads) decode_big_kernel(const __grid_constant__ BatchArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     constexpr int YS = N * static_cast<int>(sizeof(YT)) + 4;
-    grid_launch_dependents();
     grid_dependency_wait();
     const int K = a.K;
     const int Wc = EXACT ? W : a.code_words;
@@ -301,7 +300,7 @@ int launch_decode_big_t(BatchArgs& a, cudaStream_t stream) {
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
     const unsigned wpb = threads / 32;
     const unsigned grid = std::max(1u, std::min<unsigned>((tiles + wpb - 1) / wpb, di.sms * per_sm));
-    return launch_hot(kern, grid, threads, smem, stream, a);
+    return launch_hot_if(false, kern, grid, threads, smem, stream, a);
 }
 
 // ------------------------------------------------------------------------- encode

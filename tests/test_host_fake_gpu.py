@@ -163,6 +163,19 @@ def test_a_hot_call_does_not_wait_for_another_threads_build(fake):
     assert finished == 3 and done == [0, 0, 0]
 
 
+def test_which_launches_may_start_early(fake):
+    """Kernels that fill the GPU and read tables through L1 start when the one before has ended; the others early."""
+    def early():
+        return bool(fake.fake_launch_early(fake.fake_launches() - 1))
+    K = pvq.max_pulses(64, 320)          # tables in global memory, both ways
+    assert decode(fake, 64, K, rows=4096, G=64) == 0 and not early()
+    assert decode(fake, 64, K) == 0 and not early()
+    assert encode(fake, 64, K, rows=256, G=64) == 0 and not early()  # two lanes a group
+    assert encode(fake, 64, K, rows=255, G=64) == 0 and early()
+    assert decode(fake, 32, 50, rows=4096, G=128) == 0 and early()
+    assert encode(fake, 32, 50, rows=4096, G=128) == 0 and early()
+
+
 OUT_OF_HOST_MEMORY = """
 import resource, sys
 sys.path.insert(0, sys.argv[2])
