@@ -666,10 +666,16 @@ static int launch_encode_t(BatchArgs& a, cudaStream_t stream) {
     return e == cudaSuccess ? PVQ_OK : set_cuda_error(e);
 }
 
-template <int N, int W>
+template <int N, int W, bool ROT>
 static int launch_encode_nw(BatchArgs& a, int dtype, cudaStream_t s) {
-    if (a.amp_mode == 1) return PVQ_ERR_UNSUPPORTED;  // least squares: not with a rotation
-    return dtype == PVQ_DTYPE_BF16 ? launch_encode_t<N, W, true, true>(a, s) : launch_encode_t<N, W, false, true>(a, s);
+    const bool bf16 = dtype == PVQ_DTYPE_BF16;
+    if (a.amp_mode == 1) {
+        if constexpr (ROT)
+            return PVQ_ERR_UNSUPPORTED;  // least squares: not with a rotation
+        else
+            return bf16 ? launch_encode_t<N, W, true, false, true>(a, s) : launch_encode_t<N, W, false, false, true>(a, s);
+    }
+    return bf16 ? launch_encode_t<N, W, true, ROT>(a, s) : launch_encode_t<N, W, false, ROT>(a, s);
 }
 
 }  // namespace pvq

@@ -711,10 +711,23 @@ static int launch_encode_any(BatchArgs& a, int dtype, cudaStream_t s) {
             const int st = dtype == PVQ_DTYPE_BF16 ? launch_encode_lanes<E, L, W, true>(b, s) : launch_encode_lanes<E, L, W, false>(b, s);
             if (st != PVQ_ERR_UNSUPPORTED) return st;
         }
+        // More than 127 pulses, but cumulative tables that fit shared memory: the general kernel with them, but for large bf16
+        // input and the plain amplitude.  (us, general kernel and this one with tables in global memory, fp32: N = 8, 56 bits,
+        // 1024 x 4096 24.6, 57.4, 4096 x 4096 79.6, 91.9; N = 16, 90 bits 25.9, 57.6, 78.6, 88.6; bf16: N = 8 2048 x 4096 56.3,
+        // 64.9, 4096 x 4096 108.6, 89.2; N = 16 41.0, 55.3, 75.8, 73.8.)
+        if constexpr ((N == 8 && W == 2) || (N == 16 && W == 3)) {
+            long long values = 0;
+            for (int i = 0; i < a.count; ++i) values += a.m[i].rows * a.m[i].cols;
+            if (a.K > 127 && (values < (1 << 24) || dtype == PVQ_DTYPE_F32 || a.amp_mode == 1)) {
+                b = a;
+                const int st = launch_encode_nw<N, W, false>(b, dtype, s);
+                if (st != PVQ_ERR_UNSUPPORTED) return st;
+            }
+        }
         b = a;
         return launch_encode_lanes_global<N, (W <= 4 ? 4 : W)>(b, dtype, s);
     }
-    return launch_encode_nw<N, W>(a, dtype, s);
+    return launch_encode_nw<N, W, true>(a, dtype, s);
 }
 
 }  // namespace pvq
