@@ -249,15 +249,15 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
 constexpr uint32_t kNoStage = 0xffffffffu;  // no block of tables has arrived: nothing is read
 
 // All blocks from the one that PW words are first enough for: the widest first.
-template <int N, int PW, int PLANE, int KW, int W, typename Enter, typename Leave>
+template <bool STREAM, int N, int PW, int PLANE, int KW, int W, typename Enter, typename Leave>
 __device__ __forceinline__ void win_blocks(WinState<W>& st, const BatchArgs& a, const WinArgs& t, int& b, uint32_t y, Enter&& enter, Leave&& leave) {
 #pragma unroll 1
     for (; b < t.blocks_of[PW]; ++b) {
         const uint32_t stage = enter(b), yb = y + static_cast<uint32_t>(b) * 4u;
-        if (stage != kNoStage) win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
+        if (!STREAM || stage != kNoStage) win_block4<N, PW, PLANE, KW, W>(st, stage, a, t, b, yb);
         leave(b);
     }
-    if constexpr (PW > 1) win_blocks<N, PW - 1, PLANE, KW, W>(st, a, t, b, y, enter, leave);
+    if constexpr (PW > 1) win_blocks<STREAM, N, PW - 1, PLANE, KW, W>(st, a, t, b, y, enter, leave);
 }
 
 // Algorithm 3 step by step for the group at hand, from the count table in global memory: for points with a |y| of 128 or
@@ -327,8 +327,8 @@ __device__ __noinline__ bool win_walk(const uint32_t* count, int N, int K, const
 }
 
 // One tile: the 32 groups of a warp, from the code to the stored values.  enter(b) gives the shared address of block b,
-// or kNoStage, to all lanes alike; from then on `failed` is set, and the tile is not written.
-template <int N, int W, int PLANE, typename Enter, typename Leave>
+// or, streamed, kNoStage, to all lanes alike; from then on `failed` is set, and the tile is not written.
+template <bool STREAM, int N, int W, int PLANE, typename Enter, typename Leave>
 __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, const mp<W>& bound, unsigned tile, int& mi, uint32_t slots,
                                          uint32_t y, uint8_t* slot, bool& bad, const bool& failed, Enter&& enter, Leave&& leave) {
     constexpr int YS = N + 4;
@@ -382,8 +382,8 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
     st.ssy = 0u;
     st.lost = false;
     int blk = 0;
-    win_blocks<N, W, PLANE, win_key_words(N), W>(st, a, t, blk, y, enter, leave);
-    if (failed) return;
+    win_blocks<STREAM, N, W, PLANE, win_key_words(N), W>(st, a, t, blk, y, enter, leave);
+    if (STREAM && failed) return;
 
     float amp = 0.0f;
     __nv_bfloat16* out = static_cast<__nv_bfloat16*>(m.out) + static_cast<size_t>(row) * m.ld_out + static_cast<size_t>(g) * N;
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(1024, 1)
     bool bad = false;
     int mi = 0;
     for (unsigned tile = warp * gridDim.x + blockIdx.x; tile < a.total_tiles; tile += total)
-        win_tile<N, W, PLANE>(a, t, bound, tile, mi, slots, y, slot, bad, false, [&](int b) { return base + t.block_off[b]; }, [](int) {});
+        win_tile<false, N, W, PLANE>(a, t, bound, tile, mi, slots, y, slot, bad, false, [&](int b) { return base + t.block_off[b]; }, [](int) {});
     if (bad && a.status) atomicOr(a.status, PVQ_STATUS_INVALID_CODE);
 }
 
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(N == 256 ? 384 : 928, 1)
     int mi = 0, j = 0, parity = 0;
     for (int pass = 0; pass < passes; ++pass) {
         const unsigned tile = pass * step + warp * gridDim.x + blockIdx.x;  // the first tiles go to different SMs
-        win_tile<N, W, PLANE>(
+        win_tile<true, N, W, PLANE>(
             a, t, bound, tile, mi, slots, y, slot, bad, failed,
             [&](int) {
                 // (the warp as one: its lanes vote with each other further on)
