@@ -634,10 +634,12 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
         if (teams < 1) continue;
         const double per_tile = static_cast<double>(chunks_all) / tiles + (t == 32 ? 0.16 : 0.25);
         const double rounds = std::ceil(static_cast<double>(tiles) / (static_cast<double>(teams) * di.sms));
-        // an SM with fewer warps than it holds runs them faster, down to about a quarter of the time
-        const double load = std::max(0.25, std::min(1.0, static_cast<double>(teams) * t / kLaneThreads<W>));
-        const double few = rounds > 1.0 ? 1.0 : std::max(0.25, std::min(1.0, static_cast<double>(tiles) * t / (static_cast<double>(di.sms) * kLaneThreads<W>)));
-        const double cost = rounds * per_tile * load * few;
+        // In a long launch an SM with fewer warps than it holds runs them faster.  Few rounds take as long with few warps as with
+        // many: the latency of tables and barriers, not issue.  (Taken for up to four times shorter, one-warp teams with a row in
+        // many chunks won where rows are few: 1024 x 4096 at N = 64, 320 bits, 145 us instead of 84, N = 32, 96 bits 19.4
+        // instead of 14.9.  A decoder layer, 13 rounds: 402 us, 454 without the factor.)
+        const double load = rounds > 4.0 ? static_cast<double>(teams) * t / kLaneThreads<W> : 1.0;
+        const double cost = rounds * per_tile * load;
         if (best < 0.0 || cost < best) {
             best = cost;
             c.teams = static_cast<int>(std::min<long long>(teams, (tiles + di.sms - 1) / di.sms));

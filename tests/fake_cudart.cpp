@@ -66,6 +66,7 @@ int fake_launches() { return static_cast<int>(launches.size()); }
 const char* fake_launch_name(int i) { return launches[i].name.c_str(); }
 uint64_t fake_launch_table(int i, int which) { return launches[i].tables[which]; }
 unsigned fake_launch_grid(int i) { return launches[i].grid; }
+unsigned fake_launch_block(int i) { return launches[i].block; }
 int fake_launch_early(int i) { return launches[i].early; }
 int fake_live(uint64_t p) {  // does p lie in live memory?
     std::lock_guard<std::mutex> lock(mu);

@@ -176,6 +176,18 @@ def test_which_launches_may_start_early(fake):
     assert encode(fake, 32, 50, rows=4096, G=128) == 0 and early()
 
 
+@pytest.mark.parametrize("N,K,rows,G,lanes", [(8, 12, 1024, 512, 1), (16, 27, 1024, 256, 1), (32, 50, 1024, 128, 1), (64, 26, 1024, 64, 2),
+                                              (32, 1000, 600, 128, 1)])
+def test_few_rows_still_fill_the_gpu(fake, N, K, rows, G, lanes):
+    """The encoder's teams: a matrix of medium size is given as many threads as it has groups (lanes), up to what an SM
+    holds, not one warp a row that takes the row's chunks one after the other."""
+    assert encode(fake, N, K, rows=rows, G=G) == 0
+    i = fake.fake_launches() - 1
+    assert "encode_lanes" in fake.fake_launch_name(i).decode()
+    threads = fake.fake_launch_grid(i) * fake.fake_launch_block(i)
+    assert threads >= 0.75 * min(rows * G * lanes, 148 * 768)
+
+
 OUT_OF_HOST_MEMORY = """
 import resource, sys
 sys.path.insert(0, sys.argv[2])
