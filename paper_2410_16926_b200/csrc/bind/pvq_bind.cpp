@@ -14,6 +14,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <cstring>
 #include <vector>
 
 #include "pvq.h"
@@ -34,7 +35,7 @@ struct Entries {
     decltype(&pvq_scale_row_stride) scale_row_stride;
 } lib;
 PyObject* raise_error = nullptr;  // raise_error(status, where) raises PvqError
-PyObject *k_x, *k_out, *k_codes, *k_scale_idx, *k_row_norm, *k_edges, *k_levels, *k_cols;
+PyObject *k_get, *k_x, *k_out, *k_codes, *k_scale_idx, *k_row_norm, *k_edges, *k_levels, *k_cols;
 
 bool failed(int status, const char* where) {
     if (status == PVQ_OK) return false;
@@ -330,21 +331,40 @@ PyObject* bind_rotate_roundtrip(PyObject*, PyObject* const* a, Py_ssize_t n) {
     END_HANDLE_TH_ERRORS
 }
 
-// One item of a batched call (a dict of tensors).
-const at::Tensor* item_tensor(PyObject* d, PyObject* key, bool needed, bool* bad) {
-    PyObject* v = PyDict_GetItemWithError(d, key);
+// Entries of one item of a batched call: a dict, or any mapping with get().
+struct Held {  // references to what a mapping returned, as long as it is looked at
+    std::vector<PyObject*> refs;
+    ~Held() {
+        for (PyObject* o : refs) Py_DECREF(o);
+    }
+};
+PyObject* item_value(PyObject* d, PyObject* key, bool needed, Held* held) {  // null: not there, or an error
+    PyObject* v;
+    if (PyDict_CheckExact(d)) {
+        v = PyDict_GetItemWithError(d, key);
+        Py_XINCREF(v);
+        if (!v && needed && !PyErr_Occurred()) PyErr_SetObject(PyExc_KeyError, key);
+    } else {
+        v = needed ? PyObject_GetItem(d, key) : PyObject_CallMethodOneArg(d, k_get, key);
+    }
+    if (v) held->refs.push_back(v);
+    return v;
+}
+const at::Tensor* item_tensor(PyObject* d, PyObject* key, bool needed, Held* held, bool* bad) {
+    if (*bad) return nullptr;
+    PyObject* v = item_value(d, key, needed, held);
     if (!v) {
-        if (needed && !PyErr_Occurred()) PyErr_SetObject(PyExc_KeyError, key);
         *bad = PyErr_Occurred() != nullptr;
         return nullptr;
     }
     if (v == Py_None && !needed) return nullptr;
     const at::Tensor* t = tensor_of(v);
-    *bad = *bad || !t;
+    *bad = !t;
     return t;
 }
 
 bool describe(PyObject* items, std::vector<pvq_matrix_desc>* descs) {
+    if (PyObject_Length(items) < 0) return false;  // (anything that has a length and can be gone through)
     PyObject* seq = PySequence_Fast(items, "expected a sequence of matrices");
     if (!seq) return false;
     const Py_ssize_t count = PySequence_Fast_GET_SIZE(seq);
@@ -352,23 +372,18 @@ bool describe(PyObject* items, std::vector<pvq_matrix_desc>* descs) {
     bool bad = false;
     for (Py_ssize_t i = 0; i < count && !bad; ++i) {
         PyObject* it = PySequence_Fast_GET_ITEM(seq, i);
-        if (!PyDict_Check(it)) {
-            PyErr_SetString(PyExc_TypeError, "expected dicts of tensors");
-            bad = true;
-            break;
-        }
         pvq_matrix_desc& d = (*descs)[static_cast<size_t>(i)];
-        const at::Tensor* x = item_tensor(it, k_x, false, &bad);
-        const at::Tensor* out = bad ? nullptr : item_tensor(it, k_out, false, &bad);
-        const at::Tensor* edges = bad ? nullptr : item_tensor(it, k_edges, false, &bad);
-        const at::Tensor* levels = bad ? nullptr : item_tensor(it, k_levels, false, &bad);
-        const at::Tensor* codes = bad ? nullptr : item_tensor(it, k_codes, true, &bad);
-        const at::Tensor* sidx = bad ? nullptr : item_tensor(it, k_scale_idx, true, &bad);
-        const at::Tensor* rnorm = bad ? nullptr : item_tensor(it, k_row_norm, true, &bad);
+        Held held;
+        const at::Tensor* x = item_tensor(it, k_x, false, &held, &bad);
+        const at::Tensor* out = item_tensor(it, k_out, false, &held, &bad);
+        const at::Tensor* codes = item_tensor(it, k_codes, true, &held, &bad);
+        const at::Tensor* sidx = item_tensor(it, k_scale_idx, true, &held, &bad);
+        const at::Tensor* rnorm = item_tensor(it, k_row_norm, true, &held, &bad);
+        const at::Tensor* edges = item_tensor(it, k_edges, false, &held, &bad);
+        const at::Tensor* levels = item_tensor(it, k_levels, false, &held, &bad);
         if (bad) break;
-        PyObject* cols_o = PyDict_GetItemWithError(it, k_cols);
+        PyObject* cols_o = item_value(it, k_cols, true, &held);
         long long cols = 0;
-        if (!cols_o && !PyErr_Occurred()) PyErr_SetObject(PyExc_KeyError, k_cols);
         bad = !cols_o || !integer(cols_o, &cols);
         if (!bad && codes->dim() != 3) {
             PyErr_SetString(PyExc_ValueError, "expected codes of three dimensions");
@@ -457,6 +472,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_bind", nullptr, -1, methods};
 }  // namespace
 
 PyMODINIT_FUNC PyInit__bind() {
+    k_get = PyUnicode_InternFromString("get");
     k_x = PyUnicode_InternFromString("x");
     k_out = PyUnicode_InternFromString("out");
     k_codes = PyUnicode_InternFromString("codes");
