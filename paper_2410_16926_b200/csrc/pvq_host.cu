@@ -18,6 +18,7 @@ static thread_local int g_last_cuda_error = 0;
 
 int set_cuda_error(cudaError_t e) {
     g_last_cuda_error = static_cast<int>(e);
+    cudaGetLastError();  // reported by this call: not for a later one to find
     return PVQ_ERR_CUDA;
 }
 

@@ -188,6 +188,16 @@ def test_few_rows_still_fill_the_gpu(fake, N, K, rows, G, lanes):
     assert threads >= 0.75 * min(rows * G * lanes, 148 * 768)
 
 
+@pytest.mark.parametrize("call,N,K", [(decode, 32, 50), (encode, 32, 50), (decode, 64, 96), (decode, 64, 300), (encode, 64, 300)])
+def test_a_failed_launch_is_reported_once(fake, call, N, K):
+    assert build(fake, 64, 96) == 0
+    fake.fake_fail_launches(701)
+    assert call(fake, N, K) == 5 and fake.pvq_last_cuda_error() == 701
+    fake.fake_fail_launches(0)
+    assert build(fake, 32, 22) == 0, "found the error of an earlier call"
+    assert call(fake, N, K) == 0
+
+
 OUT_OF_HOST_MEMORY = """
 import resource, sys
 sys.path.insert(0, sys.argv[2])
