@@ -6,7 +6,7 @@ _bind.so, the native part of the Python binding (csrc/bind/pvq_bind.cpp).
 
 --debug builds libpvq_b200_debug.so instead: the bounds-checked variant (-DPVQ_DEBUG, see
 pvq_debug_status in include/pvq.h) of the kernels that keep their tables in shared memory;
-the global-table kernels are left out of it (calls that need them return "unsupported").
+the global-table kernels are left out of it (calls that need them return "unsupported").  The binding is the same.
 """
 import os
 import subprocess
@@ -60,8 +60,7 @@ def build_bind(force: bool = False) -> str:
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
-    if not debug:
-        build_bind(force)
+    build_bind(force)
     objdir = os.path.join(OBJDIR, "debug") if debug else OBJDIR
     lib = DEBUG_LIB if debug else LIB
     os.makedirs(objdir, exist_ok=True)

@@ -205,3 +205,15 @@ def test_c_example_round_trip_on_the_gpu(tmp_path):
     assert r.returncode == 0, r.stdout + r.stderr
     assert "status 0, QSNR" in r.stdout
 
+
+
+def test_the_bounds_checked_build_comes_with_the_binding(tmp_path, monkeypatch):
+    """PVQ_B200_LIB may point at that build where no other has been made: the binding's native part is needed all the same."""
+    from paper_2410_16926_b200 import build as lib_build
+    there = tmp_path / "libpvq_b200_debug.so"
+    there.write_bytes(b"")
+    made = []
+    monkeypatch.setattr(lib_build, "DEBUG_LIB", str(there))
+    monkeypatch.setattr(lib_build, "OBJDIR", str(tmp_path))
+    monkeypatch.setattr(lib_build, "build_bind", lambda force=False: made.append(force))
+    assert lib_build.build(debug=True) == str(there) and made == [False]
