@@ -153,18 +153,21 @@ int pvq_build_scale_codebook(int N, int64_t G, int scale_bits, float* d_edges, f
  *   d_x        rows x cols values of `dtype`, leading dimension ld (elements); 16-byte
  *              aligned, ld a multiple of 8 (bf16) or 4 (fp32) elements.
  *   N, K       group size (power of two, 8..256) and pulses (up to 8191, codes of up to 32
- *              words); cols % N == 0; 2 <= G <= 4096.  Codes of up to 2, 3, 4, 6 words at
- *              N = 8, 16, 32, 64 run on the kernels with the tables in shared memory.  Wider
- *              codes at N >= 16, and N = 128 and 256, run on slower kernels that keep the
- *              tables in global memory (the paper's grid of group sizes and direction bits,
- *              Sec. 4.1).
- *              Rows of up to 4096 groups are taken by pvq_encode proper (amplitude ||x_g||,
- *              no rotation) for codes of up to 4 words and K <= 127.  Everything else on the
- *              encode side - pvq_roundtrip, pvq_encode_amp with amp_mode 1, the rotating
- *              calls, 5- and 6-word codes, K > 127, the global-table kernels - keeps a whole
- *              row in one thread block and returns PVQ_ERR_UNSUPPORTED for G > 512 (fewer on
- *              the global-table kernels, where a row also has to fit shared memory: about
- *              G <= 256 at N = 128, 192 at N = 256).  Decoding has no such limit.
+ *              words); cols % N == 0; 2 <= G <= 4096.  Codes of up to 2, 3, 4, 4 words at
+ *              N = 8, 16, 32, 64 run on kernels with the tables in shared memory, 5 to 8 words at
+ *              N = 64, 9 to 12 at N = 128 and (decoding) 24 at N = 256 on kernels with windowed
+ *              tables (see pvq_build_count_table), the rest on slower kernels that read the tables
+ *              from global memory (the paper's grid of group sizes and direction bits, Sec. 4.1);
+ *              codes of more than 2 words at N = 8 are encoded and decoded by none
+ *              (PVQ_ERR_UNSUPPORTED), but pvq_roundtrip, which makes no codes, takes them.
+ *              Rows of up to 4096 groups are taken by every call but pvq_rotate_encode, which keeps
+ *              a whole row in one thread block: PVQ_ERR_UNSUPPORTED for G > 512 (where the tables
+ *              are in global memory a row also has to fit shared memory: about G <= 256 at N = 128,
+ *              192 at N = 256).
+ *              The windowed kernels are made for values as the paper encodes them, rotated: their
+ *              time, not their result, depends on the data.  Where many groups have most of their
+ *              l1 norm in few places, decoding takes longer: 1.3 to 7 times as long as by the walk
+ *              that needs no windows for unrotated heavy-tailed weights, 8 to 23 times for sparse ones.
  *   scale_bits 1..8 (quantile index), or 16 (see pvq_encode_amp).
  *   d_table    from pvq_build_count_table(N, K, ...).
  *   d_edges    2^scale_bits - 1 bin edges.
@@ -225,11 +228,11 @@ int pvq_encode_amp(const void* d_x, int dtype, int64_t rows, int64_t cols, int64
  * Sylvester-Walsh-Hadamard matrix; the rotated row is then encoded (pvq_rotate_encode) or
  * encoded and decoded (pvq_rotate_roundtrip) exactly as by pvq_encode / pvq_roundtrip on fp32
  * input, without the rotated matrix ever being written to memory.
- *   block      a power of two, a multiple of N, dividing cols, at most 16384.
+ *   block      a power of two, a multiple of N, dividing cols, at most 16384; for
+ *              pvq_rotate_roundtrip at N = 8 and 16 at most 4096 and 8192 where G > 512.
  * Arithmetic: fp32; the sign flip, then butterflies (a, b) -> (a + b, a - b) with strides
  * 1, 2, 4, ..., block/2, one rounding each, then one multiplication by the fp32 nearest to
- * 1/sqrt(block).  The other arguments are those of pvq_encode / pvq_roundtrip; on the kernels
- * with the tables in shared memory the fused form needs K <= 127. */
+ * 1/sqrt(block).  The other arguments are those of pvq_encode / pvq_roundtrip. */
 int pvq_rotate_encode(const void* d_x, int dtype, int64_t rows, int64_t cols, int64_t ld, int block,
                       const float* d_signs, int N, int K, int scale_bits, const uint32_t* d_table,
                       const float* d_edges, uint32_t* d_codes, uint8_t* d_scale_idx, float* d_row_norm,
