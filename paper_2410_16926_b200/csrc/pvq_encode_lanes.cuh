@@ -601,6 +601,9 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
     // Team size: the one whose rounds of tiles cost least.  A chunk costs about as much as six times
     // what a tile adds (energies, amplitude indices), eight with a barrier between warps; what
     // decides is mostly how full the last round is.
+    long long lanes = 0;
+    for (int i = 0; i < a.count; ++i) lanes += a.m[i].rows * a.m[i].G * L;
+    const bool long_launch = lanes > 8ll * di.sms * kLaneThreads<W>;
     double best = -1.0;
     LaneGeom chosen{};
     for (int t : {32, 64, 96, 128, 160, 192, 224, 256}) {
@@ -637,8 +640,8 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
         // In a long launch an SM with fewer warps than it holds runs them faster.  Few rounds take as long with few warps as with
         // many: the latency of tables and barriers, not issue.  (Taken for up to four times shorter, one-warp teams with a row in
         // many chunks won where rows are few: 1024 x 4096 at N = 64, 320 bits, 145 us instead of 84, N = 32, 96 bits 19.4
-        // instead of 14.9.  A decoder layer, 13 rounds: 402 us, 454 without the factor.)
-        const double load = rounds > 4.0 ? static_cast<double>(teams) * t / kLaneThreads<W> : 1.0;
+        // instead of 14.9.  A decoder layer, work for 51 rounds: 402 us, 454 without the factor.)
+        const double load = long_launch ? static_cast<double>(teams) * t / kLaneThreads<W> : 1.0;
         const double cost = rounds * per_tile * load;
         if (best < 0.0 || cost < best) {
             best = cost;
@@ -670,8 +673,6 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
     const unsigned grid = std::min<unsigned>(blocks, static_cast<unsigned>(di.sms * per_sm));
     // Tables in global memory: early only where the launch is small and its start counts (4096 groups at N = 16, 128 bits: 12.1 us
     // early, 14.3 in order; 32768 groups at N = 32, 200 bits, not yet a block an SM: 31.6 and 22.6).
-    long long lanes = 0;
-    for (int i = 0; i < a.count; ++i) lanes += a.m[i].rows * a.m[i].G * L;
     return launch_hot_if(RE != 0 || lanes < 32768, kern, grid, threads, smem, stream, a, g);
 }
 
