@@ -11,8 +11,8 @@
 // (N = 128, 384 bits: 760 KB; N = 256: 2.4 MB) they are streamed from L2 through a ring of buffers, block of rows
 // after block of rows, all warps of the thread block following the stream; an additional warp feeds it.
 //
-// Measured, with the walk (pvq_walk.cuh, pvq_big_impl.cuh) and now: 8192 x 28672, N = 64, 192 bits, 774 -> 364 us (79% of the
-// issue slots, 86% of the shared-memory wavefronts a cycle); 4096 x 4096, N = 128, 384 bits, 190 -> 47 us; N = 256, 768
+// Measured, with the walk (pvq_walk.cuh, pvq_big_impl.cuh) and now: 8192 x 28672, N = 64, 192 bits, 774 -> 368 us (79% of the
+// issue slots, 86% of the shared-memory wavefronts a cycle); 4096 x 4096, N = 128, 384 bits, 190 -> 48.5 us; N = 256, 768
 // bits, 601 -> 160 us.
 // (Group size 256 has a translation unit of its own: the functions that are not inlined take the registers of the
 // most generous kernel that calls them, and spill in the others.)

@@ -69,6 +69,8 @@ struct WinTables {
 __host__ __device__ constexpr uint32_t win_rows_bytes(int words, int plane) { return kWinHead + 16u * words * plane; }
 
 // The settings with windowed kernels: codes of 5 to 8 words at group size 64, 9 to 12 at 128, 24 at 256 (decoding only).
+// Those are the widths up to 4 direction bits a value at N = 64 and 3 at N = 128 and 256 that workloads here have; the
+// tables suit others too (with up to 255 pulses, or 160 thresholds a row), but every width is kernels of its own.
 constexpr bool has_window_tables(int N, int W, int K) {
     return (N == 64 && W >= 5 && W <= 8 && K <= 255) || (N == 128 && W >= 9 && W <= 12 && K <= 255) || (N == 256 && W == 24);
 }
