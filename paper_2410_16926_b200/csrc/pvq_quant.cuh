@@ -6,13 +6,15 @@
 //   the d largest residuals e_i get one more pulse, lowest index first among equals
 //   (why this is the greedy loop's result: quantize_direction in pvq_encode_impl.cuh).
 //
-// Nothing is sorted.  The residuals' leading 7 bits sit in the bytes of E / 4 words, so that one
-// subtract per word compares four of them with a threshold (bit 7 of a byte of
-// 0x80 + residual - threshold is "not below"), and a few such passes bracket the d-th largest.
-// What is left between the two ends of the bracket, at most a few residuals per lane, is
-// ranked on the exact fp32 values, fetched again from where the group came from.  A sorting
-// network over 32 fp32 residuals is 382 min / max instructions at half rate; this is about
-// five passes of 8 subtracts, 8 ands and 8 byte sums.
+// Nothing is sorted or counted twice.  The residuals' leading 8 bits, a byte each, are turned into eight bit
+// planes (a plane: one bit of every residual of the lane, in one register), and the d-th largest is found
+// a bit at a time from the top: the residuals still undecided that have the bit are either all chosen, or
+// are the undecided ones from here on.  What no bit of the eight tells apart, two residuals of a group now
+// and then, is ranked on the exact fp32 values, fetched again from where the group came from.
+// 32 values a lane: 48 instructions for the planes, 56 for the eight steps (a sorting network: 382 min / max at half
+// rate; before: about five counting passes of some 45 instructions, and four candidates to rank).  What uses it is
+// bound by issue: encoding a decoder layer at N = 32, 96 bits 403 -> 336 us, the round trip of 16384 x 4096 98 -> 77 us at
+// N = 32 and 131 -> 97 us at N = 128, encoding 4096 x 4096 at N = 128, 384 bits 66 -> 58 us.
 //
 // The result is a point packed in bytes: word j holds |y_i| of positions 4j .. 4j+3, last
 // position lowest, which is the order in which the Fischer index needs the pulses behind
@@ -195,48 +197,40 @@ struct LanePoint {
     bool has_dir;    // false: the group's point is (K, 0, ..., 0), its first coordinate positive
 };
 
-// bit of the pulse mask that belongs to position i of a lane, and the other way round: words
-// of compare results are folded into one another a bit apart
-template <int E>
-__device__ __forceinline__ int mask_bit_position(int bit) {
-    return 4 * ((bit & 7) - (8 - E / 4)) + 3 - (bit >> 3);
-}
+// Masks of a lane's residuals: bit 8b + j stands for byte b of word j.  The position that a bit belongs to:
+__device__ __forceinline__ int mask_bit_position(int bit) { return 4 * (bit & 7) + 3 - (bit >> 3); }
 
-// Bit 8b + 8-J + j: residual of byte b of word j is not below the threshold.
+// x[j] holds a byte for each of four residuals.  Afterwards bit 8b + j of (x[p % J] >> (p - p % J)), j < J, is bit p of
+// byte b of word j: in every byte the J rows of J bits that lie below one another are transposed.
 template <int J>
-__device__ __forceinline__ uint32_t not_below_mask(const uint32_t (&x)[J], uint32_t t4) {
-    uint32_t m = 0u;
+__device__ __forceinline__ void bit_planes(uint32_t (&x)[J]) {
+    static_assert(J == 2 || J == 4 || J == 8, "");
 #pragma unroll
-    for (int j = 0; j < J; ++j) m = (m >> 1) | ((x[j] - t4) & kH4);
-    return m;
-}
-
-template <int J>
-__device__ __forceinline__ int not_below_count(const uint32_t (&x)[J], uint32_t t4) {
-    unsigned c = 0u;
+    for (int s = J / 2; s >= 1; s >>= 1) {
+        const uint32_t low = s == 4 ? 0x0f0f0f0fu : (s == 2 ? 0x33333333u : 0x55555555u);
 #pragma unroll
-    for (int j = 0; j < J; ++j) c = __dp4a((x[j] - t4) & kH4, kOne4, c);
-    return static_cast<int>(c >> 7);
+        for (int j = 0; j < J; ++j)
+            if ((j & s) == 0) {
+                const uint32_t a = x[j], b = x[j + s];
+                x[j] = (a & low) | ((b << s) & ~low);
+                x[j + s] = ((a >> s) & low) | (b & ~low);
+            }
+    }
 }
 
 // The residuals of the candidates (bits of `cand`), exactly, and which of the group's candidates
 // are the r largest, lowest index first among equals.  Returns the chosen bits.  Called by
 // all lanes of a warp; a group with nothing to choose comes with cand = 0.
-//   Usual: no lane has more than C candidates; every candidate counts the better ones.
+//   Usual (rank_candidates): no lane has more than C candidates; every candidate counts the better ones.
 //   Otherwise (many equal or nearly equal residuals): one value class after the other, from the
 //   largest down, until r are chosen.
 // rotation: position i of the lane is held as position i - 8 * rotation (modulo E).
-template <int E, int L, class Fetch>
-__device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, float gsc, const Fetch& fetch, int rotation) {
-    constexpr int C = L == 1 ? 4 : 2;
+template <int E, int L, int C, class Fetch>
+__device__ __forceinline__ uint32_t rank_candidates(uint32_t cand, int r, float gsc, const Fetch& fetch, int rotation) {
     constexpr float magic = 8388608.0f;  // 2^23
-    auto residual = [&](int i) {
-        const float a = __fmul_rn(fetch(i), gsc);
-        return __fsub_rn(a, __fsub_rn(__fadd_rd(a, magic), magic));
-    };
     const int sub = static_cast<int>(threadIdx.x) & (L - 1);
     uint32_t chosen = 0u;
-    if (__all_sync(0xffffffffu, __popc(cand) <= C)) {
+    {
         float e[C];
         int pos[C], better[C];
         uint32_t bit[C];
@@ -246,7 +240,7 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
             const int b = 31 - __clz(static_cast<int>(left));  // -1: no candidate left
             bit[s] = left & (1u << (b & 31));
             left ^= bit[s];
-            pos[s] = bit[s] ? (mask_bit_position<E>(b) + 8 * rotation) & (E - 1) : 0;
+            pos[s] = bit[s] ? (mask_bit_position(b) + 8 * rotation) & (E - 1) : 0;
         }
 #pragma unroll
         for (int s = 0; s < C; ++s) e[s] = fetch(pos[s]);
@@ -279,17 +273,31 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
 #pragma unroll
         for (int s = 0; s < C; ++s)
             if (better[s] < r) chosen |= bit[s];
-        return chosen;
     }
+    return chosen;
+}
+
+template <int E, int L, class Fetch>
+__device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, float gsc, const Fetch& fetch, int rotation) {
+    constexpr float magic = 8388608.0f;  // 2^23
+    auto residual = [&](int i) {
+        const float a = __fmul_rn(fetch(i), gsc);
+        return __fsub_rn(a, __fsub_rn(__fadd_rd(a, magic), magic));
+    };
+    const int sub = static_cast<int>(threadIdx.x) & (L - 1);
+    const int mine_all = __popc(cand);
+    if (__all_sync(0xffffffffu, mine_all <= 2)) return rank_candidates<E, L, 2>(cand, r, gsc, fetch, rotation);
+    if (__all_sync(0xffffffffu, mine_all <= 4)) return rank_candidates<E, L, 4>(cand, r, gsc, fetch, rotation);
+    uint32_t chosen = 0u;
     for (int round = 0; round < E * L; ++round) {
         if (!__any_sync(0xffffffffu, cand != 0u && r > 0)) break;
         float top = -1.0f;  // the group's largest residual left
-        for (uint32_t left = cand; left; left &= left - 1u) top = fmaxf(top, residual((mask_bit_position<E>(__ffs(left) - 1) + 8 * rotation) & (E - 1)));
+        for (uint32_t left = cand; left; left &= left - 1u) top = fmaxf(top, residual((mask_bit_position(__ffs(left) - 1) + 8 * rotation) & (E - 1)));
 #pragma unroll
         for (int o = 1; o < L; o <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
         uint32_t equal = 0u;
         for (uint32_t left = cand; left; left &= left - 1u)
-            if (residual((mask_bit_position<E>(__ffs(left) - 1) + 8 * rotation) & (E - 1)) == top) equal |= left & (0u - left);
+            if (residual((mask_bit_position(__ffs(left) - 1) + 8 * rotation) & (E - 1)) == top) equal |= left & (0u - left);
         const int mine = __popc(equal);
         int before = 0, all = 0;  // of the class: in lower lanes, in the group
 #pragma unroll
@@ -304,7 +312,7 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
             int take = min(max(r - before, 0), mine);
             for (int i = 0; i < E && take > 0; ++i) {
                 const int held = (i - 8 * rotation) & (E - 1);
-                const uint32_t b = 1u << (8 * (3 - (held & 3)) + 8 - E / 4 + (held >> 2));
+                const uint32_t b = 1u << (8 * (3 - (held & 3)) + (held >> 2));
                 if (equal & b) chosen |= b, --take;
             }
         }
@@ -320,15 +328,14 @@ template <int E, int L, bool WIDE, class Fetch>
 __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, int K, const Fetch& fetch,
                                                LanePoint<E, WIDE>& pt, float minus_zero, int rotation = 0) {
     constexpr int N = E * L, J = E / 4, H = E / 2;
-    constexpr int CMAX = L == 1 ? 4 : 2;           // candidates that may be left for the exact comparison
     const float gsc = __fdiv_rn(static_cast<float>(K), l1);
     // no direction: l1 zero or not finite, or a scale that overflows
     bool has_dir = (l1 > 0.0f) && (l1 <= 3.4028234e38f) && (gsc <= 3.4028234e38f);
-    // a + 2^16 rounded down is 2^16 + floor(128 a) / 128: the floor and 7 bits of the residual
-    // sit in the low mantissa bits
+    // a + 2^15 rounded down is 2^15 + floor(256 a) / 256: 8 bits of the residual are the lowest byte, the floor
+    // begins at the next (a <= K + 1 leaves the exponent alone)
     uint32_t t[E];
     {
-        const f32x2 g2 = pack2(gsc, gsc), m2 = pack2(65536.0f, 65536.0f);
+        const f32x2 g2 = pack2(gsc, gsc), m2 = pack2(32768.0f, 32768.0f);
 #pragma unroll
         for (int i = 0; i < H; ++i) {
             float lo, hi;
@@ -337,16 +344,16 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
             t[i + H] = __float_as_uint(hi);
         }
     }
-    uint32_t x[J];  // 0x80 + leading 7 bits of the residual, a byte each
+    uint32_t x[J];  // leading 8 bits of the residuals, a byte each
     int fsum;
     if constexpr (!WIDE) {
         uint32_t sum4 = 0u;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
             const uint32_t u = __byte_perm(t[4 * j + 3], t[4 * j + 2], 0x5410), v = __byte_perm(t[4 * j + 1], t[4 * j], 0x5410);
-            x[j] = __byte_perm(u, v, 0x6420) | kH4;
-            pt.y[j] = __byte_perm(u + u, v + v, 0x7531);  // floors, below 128
-            sum4 += pt.y[j];                              // no byte passes K
+            x[j] = __byte_perm(u, v, 0x6420);
+            pt.y[j] = __byte_perm(u, v, 0x7531);  // floors, below 128
+            sum4 += pt.y[j];                      // no byte passes K
         }
         fsum = static_cast<int>(__dp4a(sum4, kOne4, 0u));
     } else {
@@ -354,9 +361,9 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
 #pragma unroll
         for (int j = 0; j < J; ++j) {
             const uint32_t u = __byte_perm(t[4 * j + 3], t[4 * j + 2], 0x0040), v = __byte_perm(t[4 * j + 1], t[4 * j], 0x0040);
-            x[j] = __byte_perm(u, v, 0x5410) | kH4;
-            pt.y[2 * j] = __byte_perm(t[4 * j + 1] << 1, t[4 * j] << 1, 0x6521);
-            pt.y[2 * j + 1] = __byte_perm(t[4 * j + 3] << 1, t[4 * j + 2] << 1, 0x6521);
+            x[j] = __byte_perm(u, v, 0x5410);
+            pt.y[2 * j] = __byte_perm(t[4 * j + 1], t[4 * j], 0x6521);
+            pt.y[2 * j + 1] = __byte_perm(t[4 * j + 3], t[4 * j + 2], 0x6521);
             sum2 += pt.y[2 * j] + pt.y[2 * j + 1];
         }
         fsum = static_cast<int>((sum2 & 0xffffu) + (sum2 >> 16));
@@ -367,40 +374,30 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
     has_dir = has_dir && d >= 0 && d <= N;
     if (!has_dir) d = 0;
 
-    // Bracket [lo, hi) of thresholds with count(lo) >= d >= count(hi), kept as count * 256 +
-    // threshold: the difference of the two ends then says in one comparison whether few enough
-    // residuals are left between them.  A group that is done goes on halving: its bracket stays
-    // one.  (d = 0 and d = N start and stay with both ends at the threshold that selects none / all.)
-    int lo = N << 8, hi = 128;
-    if (d == 0) lo = 128;
-    if (d == N) hi = lo;
-    int T = 128 - (N > 128 ? d / (N / 128) : d * (128 / (N > 128 ? 128 : N)));  // residuals are close to uniform
-    for (int it = 0; it < 12; ++it) {
-        const int c = group_add<L>(not_below_count<J>(x, static_cast<uint32_t>(T) * kOne4));
-        const int at = (c << 8) + T;
-        if (c >= d) lo = at;
-        if (c <= d) hi = at;
-        const int lo_t = lo & 255, hi_t = hi & 255;
-        if (it > 0 && !__any_sync(0xffffffffu, lo - hi > (CMAX << 8) && hi_t - lo_t > 1)) break;
-        T = (lo_t + hi_t) >> 1;
-        if (it < 2 && (lo_t == 0 || hi_t == 128)) {
-            // one end not met yet: a step by the density of the residuals and half a residual further
-            const int over = 2 * (c - d) + (c > d ? 1 : -1);  // in half residuals, 64 / N thresholds each
-            const int step = N <= 64 ? over * (64 / (N <= 64 ? N : 64)) : over / (N / 64);
-            T = min(max((at & 255) + step, lo_t), hi_t);
-        }
+    bit_planes<J>(x);
+    uint32_t sel = 0u, cand = ((1u << J) - 1u) * kOne4;  // chosen; undecided: the same in all bits so far
+    int need = d;                                        // still to be chosen among the undecided ones
+#pragma unroll
+    for (int p = 7; p >= 0; --p) {
+        const uint32_t have = cand & (x[p % J] >> (p - p % J));
+        const int c = group_add<L>(__popc(have));
+        const bool all = c <= need;
+        sel |= all ? have : 0u;
+        need -= all ? c : 0;
+        cand = all ? cand ^ have : have;
     }
-    uint32_t sel = not_below_mask<J>(x, static_cast<uint32_t>(hi & 255) * kOne4);
-    uint32_t cand = not_below_mask<J>(x, static_cast<uint32_t>(lo & 255) * kOne4) & ~sel;
-    if (__any_sync(0xffffffffu, cand != 0u)) sel |= choose_candidates<E, L>(cand, d - (hi >> 8), gsc, fetch, rotation);
+    const bool rest = group_add<L>(__popc(cand)) == need;  // (none needed: no matter)
+    if (rest) sel |= cand;
+    if (rest || need == 0) cand = 0u;
+    if (__any_sync(0xffffffffu, cand != 0u)) sel |= choose_candidates<E, L>(cand, need, gsc, fetch, rotation);
 
     if constexpr (!WIDE) {
 #pragma unroll
-        for (int j = 0; j < J; ++j) pt.y[j] += (sel >> (8 - J + j)) & kOne4;
+        for (int j = 0; j < J; ++j) pt.y[j] += (sel >> j) & kOne4;
     } else {
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const uint32_t b4 = (sel >> (8 - J + j)) & kOne4;
+            const uint32_t b4 = (sel >> j) & kOne4;
             pt.y[2 * j] += __byte_perm(b4, 0u, 0x4342);      // positions 4j+1 (low half), 4j
             pt.y[2 * j + 1] += __byte_perm(b4, 0u, 0x4140);  // positions 4j+3, 4j+2
         }
