@@ -420,14 +420,8 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
         const float s = __shfl_sync(kFull, sc, from);
         const uint32_t dst = __shfl_sync(kFull, at, from);
         const uint32_t lo = win_slot_word(src), hi = win_slot_word<4>(src);
-        float f[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {  // byte v into the low mantissa bits of 2^23: the float 2^23 + v, then minus 2^23 + 128
-            f[e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
-            f[4 + e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
-        }
-        if (dst != 0xffffffffu)
-            base[dst + sub] = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+        const uint4 v = scale_bytes8(lo, hi, s);
+        if (dst != 0xffffffffu) base[dst + sub] = v;
     }
     __syncwarp();  // the slots are free
 }

@@ -23,50 +23,12 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include "pvq_f32x2.cuh"
 #include "pvq_internal.cuh"
 
 namespace pvq {
 
 constexpr uint32_t kH4 = 0x80808080u, kOne4 = 0x01010101u;
-
-// Two fp32 in a register pair: one instruction for two roundings (same results as two scalar
-// operations; what it saves is issue slots).
-struct f32x2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 a, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ f32x2 add2_rd(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-// A product on its own.  Where an addition follows, the rounding of the product has to stay: the
-// assembler was seen to merge a mul.rn.f32x2 into a following add.rn.f32x2 (a group's energy then
-// came out an ulp off).  mul2_rounded is a multiply-add of a -0 that it cannot see (a kernel
-// argument), which changes no result and leaves nothing to merge.
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2_rounded(f32x2 a, f32x2 b, float minus_zero) { return fma2(a, b, pack2(minus_zero, minus_zero)); }
 
 // A lane's E values as they sit in memory: E/2 words of two bf16, or E words.
 template <int E, bool BF16>

@@ -25,6 +25,7 @@
 // width, whose larger entries are replaced by 2^62 (2^30): no r of that phase reaches them.
 #pragma once
 #include "mp_uint.cuh"
+#include "pvq_f32x2.cuh"
 #include "pvq_internal.cuh"
 #include "pvq_stage.cuh"
 
@@ -1075,25 +1076,19 @@ __device__ __forceinline__ void emit_scaled(const MatrixArgs& m, const YT* yslot
                                           static_cast<size_t>(g) * N);
 #pragma unroll
     for (int q = 0; q < N / 8; ++q) {
-        float f[8];
         if constexpr (sizeof(YT) == 1) {
-            // byte b into the low mantissa bits of 2^23: the float 2^23 + b, then minus 2^23 + 128
-            const uint32_t lo = y4[2 * q], hi = y4[2 * q + 1];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                f[e] = __fsub_rn(__uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7540u + e)), 8388736.0f);
-                f[4 + e] = __fsub_rn(__uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540u + e)), 8388736.0f);
-            }
+            dst[q] = scale_bytes8(y4[2 * q], y4[2 * q + 1], sc);
         } else {
+            float f[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) f[e] = static_cast<float>(static_cast<int>(yslots[8 * q + e]));
+            uint4 o;
+            o.x = pack_bf16x2(__fmul_rn(f[0], sc), __fmul_rn(f[1], sc));
+            o.y = pack_bf16x2(__fmul_rn(f[2], sc), __fmul_rn(f[3], sc));
+            o.z = pack_bf16x2(__fmul_rn(f[4], sc), __fmul_rn(f[5], sc));
+            o.w = pack_bf16x2(__fmul_rn(f[6], sc), __fmul_rn(f[7], sc));
+            dst[q] = o;
         }
-        uint4 o;
-        o.x = pack_bf16x2(__fmul_rn(f[0], sc), __fmul_rn(f[1], sc));
-        o.y = pack_bf16x2(__fmul_rn(f[2], sc), __fmul_rn(f[3], sc));
-        o.z = pack_bf16x2(__fmul_rn(f[4], sc), __fmul_rn(f[5], sc));
-        o.w = pack_bf16x2(__fmul_rn(f[6], sc), __fmul_rn(f[7], sc));
-        dst[q] = o;
     }
 }
 
@@ -1142,15 +1137,8 @@ __device__ __forceinline__ void emit_warp(const MatrixArgs& m, const uint8_t* sl
         const float s = __shfl_sync(kFull, sc, from);
         const unsigned long long dst = __shfl_sync(kFull, at, from);
         const uint32_t lo = reinterpret_cast<const uint32_t*>(src)[0], hi = reinterpret_cast<const uint32_t*>(src)[1];
-        float f[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {  // byte b into the low mantissa bits of 2^23: the float 2^23 + b, then minus 2^23 + 128
-            f[e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(lo, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
-            f[4 + e] = __fmul_rn(__fsub_rn(__uint_as_float(__byte_perm(hi, 0x4B000000u, 0x7540u + e)), 8388736.0f), s);
-        }
-        if (dst != 0ull)
-            reinterpret_cast<uint4*>(dst)[sub] =
-                make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+        const uint4 v = scale_bytes8(lo, hi, s);
+        if (dst != 0ull) reinterpret_cast<uint4*>(dst)[sub] = v;
     }
 }
 
