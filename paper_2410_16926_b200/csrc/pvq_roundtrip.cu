@@ -39,7 +39,8 @@ struct RoundArgs {
     int rot_block;
     float minus_zero;  // -0 (see mul2_rounded)
     uint32_t levels_off, ss_off, signs_off, xbuf_off;  // in shared memory, behind the bin edges
-    uint32_t ring_off, tile_bytes;                     // three buffers for input and output tiles
+    uint32_t ring_off, tile_bytes;                     // buffers for input and output tiles
+    int bufs;                                          // how many (see roundtrip_kernel)
     uint32_t* status;
     uint32_t* debug_status;
 };
@@ -102,11 +103,15 @@ __device__ __forceinline__ float amplitude(float ss, float ss_row, int b, const 
 // the input in place and leave by bulk copy: no thread waits for global memory, and the copies
 // are whole lines whatever the lanes' access pattern (64 bytes a lane, 16 at a time).  Three
 // buffers: one worked on, one arriving, one leaving.  One block-wide barrier per tile.
+// Rotated, 32 values a lane (DIRECT): every warp writes its results to memory itself, brought into whole lines in its part
+// of the rotation's buffer, so a tile's buffer is free once it is read: two buffers, or one where the rotation's
+// barriers say so early (blocks that span warps).  4096 columns: 28 KB a row, seven rows an SM.
 template <int E, int L, bool WIDE, bool ROT>
 __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __grid_constant__ RoundArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[3];
     constexpr int P = E / 8;  // 16-byte pieces a lane
+    constexpr bool DIRECT = ROT && E == 32;
     float* s_edges = reinterpret_cast<float*>(smem);
     float* s_levels = reinterpret_cast<float*>(smem + a.levels_off);
     uint32_t* s_signs = reinterpret_cast<uint32_t*>(smem + a.signs_off);
@@ -176,6 +181,9 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         float* s_ss = reinterpret_cast<float*>(smem + a.ss_off) + (i & 1) * a.rpt * a.gp;
         // (a thread that gives up works on whatever the buffer holds, as far as the next barrier)
         const bool failed = !mbarrier_wait(shared_addr(full + buf), parity, stream_polls(withheld));
+        const unsigned next = tile + gridDim.x;
+        const bool have_next = next < a.tiles;
+        const int nbuf = buf + 1 == a.bufs ? 0 : buf + 1;
         float ss;
         uint32_t neg[E / 4];
         LanePoint<E, WIDE> pt;
@@ -191,15 +199,30 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
             if constexpr (ROT) {
                 float x[E];
                 uint32_t w[E];
+                if constexpr (E == 32) {
+                    const int T0 = a.rot_block / E;
+                    const uint32_t sb = s_signs[c & (T0 - 1)];
 #pragma unroll
-                for (int k = 0; k < E; ++k) x[k] = __uint_as_float((k & 1) ? (raw[k / 2] & 0xffff0000u) : (raw[k / 2] << 16));
-                rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf, a.minus_zero);
+                    for (int k = 0; k < E / 2; ++k) raw[k] ^= (sb << k) & 0x80008000u;
+#pragma unroll
+                    for (int k = 0; k < E; ++k) x[k] = __uint_as_float((k & 1) ? (raw[k / 2] & 0xffff0000u) : (raw[k / 2] << 16));
+                    bool asked = a.bufs != 1;
+                    rotate_lanes32(x, T0, rot_scale, smem, a.xbuf_off, a.minus_zero, [&]() {
+                        __syncthreads();
+                        if (!asked && tid == 0 && have_next && !failed) request(next, nbuf);  // the tile has been read
+                        asked = true;
+                    });
+                } else {
+#pragma unroll
+                    for (int k = 0; k < E; ++k) x[k] = __uint_as_float((k & 1) ? (raw[k / 2] & 0xffff0000u) : (raw[k / 2] << 16));
+                    rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf, a.minus_zero);
+                }
 #pragma unroll
                 for (int k = 0; k < E; ++k) w[k] = __float_as_uint(x[k]);
 #pragma unroll
                 for (int j = 0; j < E / 4; ++j) neg[j] = chunk_signs4<E, false>(w, j);
                 group_norms<E, L, false>(w, ax, l1, ss, a.minus_zero);
-                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated{s_xbuf + tid, T}, pt, a.minus_zero);
+                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated<E>{smem, a.xbuf_off, rot_scale}, pt, a.minus_zero);
             } else {
 #pragma unroll
                 for (int j = 0; j < E / 4; ++j) neg[j] = chunk_signs4<E, true>(raw, j);
@@ -215,22 +238,21 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
                     if ((j & (a.gp - 1)) >= a.G) s_ss[j] = 0.0f;
         }
         // energies are in place, and the tile before this one is complete in its buffer
-        bulk_store_fence();
+        if (!DIRECT) bulk_store_fence();
         if (__syncthreads_or(failed)) {  // the copy never arrived: report and leave rather than spin, all threads
             if (a.status && failed) atomicOr(a.status, PVQ_STATUS_STAGING_TIMEOUT);
             if (tid == 0) {
-                if (i > 0) deliver(tile - gridDim.x, buf == 0 ? 2 : buf - 1);
+                if (!DIRECT && i > 0) deliver(tile - gridDim.x, buf == 0 ? a.bufs - 1 : buf - 1);
                 bulk_store_wait_read<0>();
+                // (asked for already: it has to land before the block's memory goes away)
+                if (DIRECT && a.bufs == 1 && have_next && !failed) mbarrier_wait(shared_addr(full), parity ^ 1, stream_polls(withheld));
             }
             return;
         }
-        const unsigned next = tile + gridDim.x;
-        const bool have_next = next < a.tiles;
-        const int nbuf = buf == 2 ? 0 : buf + 1;
         if (tid == 0) {
-            if (i > 0) deliver(tile - gridDim.x, buf == 0 ? 2 : buf - 1);
-            if (have_next) {
-                bulk_store_wait_read<1>();  // what was in the buffer has left it
+            if (!DIRECT && i > 0) deliver(tile - gridDim.x, buf == 0 ? a.bufs - 1 : buf - 1);
+            if (have_next && a.bufs != 1) {
+                if (!DIRECT) bulk_store_wait_read<1>();  // what was in the buffer has left it
                 request(next, nbuf);
             }
         }
@@ -245,18 +267,40 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         const int ssy = group_add<L>(lane_squares<E, WIDE>(pt));
         const float sc = __fdiv_rn(amp, __fsqrt_rn(static_cast<float>(ssy)));
         const f32x2 sc2 = pack2(sc, sc);
-        if (active) {
-            if (!pt.has_dir) {  // (K, 0, ..., 0), positive
+        if (!pt.has_dir) {  // (K, 0, ..., 0), positive
 #pragma unroll
-                for (int j = 0; j < E / 4; ++j) neg[j] = 0u;
-            }
+            for (int j = 0; j < E / 4; ++j) neg[j] = 0u;
+        }
+        auto piece_of = [&](int v) {
+            const uint2 lo = scaled_values<E, WIDE>(pt, 2 * v, neg[2 * v], sc2);
+            const uint2 hi = scaled_values<E, WIDE>(pt, 2 * v + 1, neg[2 * v + 1], sc2);
+            return make_uint4(lo.x, lo.y, hi.x, hi.y);
+        };
+        if constexpr (DIRECT) {
+            // piece p of lane l lies at 4 l + (p ^ (l / 2) % 4): the lanes of an access hit different banks
+            uint4* lines = reinterpret_cast<uint4*>(s_xbuf + (tid - lane) * E);
+            __syncwarp();  // nobody looks for residuals there any more
+#pragma unroll
+            for (int v = 0; v < P; ++v) lines[lane * P + (v ^ ((lane >> 1) & 3))] = piece_of(v);
+            const long long row = static_cast<long long>(tile) * a.rpt + rl;
+            const bool ok = active && PVQ_DEBUG_INDEX(row, a.rows, PVQ_DEBUG_GLOBAL_STORE) &&
+                            PVQ_DEBUG_INDEX(static_cast<long long>(c + 1) * E - 1, a.cols, PVQ_DEBUG_GLOBAL_STORE);
+            const unsigned long long at =
+                ok ? reinterpret_cast<unsigned long long>(static_cast<__nv_bfloat16*>(a.out) + static_cast<size_t>(row) * a.ld_out + static_cast<size_t>(c) * E) : 0ull;
+            __syncwarp();
 #pragma unroll
             for (int v = 0; v < P; ++v) {
-                const uint2 lo = scaled_values<E, WIDE>(pt, 2 * v, neg[2 * v], sc2);
-                const uint2 hi = scaled_values<E, WIDE>(pt, 2 * v + 1, neg[2 * v + 1], sc2);
+                const int l = v * (32 / P) + lane / P, p = lane % P;
+                const unsigned long long dst = __shfl_sync(0xffffffffu, at, l);
+                const uint4 q = lines[l * P + (p ^ ((l >> 1) & 3))];
+                if (dst != 0ull) reinterpret_cast<uint4*>(dst)[p] = q;
+            }
+            __syncwarp();  // free for the next tile
+        } else if (active) {
+#pragma unroll
+            for (int v = 0; v < P; ++v) {
                 const int piece = (v + rot8) & (P - 1);
-                if (PVQ_DEBUG_INDEX(tid * P + piece, a.tile_bytes / 16, PVQ_DEBUG_SHARED_INDEX))
-                    reinterpret_cast<uint4*>(mine)[piece] = make_uint4(lo.x, lo.y, hi.x, hi.y);
+                if (PVQ_DEBUG_INDEX(tid * P + piece, a.tile_bytes / 16, PVQ_DEBUG_SHARED_INDEX)) reinterpret_cast<uint4*>(mine)[piece] = piece_of(v);
             }
         }
         if (!have_next) break;
@@ -264,6 +308,7 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         buf = nbuf;
         if (buf == 0) parity ^= 1;
     }
+    if (DIRECT) return;
     bulk_store_fence();
     __syncthreads();
     if (tid == 0) {
@@ -325,7 +370,15 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_rows_kernel(const 
 #pragma unroll
             for (int i = 0; i < E; ++i)
                 x[i] = BF16 ? __uint_as_float((i & 1) ? (r[i / 2] & 0xffff0000u) : (r[i / 2] << 16)) : __uint_as_float(r[BF16 ? i / 2 : i]);
-            rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf, a.minus_zero);
+            if constexpr (E == 32) {
+                const int T0 = a.rot_block / E;
+                const uint32_t sb = s_signs[c & (T0 - 1)];
+#pragma unroll
+                for (int i = 0; i < E; ++i) x[i] = __uint_as_float(__float_as_uint(x[i]) ^ ((sb << (i / 2 + (i & 1 ? 0 : 16))) & 0x80000000u));
+                rotate_lanes32(x, T0, rot_scale, smem, a.xbuf_off, a.minus_zero, []() { __syncthreads(); });
+            } else {
+                rotate_lanes<E>(x, s_signs, a.rot_block, rot_scale, c, s_xbuf, a.minus_zero);
+            }
 #pragma unroll
             for (int i = 0; i < E; ++i) w[i] = __float_as_uint(x[i]);
         }
@@ -356,7 +409,7 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_rows_kernel(const 
             float ax[E], l1;
             group_norms<E, L, WBF16>(raw, ax, l1, ss, a.minus_zero);
             if constexpr (ROT)
-                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated{s_xbuf + tid, T}, pt, a.minus_zero);
+                quantize_group<E, L, WIDE>(ax, l1, a.K, FetchRotated<E>{smem, a.xbuf_off, rot_scale}, pt, a.minus_zero);
             else
                 quantize_group<E, L, WIDE>(ax, l1, a.K, FetchGlobal<BF16>{static_cast<const uint8_t*>(a.x) + (active ? at(c) : 0) * (BF16 ? 2 : 4)}, pt,
                                            a.minus_zero);
@@ -403,6 +456,7 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
     a.C = a.G * L;
     a.gp = 1;
     while (a.gp < a.G) a.gp <<= 1;
+    const int T0 = ROT ? a.rot_block / E : 1;
     int threads = 0;
     if (a.C > kRoundThreadsMax) {
         // 512 lanes hold whole rotation blocks (at most 16384 values at 32 a lane; for the smaller
@@ -412,13 +466,15 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
         a.rpt = 1;
         a.chunks = (a.C + threads - 1) / threads;
     } else {
-        // Whole rows: the block of up to 256 threads (more when a row needs it) that leaves the
+        // Whole rows: the block of up to 128 threads (more when a row needs it) that leaves the
         // fewest lanes idle; among equals the largest, or the smallest when the launch would
-        // not fill the SMs anyway.
+        // not fill the SMs anyway.  (Up to 256: 16384 x 4096 at N = 128 97.6 us, with 128 95.3.)  Rotated in blocks that span
+        // warps: whole blocks, and no more threads than need be, as they meet often.
         a.chunks = 1;
         const int need = (a.C + 31) / 32 * 32;
         long long best = -1;
-        for (int t = std::max(64, need); t <= std::max(256, need); t += 32) {
+        for (int t = std::max(64, need); t <= std::max(T0 > 32 ? 64 : 128, need); t += 32) {
+            if (T0 > 32 && t % T0 != 0) continue;
             const int rpt = t / a.C;
             const long long tiles = (a.rows + rpt - 1) / rpt, cost = tiles * t;
             if (best < 0 || cost < best || (cost == best && tiles >= 2 * di.sms)) {
@@ -434,16 +490,17 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
     a.levels_off = a.b <= 8 ? 4u << a.b : 0u;
     a.ss_off = (2u * a.levels_off + 15u) & ~15u;
     a.signs_off = (a.ss_off + 2u * static_cast<uint32_t>(a.rpt * a.gp) * 4u + 15u) & ~15u;
-    a.xbuf_off = a.signs_off + (ROT ? (static_cast<uint32_t>(a.rot_block / E) * 4u + 15u) & ~15u : 0u);
+    a.xbuf_off = (a.signs_off + (ROT ? static_cast<uint32_t>(a.rot_block / E) * 4u : 0u) + 127u) & ~127u;
     a.ring_off = (a.xbuf_off + (ROT ? static_cast<uint32_t>(threads) * E * 4u : 0u) + 127u) & ~127u;
     a.tile_bytes = static_cast<uint32_t>(threads) * E * 2u;
     size_t smem = a.ring_off;
     void (*kern)(RoundArgs) = roundtrip_rows_kernel<E, L, BF16, WIDE, ROT>;
     bool stays = false;  // the block stays and takes tile after tile
     if constexpr (BF16) {
-        if (a.chunks == 1 && smem + 3u * a.tile_bytes <= static_cast<size_t>(di.smem_max)) {
+        a.bufs = !ROT || E != 32 ? 3 : (T0 > 32 ? 1 : 2);
+        if (a.chunks == 1 && smem + a.bufs * a.tile_bytes <= static_cast<size_t>(di.smem_max)) {
             stays = true;
-            smem += 3u * a.tile_bytes;
+            smem += a.bufs * a.tile_bytes;
             kern = roundtrip_kernel<E, L, WIDE, ROT>;
         }
     }
