@@ -31,7 +31,8 @@ namespace {
 constexpr int kSearchThreads = 1024;
 
 // GP groups per thread: a warp takes GP consecutive tiles of 32 groups in one pass.
-template <int N, int W, int GP, int PLANE>
+// LONG: rewrites the staged buckets and has the table of the last four positions (see "long launches" in pvq_search.cuh).
+template <int N, int W, int GP, int PLANE, bool LONG>
 __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
     decode_search_kernel(const __grid_constant__ BatchArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -48,8 +49,10 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
     // (records and bucket tables, then the increments E where the blob has the thresholds T)
     const uint8_t* section = reinterpret_cast<const uint8_t*>(a.table) + a.srch_off;
     const uint32_t staged = a.srch_bytes - a.srch_t_before_e;
+    const uint32_t quad_bytes = LONG ? a.srch_quads : 0u;
     if (threadIdx.x == 0) {
-        bulk_stage_expect(stage, staged);
+        bulk_stage_expect(stage, staged + quad_bytes);
+        if (LONG && quad_bytes != 0u) bulk_stage_copy(stage, smem + staged, &kQuads, quad_bytes);
         bulk_stage_copy(stage, smem, section, a.srch_t_off);
         bulk_stage_copy(stage, smem + a.srch_t_off, section + a.srch_t_off + a.srch_t_before_e, staged - a.srch_t_off);
     }
@@ -59,7 +62,7 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     // slots: chain j of thread t at (j * blockDim.x + t) * YS behind the tables (a multiple of 16 bytes)
-    uint8_t* yslots = smem + staged + threadIdx.x * YS;
+    uint8_t* yslots = smem + staged + quad_bytes + threadIdx.x * YS;
     const uint32_t ychain = blockDim.x * YS;
 
     // N(N,K): codes at or above it are invalid
@@ -72,15 +75,19 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
         return;
     }
     int cnt[5];
-    if (!search_section_begin<N, W>(smem, a.srch_bytes, a.srch_t_before_e, K, cnt)) {  // not the table of this (N,K): refuse it
+    if (!search_section_begin<N, W>(smem, a.srch_bytes, K, cnt)) {  // not the table of this (N,K): refuse it
         if (a.status && threadIdx.x == 0) atomicOr(a.status, PVQ_STATUS_TABLE_MISMATCH);
         return;
     }
+    if constexpr (LONG)
+        search_section_long<N>(smem, a.srch_t_off, a.srch_t_before_e);
+    else
+        search_section_addresses<N>(smem, a.srch_t_before_e);
 #ifdef PVQ_DEBUG
-    debug_begin(sbase, sbase + staged, sbase + staged, YS, N, a.debug_status);
+    debug_begin(sbase, sbase + staged + quad_bytes, sbase + staged + quad_bytes, YS, N, a.debug_status);
     if (threadIdx.x == 0) {
         s_debug.slot_chain = ychain;
-        s_debug.slot_end = sbase + staged + GP * ychain;
+        s_debug.slot_end = sbase + staged + quad_bytes + GP * ychain;
     }
 #endif
     __syncthreads();
@@ -150,7 +157,21 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
         uint32_t ssy[GP];
 #pragma unroll
         for (int j = 0; j < GP; ++j) ssy[j] = 0u;
-        search_codes<N, W, GP, PLANE>(q, K, recs, t_rows, cnt, shared_addr(yslots), ychain, ssy);
+        if constexpr (LONG) {
+            uint32_t odd_one[GP];
+#pragma unroll
+            for (int j = 0; j < GP; ++j) odd_one[j] = 0u;
+            search_codes_long<N, W, GP, PLANE>(q, K, recs, cnt, quad_bytes != 0u ? sbase + staged : 0u, shared_addr(yslots), ychain, ssy, odd_one);
+#pragma unroll
+            for (int j = 0; j < GP; ++j)
+                if (active_valid[j] && (odd_one[j] & 0x80808080u) != 0u) {
+                    const MatrixArgs& m = a.m[mj[j]];
+                    const uint32_t* code = m.codes + (static_cast<size_t>(row[j]) * m.G + g[j]) * W;
+                    ssy[j] = search_exact<N, W, PLANE>(code, bw, K, recs, t_rows, cnt[4], cnt[3], cnt[2], shared_addr(yslots) + j * ychain);
+                }
+        } else {
+            search_codes<N, W, GP, PLANE>(q, K, recs, t_rows, cnt, shared_addr(yslots), ychain, ssy);
+        }
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
@@ -175,30 +196,27 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
     if (bad && a.status) atomicOr(a.status, PVQ_STATUS_INVALID_CODE);
 }
 
-template <int N, int W, int GP, int PLANE>
+template <int N, int W, int GP, int PLANE, bool LONG>
 int launch_search_t(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
     constexpr int YS = N + 4;
     constexpr int kMaxThreads = kSearchThreads / (GP > 2 ? 2 : 1);
-    unsigned tiles = 0;
-    for (int i = 0; i < a.count; ++i) {
-        a.m[i].tile_begin = tiles;
-        const long long ngroups = a.m[i].rows * a.m[i].G;
-        tiles += static_cast<unsigned>((ngroups + 31) / 32);
-    }
-    a.total_tiles = tiles;
+    const unsigned tiles = a.total_tiles;
     a.srch_off = S.off;
     a.srch_bytes = S.total;
     a.srch_t_off = S.t_off;
     a.srch_t_before_e = S.e_off - S.t_off;
-    const size_t staged = S.total - (S.e_off - S.t_off);
+    size_t staged = S.total - (S.e_off - S.t_off);
     DeviceInfo di;
     int st = device_info(&di);
     if (st != PVQ_OK) return st;
+    // (the table of the last four positions where it takes no threads away)
+    a.srch_quads = LONG && staged + sizeof(QuadTable) + static_cast<size_t>(kMaxThreads) * YS * GP <= static_cast<size_t>(di.smem_max) ? sizeof(QuadTable) : 0u;
+    staged += a.srch_quads;
     // One block per SM.  Every tile costs the same, so the launch runs in rounds of GP tiles
     // per resident warp; among the block sizes that fit, take the one whose rounds are
     // fullest, with a preference for more warps (they hide the latency of the dependent
     // table reads).
-    auto kern = decode_search_kernel<N, W, GP, PLANE>;
+    auto kern = decode_search_kernel<N, W, GP, PLANE, LONG>;
     int threads = 0;
     size_t smem = 0;
     double best_score = -1.0;
@@ -230,13 +248,27 @@ int launch_search_t(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
 
 // Two groups per thread: enough independent chains to cover the latency of the dependent
 // table reads with the warps one SM holds (one group: 389 us on the decoder-layer workload,
-// two: 333 us, four at half the threads: 455 us).
+// two: 333 us, four at half the threads: 455 us; of an earlier form of the kernel).
 template <int N, int W>
 int launch_search_g(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
+    DeviceInfo di;
+    const int st = device_info(&di);
+    if (st != PVQ_OK) return st;
+    unsigned tiles = 0;
+    for (int i = 0; i < a.count; ++i) {
+        a.m[i].tile_begin = tiles;
+        const long long ngroups = a.m[i].rows * a.m[i].G;
+        tiles += static_cast<unsigned>((ngroups + 31) / 32);
+    }
+    a.total_tiles = tiles;
+    // More than a round earns the rewriting of the buckets and the staging of the table of the last four positions, some 2 us.
+    // (Without and with, us: decoder layer, 23 rounds, 271 and 242; 4096 x 4096 at N = 16, 48 bits, 3.5 rounds, 24.6 and
+    // 22.1; at N = 32, 64 bits, 1.7 rounds, 21.5 and 20.3, 96 bits 23.5 and 23.6; one round only loses.)
+    const bool is_long = tiles > 2u * static_cast<unsigned>(di.sms) * (kSearchThreads / 32);
     switch (S.plane) {  // entries per word plane of the section's rows
-        case 64: return launch_search_t<N, W, 2, 64>(a, S, stream);
-        case 128: return launch_search_t<N, W, 2, 128>(a, S, stream);
-        case 256: return launch_search_t<N, W, 2, 256>(a, S, stream);
+        case 64: return is_long ? launch_search_t<N, W, 2, 64, true>(a, S, stream) : launch_search_t<N, W, 2, 64, false>(a, S, stream);
+        case 128: return is_long ? launch_search_t<N, W, 2, 128, true>(a, S, stream) : launch_search_t<N, W, 2, 128, false>(a, S, stream);
+        case 256: return is_long ? launch_search_t<N, W, 2, 256, true>(a, S, stream) : launch_search_t<N, W, 2, 256, false>(a, S, stream);
         default: return PVQ_ERR_UNSUPPORTED;
     }
 }

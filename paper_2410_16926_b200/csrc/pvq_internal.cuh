@@ -57,6 +57,7 @@ struct BatchArgs {
     uint32_t srch_off, srch_bytes;
     uint32_t srch_t_off;       // where the thresholds T start in the section; they stay in global memory
     uint32_t srch_t_before_e;  // bytes from a row of T to the same row of E
+    uint32_t srch_quads;       // bytes of the table of the last four positions, staged behind the section (0: without)
 };
 
 // Layout of the table blob.  Section 0 is the count table as the paper defines it,

@@ -91,13 +91,9 @@ __device__ __forceinline__ uint32_t bump_if_less(uint32_t m0, const mp<W>& t, co
 
 // Once the section has arrived in shared memory (at `sec`; `bytes` is its size in the blob): is
 // it the section of this (N,K)?  (A table built for another one would send the look-ups
-// anywhere.)  If so, the numbers of rows per width go to cnt[1..4] and threads 0..N-1 turn the
-// records' offsets into shared addresses; the caller's next block-wide barrier publishes them.
-// The thresholds T are not staged (only a 24-bit tie reads one, from global memory): the
-// increments E sit where T is in the blob, `t_before_e` bytes lower.
+// anywhere.)  If so, the numbers of rows per width go to cnt[1..4].
 template <int N, int W>
-__device__ __forceinline__ bool search_section_begin(uint8_t* sec, uint32_t bytes, uint32_t t_before_e, int K,
-                                                     int (&cnt)[5]) {
+__device__ __forceinline__ bool search_section_begin(const uint8_t* sec, uint32_t bytes, int K, int (&cnt)[5]) {
     const uint32_t* head = reinterpret_cast<const uint32_t*>(sec);
     if (head[0] != kSearchMagic || head[1] != static_cast<uint32_t>(N) || head[2] != static_cast<uint32_t>(K) ||
         head[3] != bytes)
@@ -108,13 +104,20 @@ __device__ __forceinline__ bool search_section_begin(uint8_t* sec, uint32_t byte
     if (cnt[1] + cnt[2] + cnt[3] + cnt[4] != N || ((cnt[1] | cnt[2] | cnt[3] | cnt[4]) & 3) != 0 ||
         (W < 4 && cnt[4] != 0) || (W < 3 && cnt[3] != 0) || (W < 2 && cnt[2] != 0))
         return false;
+    return true;
+}
+
+// Then threads 0..N-1 turn the records' offsets into shared addresses; the caller's next block-wide barrier publishes them.
+// The thresholds T are not staged (only a 24-bit tie reads one, from global memory): the
+// increments E sit where T is in the blob, `t_before_e` bytes lower.
+template <int N>
+__device__ __forceinline__ void search_section_addresses(uint8_t* sec, uint32_t t_before_e) {
     if (threadIdx.x < N) {
         uint32_t* rec = reinterpret_cast<uint32_t*>(sec + kSearchHeader) + 4 * threadIdx.x;
         const uint32_t base = shared_addr(sec);
         rec[1] += base - t_before_e;
         rec[2] += base;
     }
-    return true;
 }
 
 // Entry of PW words of a row stored word plane by word plane (PLANE entries a plane): word w
@@ -135,6 +138,24 @@ __device__ __forceinline__ void store_y4(uint32_t addr, uint32_t val) {
     if (!debug_slot_ok(addr, 4)) return;
 #endif
     asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(val) : "memory");
+}
+
+// From the threshold indices of four positions (a byte each, first position lowest) to their coordinates, all four at
+// a time: pulses left after a position m >> 1, before it those of the position before (k for the
+// first); their difference is |y|, and y > 0 where m is odd.  No byte borrows from or
+// carries into its neighbour: the pulses left never grow, and |y| <= 127.
+// The four y_i + 128 go to the word at y, their squares to ssy.  Returned: bit 7 of a byte set where that does not hold,
+// the pulses left having grown, or where nothing is positive (y = 0, m odd).
+__device__ __forceinline__ uint32_t search_coordinates(uint32_t m4, uint32_t& k, uint32_t y, uint32_t& ssy) {
+    const uint32_t after = (m4 >> 1) & 0x7f7f7f7fu;
+    const uint32_t before = (after << 8) | k;
+    const uint32_t mag = before - after;
+    ssy = __dp4a(mag, mag, ssy);
+    const uint32_t odd = m4 & 0x01010101u;
+    const uint32_t pos = (odd << 8) - odd;  // 0xff in the bytes with y > 0
+    store_y4(y, ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos));
+    k = after >> 24;
+    return mag | ~((mag | 0x80808080u) - odd);
 }
 
 // Four positions of GP codes (GP independent chains of dependent table reads, so that one
@@ -198,23 +219,207 @@ __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP],
             acc[j] = __funnelshift_r(acc[j], m[j], 8);  // the new byte enters at the top
         }
     }
-    // From the four indices to the four coordinates, all four bytes of a word at a time:
-    // pulses left after a position m >> 1, before it those of the position before (k for the
-    // first); their difference is |y|, and y > 0 where m is odd.  No byte borrows from or
-    // carries into its neighbour: the pulses left never grow, and |y| <= 127.
 #pragma unroll
     for (int j = 0; j < GP; ++j) {
-        const uint32_t after = (acc[j] >> 1) & 0x7f7f7f7fu;
-        const uint32_t before = (after << 8) | k[j];
-        const uint32_t mag = before - after;
-        ssy[j] = __dp4a(mag, mag, ssy[j]);
-        const uint32_t odd = acc[j] & 0x01010101u;
-        const uint32_t pos = (odd << 8) - odd;  // 0xff in the bytes with y > 0
-        store_y4(y + static_cast<uint32_t>(j) * ychain,
-                 ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos));
-        k[j] = after >> 24;
+        search_coordinates(acc[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
 #pragma unroll
         for (int w = 0; w < PW; ++w) q[j].w[w] = v[j].w[w];
+    }
+}
+
+// ---------------------------------------------------------------- long launches
+//
+// A launch of some rounds can afford to rewrite the staged buckets first (search_section_long), so that a position takes
+// fewer instructions: an entry is then what, added to the key, leaves the index in the top byte, the comparison
+// of the key with the bucket's threshold being the carry into it.  Nor does it look whether the key bits are the same as
+// a threshold's.  If they are, and q is above the threshold all the same, the index is one short and q' = T_(n-1)[2k'] + d,
+// d = q - T_n[m], is too large for the k' pulses left.  The next row then has an index of 2k' + 1 or more for it, which no q
+// of a valid code has (2k' + 1: a positive coordinate of no pulse; more: pulses left that grow), and
+// search_coordinates shows it.  (There is a next row: row 0's thresholds are their keys.)  Whatever follows is in
+// bounds: q stays above zero, as every step leaves 1 <= q <= N(n,k') for a q up to the row's last threshold, and a key above
+// the last bucket is cut off at it.  Such a group is searched once more, in full (search_exact).
+// Tried with the old entries and not kept: bucket and key bits from one wide product, and the comparison taken as the borrow of a
+// subtraction (decoder layer 271 -> 288 and 284 us: they tie up the pipes that are short).
+
+// The last four positions at once: the indices of q in row 3, of the q that follows in row 2, and so on depend on q
+// alone (no N, K or pulses left in them), and q is small there: at most N(4,k) with k pulses left, some K / 8 of them at
+// N = 32.  kQuads holds the four indices, first position lowest, of q = 1 .. N(4,kQuadPulses); a larger q is searched.
+constexpr uint32_t kQuadPulses = 16;
+constexpr uint32_t quad_count(uint32_t n, uint32_t k) {  // V(n,k) = sum over j <= k of N(n,j)
+    return n == 0 ? 1u : (n == 1 ? 2u * k + 1u : (n == 2 ? 2u * k * k + 2u * k + 1u : (2u * k + 1u) * (2u * k * k + 2u * k + 3u) / 3u));
+}
+constexpr uint32_t quad_threshold(uint32_t n, uint32_t m) {  // T_n[m]
+    return (m & 1u) ? 2u * quad_count(n, m >> 1) : quad_count(n, m >> 1) + (m > 1u ? quad_count(n, (m >> 1) - 1u) : 0u);
+}
+constexpr uint32_t kQuadEntries = quad_threshold(3, 2 * kQuadPulses);  // N(4,16) = 11008
+struct QuadTable {
+    uint32_t m4[kQuadEntries];
+};
+constexpr QuadTable make_quads() {
+    QuadTable t{};
+    uint32_t m3 = 0;
+    for (uint32_t q = 1; q <= kQuadEntries; ++q) {
+        while (quad_threshold(3, m3) < q) ++m3;
+        const uint32_t q2 = q + quad_threshold(2, m3 & ~1u) - quad_threshold(3, m3);
+        uint32_t m2 = q > 1 && (t.m4[q - 2] & 0xffu) == m3 ? (t.m4[q - 2] >> 8) & 0xffu : 0u;  // from where the q before was
+        while (quad_threshold(2, m2) < q2) ++m2;
+        const uint32_t q1 = q2 + quad_threshold(1, m2 & ~1u) - quad_threshold(2, m2);
+        const uint32_t m1 = q1 == 1 ? 0 : (q1 + 1) / 2;  // thresholds 1, 2, 4, 6, ...
+        const uint32_t q0 = q1 + quad_threshold(0, m1 & ~1u) - quad_threshold(1, m1);
+        t.m4[q - 1] = m3 | m2 << 8 | m1 << 16 | (q0 - 1) << 24;  // thresholds 1, 2
+    }
+    return t;
+}
+constexpr QuadTable kQuadsHost = make_quads();
+__device__ __align__(128) const QuadTable kQuads = kQuadsHost;
+
+// Rewrites the section that search_section_begin has accepted; all threads.  `t_off`: where its buckets end.  Records afterwards: the
+// last key of the row's buckets, the shared addresses of its row of E and of its buckets, the shift.
+template <int N>
+__device__ __forceinline__ void search_section_long(uint8_t* sec, uint32_t t_off, uint32_t t_before_e) {
+    uint32_t* recs = reinterpret_cast<uint32_t*>(sec + kSearchHeader);
+    auto first_bucket = [&](int n) { return n < N ? recs[4 * n + 2] + ((kSearchKeyOfOne >> recs[4 * n + 3]) << 2) : t_off; };
+    uint32_t last_key = 0u;
+    if (threadIdx.x < N) {
+        const int n = threadIdx.x;
+        const uint32_t sh = recs[4 * n + 3], buckets = (first_bucket(n + 1) - first_bucket(n)) >> 2;
+        last_key = (((kSearchKeyOfOne >> sh) + buckets) << sh) - 1u;
+    }
+    for (int n = threadIdx.x >> 5; n < N; n += blockDim.x >> 5) {
+        const uint32_t sh = recs[4 * n + 3], from = first_bucket(n), end = first_bucket(n + 1);
+        uint32_t* b = reinterpret_cast<uint32_t*>(sec + from);
+        for (uint32_t i = threadIdx.x & 31; from + 4u * i < end; i += 32u) {
+            const uint32_t e = b[i];
+            // (a bucket without a threshold has all ones for its key bits: the last key of the bucket, which nothing in it passes)
+            b[i] = (e << 24) + 0xffffffu - ((((kSearchKeyOfOne >> sh) + i) << sh) + (e >> (32u - sh)));
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < N) {
+        uint32_t* rec = recs + 4 * threadIdx.x;
+        const uint32_t base = shared_addr(sec);
+        rec[0] = last_key;
+        rec[1] += base - t_before_e;
+        rec[2] += base;
+    }
+}
+
+// Four positions, as search_block4; `odd_one`: bit 7 of a byte set if the group has to be searched in full.
+template <int W, int PW, int GP, int PLANE>
+__device__ __forceinline__ void search_block4_long(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, uint32_t y, uint32_t ychain,
+                                                   uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
+    uint32_t acc[GP];
+    mp<PW> v[GP];
+#pragma unroll
+    for (int j = 0; j < GP; ++j) {
+        acc[j] = 0u;
+#pragma unroll
+        for (int w = 0; w < PW; ++w) v[j].w[w] = q[j].w[w];
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        const uint4 r = load_record(rec - static_cast<uint32_t>(s) * 16u);  // last key, E row, buckets, shift
+        uint32_t sum[GP];
+#pragma unroll
+        for (int j = 0; j < GP; ++j) {
+            const uint32_t key = min(search_key<PW>(v[j].w), r.x);
+            sum[j] = key + load_bucket(r.z + ((key >> r.w) << 2));
+        }
+#pragma unroll
+        for (int j = 0; j < GP; ++j) {
+            const mp<PW> e = load_planes<PW, PLANE>(r.y + ((sum[j] >> 24) << 2));
+            mp_add<PW>(v[j], e);
+            acc[j] = __byte_perm(acc[j], sum[j], 0x7321);  // the new byte enters at the top
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < GP; ++j) {
+        odd_one[j] |= search_coordinates(acc[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
+#pragma unroll
+        for (int w = 0; w < PW; ++w) q[j].w[w] = v[j].w[w];
+    }
+}
+
+// One group, position by position, every comparison in full.  Returns the sum of the squares.
+template <int N, int W, int PLANE>
+__device__ __noinline__ uint32_t search_exact(const uint32_t* code, const uint32_t* bound, int K, uint32_t recs, const uint8_t* t_rows,
+                                              int rows4, int rows3, int rows2, uint32_t y) {
+    uint32_t q[W];
+    long long c = 0;
+    for (int w = 0; w < W; ++w) {
+        c += static_cast<long long>(bound[w]) - code[w];
+        q[w] = static_cast<uint32_t>(c);
+        c >>= 32;
+    }
+    uint32_t ssy = 0u, y4 = 0u;
+    int k = K;
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+        const int words = min(W, i < rows4 ? 4 : (i < rows4 + rows3 ? 3 : (i < rows4 + rows3 + rows2 ? 2 : 1)));
+        const uint4 r = load_record(recs + static_cast<uint32_t>(N - 1 - i) * 16u);
+        const uint32_t key = min(search_key(q, W), r.x);
+        const uint32_t sum = key + load_bucket(r.z + ((key >> r.w) << 2));
+        uint32_t m = sum >> 24;
+        if ((sum & 0xffffffu) == 0xffffffu) {  // the key bits of T[m]; the row of T in global memory lies where that of E lies in shared memory
+            const uint32_t* t = reinterpret_cast<const uint32_t*>(t_rows + r.y + m * 4u);
+            c = 0;
+            for (int w = 0; w < words; ++w) c = (c + static_cast<long long>(t[w * PLANE]) - q[w]) >> 32;
+            if (c < 0) ++m;
+        }
+        unsigned long long carry = 0;
+        for (int w = 0; w < words; ++w) {
+            carry += static_cast<unsigned long long>(q[w]) + load_bucket(r.y + (m + static_cast<uint32_t>(w) * PLANE) * 4u);
+            q[w] = static_cast<uint32_t>(carry);
+            carry >>= 32;
+        }
+        const int left = static_cast<int>(m >> 1), mag = k - left;
+        ssy += static_cast<uint32_t>(mag * mag);
+        y4 |= (static_cast<uint32_t>((m & 1u) ? 128 + mag : 128 - mag) & 0xffu) << (8 * (i & 3));
+        if ((i & 3) == 3) {
+            store_y4(y + static_cast<uint32_t>(i & ~3), y4);
+            y4 = 0u;
+        }
+        k = left;
+    }
+    return ssy;
+}
+
+// search_codes for a rewritten section; quads: shared address of kQuads, or 0: without.
+template <int N, int W, int GP, int PLANE>
+__device__ __forceinline__ void search_codes_long(mp<W> (&q)[GP], int K, uint32_t recs, const int (&cnt)[5], uint32_t quads, uint32_t y,
+                                                  uint32_t ychain, uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
+    uint32_t k[GP];
+#pragma unroll
+    for (int j = 0; j < GP; ++j) k[j] = static_cast<uint32_t>(K);
+    uint32_t rec = recs + static_cast<uint32_t>(N - 1) * 16u;
+    if constexpr (W >= 4) {
+#pragma unroll 1
+        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4_long<W, 4, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+    }
+    if constexpr (W >= 3) {
+#pragma unroll 1
+        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4_long<W, 3, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+    }
+    if constexpr (W >= 2) {
+#pragma unroll 1
+        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4_long<W, 2, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+    }
+#pragma unroll 1
+    for (int b = 0; b < cnt[1]; b += 4, rec -= 64u, y += 4u) {
+        if (b + 4 == cnt[1] && quads != 0u) {  // the last four (N(4,K) is below 2^32: a block of one word)
+            uint32_t most = q[0].w[0];
+#pragma unroll
+            for (int j = 1; j < GP; ++j) most = max(most, q[j].w[0]);
+            if (!__any_sync(kFull, most > kQuadEntries)) {
+                uint32_t m4[GP];
+#pragma unroll
+                for (int j = 0; j < GP; ++j) m4[j] = load_bucket(quads + ((q[j].w[0] - 1u) << 2));
+#pragma unroll
+                for (int j = 0; j < GP; ++j) odd_one[j] |= search_coordinates(m4[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
+                break;
+            }
+        }
+        search_block4_long<W, 1, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
     }
 }
 
