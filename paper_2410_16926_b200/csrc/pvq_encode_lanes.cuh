@@ -38,7 +38,8 @@ constexpr int kSplitBit = 48;
 
 struct LaneGeom {
     int team, teams;                // threads per team, teams per block
-    uint32_t team_off, team_bytes;  // the teams' areas: [2 input buffers], then one (a team of one warp) or two each of [energies][LS amplitudes][index words]
+    int in_bufs;                    // 2: the next chunk's input is asked for a chunk ahead; 1: as soon as the chunk's point is there
+    uint32_t team_off, team_bytes;  // the teams' areas: [input buffers], then one (a team of one warp) or two each of [energies][LS amplitudes][index words]
     uint32_t in_bytes;              // of one input buffer
     uint32_t ss_off, amp_off, idx_off;  // inside a team's area
     int ss_floats, idx_words;       // per buffer
@@ -441,8 +442,9 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
     const int wide_blocks = g.wide_blocks;
 
     int in_buf = 0, buf = 0;
+    const int in_flip = g.in_bufs - 1;
     int done_mi = -1;  // matrix of the tile before, whose index words are still to be written out
-    for (;; in_buf ^= 1) {
+    for (;; in_buf ^= in_flip) {
         copy_async_wait<0>();
         __syncwarp();
         const LanePlace cur = at;
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
                 enter_matrix(a, at, ni, tid, L);
             }
         }
-        if (more) request_input<E, L, BF16>(a, at, shared_addr(area + (in_buf ^ 1) * g.in_bytes), T, tid);
+        if (more && in_flip != 0) request_input<E, L, BF16>(a, at, shared_addr(area + (in_buf ^ 1) * g.in_bytes), T, tid);
 
         const int G = m.G, C = G * L, gp = G > 1 ? 1 << (32 - __clz(G - 1)) : 1;
         const long long row = static_cast<long long>(cur.tile - m.tile_begin) * m.rows_per_tile + cur.rl;
@@ -498,6 +500,10 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
             if constexpr (LS) {
                 const float ls = least_squares_amplitude<E, L, BF16, GLOBAL>(pt, mine);
                 if (leader) s_amp[slot] = ls;
+            }
+            if (more && in_flip == 0) {
+                __syncwarp();  // (the warp's lanes asked for the input, and are through with it)
+                request_input<E, L, BF16>(a, at, shared_addr(area), T, tid);
             }
             if (!pt.has_dir) {  // (K, 0, ..., 0), positive
 #pragma unroll
@@ -627,13 +633,19 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
         c.ss_floats = (ss_floats + 3) & ~3;
         c.idx_words = idx_words;
         const uint32_t bufs = t == 32 ? 1u : 2u;
-        c.ss_off = 2u * c.in_bytes;
-        c.amp_off = c.ss_off + bufs * static_cast<uint32_t>(c.ss_floats) * 4u;
-        c.idx_off = c.amp_off + (LS ? bufs * static_cast<uint32_t>(c.ss_floats) * 4u : 0u);
-        c.team_bytes = (c.idx_off + bufs * static_cast<uint32_t>(idx_words) * 4u + 127u) & ~127u;
-        // as many teams as the threads, the shared memory and (larger than a warp) the named barriers hold
-        long long teams = std::min(kLaneThreads<W> / t, t == 32 ? 32 : 15);
-        teams = std::min(teams, (static_cast<long long>(di.smem_max) - c.team_off) / c.team_bytes);
+        // As many teams as the threads, the shared memory and (larger than a warp) the named barriers hold.  Where the
+        // shared memory is what limits them, a long launch makes do with one input buffer a team: the wait for the input is
+        // covered by the other warps.  (A decoder layer at N = 32, 96 bits: 23 warps and two buffers 336 us, 28 and one 286.)
+        const long long most_teams = std::min(kLaneThreads<W> / t, t == 32 ? 32 : 15);
+        long long teams = 0;
+        for (int n = 2; n >= (long_launch ? 1 : 2) && teams < most_teams; --n) {
+            c.in_bufs = n;
+            c.ss_off = static_cast<uint32_t>(n) * c.in_bytes;
+            c.amp_off = c.ss_off + bufs * static_cast<uint32_t>(c.ss_floats) * 4u;
+            c.idx_off = c.amp_off + (LS ? bufs * static_cast<uint32_t>(c.ss_floats) * 4u : 0u);
+            c.team_bytes = (c.idx_off + bufs * static_cast<uint32_t>(idx_words) * 4u + 127u) & ~127u;
+            teams = std::min(most_teams, (static_cast<long long>(di.smem_max) - c.team_off) / c.team_bytes);
+        }
         if (teams < 1) continue;
         const double per_tile = static_cast<double>(chunks_all) / tiles + (t == 32 ? 0.16 : 0.25);
         const double rounds = std::ceil(static_cast<double>(tiles) / (static_cast<double>(teams) * di.sms));
