@@ -7,8 +7,8 @@
 // points in shared memory, a signed byte a value; then the amplitudes, once the rows' energies are complete;
 // then every thread sums its group's index from the windowed tables (pvq_window.cuh), one entry of E a position, read
 // word plane by word plane from the ring that a feeding warp keeps filled, the last block of rows first.  With q the
-// number that the decoder searches, the code is N(N,K) - q: the sum of all E is 1 - q.  Same matrix: 66 us; the two phases
-// do not overlap (62% of the issue slots used).
+// number that the decoder searches, the code is N(N,K) - q: the sum of all E is 1 - q.  Same matrix: 56 us; the two phases
+// do not overlap (61% of the issue slots used).
 #include <algorithm>
 #include <cstring>
 
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
     __shared__ int s_failed, s_gave_up;  // s_gave_up: written and read between the working warps' barriers only
     __shared__ uint8_t s_words[N];
     constexpr int E = 32, L = N / E, BLOCKS = N / 4, YS = N + 4, GW = 32 / L;
-    constexpr bool WIDE = N == 64 ? W >= 7 : W >= 10;  // K may pass 127
+    constexpr bool LARGE = N == 64 ? W >= 7 : W >= 10;  // K may pass 127 (it is at most 255: a byte holds a coordinate's pulses)
     constexpr int P = E * (BF16 ? 2 : 4) / 16, RUN = kLaneRun<E, BF16>;
     grid_launch_dependents();
     if (threadIdx.x == 0) {
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
     }
     const int T = g.warps * 32, K = a.K, b = a.scale_bits;
     const TableLayout TL = table_layout(N, K, W);
-    for (int i = threadIdx.x; i < N; i += T) {  // words of N(n+1,K), which no term of the position exceeds
+    for (int i = threadIdx.x; LARGE && i < N; i += T) {  // words of N(n+1,K), which no term of the position exceeds
         const uint32_t* u = a.table + TL.enc_off[0] / 4 + (static_cast<size_t>(i) * (K + 2) + K + 1) * TL.top_words;
         int words = W;
         while (i > 0 && words > 1 && __ldg(u + words - 1) == 0u) --words;
@@ -217,7 +217,8 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
         ew_barrier(T);  // the tile before is done with shared memory
 
         // the points
-        for (int g0 = warp * GW; warp < g.quant_warps && g0 < groups; g0 += g.quant_warps * GW) {
+        const int g_step = g.quant_warps * GW, g_first = warp < g.quant_warps ? warp * GW : groups;
+        auto request = [&](int g0) {
 #pragma unroll
             for (int v = 0; v < P; ++v) {
                 const int q = v * 32 + lane, l = q / P, gi = g0 + l / L;  // 16-byte piece; the lane and group it belongs to
@@ -228,11 +229,14 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
                 }
             }
             copy_async_commit();
+        };
+        if (g_first < groups) request(g_first);
+        for (int g0 = g_first; g0 < groups; g0 += g_step) {
             copy_async_wait<0>();
             __syncwarp();
             const uint8_t* mine = in + lane * RUN;
             uint32_t neg[E / 4];
-            LanePoint<E, WIDE> pt;
+            LanePoint<E, false> pt;
             float ss;
             {
                 uint32_t raw[kRawWords<E, BF16>];
@@ -246,27 +250,36 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
                 for (int i = 0; i < E / 4; ++i) neg[i] = chunk_signs4<E, BF16>(raw, i);
                 group_norms<E, L, BF16>(raw, ax, l1, ss, g.minus_zero);
                 if constexpr (BF16)
-                    quantize_group<E, L, WIDE>(ax, l1, K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, g.minus_zero);
+                    quantize_group<E, L, false>(ax, l1, K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, g.minus_zero);
                 else
-                    quantize_group<E, L, WIDE>(ax, l1, K, FetchSharedF32{reinterpret_cast<const float*>(mine)}, pt, g.minus_zero);
+                    quantize_group<E, L, false>(ax, l1, K, FetchSharedF32{reinterpret_cast<const float*>(mine)}, pt, g.minus_zero);
             }
             const int gi = g0 + lane / L, sub = lane % L;
             const bool ok = gi < groups, leader = ok && sub == 0;
             const int r = gi / G, gr = gi - r * G;
             if (leader && PVQ_DEBUG_INDEX(r * gp + gr, (g.amp_off - g.ss_off) / 4, PVQ_DEBUG_SHARED_INDEX)) s_ss[r * gp + gr] = ss;
             if (ls_mode) {
-                const float ls = least_squares_amplitude<E, L, BF16, WIDE>(pt, mine);
+                const float ls = least_squares_amplitude<E, L, BF16, false>(pt, mine);
                 if (leader) s_amp[r * gp + gr] = ls;
             }
+            __syncwarp();  // the input buffer is free
+            if (g0 + g_step < groups) request(g0 + g_step);
             uint32_t kind = pt.has_dir ? kEwPoint : kEwZero;
-            if constexpr (WIDE) {
+            if constexpr (LARGE) {
                 uint32_t high = 0u;
 #pragma unroll
-                for (int h = 0; h < E / 2; ++h) high |= pt.y[h];
-                const int lanes_high = group_add<L>((high & 0xff80ff80u) != 0u ? 1 : 0);  // (every lane takes part)
+                for (int i = 0; i < E / 4; ++i) high |= pt.y[i];
+                const int lanes_high = group_add<L>((high & kH4) != 0u ? 1 : 0);  // (every lane takes part)
                 const bool large = pt.has_dir && ok && lanes_high != 0;
-                if (__any_sync(kFull, large)) {  // a value of 128 pulses and more has no byte: its index right here
-                    const mp<W> code = lanes_index_global<E, L, W>(pt, neg, K, a.table + TL.enc_off[0] / 4, a.table + TL.enc_off[1] / 4, TL.top_words, s_words);
+                if (__any_sync(kFull, large)) {  // 128 pulses and more leave no room for a sign in the byte: its index right here
+                    LanePoint<E, true> halves;
+                    halves.has_dir = pt.has_dir;
+#pragma unroll
+                    for (int i = 0; i < E / 4; ++i) {
+                        halves.y[2 * i] = __byte_perm(pt.y[i], 0u, 0x4342);
+                        halves.y[2 * i + 1] = __byte_perm(pt.y[i], 0u, 0x4140);
+                    }
+                    const mp<W> code = lanes_index_global<E, L, W>(halves, neg, K, a.table + TL.enc_off[0] / 4, a.table + TL.enc_off[1] / 4, TL.top_words, s_words);
                     if (large) kind = kEwWritten;
                     if (large && leader) {
                         uint32_t* cp = m.codes + (static_cast<size_t>(row0 + r) * G + gr) * W;
@@ -278,17 +291,9 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
             if (ok && PVQ_DEBUG_INDEX(gi, T, PVQ_DEBUG_SLOT_WRITE)) {
                 uint32_t* slot = reinterpret_cast<uint32_t*>(smem + g.slots_off + gi * YS) + sub * (E / 4);
 #pragma unroll
-                for (int i = 0; i < E / 4; ++i) {
-                    uint32_t y;
-                    if constexpr (WIDE)
-                        y = __byte_perm(pt.y[2 * i + 1], pt.y[2 * i], 0x6420);
-                    else
-                        y = pt.y[i];
-                    slot[i] = y | (neg[i] & kH4);
-                }
+                for (int i = 0; i < E / 4; ++i) slot[i] = pt.y[i] | (neg[i] & kH4);
                 if (sub == L - 1) slot[E / 4] = kind;
             }
-            __syncwarp();  // the input buffer is free
         }
         bulk_store_fence();  // the ring's buffers are written by bulk copies next
         __syncwarp();
