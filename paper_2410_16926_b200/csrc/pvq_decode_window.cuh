@@ -225,7 +225,7 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
     const uint32_t after = (acc >> 1) & 0x7f7f7f7fu;
     const uint32_t mag = (after << 8) + win_load<kWinDlo4>(stage) - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;
-    uint32_t y4 = ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos);
+    uint32_t y4 = (mag ^ ~pos) + 0x80808081u + pos;  // 128 + |y|; else 255 - |y| + 128 - 255: no byte of the sum leaves 1 .. 255
     if (__any_sync(kFull, top == 0xffffffffu || (((mag | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
         WinExact<PW> x;
         x.v = v;

@@ -248,7 +248,15 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
     };
     const int sub = static_cast<int>(threadIdx.x) & (L - 1);
     const int mine_all = __popc(cand);
-    if (__all_sync(0xffffffffu, mine_all <= 2)) return rank_candidates<E, L, 2>(cand, r, gsc, fetch, rotation);
+    if (__all_sync(0xffffffffu, mine_all <= 2)) {
+        if constexpr (L > 1) return rank_candidates<E, L, 2>(cand, r, gsc, fetch, rotation);
+        // two, or none, of which one is chosen
+        const uint32_t one = cand & (0u - cand), two = cand ^ one;
+        const int i = (mask_bit_position(31 - __clz(static_cast<int>(one))) + 8 * rotation) & (E - 1);
+        const int j = (mask_bit_position(31 - __clz(static_cast<int>(two))) + 8 * rotation) & (E - 1);
+        const float a = residual(i), b = residual(j);
+        return a > b || (a == b && i < j) ? one : two;
+    }
     if (__all_sync(0xffffffffu, mine_all <= 4)) return rank_candidates<E, L, 4>(cand, r, gsc, fetch, rotation);
     uint32_t chosen = 0u;
     for (int round = 0; round < E * L; ++round) {
@@ -283,6 +291,22 @@ __device__ __forceinline__ uint32_t choose_candidates(uint32_t cand, int r, floa
         if (r == 0) cand = 0u;
     }
     return chosen;
+}
+
+// One step of the selection: `have`, c in the group, are the undecided residuals with the bit.  All of them are taken if no more
+// are needed than that, and those without the bit stay undecided; else those with it do.  (Predicates: a selection
+// and an operation each otherwise.)
+__device__ __forceinline__ void take_or_keep(int c, uint32_t have, uint32_t plane, uint32_t& sel, int& need, uint32_t& cand) {
+    uint32_t rest;
+    asm("{\n\t.reg .pred p;\n\t"
+        "setp.le.s32 p, %3, %1;\n\t"
+        "mov.b32 %2, %4;\n\t"
+        "@p lop3.b32 %2, %5, %6, 0, 0x30;\n\t"
+        "@p or.b32 %0, %0, %4;\n\t"
+        "@p sub.s32 %1, %1, %3;\n\t}"
+        : "+r"(sel), "+r"(need), "=&r"(rest)
+        : "r"(c), "r"(have), "r"(cand), "r"(plane));
+    cand = rest;
 }
 
 // ax: |x_i| of the lane's values; l1: of the whole group.
@@ -341,12 +365,9 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
     int need = d;                                        // still to be chosen among the undecided ones
 #pragma unroll
     for (int p = 7; p >= 0; --p) {
-        const uint32_t have = cand & (x[p % J] >> (p - p % J));
+        const uint32_t plane = x[p % J] >> (p - p % J), have = cand & plane;
         const int c = group_add<L>(__popc(have));
-        const bool all = c <= need;
-        sel |= all ? have : 0u;
-        need -= all ? c : 0;
-        cand = all ? cand ^ have : have;
+        take_or_keep(c, have, plane, sel, need, cand);
     }
     const bool rest = group_add<L>(__popc(cand)) == need;  // (none needed: no matter)
     if (rest) sel |= cand;

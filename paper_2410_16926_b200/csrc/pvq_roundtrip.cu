@@ -53,14 +53,15 @@ __device__ __forceinline__ uint2 scaled_values(const LanePoint<E, WIDE>& pt, int
     float f[4];
     if constexpr (!WIDE) {
         // 128 + y_i in a byte; as the low mantissa bits of 2^23 it becomes a float by one subtraction
-        const uint32_t biased = ((kH4 + pt.y[j]) & ~neg) | ((kH4 - pt.y[j]) & neg);
+        // (128 + y, or 128 + 255 - y - 255: no byte of the sum leaves 1 .. 255)
+        const uint32_t biased = (pt.y[j] ^ neg) + kH4 - neg;
 #pragma unroll
         for (int e = 0; e < 4; ++e) f[e] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7540u + 3 - e));
     } else {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {  // positions 4j + 2h (high half), 4j + 2h + 1
             const uint32_t y = pt.y[2 * j + h], n2 = __byte_perm(neg, 0u, h == 0 ? 0x3322 : 0x1100);
-            const uint32_t biased = ((0x80008000u + y) & ~n2) | ((0x80008000u - y) & n2);
+            const uint32_t biased = (y ^ n2) + 0x80008000u - n2;
             f[2 * h] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7532u));
             f[2 * h + 1] = __uint_as_float(__byte_perm(biased, 0x4B000000u, 0x7510u));
         }

@@ -153,7 +153,7 @@ __device__ __forceinline__ uint32_t search_coordinates(uint32_t m4, uint32_t& k,
     ssy = __dp4a(mag, mag, ssy);
     const uint32_t odd = m4 & 0x01010101u;
     const uint32_t pos = (odd << 8) - odd;  // 0xff in the bytes with y > 0
-    store_y4(y, ((0x80808080u + mag) & pos) | ((0x80808080u - mag) & ~pos));
+    store_y4(y, (mag ^ ~pos) + 0x80808081u + pos);  // 128 + |y|; else 255 - |y| + 128 - 255: no byte of the sum leaves 1 .. 255
     k = after >> 24;
     return mag | ~((mag | 0x80808080u) - odd);
 }
