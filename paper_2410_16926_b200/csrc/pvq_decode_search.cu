@@ -31,7 +31,7 @@ namespace {
 constexpr int kSearchThreads = 1024;
 
 // GP groups per thread: a warp takes GP consecutive tiles of 32 groups in one pass.
-// LONG: rewrites the staged buckets and has the table of the last four positions (see "long launches" in pvq_search.cuh).
+// LONG: rewrites the staged buckets and has the table of the last four positions (pvq_search.cuh).
 template <int N, int W, int GP, int PLANE, bool LONG>
 __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
     decode_search_kernel(const __grid_constant__ BatchArgs a) {
@@ -79,10 +79,7 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
         if (a.status && threadIdx.x == 0) atomicOr(a.status, PVQ_STATUS_TABLE_MISMATCH);
         return;
     }
-    if constexpr (LONG)
-        search_section_long<N>(smem, a.srch_t_off, a.srch_t_before_e);
-    else
-        search_section_addresses<N>(smem, a.srch_t_before_e);
+    search_section_ready<N, LONG>(smem, a.srch_t_off, a.srch_t_before_e);
 #ifdef PVQ_DEBUG
     debug_begin(sbase, sbase + staged + quad_bytes, sbase + staged + quad_bytes, YS, N, a.debug_status);
     if (threadIdx.x == 0) {
@@ -157,21 +154,17 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
         uint32_t ssy[GP];
 #pragma unroll
         for (int j = 0; j < GP; ++j) ssy[j] = 0u;
-        if constexpr (LONG) {
-            uint32_t odd_one[GP];
+        uint32_t odd_one[GP];
 #pragma unroll
-            for (int j = 0; j < GP; ++j) odd_one[j] = 0u;
-            search_codes_long<N, W, GP, PLANE>(q, K, recs, cnt, quad_bytes != 0u ? sbase + staged : 0u, shared_addr(yslots), ychain, ssy, odd_one);
+        for (int j = 0; j < GP; ++j) odd_one[j] = 0u;
+        search_codes<N, W, GP, PLANE, LONG>(q, K, recs, cnt, quad_bytes != 0u ? sbase + staged : 0u, shared_addr(yslots), ychain, ssy, odd_one);
 #pragma unroll
-            for (int j = 0; j < GP; ++j)
-                if (active_valid[j] && (odd_one[j] & 0x80808080u) != 0u) {
-                    const MatrixArgs& m = a.m[mj[j]];
-                    const uint32_t* code = m.codes + (static_cast<size_t>(row[j]) * m.G + g[j]) * W;
-                    ssy[j] = search_exact<N, W, PLANE>(code, bw, K, recs, t_rows, cnt[4], cnt[3], cnt[2], shared_addr(yslots) + j * ychain);
-                }
-        } else {
-            search_codes<N, W, GP, PLANE>(q, K, recs, t_rows, cnt, shared_addr(yslots), ychain, ssy);
-        }
+        for (int j = 0; j < GP; ++j)
+            if (active_valid[j] && (odd_one[j] & 0x80808080u) != 0u) {
+                const MatrixArgs& m = a.m[mj[j]];
+                const uint32_t* code = m.codes + (static_cast<size_t>(row[j]) * m.G + g[j]) * W;
+                ssy[j] = search_exact<N, W, PLANE, LONG>(code, bw, K, recs, t_rows, cnt[4], cnt[3], cnt[2], shared_addr(yslots) + j * ychain);
+            }
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
@@ -262,7 +255,7 @@ int launch_search_g(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
     }
     a.total_tiles = tiles;
     // More than a round earns the rewriting of the buckets and the staging of the table of the last four positions, some 2 us.
-    // (Without and with, us: decoder layer, 23 rounds, 271 and 242; 4096 x 4096 at N = 16, 48 bits, 3.5 rounds, 24.6 and
+    // (Without and with, us: decoder layer, 23 rounds, 271 and 240; 4096 x 4096 at N = 16, 48 bits, 3.5 rounds, 24.6 and
     // 22.1; at N = 32, 64 bits, 1.7 rounds, 21.5 and 20.3, 96 bits 23.5 and 23.6; one round only loses.)
     const bool is_long = tiles > 2u * static_cast<unsigned>(di.sms) * (kSearchThreads / 32);
     switch (S.plane) {  // entries per word plane of the section's rows

@@ -45,50 +45,6 @@ __device__ __forceinline__ uint32_t load_bucket(uint32_t addr) {
     return v;
 }
 
-// m0 + (t < q): minus the borrow of t - q, which the last link of the chain leaves as 0 or -1
-template <int W>
-__device__ __forceinline__ uint32_t bump_if_less(uint32_t m0, const mp<W>& t, const mp<W>& q) {
-    uint32_t m;
-    if constexpr (W == 1) {
-        asm("{\n\t.reg .u32 d;\n\t"
-            "sub.cc.u32 d, %2, %3;\n\t"
-            "subc.u32 d, 0, 0;\n\t"
-            "sub.u32 %0, %1, d;\n\t}"
-            : "=r"(m)
-            : "r"(m0), "r"(t.w[0]), "r"(q.w[0]));
-    } else if constexpr (W == 2) {
-        asm("{\n\t.reg .u32 d;\n\t"
-            "sub.cc.u32 d, %2, %4;\n\t"
-            "subc.cc.u32 d, %3, %5;\n\t"
-            "subc.u32 d, 0, 0;\n\t"
-            "sub.u32 %0, %1, d;\n\t}"
-            : "=r"(m)
-            : "r"(m0), "r"(t.w[0]), "r"(t.w[1]), "r"(q.w[0]), "r"(q.w[1]));
-    } else if constexpr (W == 3) {
-        asm("{\n\t.reg .u32 d;\n\t"
-            "sub.cc.u32 d, %2, %5;\n\t"
-            "subc.cc.u32 d, %3, %6;\n\t"
-            "subc.cc.u32 d, %4, %7;\n\t"
-            "subc.u32 d, 0, 0;\n\t"
-            "sub.u32 %0, %1, d;\n\t}"
-            : "=r"(m)
-            : "r"(m0), "r"(t.w[0]), "r"(t.w[1]), "r"(t.w[2]), "r"(q.w[0]), "r"(q.w[1]), "r"(q.w[2]));
-    } else {
-        static_assert(W == 4, "codes of up to four words");
-        asm("{\n\t.reg .u32 d;\n\t"
-            "sub.cc.u32 d, %2, %6;\n\t"
-            "subc.cc.u32 d, %3, %7;\n\t"
-            "subc.cc.u32 d, %4, %8;\n\t"
-            "subc.cc.u32 d, %5, %9;\n\t"
-            "subc.u32 d, 0, 0;\n\t"
-            "sub.u32 %0, %1, d;\n\t}"
-            : "=r"(m)
-            : "r"(m0), "r"(t.w[0]), "r"(t.w[1]), "r"(t.w[2]), "r"(t.w[3]), "r"(q.w[0]), "r"(q.w[1]), "r"(q.w[2]),
-              "r"(q.w[3]));
-    }
-    return m;
-}
-
 // Once the section has arrived in shared memory (at `sec`; `bytes` is its size in the blob): is
 // it the section of this (N,K)?  (A table built for another one would send the look-ups
 // anywhere.)  If so, the numbers of rows per width go to cnt[1..4].
@@ -105,19 +61,6 @@ __device__ __forceinline__ bool search_section_begin(const uint8_t* sec, uint32_
         (W < 4 && cnt[4] != 0) || (W < 3 && cnt[3] != 0) || (W < 2 && cnt[2] != 0))
         return false;
     return true;
-}
-
-// Then threads 0..N-1 turn the records' offsets into shared addresses; the caller's next block-wide barrier publishes them.
-// The thresholds T are not staged (only a 24-bit tie reads one, from global memory): the
-// increments E sit where T is in the blob, `t_before_e` bytes lower.
-template <int N>
-__device__ __forceinline__ void search_section_addresses(uint8_t* sec, uint32_t t_before_e) {
-    if (threadIdx.x < N) {
-        uint32_t* rec = reinterpret_cast<uint32_t*>(sec + kSearchHeader) + 4 * threadIdx.x;
-        const uint32_t base = shared_addr(sec);
-        rec[1] += base - t_before_e;
-        rec[2] += base;
-    }
 }
 
 // Entry of PW words of a row stored word plane by word plane (PLANE entries a plane): word w
@@ -158,87 +101,19 @@ __device__ __forceinline__ uint32_t search_coordinates(uint32_t m4, uint32_t& k,
     return mag | ~((mag | 0x80808080u) - odd);
 }
 
-// Four positions of GP codes (GP independent chains of dependent table reads, so that one
-// thread keeps several reads in flight), in PW-word arithmetic on rows of PW word planes.
-// `rec` is the shared address of the record of the first of the four rows (the rows of the
-// following positions have the records before it); a record is read once for all chains.
-// `t_rows` plus the shared address of a row of E is the global address of the same row of T.
-// The four y_i + 128 of chain j go to the word at y + j * ychain, their squares to ssy[j].
+// How a position is searched: the key of q selects a bucket; its entry holds the low key bits of the threshold T[m0] in it, and m0.
+// q's own low key bits being larger means q > T[m0] and the index m0 + 1, else it is m0 (a bucket without a threshold
+// holds all ones there).  A launch of some rounds can afford to rewrite the staged buckets first (LONG): an entry is then what,
+// added to the key, leaves the index in the top byte, the comparison being the carry into it.
 //
-// Per position: the key of q selects a bucket; its entry is m0 and the low key bits of the
-// threshold T[m0]; q's own low key bits being larger means q > T[m0], smaller means q <= T[m0]
-// (a bucket without a threshold holds all ones there).  Equal bits leave it open: then, and
-// that is rare, the threads of the warp whose bits were equal compare q with T[m0] in full.
-template <int W, int PW, int GP, int PLANE>
-__device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, const uint8_t* t_rows,
-                                              uint32_t y, uint32_t ychain, uint32_t (&ssy)[GP]) {
-    uint32_t acc[GP];  // the four threshold indices m, a byte each, first position lowest
-    mp<PW> v[GP];      // the low PW words of q: the rest is zero by now
-#pragma unroll
-    for (int j = 0; j < GP; ++j) {
-        acc[j] = 0u;
-#pragma unroll
-        for (int w = 0; w < PW; ++w) v[j].w[w] = q[j].w[w];
-    }
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const uint4 r = load_record(rec - static_cast<uint32_t>(s) * 16u);  // 32 - shift, E row, buckets, shift
-        uint32_t key[GP], entry[GP], m[GP];
-        mp<PW> e[GP];
-        bool open = false;
-#pragma unroll
-        for (int j = 0; j < GP; ++j) {
-            key[j] = search_key<PW>(v[j].w);
-            entry[j] = load_bucket(r.z + ((key[j] >> r.w) << 2));
-        }
-#pragma unroll
-        for (int j = 0; j < GP; ++j) {
-            const uint32_t x = key[j] << r.x;  // the key bits below the shift, left-aligned like the entry's
-            m[j] = (entry[j] & 0xffu) + (x > entry[j] ? 1u : 0u);
-            open = open || (entry[j] - x < 256u);
-        }
-        if (__any_sync(kFull, open)) {
-#pragma unroll
-            for (int j = 0; j < GP; ++j) {
-                const uint32_t m0 = entry[j] & 0xffu;
-                if (entry[j] - (key[j] << r.x) < 256u) {
-                    // the row of T in global memory lies where the row of E lies in shared memory
-                    const uint32_t* tp = reinterpret_cast<const uint32_t*>(t_rows + r.y + m0 * 4u);
-                    mp<PW> t;
-#pragma unroll
-                    for (int w = 0; w < PW; ++w) t.w[w] = tp[w * PLANE];
-                    m[j] = bump_if_less<PW>(m0, t, v[j]);
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < GP; ++j) e[j] = load_planes<PW, PLANE>(r.y + (m[j] << 2));
-#pragma unroll
-        for (int j = 0; j < GP; ++j) {
-            mp_add<PW>(v[j], e[j]);
-            acc[j] = __funnelshift_r(acc[j], m[j], 8);  // the new byte enters at the top
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < GP; ++j) {
-        search_coordinates(acc[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
-#pragma unroll
-        for (int w = 0; w < PW; ++w) q[j].w[w] = v[j].w[w];
-    }
-}
-
-// ---------------------------------------------------------------- long launches
-//
-// A launch of some rounds can afford to rewrite the staged buckets first (search_section_long), so that a position takes
-// fewer instructions: an entry is then what, added to the key, leaves the index in the top byte, the comparison
-// of the key with the bucket's threshold being the carry into it.  Nor does it look whether the key bits are the same as
-// a threshold's.  If they are, and q is above the threshold all the same, the index is one short and q' = T_(n-1)[2k'] + d,
-// d = q - T_n[m], is too large for the k' pulses left.  The next row then has an index of 2k' + 1 or more for it, which no q
-// of a valid code has (2k' + 1: a positive coordinate of no pulse; more: pulses left that grow), and
-// search_coordinates shows it.  (There is a next row: row 0's thresholds are their keys.)  Whatever follows is in
+// Key bits that are the same as the threshold's are not looked for.  If they are, and q is above the threshold all the same, the
+// index is one short and q' = T_(n-1)[2k'] + d, d = q - T_n[m], is too large for the k' pulses left.  The next row then has an
+// index of 2k' + 1 or more for it, which no q of a valid code has (2k' + 1: a positive coordinate of no pulse; more: pulses left
+// that grow), and search_coordinates shows it.  (There is a next row: row 0's thresholds are their keys.)  Whatever follows is in
 // bounds: q stays above zero, as every step leaves 1 <= q <= N(n,k') for a q up to the row's last threshold, and a key above
-// the last bucket is cut off at it.  Such a group is searched once more, in full (search_exact).
-// Tried with the old entries and not kept: bucket and key bits from one wide product, and the comparison taken as the borrow of a
+// the last bucket is cut off at it.  Such a group is searched once more, in full (search_exact).  (A vote of the warp a position,
+// and the full comparison right there: decoder layer 271 us, this way and LONG 240; 512 x 512, one round, 6.7 and 6.3 us.)
+// Tried and not kept: bucket and key bits from one wide product, and the comparison taken as the borrow of a
 // subtraction (decoder layer 271 -> 288 and 284 us: they tie up the pipes that are short).
 
 // The last four positions at once: the indices of q in row 3, of the q that follows in row 2, and so on depend on q
@@ -273,10 +148,12 @@ constexpr QuadTable make_quads() {
 constexpr QuadTable kQuadsHost = make_quads();
 __device__ __align__(128) const QuadTable kQuads = kQuadsHost;
 
-// Rewrites the section that search_section_begin has accepted; all threads.  `t_off`: where its buckets end.  Records afterwards: the
-// last key of the row's buckets, the shared addresses of its row of E and of its buckets, the shift.
-template <int N>
-__device__ __forceinline__ void search_section_long(uint8_t* sec, uint32_t t_off, uint32_t t_before_e) {
+// Makes the accepted section ready for the search; all threads, a barrier follows.  `t_off`: where its buckets end.  Records
+// afterwards: the last key of the row's buckets, the shared addresses of its row of E and of its buckets, the shift.
+// The thresholds T are not staged (search_exact reads some, from global memory): the
+// increments E sit where T is in the blob, `t_before_e` bytes lower.
+template <int N, bool LONG>
+__device__ __forceinline__ void search_section_ready(uint8_t* sec, uint32_t t_off, uint32_t t_before_e) {
     uint32_t* recs = reinterpret_cast<uint32_t*>(sec + kSearchHeader);
     auto first_bucket = [&](int n) { return n < N ? recs[4 * n + 2] + ((kSearchKeyOfOne >> recs[4 * n + 3]) << 2) : t_off; };
     uint32_t last_key = 0u;
@@ -285,13 +162,15 @@ __device__ __forceinline__ void search_section_long(uint8_t* sec, uint32_t t_off
         const uint32_t sh = recs[4 * n + 3], buckets = (first_bucket(n + 1) - first_bucket(n)) >> 2;
         last_key = (((kSearchKeyOfOne >> sh) + buckets) << sh) - 1u;
     }
-    for (int n = threadIdx.x >> 5; n < N; n += blockDim.x >> 5) {
-        const uint32_t sh = recs[4 * n + 3], from = first_bucket(n), end = first_bucket(n + 1);
-        uint32_t* b = reinterpret_cast<uint32_t*>(sec + from);
-        for (uint32_t i = threadIdx.x & 31; from + 4u * i < end; i += 32u) {
-            const uint32_t e = b[i];
-            // (a bucket without a threshold has all ones for its key bits: the last key of the bucket, which nothing in it passes)
-            b[i] = (e << 24) + 0xffffffu - ((((kSearchKeyOfOne >> sh) + i) << sh) + (e >> (32u - sh)));
+    if constexpr (LONG) {
+        for (int n = threadIdx.x >> 5; n < N; n += blockDim.x >> 5) {
+            const uint32_t sh = recs[4 * n + 3], from = first_bucket(n), end = first_bucket(n + 1);
+            uint32_t* b = reinterpret_cast<uint32_t*>(sec + from);
+            for (uint32_t i = threadIdx.x & 31; from + 4u * i < end; i += 32u) {
+                const uint32_t e = b[i];
+                // (all ones: the last key of the bucket, which nothing in it passes)
+                b[i] = (e << 24) + 0xffffffu - ((((kSearchKeyOfOne >> sh) + i) << sh) + (e >> (32u - sh)));
+            }
         }
     }
     __syncthreads();
@@ -304,12 +183,26 @@ __device__ __forceinline__ void search_section_long(uint8_t* sec, uint32_t t_off
     }
 }
 
-// Four positions, as search_block4; `odd_one`: bit 7 of a byte set if the group has to be searched in full.
-template <int W, int PW, int GP, int PLANE>
-__device__ __forceinline__ void search_block4_long(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, uint32_t y, uint32_t ychain,
-                                                   uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
-    uint32_t acc[GP];
-    mp<PW> v[GP];
+// The index that a bucket's entry leads to; top: it sits in the top byte of the result, else in the lowest.
+template <bool LONG>
+__device__ __forceinline__ uint32_t search_index(uint32_t key, uint32_t entry, uint32_t shift) {
+    if constexpr (LONG)
+        return key + entry;
+    else  // (funnel: key << (32 - shift))
+        return (entry & 0xffu) + (__funnelshift_r(0u, key, shift) > entry ? 1u : 0u);
+}
+
+// Four positions of GP codes (GP independent chains of dependent table reads, so that one
+// thread keeps several reads in flight), in PW-word arithmetic on rows of PW word planes.
+// `rec` is the shared address of the record of the first of the four rows (the rows of the
+// following positions have the records before it); a record is read once for all chains.
+// The four y_i + 128 of chain j go to the word at y + j * ychain, their squares to ssy[j]; odd_one[j]: bit 7 of a
+// byte set if the group has to be searched in full.
+template <int W, int PW, int GP, int PLANE, bool LONG>
+__device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, uint32_t y, uint32_t ychain,
+                                              uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
+    uint32_t acc[GP];  // the four threshold indices m, a byte each, first position lowest
+    mp<PW> v[GP];      // the low PW words of q: the rest is zero by now
 #pragma unroll
     for (int j = 0; j < GP; ++j) {
         acc[j] = 0u;
@@ -319,17 +212,17 @@ __device__ __forceinline__ void search_block4_long(mp<W> (&q)[GP], uint32_t (&k)
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
         const uint4 r = load_record(rec - static_cast<uint32_t>(s) * 16u);  // last key, E row, buckets, shift
-        uint32_t sum[GP];
+        uint32_t m[GP];
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
             const uint32_t key = min(search_key<PW>(v[j].w), r.x);
-            sum[j] = key + load_bucket(r.z + ((key >> r.w) << 2));
+            m[j] = search_index<LONG>(key, load_bucket(r.z + ((key >> r.w) << 2)), r.w);
         }
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
-            const mp<PW> e = load_planes<PW, PLANE>(r.y + ((sum[j] >> 24) << 2));
+            const mp<PW> e = load_planes<PW, PLANE>(r.y + ((LONG ? m[j] >> 24 : m[j]) << 2));
             mp_add<PW>(v[j], e);
-            acc[j] = __byte_perm(acc[j], sum[j], 0x7321);  // the new byte enters at the top
+            acc[j] = LONG ? __byte_perm(acc[j], m[j], 0x7321) : __funnelshift_r(acc[j], m[j], 8);  // the new byte enters at the top
         }
     }
 #pragma unroll
@@ -341,7 +234,7 @@ __device__ __forceinline__ void search_block4_long(mp<W> (&q)[GP], uint32_t (&k)
 }
 
 // One group, position by position, every comparison in full.  Returns the sum of the squares.
-template <int N, int W, int PLANE>
+template <int N, int W, int PLANE, bool LONG>
 __device__ __noinline__ uint32_t search_exact(const uint32_t* code, const uint32_t* bound, int K, uint32_t recs, const uint8_t* t_rows,
                                               int rows4, int rows3, int rows2, uint32_t y) {
     uint32_t q[W];
@@ -358,14 +251,14 @@ __device__ __noinline__ uint32_t search_exact(const uint32_t* code, const uint32
         const int words = min(W, i < rows4 ? 4 : (i < rows4 + rows3 ? 3 : (i < rows4 + rows3 + rows2 ? 2 : 1)));
         const uint4 r = load_record(recs + static_cast<uint32_t>(N - 1 - i) * 16u);
         const uint32_t key = min(search_key(q, W), r.x);
-        const uint32_t sum = key + load_bucket(r.z + ((key >> r.w) << 2));
-        uint32_t m = sum >> 24;
-        if ((sum & 0xffffffu) == 0xffffffu) {  // the key bits of T[m]; the row of T in global memory lies where that of E lies in shared memory
-            const uint32_t* t = reinterpret_cast<const uint32_t*>(t_rows + r.y + m * 4u);
-            c = 0;
-            for (int w = 0; w < words; ++w) c = (c + static_cast<long long>(t[w * PLANE]) - q[w]) >> 32;
-            if (c < 0) ++m;
-        }
+        uint32_t m = search_index<LONG>(key, load_bucket(r.z + ((key >> r.w) << 2)), r.w);
+        if (LONG) m >>= 24;
+        // (m is right or, where the key bits are the same, one short; the row of T in global memory lies where that of E lies in
+        // shared memory)
+        const uint32_t* t = reinterpret_cast<const uint32_t*>(t_rows + r.y + m * 4u);
+        c = 0;
+        for (int w = 0; w < words; ++w) c = (c + static_cast<long long>(t[w * PLANE]) - q[w]) >> 32;
+        if (c < 0) ++m;
         unsigned long long carry = 0;
         for (int w = 0; w < words; ++w) {
             carry += static_cast<unsigned long long>(q[w]) + load_bucket(r.y + (m + static_cast<uint32_t>(w) * PLANE) * 4u);
@@ -384,9 +277,11 @@ __device__ __noinline__ uint32_t search_exact(const uint32_t* code, const uint32
     return ssy;
 }
 
-// search_codes for a rewritten section; quads: shared address of kQuads, or 0: without.
-template <int N, int W, int GP, int PLANE>
-__device__ __forceinline__ void search_codes_long(mp<W> (&q)[GP], int K, uint32_t recs, const int (&cnt)[5], uint32_t quads, uint32_t y,
+// The points of GP codes: q = N(N,K) - code on entry.  `recs` is the shared address of the
+// row records (absolute shared addresses by now), cnt[w] the number of rows done in w words; quads: shared address of kQuads,
+// or 0: without.
+template <int N, int W, int GP, int PLANE, bool LONG>
+__device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t recs, const int (&cnt)[5], uint32_t quads, uint32_t y,
                                                   uint32_t ychain, uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
     uint32_t k[GP];
 #pragma unroll
@@ -394,19 +289,19 @@ __device__ __forceinline__ void search_codes_long(mp<W> (&q)[GP], int K, uint32_
     uint32_t rec = recs + static_cast<uint32_t>(N - 1) * 16u;
     if constexpr (W >= 4) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4_long<W, 4, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4<W, 4, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
     }
     if constexpr (W >= 3) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4_long<W, 3, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4<W, 3, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
     }
     if constexpr (W >= 2) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4_long<W, 2, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4<W, 2, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
     }
 #pragma unroll 1
     for (int b = 0; b < cnt[1]; b += 4, rec -= 64u, y += 4u) {
-        if (b + 4 == cnt[1] && quads != 0u) {  // the last four (N(4,K) is below 2^32: a block of one word)
+        if (LONG && b + 4 == cnt[1] && quads != 0u) {  // the last four (N(4,K) is below 2^32: a block of one word)
             uint32_t most = q[0].w[0];
 #pragma unroll
             for (int j = 1; j < GP; ++j) most = max(most, q[j].w[0]);
@@ -419,33 +314,8 @@ __device__ __forceinline__ void search_codes_long(mp<W> (&q)[GP], int K, uint32_
                 break;
             }
         }
-        search_block4_long<W, 1, GP, PLANE>(q, k, rec, y, ychain, ssy, odd_one);
+        search_block4<W, 1, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
     }
-}
-
-// The points of GP codes: q = N(N,K) - code on entry.  `recs` is the shared address of the
-// row records (absolute shared addresses by now), cnt[w] the number of rows done in w words.
-template <int N, int W, int GP, int PLANE>
-__device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t recs, const uint8_t* t_rows,
-                                             const int (&cnt)[5], uint32_t y, uint32_t ychain, uint32_t (&ssy)[GP]) {
-    uint32_t k[GP];
-#pragma unroll
-    for (int j = 0; j < GP; ++j) k[j] = static_cast<uint32_t>(K);
-    uint32_t rec = recs + static_cast<uint32_t>(N - 1) * 16u;
-    if constexpr (W >= 4) {
-#pragma unroll 1
-        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4<W, 4, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
-    }
-    if constexpr (W >= 3) {
-#pragma unroll 1
-        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4<W, 3, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
-    }
-    if constexpr (W >= 2) {
-#pragma unroll 1
-        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4<W, 2, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
-    }
-#pragma unroll 1
-    for (int b = 0; b < cnt[1]; b += 4, rec -= 64u, y += 4u) search_block4<W, 1, GP, PLANE>(q, k, rec, t_rows, y, ychain, ssy);
 }
 
 }  // namespace pvq
