@@ -561,10 +561,8 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
             if (b == 16) {  // the amplitude itself, as binary16
                 q = __half_as_ushort(__float2half_rn(LS ? ls : __fsqrt_rn(ss)));
             } else {
-                // Step 5: q = floor(CDF(u) 2^b) as the number of bin edges <= u
                 const float u = ss_row > 0.0f ? __fdiv_rn(LS ? __fmul_rn(ls, ls) : ss, ss_row) : 0.0f;
-                for (int step = 1 << (b - 1); step >= 1; step >>= 1)
-                    if (__ldg(edges + q + step - 1) <= u) q += step;
+                q = amplitude_bin(u, b, [&](int i) { return __ldg(edges + i); });
             }
             if (gi == 0 && PVQ_DEBUG_INDEX(row, m.rows, PVQ_DEBUG_GLOBAL_STORE)) m.row_norm[row] = __fsqrt_rn(ss_row);
             const unsigned bit = static_cast<unsigned>(gi) * b;

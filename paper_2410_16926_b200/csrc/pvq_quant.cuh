@@ -30,6 +30,25 @@ namespace pvq {
 
 constexpr uint32_t kH4 = 0x80808080u, kOne4 = 0x01010101u;
 
+// Step 5: q = floor(CDF(u) 2^b) as the number of bin edges <= u, for b <= 8 bits; edge(i): the i-th of 2^b - 1.
+// (Unrolled: three or four instructions a step instead of eight with a counter; decoder layer 286 -> 284.5 us, 4096 x 4096 fp32
+// 39.5 -> 39.1.)
+template <class Edge>
+__device__ __forceinline__ int amplitude_bin(float u, int b, const Edge& edge) {
+    int q = 0;
+    switch (b) {
+        case 8: if (edge(127) <= u) q = 128; [[fallthrough]];
+        case 7: if (edge(q + 63) <= u) q += 64; [[fallthrough]];
+        case 6: if (edge(q + 31) <= u) q += 32; [[fallthrough]];
+        case 5: if (edge(q + 15) <= u) q += 16; [[fallthrough]];
+        case 4: if (edge(q + 7) <= u) q += 8; [[fallthrough]];
+        case 3: if (edge(q + 3) <= u) q += 4; [[fallthrough]];
+        case 2: if (edge(q + 1) <= u) q += 2; [[fallthrough]];
+        default: if (edge(q) <= u) q += 1;
+    }
+    return q;
+}
+
 // A lane's E values as they sit in memory: E/2 words of two bf16, or E words.
 template <int E, bool BF16>
 constexpr int kRawWords = BF16 ? E / 2 : E;

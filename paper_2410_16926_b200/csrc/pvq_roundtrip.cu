@@ -23,6 +23,7 @@ namespace pvq {
 namespace {
 
 constexpr int kRoundThreadsMax = 512;
+constexpr int kCodebookMax = 256;  // levels of an amplitude codebook
 
 struct RoundArgs {
     const void* x;
@@ -91,10 +92,18 @@ __device__ __forceinline__ int lane_squares(const LanePoint<E, WIDE>& pt) {
 // The group's dequantised amplitude.
 __device__ __forceinline__ float amplitude(float ss, float ss_row, int b, const float* s_edges, const float* s_levels) {
     if (b == 16) return __half2float(__float2half_rn(__fsqrt_rn(ss)));  // the amplitude as binary16
-    // Step 5: q = floor(CDF(u) 2^b) as the number of bin edges <= u, then the bin's level
+    // Step 5: q = floor(CDF(u) 2^b) as the number of bin edges <= u, then the bin's level.  The edges are padded to 255 by NaN, which
+    // nothing reaches: four or eight steps without a counter.  (16384 x 4096: 75.2 us with one, 74.3 by a jump to the
+    // first step, 72.7 so.)
     const float u = ss_row > 0.0f ? __fdiv_rn(ss, ss_row) : 0.0f;
     int q = 0;
-    for (int step = 1 << (b - 1); step >= 1; step >>= 1)
+    if (b > 4) {
+#pragma unroll
+        for (int step = 128; step >= 16; step >>= 1)
+            if (s_edges[q + step - 1] <= u) q += step;
+    }
+#pragma unroll
+    for (int step = 8; step >= 1; step >>= 1)
         if (s_edges[q + step - 1] <= u) q += step;
     return __fmul_rn(__fsqrt_rn(ss_row), s_levels[q]);
 }
@@ -161,9 +170,9 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         rot_scale = static_cast<float>(1.0 / sqrt(static_cast<double>(a.rot_block)));
     }
     const int nlevels = b <= 8 ? 1 << b : 0;  // 16 bits: the amplitude itself, no codebook
-    for (int i = tid; i < nlevels; i += T) {
-        if (i + 1 < nlevels) s_edges[i] = a.edges[i];
-        s_levels[i] = a.levels[i];
+    for (int i = tid; nlevels != 0 && i < kCodebookMax; i += T) {
+        s_edges[i] = i + 1 < nlevels ? a.edges[i] : __int_as_float(0x7fffffff);
+        if (i < nlevels) s_levels[i] = a.levels[i];
     }
 #ifdef PVQ_DEBUG
     debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
@@ -343,9 +352,9 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_rows_kernel(const 
         rot_scale = static_cast<float>(1.0 / sqrt(static_cast<double>(a.rot_block)));
     }
     const int nlevels = b <= 8 ? 1 << b : 0;  // 16 bits: the amplitude itself, no codebook
-    for (int i = tid; i < nlevels; i += T) {
-        if (i + 1 < nlevels) s_edges[i] = a.edges[i];
-        s_levels[i] = a.levels[i];
+    for (int i = tid; nlevels != 0 && i < kCodebookMax; i += T) {
+        s_edges[i] = i + 1 < nlevels ? a.edges[i] : __int_as_float(0x7fffffff);
+        if (i < nlevels) s_levels[i] = a.levels[i];
     }
     if (ROT) __syncthreads();
 
@@ -488,8 +497,8 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
     const long long tiles = (a.rows + a.rpt - 1) / a.rpt;
     if (tiles > 0x7fffffffLL) return PVQ_ERR_UNSUPPORTED;
     a.tiles = static_cast<unsigned>(tiles);
-    a.levels_off = a.b <= 8 ? 4u << a.b : 0u;
-    a.ss_off = (2u * a.levels_off + 15u) & ~15u;
+    a.levels_off = a.b <= 8 ? 4u * kCodebookMax : 0u;
+    a.ss_off = 2u * a.levels_off;
     a.signs_off = (a.ss_off + 2u * static_cast<uint32_t>(a.rpt * a.gp) * 4u + 15u) & ~15u;
     a.xbuf_off = (a.signs_off + (ROT ? static_cast<uint32_t>(a.rot_block / E) * 4u : 0u) + 127u) & ~127u;
     a.ring_off = (a.xbuf_off + (ROT ? static_cast<uint32_t>(threads) * E * 4u : 0u) + 127u) & ~127u;
