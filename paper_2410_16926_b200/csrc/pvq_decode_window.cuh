@@ -69,6 +69,17 @@ __device__ __forceinline__ uint4 win_record(uint32_t addr) {
     return v;
 }
 
+// Two neighbouring words of a block's head.
+template <int OFF>
+__device__ __forceinline__ uint2 win_load2(uint32_t addr) {
+    uint2 v;
+#ifdef PVQ_DEBUG
+    if (!debug_table_ok(addr + OFF, 8u)) return make_uint2(0u, 0u);
+#endif
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2+%3];" : "=r"(v.x), "=r"(v.y) : "r"(addr), "n"(OFF));
+    return v;
+}
+
 // The key of q: its KW leading words as an fp32, every step rounded towards zero.
 template <int PW, int KW>
 __device__ __forceinline__ uint32_t win_key(const mp<PW>& v) {
@@ -192,12 +203,12 @@ struct WinState {
     bool lost;      // some |y| has no byte, or q no room: the group is walked
 };
 
+// `sum`: all ones but for the top byte where the key bits are the same as the threshold's.
 template <int PW, int PLANE, int KW, int S>
-__device__ __forceinline__ void win_position(mp<PW>& v, uint32_t& acc, uint32_t& top, uint32_t stage) {
+__device__ __forceinline__ void win_position(mp<PW>& v, uint32_t& acc, uint32_t& sum, uint32_t stage) {
     const uint4 r = win_record(stage + 16u * S);
     const uint32_t key = min(win_key<PW, KW>(v) - r.x, r.y);
-    const uint32_t sum = key + win_load(stage + r.w + ((key >> r.z) << 2));
-    top = max(top, sum | 0xff000000u);
+    sum = key + win_load(stage + r.w + ((key >> r.z) << 2));
     acc = __byte_perm(acc, sum, 0x7321);
     mp<PW> e;
     win_entry<PW, PLANE, S * PW>(e, stage + kWinHead + ((sum >> 24) << 2));
@@ -207,26 +218,32 @@ __device__ __forceinline__ void win_position(mp<PW>& v, uint32_t& acc, uint32_t&
 template <int N, int PW, int PLANE, int KW, int W>
 __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, const BatchArgs& a, const WinArgs& t, int b, uint32_t y) {
     mp<PW> v;
+    static_assert(kWinDelta == kWinDlo4 + 4, "one read");
+    const uint2 head = win_load2<kWinDlo4>(stage);
     {
-        const uint32_t delta = win_load<kWinDelta>(stage);
+        const uint32_t delta = head.y;
         st.over = __funnelshift_l(st.a[0], st.over, delta);
 #pragma unroll
         for (int j = 0; j < PW; ++j) v.w[PW - 1 - j] = __funnelshift_l(st.a[j + 1], st.a[j], delta);
         st.a[PW] = 0u;
     }
-    uint32_t acc = 0u, top = 0u;
-    win_position<PW, PLANE, KW, 0>(v, acc, top, stage);
-    win_position<PW, PLANE, KW, 1>(v, acc, top, stage);
-    win_position<PW, PLANE, KW, 2>(v, acc, top, stage);
-    win_position<PW, PLANE, KW, 3>(v, acc, top, stage);
+    uint32_t acc = 0u, sum;
+    win_position<PW, PLANE, KW, 0>(v, acc, sum, stage);
+    win_position<PW, PLANE, KW, 1>(v, acc, sum, stage);
+    win_position<PW, PLANE, KW, 2>(v, acc, sum, stage);
+    win_position<PW, PLANE, KW, 3>(v, acc, sum, stage);
     // |y|: pulses left before the position minus those left after it, a byte each: one sum, whose bytes do not
     // touch each other while all of them are 0..127 (else some bit 7 shows, unless the position before was out of the
     // window too, and then h shows it); y > 0 where the index is odd
     const uint32_t after = (acc >> 1) & 0x7f7f7f7fu;
-    const uint32_t mag = (after << 8) + win_load<kWinDlo4>(stage) - after + static_cast<uint32_t>(st.h);
+    const uint32_t mag = (after << 8) + head.x - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;
     uint32_t y4 = (mag ^ ~pos) + 0x80808081u + pos;  // 128 + |y|; else 255 - |y| + 128 - 255: no byte of the sum leaves 1 .. 255
-    if (__any_sync(kFull, top == 0xffffffffu || (((mag | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
+    // Key bits the same as a threshold's, and q above it all the same: the index is one short, and the next position's is one
+    // that a valid q cannot have, y = 0 with an odd index, or pulses that grow (see pvq_search.cuh); looked for at the last
+    // position, whose next is in another block.
+    const uint32_t odd_zero = ~((mag | 0x80808080u) - odd);
+    if (__any_sync(kFull, (sum | 0xff000000u) == 0xffffffffu || (((mag | odd_zero | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
         WinExact<PW> x;
         x.v = v;
         x.over = st.over, x.h = st.h, x.ssy = st.ssy, x.lost = st.lost;

@@ -7,7 +7,7 @@
 // points in shared memory, a signed byte a value; then the amplitudes, once the rows' energies are complete;
 // then every thread sums its group's index from the windowed tables (pvq_window.cuh), one entry of E a position, read
 // word plane by word plane from the ring that a feeding warp keeps filled, the last block of rows first.  With q the
-// number that the decoder searches, the code is N(N,K) - q: the sum of all E is 1 - q.  Same matrix: 56 us; the two phases
+// number that the decoder searches, the code is N(N,K) - q: the sum of all E is 1 - q.  Same matrix: 54 us; the two phases
 // do not overlap (61% of the issue slots used).
 #include <algorithm>
 #include <cstring>
@@ -56,6 +56,17 @@ __device__ __forceinline__ void ew_entry(mp<PW>& e, uint32_t addr) {
     }
 }
 
+// The last four words of a block's head: x (not used here), y delta, z klo, w khi - klo.
+__device__ __forceinline__ uint4 ew_head(uint32_t stage) {
+    static_assert(kWinDlo4 % 16 == 0 && kWinDelta == kWinDlo4 + 4 && kWinKlo4 == kWinDlo4 + 8 && kWinWidth4 == kWinDlo4 + 12, "one read");
+    uint4 v;
+#ifdef PVQ_DEBUG
+    if (!debug_table_ok(stage + kWinDlo4, 16u)) return make_uint4(0u, 0u, 0u, 0u);
+#endif
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4+%5];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(stage), "n"(kWinDlo4));
+    return v;
+}
+
 // a[0] is the leading word of -q (the words above it are all ones, those below the block's are zero).
 template <int W>
 struct EwState {
@@ -71,12 +82,13 @@ __device__ __forceinline__ void ew_block4(EwState<W>& st, uint32_t stage, uint32
     v.w[PW - 1] = __funnelshift_r(st.a[0], 0xffffffffu, st.delta);
 #pragma unroll
     for (int j = 1; j < PW; ++j) v.w[PW - 1 - j] = __funnelshift_r(st.a[j], st.a[j - 1], st.delta);
-    st.delta = ew_load(stage + kWinDelta);
+    const uint4 head = ew_head(stage);
+    st.delta = head.y;
     // pulses behind each of the four positions: running sums, first position in the highest byte
     const uint32_t mag = point & 0x7f7f7f7fu;
     const uint32_t positive = (((mag + 0x7f7f7f7fu) & ~point) >> 7) & kOne4;
-    const uint32_t local = __byte_perm(mag, st.behind, 0x2104) * kOne4 - ew_load(stage + kWinKlo4);
-    st.flag |= local | (ew_load(stage + kWinWidth4) - local);
+    const uint32_t local = __byte_perm(mag, st.behind, 0x2104) * kOne4 - head.z;
+    st.flag |= local | (head.w - local);
     st.behind = __dp4a(mag, kOne4, st.behind);
     const uint32_t m4 = local + local + positive, rows = stage + kWinHead;
     mp<PW> e;
@@ -209,6 +221,9 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
         while (mi + 1 < a.count && tile >= a.m[mi + 1].tile_begin) ++mi;
         const MatrixArgs& m = a.m[mi];
         const int G = m.G, gp = 1 << (32 - __clz(G - 1)), rpt = m.rows_per_tile;
+        // row of a group: i / G as a product, exact as i and G are below 1024 (i * (per_row * G - 2^22) < 2^22)
+        const unsigned per_row = (1u << 22) / static_cast<unsigned>(G) + 1u;
+        auto row_of = [&](int i) { return static_cast<int>((static_cast<unsigned>(i) * per_row) >> 22); };
         const long long row0 = static_cast<long long>(tile - m.tile_begin) * rpt;
         const int nr = static_cast<int>(min(static_cast<long long>(rpt), m.rows - row0)), groups = nr * G;
         const int idx_words = m.sstride >> 2;
@@ -223,7 +238,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
             for (int v = 0; v < P; ++v) {
                 const int q = v * 32 + lane, l = q / P, gi = g0 + l / L;  // 16-byte piece; the lane and group it belongs to
                 if (gi < groups) {
-                    const int r = gi / G;
+                    const int r = row_of(gi);
                     const size_t off = static_cast<size_t>(row0 + r) * m.ld + static_cast<size_t>(gi - r * G) * N + (l % L) * E;
                     copy16_async(shared_addr(in) + l * RUN + (q & (P - 1)) * 16, static_cast<const uint8_t*>(m.x) + off * (BF16 ? 2 : 4) + (q & (P - 1)) * 16);
                 }
@@ -256,7 +271,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
             }
             const int gi = g0 + lane / L, sub = lane % L;
             const bool ok = gi < groups, leader = ok && sub == 0;
-            const int r = gi / G, gr = gi - r * G;
+            const int r = row_of(gi), gr = gi - r * G;
             if (leader && PVQ_DEBUG_INDEX(r * gp + gr, (g.amp_off - g.ss_off) / 4, PVQ_DEBUG_SHARED_INDEX)) s_ss[r * gp + gr] = ss;
             if (ls_mode) {
                 const float ls = least_squares_amplitude<E, L, BF16, false>(pt, mine);
@@ -301,7 +316,7 @@ __global__ void __launch_bounds__((kEwWarps + 1) * 32, 1)
         ew_barrier(T);
 
         // the amplitudes
-        const int gi = threadIdx.x, rl = gi / G, gr = gi - rl * G;
+        const int gi = threadIdx.x, rl = row_of(gi), gr = gi - rl * G;
         const bool active = gi < groups;
         const long long row = row0 + rl;
         const float ss_row = row_energy(s_ss, gp, rl, rpt, lane);
