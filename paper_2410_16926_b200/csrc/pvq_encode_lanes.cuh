@@ -94,13 +94,17 @@ __device__ __forceinline__ T lane_entry(const uint8_t* p) {
     return *reinterpret_cast<const T*>(p);
 }
 
-// Stages the tables: entry (i, m) from the blob's telescoped word planes.  A barrier has to follow.
+// The block's threads meet once, when the tables are staged: those that go on wait, the others only say that they are done.
+__device__ __forceinline__ void tables_done() { asm volatile("bar.arrive 0, %0;" ::"r"(blockDim.x) : "memory"); }
+__device__ __forceinline__ void tables_wait() { asm volatile("bar.sync 0, %0;" ::"r"(blockDim.x) : "memory"); }
+
+// Stages the tables, with `threads` threads of which this is the `first`-th: entry (i, m) from the blob's telescoped word planes.
 template <int N, int W, int RE>
-__device__ __forceinline__ void stage_lane_table(uint8_t* tab, const uint32_t* blob, const TableLayout& L, int K, int wide_blocks) {
+__device__ __forceinline__ void stage_lane_table(uint8_t* tab, const uint32_t* blob, const TableLayout& L, int K, int wide_blocks, int first, int threads) {
     constexpr int TW = W <= 2 ? W : 4;
     // entry by entry, several loads in flight: a small launch consists mostly of this
 #pragma unroll 4
-    for (int e = threadIdx.x; e < N * RE; e += blockDim.x) {
+    for (int e = first; e < N * RE; e += threads) {
         const int i = e / RE, m = e - i * RE;
         if (m >= 2 * K + 2) continue;
         const uint32_t* src = blob + ((m & 1) ? L.cenc_off[1] : L.cenc_off[0]) / 4 + static_cast<size_t>(i) * TW * L.crow + (m >> 1);
@@ -388,8 +392,8 @@ __device__ __forceinline__ void flush_index_words(const MatrixArgs& m, unsigned 
 }
 
 // RE: entries per row of the staged table (codes of exactly W words); 0: the tables stay in global memory,
-// codes of up to W words.
-template <int E, int L, int W, int RE, bool BF16, bool LS>
+// codes of up to W words.  LATE: for small launches, whose staging of the tables it hides.
+template <int E, int L, int W, int RE, bool BF16, bool LS, bool LATE>
 __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const __grid_constant__ BatchArgs a,
                                                                            const __grid_constant__ LaneGeom g) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -430,15 +434,27 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
         debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
 #endif
     } else {
-        stage_lane_table<N, W, GLOBAL ? 64 : RE>(smem, a.table, TL, K, g.wide_blocks);
+        // LATE: most threads have no values.  They stage the tables while the others quantise, which wait half way through
+        // their first chunk.
+        const int busy = g.team * static_cast<int>(min(static_cast<unsigned>(g.teams), (a.total_tiles - blockIdx.x + gridDim.x - 1u) / gridDim.x));
+        const int skip = LATE ? busy : 0, first = static_cast<int>(threadIdx.x) - skip;
+        if (first >= 0) stage_lane_table<N, W, GLOBAL ? 64 : RE>(smem, a.table, TL, K, g.wide_blocks, first, static_cast<int>(blockDim.x) - skip);
 #pragma unroll
         for (int w = 0; w < W; ++w) start.w[GLOBAL ? 0 : w] = a.table[TL.start_off / 4 + w];
 #ifdef PVQ_DEBUG
         debug_begin(shared_addr(smem), shared_addr(smem) + lane_table_bytes<N, W, GLOBAL ? 64 : RE>(g.wide_blocks), 0u, 0u, 0u, a.debug_status);
 #endif
     }
-    __syncthreads();  // the tables; from here on the teams go their own way
-    if (!works) return;
+    if constexpr (LATE) {
+        if (!works) {
+            tables_done();
+            return;
+        }
+    } else {
+        __syncthreads();  // the tables; from here on the teams go their own way
+        if (!works) return;
+    }
+    bool tables_here = !LATE;
     const int wide_blocks = g.wide_blocks;
 
     int in_buf = 0, buf = 0;
@@ -489,10 +505,17 @@ __global__ void __launch_bounds__(kLaneThreads<W>, 1) encode_lanes_kernel(const 
 #pragma unroll
                 for (int j = 0; j < E / 4; ++j) neg[j] = chunk_signs4<E, BF16>(raw, j);
                 group_norms<E, L, BF16>(raw, ax, l1, ss, g.minus_zero);
+                auto tables = [&]() {
+                    if (LATE && !tables_here) {
+                        __syncwarp();
+                        tables_wait();
+                        tables_here = true;
+                    }
+                };
                 if constexpr (BF16)
-                    quantize_group<E, L, GLOBAL>(ax, l1, K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, g.minus_zero);
+                    quantize_group<E, L, GLOBAL>(ax, l1, K, FetchShared{reinterpret_cast<const unsigned short*>(mine)}, pt, g.minus_zero, 0, tables);
                 else
-                    quantize_group<E, L, GLOBAL>(ax, l1, K, FetchSharedF32{reinterpret_cast<const float*>(mine)}, pt, g.minus_zero);
+                    quantize_group<E, L, GLOBAL>(ax, l1, K, FetchSharedF32{reinterpret_cast<const float*>(mine)}, pt, g.minus_zero, 0, tables);
             }
             const bool leader = row_ok && c < C && (c & (L - 1)) == 0;
             const int slot = cur.rl * gp + c / L;
@@ -675,11 +698,18 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
     const size_t smem = g.team_off + static_cast<size_t>(g.teams) * g.team_bytes;
     // at least sixteen warps to share the staging of the tables
     const int threads = std::max(g.team * g.teams, RE == 0 ? 64 : 512);
-    auto kern = encode_lanes_kernel<E, L, W, RE, BF16, LS>;
+    const unsigned blocks = (tiles + g.teams - 1) / g.teams;
+    // (512 x 512 fp32 7.3 -> 6.5 us.  In large launches the wait further on costs: 4096 x 4096 at N = 32 29.8 -> 30.1 us, fp32
+    // 38.7 -> 39.4.)
+    auto kern = encode_lanes_kernel<E, L, W, RE, BF16, LS, false>;
+    if constexpr (RE != 0 && !LS) {
+        const unsigned share = std::min<unsigned>(blocks, static_cast<unsigned>(di.sms));  // blocks, one an SM
+        const int busy = g.team * static_cast<int>(std::min<unsigned>(static_cast<unsigned>(g.teams), (tiles + share - 1) / share));
+        if (threads - busy >= 256) kern = encode_lanes_kernel<E, L, W, RE, BF16, LS, true>;
+    }
     int per_sm = 0;
     if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
-    const unsigned blocks = (tiles + g.teams - 1) / g.teams;
     const unsigned grid = std::min<unsigned>(blocks, static_cast<unsigned>(di.sms * per_sm));
     // Tables in global memory: early only where the launch is small and its start counts (4096 groups at N = 16, 128 bits: 12.1 us
     // early, 14.3 in order; 32768 groups at N = 32, 200 bits, not yet a block an SM: 31.6 and 22.6).

@@ -328,10 +328,15 @@ __device__ __forceinline__ void take_or_keep(int c, uint32_t have, uint32_t plan
     cand = rest;
 }
 
-// ax: |x_i| of the lane's values; l1: of the whole group.
-template <int E, int L, bool WIDE, class Fetch>
+struct NoHook {
+    __device__ __forceinline__ void operator()() const {}
+};
+
+// ax: |x_i| of the lane's values; l1: of the whole group.  `hook` is called by the warp half way, where few registers
+// are in use.
+template <int E, int L, bool WIDE, class Fetch, class Hook = NoHook>
 __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, int K, const Fetch& fetch,
-                                               LanePoint<E, WIDE>& pt, float minus_zero, int rotation = 0) {
+                                               LanePoint<E, WIDE>& pt, float minus_zero, int rotation = 0, Hook&& hook = Hook()) {
     constexpr int N = E * L, J = E / 4, H = E / 2;
     const float gsc = __fdiv_rn(static_cast<float>(K), l1);
     // no direction: l1 zero or not finite, or a scale that overflows
@@ -379,6 +384,7 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
     has_dir = has_dir && d >= 0 && d <= N;
     if (!has_dir) d = 0;
 
+    hook();
     bit_planes<J>(x);
     uint32_t sel = 0u, cand = ((1u << J) - 1u) * kOne4;  // chosen; undecided: the same in all bits so far
     int need = d;                                        // still to be chosen among the undecided ones
