@@ -154,17 +154,7 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
         uint32_t ssy[GP];
 #pragma unroll
         for (int j = 0; j < GP; ++j) ssy[j] = 0u;
-        uint32_t odd_one[GP];
-#pragma unroll
-        for (int j = 0; j < GP; ++j) odd_one[j] = 0u;
-        search_codes<N, W, GP, PLANE, LONG>(q, K, recs, cnt, quad_bytes != 0u ? sbase + staged : 0u, shared_addr(yslots), ychain, ssy, odd_one);
-#pragma unroll
-        for (int j = 0; j < GP; ++j)
-            if (active_valid[j] && (odd_one[j] & 0x80808080u) != 0u) {
-                const MatrixArgs& m = a.m[mj[j]];
-                const uint32_t* code = m.codes + (static_cast<size_t>(row[j]) * m.G + g[j]) * W;
-                ssy[j] = search_exact<N, W, PLANE, LONG>(code, bw, K, recs, t_rows, cnt[4], cnt[3], cnt[2], shared_addr(yslots) + j * ychain);
-            }
+        search_codes<N, W, GP, PLANE, LONG>(q, K, recs, t_rows, cnt, quad_bytes != 0u ? sbase + staged : 0u, shared_addr(yslots), ychain, ssy);
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
@@ -254,10 +244,10 @@ int launch_search_g(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
         tiles += static_cast<unsigned>((ngroups + 31) / 32);
     }
     a.total_tiles = tiles;
-    // More than a round earns the rewriting of the buckets and the staging of the table of the last four positions, some 2 us.
-    // (Without and with, us: decoder layer, 23 rounds, 271 and 240; 4096 x 4096 at N = 16, 48 bits, 3.5 rounds, 24.6 and
-    // 22.1; at N = 32, 64 bits, 1.7 rounds, 21.5 and 20.3, 96 bits 23.5 and 23.6; one round only loses.)
-    const bool is_long = tiles > 2u * static_cast<unsigned>(di.sms) * (kSearchThreads / 32);
+    // More than two rounds earn the rewriting of the buckets and the staging of the table of the last four positions, some 2 us.
+    // (Without and with, us: decoder layer, 23 rounds, 271 and 257; 4096 x 4096 at N = 16, 48 bits, 3.5 rounds, 24.6 and
+    // 23.2; at N = 32, 96 bits, 1.7 rounds, 23.5 and 24.9.)
+    const bool is_long = tiles > 4u * static_cast<unsigned>(di.sms) * (kSearchThreads / 32);
     switch (S.plane) {  // entries per word plane of the section's rows
         case 64: return is_long ? launch_search_t<N, W, 2, 64, true>(a, S, stream) : launch_search_t<N, W, 2, 64, false>(a, S, stream);
         case 128: return is_long ? launch_search_t<N, W, 2, 128, true>(a, S, stream) : launch_search_t<N, W, 2, 128, false>(a, S, stream);

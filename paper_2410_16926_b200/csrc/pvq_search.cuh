@@ -87,9 +87,8 @@ __device__ __forceinline__ void store_y4(uint32_t addr, uint32_t val) {
 // a time: pulses left after a position m >> 1, before it those of the position before (k for the
 // first); their difference is |y|, and y > 0 where m is odd.  No byte borrows from or
 // carries into its neighbour: the pulses left never grow, and |y| <= 127.
-// The four y_i + 128 go to the word at y, their squares to ssy.  Returned: bit 7 of a byte set where that does not hold,
-// the pulses left having grown, or where nothing is positive (y = 0, m odd).
-__device__ __forceinline__ uint32_t search_coordinates(uint32_t m4, uint32_t& k, uint32_t y, uint32_t& ssy) {
+// The four y_i + 128 go to the word at y, their squares to ssy.
+__device__ __forceinline__ void search_coordinates(uint32_t m4, uint32_t& k, uint32_t y, uint32_t& ssy) {
     const uint32_t after = (m4 >> 1) & 0x7f7f7f7fu;
     const uint32_t before = (after << 8) | k;
     const uint32_t mag = before - after;
@@ -98,23 +97,19 @@ __device__ __forceinline__ uint32_t search_coordinates(uint32_t m4, uint32_t& k,
     const uint32_t pos = (odd << 8) - odd;  // 0xff in the bytes with y > 0
     store_y4(y, (mag ^ ~pos) + 0x80808081u + pos);  // 128 + |y|; else 255 - |y| + 128 - 255: no byte of the sum leaves 1 .. 255
     k = after >> 24;
-    return mag | ~((mag | 0x80808080u) - odd);
 }
 
 // How a position is searched: the key of q selects a bucket; its entry holds the low key bits of the threshold T[m0] in it, and m0.
-// q's own low key bits being larger means q > T[m0] and the index m0 + 1, else it is m0 (a bucket without a threshold
-// holds all ones there).  A launch of some rounds can afford to rewrite the staged buckets first (LONG): an entry is then what,
-// added to the key, leaves the index in the top byte, the comparison being the carry into it.
-//
-// Key bits that are the same as the threshold's are not looked for.  If they are, and q is above the threshold all the same, the
-// index is one short and q' = T_(n-1)[2k'] + d, d = q - T_n[m], is too large for the k' pulses left.  The next row then has an
-// index of 2k' + 1 or more for it, which no q of a valid code has (2k' + 1: a positive coordinate of no pulse; more: pulses left
-// that grow), and search_coordinates shows it.  (There is a next row: row 0's thresholds are their keys.)  Whatever follows is in
-// bounds: q stays above zero, as every step leaves 1 <= q <= N(n,k') for a q up to the row's last threshold, and a key above
-// the last bucket is cut off at it.  Such a group is searched once more, in full (search_exact).  (A vote of the warp a position,
-// and the full comparison right there: decoder layer 271 us, this way and LONG 240; 512 x 512, one round, 6.7 and 6.3 us.)
+// q's own low key bits being larger means q > T[m0] and the index m0 + 1, smaller that it is m0 (a bucket without a threshold
+// holds all ones there).  Equal bits leave it open, unless the threshold is its key (below 2^24): then the threads of the warp
+// whose bits were equal compare q with T[m0] in full.  A launch of some rounds can afford to rewrite the staged buckets first
+// (LONG): an entry is then what, added to twice the key, leaves the index in the top byte, the comparison being the carry into
+// it, and all ones below it where the comparison is open (an even number where the threshold is its key).  Four instructions
+// less a position; with them and the last four positions looked up, decoder layer 271 -> 257 us.
 // Tried and not kept: bucket and key bits from one wide product, and the comparison taken as the borrow of a
-// subtraction (decoder layer 271 -> 288 and 284 us: they tie up the pipes that are short).
+// subtraction (decoder layer 271 -> 288 and 284 us: they tie up the pipes that are short); equal bits not looked for but found out
+// from the position that follows, and such a group searched again (237 us, but heavy-tailed data have many: N = 32, 96
+// bits, Student's t with 3 degrees of freedom, 4096 x 4096 25 -> 70 us); E read before the vote (257 -> 259 us).
 
 // The last four positions at once: the indices of q in row 3, of the q that follows in row 2, and so on depend on q
 // alone (no N, K or pulses left in them), and q is small there: at most N(4,k) with k pulses left, some K / 8 of them at
@@ -149,58 +144,42 @@ constexpr QuadTable kQuadsHost = make_quads();
 __device__ __align__(128) const QuadTable kQuads = kQuadsHost;
 
 // Makes the accepted section ready for the search; all threads, a barrier follows.  `t_off`: where its buckets end.  Records
-// afterwards: the last key of the row's buckets, the shared addresses of its row of E and of its buckets, the shift.
-// The thresholds T are not staged (search_exact reads some, from global memory): the
+// afterwards: 32 - shift, the shared addresses of its row of E and of its buckets, the shift.
+// The thresholds T are not staged (open comparisons read some, from global memory): the
 // increments E sit where T is in the blob, `t_before_e` bytes lower.
 template <int N, bool LONG>
 __device__ __forceinline__ void search_section_ready(uint8_t* sec, uint32_t t_off, uint32_t t_before_e) {
     uint32_t* recs = reinterpret_cast<uint32_t*>(sec + kSearchHeader);
-    auto first_bucket = [&](int n) { return n < N ? recs[4 * n + 2] + ((kSearchKeyOfOne >> recs[4 * n + 3]) << 2) : t_off; };
-    uint32_t last_key = 0u;
-    if (threadIdx.x < N) {
-        const int n = threadIdx.x;
-        const uint32_t sh = recs[4 * n + 3], buckets = (first_bucket(n + 1) - first_bucket(n)) >> 2;
-        last_key = (((kSearchKeyOfOne >> sh) + buckets) << sh) - 1u;
-    }
     if constexpr (LONG) {
+        auto first_bucket = [&](int n) { return n < N ? recs[4 * n + 2] + ((kSearchKeyOfOne >> recs[4 * n + 3]) << 2) : t_off; };
         for (int n = threadIdx.x >> 5; n < N; n += blockDim.x >> 5) {
             const uint32_t sh = recs[4 * n + 3], from = first_bucket(n), end = first_bucket(n + 1);
             uint32_t* b = reinterpret_cast<uint32_t*>(sec + from);
             for (uint32_t i = threadIdx.x & 31; from + 4u * i < end; i += 32u) {
                 const uint32_t e = b[i];
-                // (all ones: the last key of the bucket, which nothing in it passes)
-                b[i] = (e << 24) + 0xffffffu - ((((kSearchKeyOfOne >> sh) + i) << sh) + (e >> (32u - sh)));
+                // (no threshold: the last key of the bucket, which nothing in it passes, and bit 8, as for one that is its key)
+                b[i] = (e << 24) + 0xffffffu - ((e >> 8) & 1u) - 2u * ((((kSearchKeyOfOne >> sh) + i) << sh) + (e >> (32u - sh)));
             }
         }
+        __syncthreads();
     }
-    __syncthreads();
     if (threadIdx.x < N) {
         uint32_t* rec = recs + 4 * threadIdx.x;
         const uint32_t base = shared_addr(sec);
-        rec[0] = last_key;
         rec[1] += base - t_before_e;
         rec[2] += base;
     }
-}
-
-// The index that a bucket's entry leads to; top: it sits in the top byte of the result, else in the lowest.
-template <bool LONG>
-__device__ __forceinline__ uint32_t search_index(uint32_t key, uint32_t entry, uint32_t shift) {
-    if constexpr (LONG)
-        return key + entry;
-    else  // (funnel: key << (32 - shift))
-        return (entry & 0xffu) + (__funnelshift_r(0u, key, shift) > entry ? 1u : 0u);
 }
 
 // Four positions of GP codes (GP independent chains of dependent table reads, so that one
 // thread keeps several reads in flight), in PW-word arithmetic on rows of PW word planes.
 // `rec` is the shared address of the record of the first of the four rows (the rows of the
 // following positions have the records before it); a record is read once for all chains.
-// The four y_i + 128 of chain j go to the word at y + j * ychain, their squares to ssy[j]; odd_one[j]: bit 7 of a
-// byte set if the group has to be searched in full.
+// `t_rows` plus the shared address of a row of E is the global address of the same row of T.
+// The four y_i + 128 of chain j go to the word at y + j * ychain, their squares to ssy[j].
 template <int W, int PW, int GP, int PLANE, bool LONG>
-__device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, uint32_t y, uint32_t ychain,
-                                              uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
+__device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP], uint32_t rec, const uint8_t* t_rows,
+                                              uint32_t y, uint32_t ychain, uint32_t (&ssy)[GP]) {
     uint32_t acc[GP];  // the four threshold indices m, a byte each, first position lowest
     mp<PW> v[GP];      // the low PW words of q: the rest is zero by now
 #pragma unroll
@@ -211,12 +190,38 @@ __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP],
     }
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-        const uint4 r = load_record(rec - static_cast<uint32_t>(s) * 16u);  // last key, E row, buckets, shift
-        uint32_t m[GP];
+        const uint4 r = load_record(rec - static_cast<uint32_t>(s) * 16u);  // 32 - shift, E row, buckets, shift
+        uint32_t key[GP], m[GP];  // m: the index; LONG: in the top byte
+        bool open[GP], any = false;
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
-            const uint32_t key = min(search_key<PW>(v[j].w), r.x);
-            m[j] = search_index<LONG>(key, load_bucket(r.z + ((key >> r.w) << 2)), r.w);
+            key[j] = search_key<PW>(v[j].w);
+            m[j] = load_bucket(r.z + ((key[j] >> r.w) << 2));
+        }
+#pragma unroll
+        for (int j = 0; j < GP; ++j) {
+            if constexpr (LONG) {
+                m[j] += key[j] + key[j];
+                open[j] = (~m[j] & 0xffffffu) == 0u;
+            } else {
+                const uint32_t low = key[j] << r.x;  // the key bits below the shift, left-aligned like the entry's
+                open[j] = m[j] - low < 256u;
+                m[j] = (m[j] & 0xffu) + (low > m[j] ? 1u : 0u);
+            }
+            any = any || open[j];
+        }
+        if (__any_sync(kFull, any)) {
+#pragma unroll
+            for (int j = 0; j < GP; ++j) {
+                if (open[j]) {
+                    // the row of T in global memory lies where the row of E lies in shared memory
+                    const uint32_t* tp = reinterpret_cast<const uint32_t*>(t_rows + r.y + (LONG ? m[j] >> 24 : m[j]) * 4u);
+                    mp<PW> t, d;
+#pragma unroll
+                    for (int w = 0; w < PW; ++w) t.w[w] = tp[w * PLANE];
+                    if (mp_sub_borrow<PW>(d, t, v[j])) m[j] += LONG ? 1u << 24 : 1u;
+                }
+            }
         }
 #pragma unroll
         for (int j = 0; j < GP; ++j) {
@@ -227,77 +232,33 @@ __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP],
     }
 #pragma unroll
     for (int j = 0; j < GP; ++j) {
-        odd_one[j] |= search_coordinates(acc[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
+        search_coordinates(acc[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
 #pragma unroll
         for (int w = 0; w < PW; ++w) q[j].w[w] = v[j].w[w];
     }
-}
-
-// One group, position by position, every comparison in full.  Returns the sum of the squares.
-template <int N, int W, int PLANE, bool LONG>
-__device__ __noinline__ uint32_t search_exact(const uint32_t* code, const uint32_t* bound, int K, uint32_t recs, const uint8_t* t_rows,
-                                              int rows4, int rows3, int rows2, uint32_t y) {
-    uint32_t q[W];
-    long long c = 0;
-    for (int w = 0; w < W; ++w) {
-        c += static_cast<long long>(bound[w]) - code[w];
-        q[w] = static_cast<uint32_t>(c);
-        c >>= 32;
-    }
-    uint32_t ssy = 0u, y4 = 0u;
-    int k = K;
-#pragma unroll 1
-    for (int i = 0; i < N; ++i) {
-        const int words = min(W, i < rows4 ? 4 : (i < rows4 + rows3 ? 3 : (i < rows4 + rows3 + rows2 ? 2 : 1)));
-        const uint4 r = load_record(recs + static_cast<uint32_t>(N - 1 - i) * 16u);
-        const uint32_t key = min(search_key(q, W), r.x);
-        uint32_t m = search_index<LONG>(key, load_bucket(r.z + ((key >> r.w) << 2)), r.w);
-        if (LONG) m >>= 24;
-        // (m is right or, where the key bits are the same, one short; the row of T in global memory lies where that of E lies in
-        // shared memory)
-        const uint32_t* t = reinterpret_cast<const uint32_t*>(t_rows + r.y + m * 4u);
-        c = 0;
-        for (int w = 0; w < words; ++w) c = (c + static_cast<long long>(t[w * PLANE]) - q[w]) >> 32;
-        if (c < 0) ++m;
-        unsigned long long carry = 0;
-        for (int w = 0; w < words; ++w) {
-            carry += static_cast<unsigned long long>(q[w]) + load_bucket(r.y + (m + static_cast<uint32_t>(w) * PLANE) * 4u);
-            q[w] = static_cast<uint32_t>(carry);
-            carry >>= 32;
-        }
-        const int left = static_cast<int>(m >> 1), mag = k - left;
-        ssy += static_cast<uint32_t>(mag * mag);
-        y4 |= (static_cast<uint32_t>((m & 1u) ? 128 + mag : 128 - mag) & 0xffu) << (8 * (i & 3));
-        if ((i & 3) == 3) {
-            store_y4(y + static_cast<uint32_t>(i & ~3), y4);
-            y4 = 0u;
-        }
-        k = left;
-    }
-    return ssy;
 }
 
 // The points of GP codes: q = N(N,K) - code on entry.  `recs` is the shared address of the
 // row records (absolute shared addresses by now), cnt[w] the number of rows done in w words; quads: shared address of kQuads,
 // or 0: without.
 template <int N, int W, int GP, int PLANE, bool LONG>
-__device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t recs, const int (&cnt)[5], uint32_t quads, uint32_t y,
-                                                  uint32_t ychain, uint32_t (&ssy)[GP], uint32_t (&odd_one)[GP]) {
+__device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t recs, const uint8_t* t_rows, const int (&cnt)[5], uint32_t quads,
+                                             uint32_t y, uint32_t ychain, uint32_t (&ssy)[GP]) {
     uint32_t k[GP];
 #pragma unroll
     for (int j = 0; j < GP; ++j) k[j] = static_cast<uint32_t>(K);
     uint32_t rec = recs + static_cast<uint32_t>(N - 1) * 16u;
     if constexpr (W >= 4) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4<W, 4, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
+        for (int b = 0; b < cnt[4]; b += 4, rec -= 64u, y += 4u) search_block4<W, 4, GP, PLANE, LONG>(q, k, rec, t_rows, y, ychain, ssy);
     }
     if constexpr (W >= 3) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4<W, 3, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
+        for (int b = 0; b < cnt[3]; b += 4, rec -= 64u, y += 4u) search_block4<W, 3, GP, PLANE, LONG>(q, k, rec, t_rows, y, ychain, ssy);
     }
     if constexpr (W >= 2) {
 #pragma unroll 1
-        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4<W, 2, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
+        for (int b = 0; b < cnt[2]; b += 4, rec -= 64u, y += 4u) search_block4<W, 2, GP, PLANE, LONG>(q, k, rec, t_rows, y, ychain, ssy);
     }
 #pragma unroll 1
     for (int b = 0; b < cnt[1]; b += 4, rec -= 64u, y += 4u) {
@@ -310,11 +271,11 @@ __device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t rec
 #pragma unroll
                 for (int j = 0; j < GP; ++j) m4[j] = load_bucket(quads + ((q[j].w[0] - 1u) << 2));
 #pragma unroll
-                for (int j = 0; j < GP; ++j) odd_one[j] |= search_coordinates(m4[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
+                for (int j = 0; j < GP; ++j) search_coordinates(m4[j], k[j], y + static_cast<uint32_t>(j) * ychain, ssy[j]);
                 break;
             }
         }
-        search_block4<W, 1, GP, PLANE, LONG>(q, k, rec, y, ychain, ssy, odd_one);
+        search_block4<W, 1, GP, PLANE, LONG>(q, k, rec, t_rows, y, ychain, ssy);
     }
 }
 

@@ -1,6 +1,6 @@
-"""Decoding in launches of several rounds (codes of up to four words): the searching decoder then rewrites its buckets, looks
-up the last four positions at once, and finds out afterwards that key bits could not decide.  Codes that sit on thresholds
-among random ones, the first and the last code, against the oracle; and on the CPU that what is not decided does show."""
+"""Decoding in launches of several rounds (codes of up to four words): the searching decoder then rewrites its buckets and looks
+up the last four positions at once.  Codes that sit on thresholds among random ones, the first and the last code, against
+the oracle; and on the CPU that a rewritten entry leads to the index or says that the key bits leave it open."""
 import numpy as np
 import pytest
 import torch
@@ -34,43 +34,36 @@ def threshold_codes(rng, N, K, want):
 
 
 @pytest.mark.parametrize("N,K", SETTINGS)
-def test_undecided_key_bits_show(N, K):
+def test_rewritten_entries(N, K):
     count = pr.count_table(N, K)
     sec = bs.section(count, N, K, pvq.code_words(N, K), 0)
     rng = np.random.default_rng(N + K)
-    missed = 0
+    left_open = 0
     for c in threshold_codes(rng, N, K, 300):
-        q, k, shown, m_all = count[N][K] - c, K, False, []
+        q = count[N][K] - c
         for i in range(N):
             n = N - 1 - i
-            sh, tab = sec["shifts"][n], sec["tables"][n]
-            last = (((bs.KEY_OF_ONE >> sh) + len(tab)) << sh) - 1
-            assert q >= 1
-            key = min(bs.key_bits(q), last)
+            sh, tab, T = sec["shifts"][n], sec["tables"][n], sec["T"][n]
+            key = bs.key_bits(q)
             b = (key >> sh) - (bs.KEY_OF_ONE >> sh)
-            entry = ((tab[b] << 24) + 0xFFFFFF - ((((bs.KEY_OF_ONE >> sh) + b) << sh) + (tab[b] >> (32 - sh)))) & 0xFFFFFFFF
-            m = ((key + entry) & 0xFFFFFFFF) >> 24
-            assert m <= 2 * K + 1
-            shown = shown or m > 2 * k
-            m_all.append(m)
-            e = sec["E"][n][m] if m <= 2 * K else 0     # (the entry behind the last threshold is zero)
-            q = (q + e) % (1 << (32 * sec["words"][n]))
-            k = m >> 1
-        right = bs.decode_with(sec, count, c, N, K)
-        k, y = K, []
-        for m in m_all:
-            y.append(k - (m >> 1) if m & 1 else (m >> 1) - k)
-            k = m >> 1
-        assert shown or list(y) == list(right)
-        missed += list(y) != list(right)
+            e = tab[b]
+            entry = ((e << 24) + 0xFFFFFF - ((e >> 8) & 1) - 2 * ((((bs.KEY_OF_ONE >> sh) + b) << sh) + (e >> (32 - sh)))) & 0xFFFFFFFF
+            total = (2 * key + entry) & 0xFFFFFFFF
+            m = total >> 24
+            if total & 0xFFFFFF == 0xFFFFFF:
+                assert T[m] >= 1 << 24 and bs.key_bits(T[m]) == key
+                left_open += 1
+                m += 1 if T[m] < q else 0
+            assert T[m] >= q and (m == 0 or T[m - 1] < q)
+            q += (sec["T"][n - 1][2 * (m >> 1)] if n >= 1 else 0) - T[m]
     if pvq.code_words(N, K) > 1:
-        assert missed > 0           # these codes do reach the case
+        assert left_open > 0           # these codes do reach the case
 
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("N,K", SETTINGS)
 def test_long_launch(N, K):
-    G, rows, b = 64, 5001, 8        # 320064 groups: more than a round of 148 x 32 warps of two tiles
+    G, rows, b = 64, 9601, 8        # 614464 groups: more than two rounds of 148 x 32 warps of two tiles
     W = pvq.code_words(N, K)
     rng = np.random.default_rng(3 * N + K)
     total = pr.count_table(N, K)[N][K]
