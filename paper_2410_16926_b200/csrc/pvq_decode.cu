@@ -69,13 +69,13 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
         const unsigned gi = g0 + lane;
         const bool active = gi < ngroups;
         // row and group-in-row: one division per tile, the threads follow from the first group
-        unsigned row = g0 / G;
+        unsigned row = group_row(m, g0);
         unsigned g = g0 - row * G + lane;
         if (g >= G) {
             g -= G;
             row += 1;
             if (g >= G) {  // rows shorter than a tile
-                const unsigned q = g / G;
+                const unsigned q = group_row(m, g);
                 row += q;
                 g -= q * G;
             }

@@ -118,13 +118,13 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
             active[j] = tile < a.total_tiles && gi < ngroups;
             active_valid[j] = active[j];
             // row and group-in-row: one division per tile, the threads follow from the first group
-            row[j] = g0 / G;
+            row[j] = group_row(m, g0);
             g[j] = g0 - row[j] * G + lane;
             if (g[j] >= G) {
                 g[j] -= G;
                 row[j] += 1;
                 if (g[j] >= G) {  // rows shorter than a tile
-                    const unsigned qq = g[j] / G;
+                    const unsigned qq = group_row(m, g[j]);
                     row[j] += qq;
                     g[j] -= qq * G;
                 }

@@ -358,7 +358,7 @@ __device__ __forceinline__ void win_tile(const BatchArgs& a, const WinArgs& t, c
     const unsigned ngroups = static_cast<unsigned>(m.rows) * G;
     const unsigned gi = (tile - m.tile_begin) * 32u + lane;
     const bool active = any && gi < ngroups;
-    const unsigned row = gi / G, g = gi - row * G;
+    const unsigned row = group_row(m, gi), g = gi - row * G;
     mp<W> c;
     mp_zero(c);
     unsigned sbits = 0u;

@@ -392,6 +392,7 @@ int fill_matrix(const pvq_matrix_desc& d, int need, int dtype, const Common& c, 
     m->ld = d.ld;
     m->ld_out = d.ld_out;
     m->G = static_cast<int>(G);
+    set_group_division(m, m->G);
     m->sstride = static_cast<int>(pvq_scale_row_stride(G, c.scale_bits));
     m->rows_per_tile = 1;
     m->tile_begin = 0;

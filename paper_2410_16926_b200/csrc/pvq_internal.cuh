@@ -28,11 +28,24 @@ struct MatrixArgs {
     const float* levels;
     long long rows, cols, ld, ld_out;
     int G;                // groups per row
+    uint32_t g_mul;       // i / G for i < 2^31 is the upper word of i * g_mul, shifted right by g_shift (group_row)
+    int g_shift;
     int sstride;          // bytes per row of scale_idx
     int rows_per_tile;    // encode: rows one thread block covers
     int chunks;           // encode: pieces a row longer than the block is taken in (else 1)
     unsigned tile_begin;  // first tile of this matrix in the launch
 };
+
+// The row of a group of the matrix: a division is some 20 instructions, several times a tile.  With s = ceil(log2 G) and
+// g_mul = ceil(2^(31+s) / G), which is below 2^32, i * g_mul / 2^(31+s) exceeds i / G by less than 1 / G
+// (i * (g_mul * G - 2^(31+s)) < i * G <= i * 2^s < 2^(31+s) for i < 2^31), so the floors agree.
+inline void set_group_division(MatrixArgs* m, int G) {
+    int s = 1;  // (G >= 2)
+    while ((1ll << s) < G) ++s;
+    const unsigned long long one = 1ull << (31 + s);
+    m->g_mul = static_cast<uint32_t>((one + G - 1) / G);
+    m->g_shift = s - 1;
+}
 
 struct BatchArgs {
     MatrixArgs m[kMaxBatch];
@@ -286,6 +299,8 @@ int launch_roundtrip(const MatrixArgs& m, int dtype, int N, int K, int scale_bit
 // ---------------------------------------------------------------- device bits
 
 #ifdef __CUDACC__
+
+__device__ __forceinline__ unsigned group_row(const MatrixArgs& m, unsigned i) { return __umulhi(i, m.g_mul) >> m.g_shift; }
 
 // Launch of a hot-path kernel so that it may be set up while the kernel before it in the stream still runs
 // (programmatic dependent launch): between two small calls that hides most of the launch.  Such a
