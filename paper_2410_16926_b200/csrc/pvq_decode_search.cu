@@ -244,10 +244,12 @@ int launch_search_g(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
         tiles += static_cast<unsigned>((ngroups + 31) / 32);
     }
     a.total_tiles = tiles;
-    // More than two rounds earn the rewriting of the buckets and the staging of the table of the last four positions, some 2 us.
-    // (Without and with, us: decoder layer, 23 rounds, 271 and 257; 4096 x 4096 at N = 16, 48 bits, 3.5 rounds, 24.6 and
-    // 23.2; at N = 32, 96 bits, 1.7 rounds, 23.5 and 24.9.)
-    const bool is_long = tiles > 4u * static_cast<unsigned>(di.sms) * (kSearchThreads / 32);
+    // Rewriting the buckets costs some 0.2 us a thousand, and saves some 0.017 us a position and round; a few rounds for the
+    // staging of the table of the last four positions.  (Without and with, us: N = 32, 96 bits, 14800 buckets, decoder layer, 23
+    // rounds, 266.5 and 257.1, 8192 x 4096, 3.5 rounds, 43.4 and 44.5; as large, N = 32, 64 bits 39.8 and 38.6; N = 16, 64 bits, 25.9
+    // and 27.8, 48 bits 23.8 and 22.9; N = 8, 24 bits 14.7 and 13.4.)
+    const double rounds = tiles / (2.0 * di.sms * (kSearchThreads / 32)), buckets = (S.t_off - S.b_off) / 4.0;
+    const bool is_long = rounds > 3.0 && rounds * N * 80.0 > buckets;
     switch (S.plane) {  // entries per word plane of the section's rows
         case 64: return is_long ? launch_search_t<N, W, 2, 64, true>(a, S, stream) : launch_search_t<N, W, 2, 64, false>(a, S, stream);
         case 128: return is_long ? launch_search_t<N, W, 2, 128, true>(a, S, stream) : launch_search_t<N, W, 2, 128, false>(a, S, stream);

@@ -63,7 +63,11 @@ def test_rewritten_entries(N, K):
 @pytest.mark.gpu
 @pytest.mark.parametrize("N,K", SETTINGS)
 def test_long_launch(N, K):
-    G, rows, b = 64, 9601, 8        # 614464 groups: more than two rounds of 148 x 32 warps of two tiles
+    # enough rounds of two tiles of 32 groups for each of 32 warps an SM that the buckets are rewritten (launch_search_g)
+    sec = bs.section(pr.count_table(N, K), N, K, pvq.code_words(N, K), 0)
+    rounds = 1.02 * max(3.0, (sec["t_off"] - sec["b_off"]) / 4 / (80 * N))
+    G, b = 64, 8
+    rows = int(rounds * 2 * torch.cuda.get_device_properties(0).multi_processor_count * 32 * 32 / G) + 1
     W = pvq.code_words(N, K)
     rng = np.random.default_rng(3 * N + K)
     total = pr.count_table(N, K)[N][K]
