@@ -11,9 +11,9 @@
 // (N = 128, 384 bits: 760 KB; N = 256: 2.4 MB) they are streamed from L2 through a ring of buffers, block of rows
 // after block of rows, all warps of the thread block following the stream; an additional warp feeds it.
 //
-// Measured, with the walk (pvq_walk.cuh, pvq_big_impl.cuh) and now: 8192 x 28672, N = 64, 192 bits, 774 -> 368 us (79% of the
-// issue slots, 86% of the shared-memory wavefronts a cycle); 4096 x 4096, N = 128, 384 bits, 190 -> 48.5 us; N = 256, 768
-// bits, 601 -> 160 us.
+// Measured, with the walk (pvq_walk.cuh, pvq_big_impl.cuh) and now: 8192 x 28672, N = 64, 192 bits, 774 -> 356 us (77% of the
+// issue slots, 88% of the shared-memory wavefronts a cycle); 4096 x 4096, N = 128, 384 bits, 190 -> 47.6 us; N = 256, 768
+// bits, 601 -> 155 us.
 // (Group size 256 has a translation unit of its own: the functions that are not inlined take the registers of the
 // most generous kernel that calls them, and spill in the others.)
 #pragma once
@@ -239,9 +239,10 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
     const uint32_t mag = (after << 8) + head.x - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;
     uint32_t y4 = (mag ^ ~pos) + 0x80808081u + pos;  // 128 + |y|; else 255 - |y| + 128 - 255: no byte of the sum leaves 1 .. 255
-    // Key bits the same as a threshold's, and q above it all the same: the index is one short, and the next position's is one
-    // that a valid q cannot have, y = 0 with an odd index, or pulses that grow (see pvq_search.cuh); looked for at the last
-    // position, whose next is in another block.
+    // Key bits the same as a threshold's, and q above it all the same: the index is one short, and q' = T_(n-1)[2k'] + d with d =
+    // q - T_n[m] is too large for the k' pulses left.  The next position's index is then 2k' + 1 or more, which no q of a valid code
+    // has: y = 0 with an odd index, or pulses that grow.  At the last position, whose next is in another block, the bits are
+    // looked at.
     const uint32_t odd_zero = ~((mag | 0x80808080u) - odd);
     if (__any_sync(kFull, (sum | 0xff000000u) == 0xffffffffu || (((mag | odd_zero | static_cast<uint32_t>(st.h)) & 0x80808080u) | st.over) != 0u)) {
         WinExact<PW> x;

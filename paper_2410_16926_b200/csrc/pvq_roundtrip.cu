@@ -9,7 +9,7 @@
 //
 // A group lies on L = N / 32 neighbouring lanes (pvq_quant.cuh): the work and the bytes per lane are the
 // same from group size 32 up.  What bounds it: issue slots and the half-rate integer pipe (about
-// 1300 warp instructions per 1024 values), not the 4 bytes a value moves.
+// 840 warp instructions per 1024 values), not the 4 bytes a value moves.
 #include <algorithm>
 
 #include <cuda_fp16.h>
