@@ -89,6 +89,10 @@ __device__ __forceinline__ uint32_t win_key(const mp<PW>& v) {
     return __float_as_uint(x);
 }
 
+// Marks pulses left that an index outside the window might pass for: the local index 255 says 127 left, and with 127 or more
+// before the position that is no growth.  (A bit that the packed test looks at, above any number of pulses.)
+constexpr int kWinFar = 0x800000;
+
 // What the repeated search of a block works on: q (`over`: the word above the block's, for paths above the windows), the
 // local pulses left, and what it hands back.
 template <int PW>
@@ -128,7 +132,7 @@ __device__ __noinline__ void win_exact4(WinExact<PW>& st, uint32_t acc, uint32_t
     }
     const TableLayout L = table_layout(N, K, Wc);
     const int up = t.up[b];
-    int k = (b > 0 ? t.klo[4 * b - 1] : K) + st.h;  // pulses left before the position
+    int k = (b > 0 ? t.klo[4 * b - 1] : K) + (st.h >= kWinFar ? st.h - kWinFar : st.h);  // pulses left before the position
     st.y4 = 0u;
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
@@ -189,6 +193,7 @@ __device__ __noinline__ void win_exact4(WinExact<PW>& st, uint32_t acc, uint32_t
         k = left;
     }
     st.h = k - t.klo[4 * b + 3];
+    if (4 * b + 4 < N && k - t.klo[4 * b + 4] >= 127) st.h += kWinFar;  // (only a repeated search can leave so many)
     if (st.over >= 0x10000u) st.lost = true;  // the next block's shift (16 bits at most) would push bits out
     if (st.lost) st.over = 0u, st.h = 0;
 }
@@ -198,7 +203,7 @@ template <int W>
 struct WinState {
     uint32_t a[W + 1];
     uint32_t over;  // the word above a[0]: zero but for paths above the windows
-    int h;          // pulses left after the position before, minus its klo
+    int h;          // pulses left after the position before, minus its klo (kWinFar added where they are too many)
     uint32_t ssy;   // sum of y^2
     bool lost;      // some |y| has no byte, or q no room: the group is walked
 };
@@ -234,7 +239,7 @@ __device__ __forceinline__ void win_block4(WinState<W>& st, uint32_t stage, cons
     win_position<PW, PLANE, KW, 3>(v, acc, sum, stage);
     // |y|: pulses left before the position minus those left after it, a byte each: one sum, whose bytes do not
     // touch each other while all of them are 0..127 (else some bit 7 shows, unless the position before was out of the
-    // window too, and then h shows it); y > 0 where the index is odd
+    // window too: in the block, its own bit 7 shows; in the block before, h shows it); y > 0 where the index is odd
     const uint32_t after = (acc >> 1) & 0x7f7f7f7fu;
     const uint32_t mag = (after << 8) + head.x - after + static_cast<uint32_t>(st.h);
     const uint32_t odd = acc & 0x01010101u, pos = (odd << 8) - odd;

@@ -135,7 +135,7 @@ struct Builder {
             for (int s = 0; s < 4; ++s) {
                 const int i = 4 * b + s, n = N - 1 - i;
                 const int dlo = (i > 0 ? lo[i - 1] : K) - lo[i];
-                // |y| and the sums of the packed arithmetic stay below 256, and an out-of-window index always shows
+                // |y| and the sums of the packed arithmetic stay below 256, and an out-of-window index behind one inside shows
                 if (dlo < 0 || dlo > 127 || before(i) - lo[i] >= 127 || last_m[i] - 2 * lo[i] + 1 > plane) return false;
                 t.args.klo[i] = static_cast<int16_t>(lo[i]);
                 klo4 |= static_cast<uint32_t>(lo[i] & 255) << (8 * (3 - s));  // (read where K <= 255)

@@ -107,6 +107,42 @@ def test_codes_on_thresholds(N, bits):
     assert np.array_equal(bf16_bits(out), o_out)
 
 
+# position: value.  The pulses left at the beginning of a block of positions are 125 to 127 above the window's lower end, and the
+# positions that follow are outside the window.
+MANY_LEFT = [
+    (64, 140, {1: -5, 48: 50, 52: 85}), (64, 140, {22: 4, 48: 51, 50: 85}), (64, 140, {29: 1, 46: 1, 48: 53, 54: -52, 62: 33}),
+    (64, 165, {21: 23, 48: 36, 53: -46, 63: 60}), (64, 165, {2: -17, 9: 3, 17: -5, 48: 34, 51: 83, 63: 23}),
+    (64, 169, {16: -33, 48: 30, 51: 20, 53: -35, 60: 51}), (64, 169, {21: -5, 32: 25, 48: 33, 50: 30, 51: 70, 59: 6}),
+    (64, 180, {32: 39, 33: -4, 42: 39, 54: 7, 55: -16, 63: -75}), (64, 199, {7: -29, 22: 43, 61: -127}),
+    (128, 187, {32: 34, 84: -1, 103: 14, 104: -68, 119: -70}), (128, 187, {3: -1, 6: 5, 40: -5, 66: 27, 92: -59, 95: 28, 97: 11, 109: 51}),
+]
+
+
+@pytest.mark.parametrize("N,K", sorted({p[:2] for p in MANY_LEFT}))
+def test_many_pulses_left(N, K):
+    """Points whose path is as far above the windows as an index outside of them says.  Each beside 31 ordinary ones: a warp
+    looks closer for all its groups when it does for one."""
+    W = pvq.code_words(N, K)
+    rng = np.random.default_rng(N + K)
+    points = []
+    for value in (p[2] for p in MANY_LEFT if p[:2] == (N, K)):
+        y = np.zeros((32, N), dtype=np.int32)
+        y[:] = np.diff(np.arange(N + 1) * K // N)
+        y *= rng.choice([-1, 1], size=y.shape).astype(np.int32)
+        y[11] = 0
+        y[11, list(value)] = list(value.values())
+        points.append(y)
+    codes = np.stack([[po.enumerate_point(y, K, W) for y in tile] for tile in points])
+    rows = len(points)
+    sidx = rng.integers(0, 120, size=(rows, int(pvq.scale_row_stride(32, 16))), dtype=np.uint8)  # finite binary16 amplitudes
+    rnorm = np.ones(rows, dtype=np.float32)
+    o_out, _ = po.decode(codes, sidx, rnorm, N, K, 16, None)
+    out = pvq.decode(torch.from_numpy(codes.view(np.int32)).to(DEV), torch.from_numpy(sidx).to(DEV), torch.from_numpy(rnorm).to(DEV), N, K, 16,
+                     pvq.build_count_table(N, K), None)
+    torch.cuda.synchronize()
+    assert np.array_equal(bf16_bits(out), o_out)
+
+
 def test_several_matrices_and_streams():
     N, bits, b = 64, 192, 6
     K = pvq.max_pulses(N, bits)
