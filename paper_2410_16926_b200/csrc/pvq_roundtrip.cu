@@ -531,6 +531,16 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
     int per_sm = 0;
     if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
+    // A launch of a few blocks an SM asks for the shared memory that keeps more than its share of them off an SM: where calls follow
+    // one another, the blocks of one are placed while those of the one before still run, and several came to lie on one SM while
+    // others had none.  (us, without and with: 100 x 8192 rotated, B = 8192, 16.5 and 7.7, B = 4096 13.1 and 8.0; 600 x 2048, B = 2048,
+    // 15.9 and 8.7; not rotated, N = 128, 256 x 4096 8.2 and 4.7.  From some 2 M values on it makes no difference.)
+    const int share = static_cast<int>((tiles + di.sms - 1) / di.sms);
+    if (share < per_sm) {
+        const size_t sm_bytes = static_cast<size_t>(di.smem_max) + 1280;  // of an SM; 1024 are added for every block
+        smem = std::max(smem, (sm_bytes / (share + 1) - 1024 + 255) & ~size_t(127));
+        if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
+    }
     const unsigned grid = stays ? std::min(a.tiles, static_cast<unsigned>(di.sms * per_sm)) : a.tiles;
     return launch_hot(kern, grid, threads, smem, stream, a);
 }

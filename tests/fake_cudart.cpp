@@ -2,6 +2,7 @@
 // device memory is host memory that is kept track of, uploads from pageable memory are on their way until
 // something waits for them, calls can be made to fail or to wait.  Linked with the library's objects by
 // tests/test_host_fake_gpu.py.
+#include <algorithm>
 #include <condition_variable>
 #include <cstdint>
 #include <cstdlib>
@@ -26,6 +27,7 @@ struct Launch {
     std::string name;
     uint64_t tables[2];  // the first words of a windowed kernel's second argument: its tables' addresses
     unsigned grid, block;
+    size_t shared;
     bool early;  // may start before the kernel in front has ended
 };
 std::vector<Launch> launches;
@@ -49,11 +51,11 @@ void wait_while(bool& flag, std::unique_lock<std::mutex>& lock) {
     cv.wait(lock, [&] { return !flag; });
     --held;
 }
-cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, bool early) {
+cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, size_t shared, bool early) {
     std::unique_lock<std::mutex> lock(mu);
     if (kernels()[f].find("code_window") != std::string::npos) wait_while(hold_launch, lock);
     if (fail_launch != cudaSuccess) return ret(fail_launch);
-    Launch l{kernels()[f], {0, 0}, grid.x, block.x, early};
+    Launch l{kernels()[f], {0, 0}, grid.x, block.x, shared, early};
     if (l.name.find("code_window") != std::string::npos) std::memcpy(l.tables, args[1], sizeof l.tables);
     launches.push_back(l);
     return cudaSuccess;
@@ -67,6 +69,7 @@ const char* fake_launch_name(int i) { return launches[i].name.c_str(); }
 uint64_t fake_launch_table(int i, int which) { return launches[i].tables[which]; }
 unsigned fake_launch_grid(int i) { return launches[i].grid; }
 unsigned fake_launch_block(int i) { return launches[i].block; }
+unsigned fake_launch_shared(int i) { return static_cast<unsigned>(launches[i].shared); }
 int fake_launch_early(int i) { return launches[i].early; }
 int fake_live(uint64_t p) {  // does p lie in live memory?
     std::lock_guard<std::mutex> lock(mu);
@@ -127,12 +130,14 @@ cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* shared, 
     *static_cast<void**>(stream) = config.stream;
     return cudaSuccess;
 }
-cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3 block, void** args, size_t, cudaStream_t) { return launch(f, grid, block, args, false); }
+cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3 block, void** args, size_t shared, cudaStream_t) {
+    return launch(f, grid, block, args, shared, false);
+}
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
     bool early = false;
     for (unsigned i = 0; i < c->numAttrs; ++i)
         early = early || (c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization && c->attrs[i].val.programmaticStreamSerializationAllowed);
-    return launch(f, c->gridDim, c->blockDim, args, early);
+    return launch(f, c->gridDim, c->blockDim, args, c->dynamicSmemBytes, early);
 }
 cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
@@ -140,7 +145,10 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
     return cudaSuccess;
 }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
-cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t) { return *n = 1, cudaSuccess; }
+// (64 registers a thread)
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int threads, size_t shared) {
+    return *n = static_cast<int>(std::min<size_t>(1024 / threads, 233472 / (shared + 1024))), cudaSuccess;
+}
 cudaError_t cudaGetLastError() {
     const cudaError_t e = last_error;
     last_error = cudaSuccess;

@@ -50,6 +50,8 @@ def load(path):
     L.pvq_build_count_table.argtypes = [i32, i32, vp, C.c_size_t, vp]
     L.pvq_encode.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, vp, vp, vp, vp, vp, vp]
     L.pvq_decode.argtypes = [vp, vp, vp, i64, i64, i32, i32, i32, vp, vp, vp, i64, vp, vp]
+    L.pvq_roundtrip.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, vp, vp, vp, vp, i64, vp]
+    L.pvq_rotate_roundtrip.argtypes = [vp, i32, i64, i64, i64, i32, vp, i32, i32, i32, vp, vp, vp, vp, i64, vp]
     L.fake_capture.argtypes = [vp, i32]
     L.fake_launch_name.restype = C.c_char_p
     L.fake_launch_table.restype = C.c_uint64
@@ -67,6 +69,13 @@ def encode(L, N, K, stream=PLAIN, rows=8, G=4):
 
 def decode(L, N, K, stream=PLAIN, rows=8, G=4):
     return L.pvq_decode(P, P, P, rows, G * N, N, K, 16, P, None, P, G * N, None, stream)
+
+
+def roundtrip(L, N, K, rows, cols, bf16=True, block=0):
+    dtype = 1 if bf16 else 0
+    if block:
+        return L.pvq_rotate_roundtrip(P, dtype, rows, cols, cols, block, P, N, K, 16, P, None, None, P, cols, PLAIN)
+    return L.pvq_roundtrip(P, dtype, rows, cols, cols, N, K, 16, P, None, None, P, cols, PLAIN)
 
 
 def last_tables(L):
@@ -186,6 +195,18 @@ def test_few_rows_still_fill_the_gpu(fake, N, K, rows, G, lanes):
     assert "encode_lanes" in fake.fake_launch_name(i).decode()
     threads = fake.fake_launch_grid(i) * fake.fake_launch_block(i)
     assert threads >= 0.75 * min(rows * G * lanes, 148 * 768)
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("N,K,rows,cols,block", [(32, 22, 100, 8192, 8192), (32, 22, 600, 2048, 2048), (32, 22, 100, 8192, 0), (128, 155, 256, 4096, 0),
+                                                 (16, 27, 100, 1664, 0), (32, 22, 1, 512, 0), (32, 22, 2000, 512, 512)])
+def test_a_round_trip_of_few_blocks_spreads(fake, N, K, rows, cols, block, bf16):
+    """No more blocks fit an SM than its share of the launch."""
+    assert roundtrip(fake, N, K, rows, cols, bf16, block) == 0
+    i = fake.fake_launches() - 1
+    grid, shared = fake.fake_launch_grid(i), fake.fake_launch_shared(i)
+    share = -(-grid // 148)
+    assert shared <= 232448 and 233472 // (shared + 1024) <= share or grid >= 148 * (1024 // fake.fake_launch_block(i))
 
 
 @pytest.mark.parametrize("call,N,K", [(decode, 32, 50), (encode, 32, 50), (decode, 64, 96), (decode, 64, 300), (encode, 64, 300)])
