@@ -489,18 +489,25 @@ int launch_round_t(RoundArgs& a, cudaStream_t stream) {
         a.rpt = 1;
         a.chunks = (a.C + threads - 1) / threads;
     } else {
-        // Whole rows: the block of up to 128 threads (more when a row needs it) that leaves the
-        // fewest lanes idle; among equals the largest, or the smallest when the launch would
-        // not fill the SMs anyway.  (Up to 256: 16384 x 4096 at N = 128 97.6 us, with 128 95.3.)  Rotated in blocks that span
-        // warps: whole blocks, and no more threads than need be, as they meet often.
+        // Whole rows: the block that leaves the fewest lanes idle; among equals the largest, or the smallest when the launch
+        // would not fill the SMs anyway.  Blocks of up to 128 threads, and of up to 256 where such blocks stay and there is work for
+        // one of 128 threads an SM: those above 128 are counted 3 % dearer (N = 128, 16384 x 4096: 95.3 us with 128, 97.6 with 256), but
+        // for groups on eight lanes (4096 x 4096: 32.9 and 30.8).  (With at most 128, us: 6553 x 2560 at N = 32 26.7 instead
+        // of 21.9, 7281 x 2304 at N = 128 36.5 instead of 29.6.  Less work, 100 x 1152 at N = 64, 4.6 with 128, 5.1 with 256.
+        // Blocks that take one tile, fp32: 4096 x 1024 at N = 128 11.1 with 128, 13.6 with 256.)  Rotated in blocks that span
+        // warps: whole blocks, and no more threads than need be, as they meet often (B = 2048, 8192 rows: 64 threads
+        // 41.5, 128 38.2, 256 39.2).
         a.chunks = 1;
         const int need = (a.C + 31) / 32 * 32;
-        long long best = -1;
-        for (int t = std::max(64, need); t <= std::max(T0 > 32 ? 64 : 128, need); t += 32) {
+        const bool large = BF16 && a.rows * a.C >= 128ll * di.sms;
+        const int most = std::max(need, T0 > 32 ? (BF16 ? 128 : 64) : (large ? 256 : 128));
+        double best = -1.0;
+        for (int t = std::max(64, need); t <= most; t += 32) {
             if (T0 > 32 && t % T0 != 0) continue;
             const int rpt = t / a.C;
-            const long long tiles = (a.rows + rpt - 1) / rpt, cost = tiles * t;
-            if (best < 0 || cost < best || (cost == best && tiles >= 2 * di.sms)) {
+            const long long tiles = (a.rows + rpt - 1) / rpt;
+            const double cost = static_cast<double>(tiles * t) * (L < 8 && t > 128 ? 1.03 : 1.0);
+            if (best < 0.0 || cost < best || (cost == best && tiles >= 2 * di.sms)) {
                 best = cost;
                 threads = t;
             }

@@ -209,6 +209,22 @@ def test_a_round_trip_of_few_blocks_spreads(fake, N, K, rows, cols, block, bf16)
     assert shared <= 232448 and 233472 // (shared + 1024) <= share or grid >= 148 * (1024 // fake.fake_launch_block(i))
 
 
+@pytest.mark.parametrize("N,K", [(16, 27), (32, 22), (64, 199), (128, 155)])
+@pytest.mark.parametrize("cols", [1152, 1664, 2304, 2560, 3072, 3328, 3584, 4096])
+def test_round_trip_blocks_waste_few_lanes(fake, N, K, cols):
+    """bf16, rows enough: the lanes without values are no more than in the best block of up to 256 threads, but for the 3 %
+    that those above 128 cost."""
+    rows, lanes = (1 << 24) // cols, cols // min(N, 32)
+
+    def cost(threads):
+        return -(-rows // (threads // lanes)) * threads
+
+    assert roundtrip(fake, N, K, rows, cols) == 0
+    threads = fake.fake_launch_block(fake.fake_launches() - 1)
+    need = -(-lanes // 32) * 32
+    assert cost(threads) <= 1.03 * min(cost(t) for t in range(max(64, need), max(256, need) + 1, 32))
+
+
 @pytest.mark.parametrize("call,N,K", [(decode, 32, 50), (encode, 32, 50), (decode, 64, 96), (decode, 64, 300), (encode, 64, 300)])
 def test_a_failed_launch_is_reported_once(fake, call, N, K):
     assert build(fake, 64, 96) == 0
