@@ -89,6 +89,18 @@ __device__ __forceinline__ int lane_squares(const LanePoint<E, WIDE>& pt) {
     return static_cast<int>(s);
 }
 
+// The amplitude codebook, edges padded to the 15 or 255 that amplitude() looks at; a barrier follows.
+__device__ __forceinline__ void stage_codebook(const RoundArgs& a, float* s_edges, float* s_levels, int tid, int T) {
+    if (a.b == 16) return;  // the amplitude itself
+    const int levels = 1 << a.b, entries = a.b > 4 ? kCodebookMax : 16;
+#pragma unroll 4
+    for (int i = tid; i < entries; i += T) {
+        const float edge = i + 1 < levels ? a.edges[i] : __int_as_float(0x7fffffff), level = i < levels ? a.levels[i] : 0.0f;
+        s_edges[i] = edge;
+        s_levels[i] = level;
+    }
+}
+
 // The group's dequantised amplitude.
 __device__ __forceinline__ float amplitude(float ss, float ss_row, int b, const float* s_edges, const float* s_levels) {
     if (b == 16) return __half2float(__float2half_rn(__fsqrt_rn(ss)));  // the amplitude as binary16
@@ -169,11 +181,7 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
         pack_signs<E>(s_signs, a.signs, a.rot_block);
         rot_scale = static_cast<float>(1.0 / sqrt(static_cast<double>(a.rot_block)));
     }
-    const int nlevels = b <= 8 ? 1 << b : 0;  // 16 bits: the amplitude itself, no codebook
-    for (int i = tid; nlevels != 0 && i < kCodebookMax; i += T) {
-        s_edges[i] = i + 1 < nlevels ? a.edges[i] : __int_as_float(0x7fffffff);
-        if (i < nlevels) s_levels[i] = a.levels[i];
-    }
+    stage_codebook(a, s_edges, s_levels, tid, T);
 #ifdef PVQ_DEBUG
     debug_begin(0u, 0u, 0u, 0u, 0u, a.debug_status);
 #endif
@@ -364,11 +372,7 @@ __global__ void __launch_bounds__(kRoundThreadsMax) roundtrip_rows_kernel(const 
         pack_signs<E>(s_signs, a.signs, a.rot_block);
         rot_scale = static_cast<float>(1.0 / sqrt(static_cast<double>(a.rot_block)));
     }
-    const int nlevels = b <= 8 ? 1 << b : 0;  // 16 bits: the amplitude itself, no codebook
-    for (int i = tid; nlevels != 0 && i < kCodebookMax; i += T) {
-        s_edges[i] = i + 1 < nlevels ? a.edges[i] : __int_as_float(0x7fffffff);
-        if (i < nlevels) s_levels[i] = a.levels[i];
-    }
+    stage_codebook(a, s_edges, s_levels, tid, T);
     if (ROT) __syncthreads();
 
     const int rl = a.chunks == 1 ? tid / a.C : 0;
