@@ -658,14 +658,18 @@ static int launch_encode_lanes_t(BatchArgs& a, cudaStream_t stream) {
         // shared memory is what limits them, a long launch makes do with one input buffer a team: the wait for the input is
         // covered by the other warps.  (A decoder layer at N = 32, 96 bits: 23 warps and two buffers 336 us, 28 and one 286.)
         const long long most_teams = std::min(kLaneThreads<W> / t, t == 32 ? 32 : 15);
-        long long teams = 0;
-        for (int n = 2; n >= (long_launch ? 1 : 2) && teams < most_teams; --n) {
-            c.in_bufs = n;
-            c.ss_off = static_cast<uint32_t>(n) * c.in_bytes;
+        auto place = [&](int in_bufs) {  // the team's area, and how many of them fit
+            c.in_bufs = in_bufs;
+            c.ss_off = static_cast<uint32_t>(in_bufs) * c.in_bytes;
             c.amp_off = c.ss_off + bufs * static_cast<uint32_t>(c.ss_floats) * 4u;
             c.idx_off = c.amp_off + (LS ? bufs * static_cast<uint32_t>(c.ss_floats) * 4u : 0u);
             c.team_bytes = (c.idx_off + bufs * static_cast<uint32_t>(idx_words) * 4u + 127u) & ~127u;
-            teams = std::min(most_teams, (static_cast<long long>(di.smem_max) - c.team_off) / c.team_bytes);
+            return std::min(most_teams, (static_cast<long long>(di.smem_max) - c.team_off) / c.team_bytes);
+        };
+        long long teams = place(2);
+        if (long_launch && teams < most_teams) {
+            const long long more = place(1);
+            teams = more > teams ? more : place(2);
         }
         if (teams < 1) continue;
         const double per_tile = static_cast<double>(chunks_all) / tiles + (t == 32 ? 0.16 : 0.25);

@@ -26,6 +26,7 @@ std::map<const void*, std::string>& kernels() {
 struct Launch {
     std::string name;
     uint64_t tables[2];  // the first words of a windowed kernel's second argument: its tables' addresses
+    int teams[3];        // of encode_lanes_kernel's: threads a team, teams, input buffers a team
     unsigned grid, block;
     size_t shared;
     bool early;  // may start before the kernel in front has ended
@@ -55,8 +56,9 @@ cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, size_t sha
     std::unique_lock<std::mutex> lock(mu);
     if (kernels()[f].find("code_window") != std::string::npos) wait_while(hold_launch, lock);
     if (fail_launch != cudaSuccess) return ret(fail_launch);
-    Launch l{kernels()[f], {0, 0}, grid.x, block.x, shared, early};
+    Launch l{kernels()[f], {0, 0}, {0, 0, 0}, grid.x, block.x, shared, early};
     if (l.name.find("code_window") != std::string::npos) std::memcpy(l.tables, args[1], sizeof l.tables);
+    if (l.name.find("encode_lanes") != std::string::npos) std::memcpy(l.teams, args[1], sizeof l.teams);
     launches.push_back(l);
     return cudaSuccess;
 }
@@ -67,6 +69,7 @@ extern "C" {
 int fake_launches() { return static_cast<int>(launches.size()); }
 const char* fake_launch_name(int i) { return launches[i].name.c_str(); }
 uint64_t fake_launch_table(int i, int which) { return launches[i].tables[which]; }
+int fake_launch_teams(int i, int which) { return launches[i].teams[which]; }
 unsigned fake_launch_grid(int i) { return launches[i].grid; }
 unsigned fake_launch_block(int i) { return launches[i].block; }
 unsigned fake_launch_shared(int i) { return static_cast<unsigned>(launches[i].shared); }

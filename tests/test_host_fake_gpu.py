@@ -50,6 +50,7 @@ def load(path):
     L.pvq_build_count_table.argtypes = [i32, i32, vp, C.c_size_t, vp]
     L.pvq_encode.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, vp, vp, vp, vp, vp, vp]
     L.pvq_decode.argtypes = [vp, vp, vp, i64, i64, i32, i32, i32, vp, vp, vp, i64, vp, vp]
+    L.pvq_encode_amp.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, i32, vp, vp, vp, vp, vp, vp]
     L.pvq_roundtrip.argtypes = [vp, i32, i64, i64, i64, i32, i32, i32, vp, vp, vp, vp, i64, vp]
     L.pvq_rotate_roundtrip.argtypes = [vp, i32, i64, i64, i64, i32, vp, i32, i32, i32, vp, vp, vp, vp, i64, vp]
     L.fake_capture.argtypes = [vp, i32]
@@ -195,6 +196,16 @@ def test_few_rows_still_fill_the_gpu(fake, N, K, rows, G, lanes):
     assert "encode_lanes" in fake.fake_launch_name(i).decode()
     threads = fake.fake_launch_grid(i) * fake.fake_launch_block(i)
     assert threads >= 0.75 * min(rows * G * lanes, 148 * 768)
+
+
+@pytest.mark.parametrize("K,G,bf16,amp_mode,bufs", [(50, 4096, 1, 0, 2), (50, 4096, 1, 1, 2), (63, 4096, 1, 0, 2), (63, 128, 1, 1, 1), (50, 128, 0, 0, 1)])
+def test_one_input_buffer_only_for_more_teams(fake, K, G, bf16, amp_mode, bufs):
+    """Long encoder launches: a team gives up the buffer that its next input is asked for ahead only where more teams fit
+    without.  (Rows of 4096 groups: as many either way.)"""
+    assert fake.pvq_encode_amp(P, bf16, 2000000 // G, G * 32, G * 32, 32, K, 8, amp_mode, P, P, P, P, P, PLAIN) == 0
+    i = fake.fake_launches() - 1
+    assert "encode_lanes" in fake.fake_launch_name(i).decode()
+    assert fake.fake_launch_teams(i, 2) == bufs
 
 
 @pytest.mark.parametrize("bf16", [True, False])
