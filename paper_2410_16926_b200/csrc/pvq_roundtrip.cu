@@ -93,11 +93,10 @@ __device__ __forceinline__ int lane_squares(const LanePoint<E, WIDE>& pt) {
 __device__ __forceinline__ void stage_codebook(const RoundArgs& a, float* s_edges, float* s_levels, int tid, int T) {
     if (a.b == 16) return;  // the amplitude itself
     const int levels = 1 << a.b, entries = a.b > 4 ? kCodebookMax : 16;
-#pragma unroll 4
+#pragma unroll 1  // (four at a time: small calls 0.1 to 0.4 us slower)
     for (int i = tid; i < entries; i += T) {
-        const float edge = i + 1 < levels ? a.edges[i] : __int_as_float(0x7fffffff), level = i < levels ? a.levels[i] : 0.0f;
-        s_edges[i] = edge;
-        s_levels[i] = level;
+        s_edges[i] = i + 1 < levels ? a.edges[i] : __int_as_float(0x7fffffff);
+        if (i < levels) s_levels[i] = a.levels[i];
     }
 }
 
