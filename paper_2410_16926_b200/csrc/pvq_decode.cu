@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
         const unsigned g0 = (tile - m.tile_begin) * 32u;             // first group of the tile
         const unsigned gi = g0 + lane;
         const bool active = gi < ngroups;
-        // row and group-in-row: one division per tile, the threads follow from the first group
+        // row and group-in-row: found once a tile, the threads follow from the first group
         unsigned row = group_row(m, g0);
         unsigned g = g0 - row * G + lane;
         if (g >= G) {

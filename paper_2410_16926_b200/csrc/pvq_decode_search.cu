@@ -9,9 +9,10 @@
 // thresholds of row n, which do not depend on k (SearchLayout in pvq_internal.cuh): the first
 // threshold index m with T_n[m] >= q gives the pulses left after the position (m >> 1) and
 // the sign (m odd: positive), and q + E_n[m] is the q of the next position.  The search is one
-// table look-up and one multi-word compare: the leading bits of q, as an fp32 key shifted
-// by a per-row amount, select a bucket whose byte entry is the first index that can be
-// right, and the buckets are fine enough that the only other candidate is the next index.
+// table look-up: the leading bits of q, as an fp32 key shifted by a per-row amount, select a bucket, which
+// holds one threshold at most; its entry has the index of the first threshold that can be right and the key bits of
+// that threshold, which decide against the next index.  Where they are q's own, q and the threshold are
+// compared in full (pvq_search.cuh).
 //
 // All threads of a warp are at the same position, so nothing diverges; table reads of a warp
 // go to one row (neighbouring entries for similar q).  Threads collect their point in shared
@@ -27,6 +28,9 @@
 namespace pvq {
 
 namespace {
+
+constexpr QuadTable kQuadsHost = make_quads();
+__device__ __align__(128) const QuadTable kQuads = kQuadsHost;
 
 constexpr int kSearchThreads = 1024;
 
@@ -117,7 +121,7 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
             const unsigned gi = g0 + lane;
             active[j] = tile < a.total_tiles && gi < ngroups;
             active_valid[j] = active[j];
-            // row and group-in-row: one division per tile, the threads follow from the first group
+            // row and group-in-row: found once a tile, the threads follow from the first group
             row[j] = group_row(m, g0);
             g[j] = g0 - row[j] * G + lane;
             if (g[j] >= G) {

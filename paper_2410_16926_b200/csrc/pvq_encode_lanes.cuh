@@ -2,8 +2,8 @@
 // Algorithms 1 and 2): group sizes 8 to 64, the tables of the Fischer index in shared memory.
 //
 // What bounds it: issue slots and the half-rate integer pipe.  So:
-//   - the direction comes from counting passes over packed residuals (pvq_quant.cuh), not from a
-//     sorting network;
+//   - the last pulses of the direction are found bit by bit in bit planes of the residuals (pvq_quant.cuh),
+//     not by a sorting network;
 //   - the index is summed from one table entry per position, E(i, m) with m = 2 k' + (y_i > 0), k' the
 //     pulses behind position i (the telescoped tables, `cenc` of TableLayout, interleaved).  The
 //     k' of four positions are one multiplication (a running sum over the bytes of the packed
@@ -11,8 +11,9 @@
 //   - for codes of two and three words M = -E is kept as doubles, 48 bits each (32 of them add up
 //     exactly), so that the additions are one or two instructions on the fp64 pipe, which nothing
 //     else uses, without carries; positions whose M stays below 2^48 have no upper half to read;
-//   - the input arrives in shared memory by asynchronous copies of whole lines, a chunk ahead, each
-//     lane's run padded by 16 bytes so that the lanes' 16-byte reads hit different banks.
+//   - the input arrives in shared memory by asynchronous copies of whole lines, a chunk ahead (or as soon as the
+//     chunk before has been read, LaneGeom::in_bufs), each lane's run padded by 16 bytes so that the
+//     lanes' 16-byte reads hit different banks.
 // Larger groups and wider codes (any group size, up to 32 words, any K): the same kernel with a group on up
 // to 8 lanes, the point in 16-bit halves, and Algorithm 2's two terms per position read from the cumulative
 // tables in global memory (L1, L2), only as many words as the position's counts have.

@@ -8,7 +8,7 @@
 // then every thread sums its group's index from the windowed tables (pvq_window.cuh), one entry of E a position, read
 // word plane by word plane from the ring that a feeding warp keeps filled, the last block of rows first.  With q the
 // number that the decoder searches, the code is N(N,K) - q: the sum of all E is 1 - q.  Same matrix: 54 us; the two phases
-// do not overlap (61% of the issue slots used).
+// do not overlap (59% of the issue slots used).
 #include <algorithm>
 #include <cstring>
 
@@ -477,6 +477,7 @@ int launch_ew(BatchArgs& a, int dtype, const WinTables& t, cudaStream_t s) {
 }  // namespace
 
 int launch_encode_window(const BatchArgs& args, int dtype, int N, int W, cudaStream_t stream) {
+    static_assert(!has_window_tables(64, 8, 256) && !has_window_tables(128, 12, 256), "a coordinate's pulses and the sums of four have a byte each");
     if (N == 256 || !has_window_tables(N, W, args.K)) return PVQ_ERR_UNSUPPORTED;
     const auto t = window_tables(N, args.K, stream);
     if (!t || t->args.words[N / 4 - 1] != 1) return PVQ_ERR_UNSUPPORTED;

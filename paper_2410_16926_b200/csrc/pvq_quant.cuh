@@ -332,7 +332,9 @@ struct NoHook {
     __device__ __forceinline__ void operator()() const {}
 };
 
-// ax: |x_i| of the lane's values; l1: of the whole group.  `hook` is called by the warp half way, where few registers
+// ax: |x_i| of the lane's values; l1: of the whole group.  Points in bytes (not WIDE) hold up to 255 pulses: no coordinate, and no
+// sum of the lane's floors over the words, which is an integer of at most K as their sum is below K + 1, leaves its byte.  (What
+// reads a sign or a comparison from a byte's top bit has to see to K <= 127 itself.)  `hook` is called by the warp half way, where few registers
 // are in use.
 template <int E, int L, bool WIDE, class Fetch, class Hook = NoHook>
 __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, int K, const Fetch& fetch,
@@ -342,7 +344,8 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
     // no direction: l1 zero or not finite, or a scale that overflows
     bool has_dir = (l1 > 0.0f) && (l1 <= 3.4028234e38f) && (gsc <= 3.4028234e38f);
     // a + 2^15 rounded down is 2^15 + floor(256 a) / 256: 8 bits of the residual are the lowest byte, the floor
-    // begins at the next (a <= K + 1 leaves the exponent alone)
+    // begins at the next (a < K + 1 leaves the exponent alone)
+    static_assert(kMaxPulses + 1 < 32768, "2^15 + a below 2^16");
     uint32_t t[E];
     {
         const f32x2 g2 = pack2(gsc, gsc), m2 = pack2(32768.0f, 32768.0f);
@@ -362,8 +365,8 @@ __device__ __forceinline__ void quantize_group(const float (&ax)[E], float l1, i
         for (int j = 0; j < J; ++j) {
             const uint32_t u = __byte_perm(t[4 * j + 3], t[4 * j + 2], 0x5410), v = __byte_perm(t[4 * j + 1], t[4 * j], 0x5410);
             x[j] = __byte_perm(u, v, 0x6420);
-            pt.y[j] = __byte_perm(u, v, 0x7531);  // floors, below 128
-            sum4 += pt.y[j];                      // no byte passes K
+            pt.y[j] = __byte_perm(u, v, 0x7531);  // floors, at most K
+            sum4 += pt.y[j];                      // ... as are these
         }
         fsum = static_cast<int>(__dp4a(sum4, kOne4, 0u));
     } else {

@@ -113,7 +113,7 @@ __device__ __forceinline__ void search_coordinates(uint32_t m4, uint32_t& k, uin
 
 // The last four positions at once: the indices of q in row 3, of the q that follows in row 2, and so on depend on q
 // alone (no N, K or pulses left in them), and q is small there: at most N(4,k) with k pulses left, some K / 8 of them at
-// N = 32.  kQuads holds the four indices, first position lowest, of q = 1 .. N(4,kQuadPulses); a larger q is searched.
+// N = 32.  A QuadTable holds the four indices, first position lowest, of q = 1 .. N(4,kQuadPulses); a larger q is searched.
 constexpr uint32_t kQuadPulses = 16;
 constexpr uint32_t quad_count(uint32_t n, uint32_t k) {  // V(n,k) = sum over j <= k of N(n,j)
     return n == 0 ? 1u : (n == 1 ? 2u * k + 1u : (n == 2 ? 2u * k * k + 2u * k + 1u : (2u * k + 1u) * (2u * k * k + 2u * k + 3u) / 3u));
@@ -140,8 +140,6 @@ constexpr QuadTable make_quads() {
     }
     return t;
 }
-constexpr QuadTable kQuadsHost = make_quads();
-__device__ __align__(128) const QuadTable kQuads = kQuadsHost;
 
 // Makes the accepted section ready for the search; all threads, a barrier follows.  `t_off`: where its buckets end.  Records
 // afterwards: 32 - shift, the shared addresses of its row of E and of its buckets, the shift.
@@ -239,7 +237,7 @@ __device__ __forceinline__ void search_block4(mp<W> (&q)[GP], uint32_t (&k)[GP],
 }
 
 // The points of GP codes: q = N(N,K) - code on entry.  `recs` is the shared address of the
-// row records (absolute shared addresses by now), cnt[w] the number of rows done in w words; quads: shared address of kQuads,
+// row records (absolute shared addresses by now), cnt[w] the number of rows done in w words; quads: shared address of a QuadTable,
 // or 0: without.
 template <int N, int W, int GP, int PLANE, bool LONG>
 __device__ __forceinline__ void search_codes(mp<W> (&q)[GP], int K, uint32_t recs, const uint8_t* t_rows, const int (&cnt)[5], uint32_t quads,
