@@ -62,3 +62,34 @@ def test_rotated_round_trip(N, bits, G, block):
     want = po.decode(*o, N, K, b, None)[0]
     got = pvq.rotate_roundtrip(torch.from_numpy(x).cuda(), block, torch.from_numpy(signs).cuda(), N, K, b, pvq.build_count_table(N, K), None, None)
     assert np.array_equal(bf16_bits(got), want)
+
+
+# Rows of whole warps, a power of two of them or not (lanes a row; N / 32 lanes a group): a warp's part of a row's energy and the
+# zeros between the rows' parts; rows that leave a thread block's lanes idle; input and output in wider rows.
+@pytest.mark.parametrize("N,bits,b", [(32, 64, 8), (64, 256, 3), (128, 512, 16), (256, 768, 5)])
+@pytest.mark.parametrize("lanes", [32, 64, 72, 80, 96, 160, 352])
+@pytest.mark.parametrize("block", [0, 256])
+def test_round_trip_lanes(N, bits, b, lanes, block):
+    rows, cols = 401, lanes * 32
+    if cols % max(block, N) != 0:
+        pytest.skip("rows of whole groups and rotation blocks")
+    G = cols // N
+    K = pvq.max_pulses(N, bits)
+    rng = np.random.default_rng(N + lanes)
+    x = np.zeros((rows, cols + 24), dtype=np.uint16)
+    x[:, :cols] = inputs.f32_to_bf16_bits(rng.standard_normal((rows, cols)).astype(np.float32))
+    e_np, l_np = (None, None) if b == 16 else (bc.edges_f32(N, G, b), bc.levels_amp_f32(N, G, b))
+    edges, levels = (None, None) if b == 16 else (torch.from_numpy(e_np).cuda(), torch.from_numpy(l_np).cuda())
+    table = pvq.build_count_table(N, K)
+    out = torch.full((rows, cols + 8), 7.0, dtype=torch.bfloat16, device="cuda")
+    x_dev = torch.from_numpy(x.view(np.int16)).cuda().view(torch.bfloat16)[:, :cols]
+    values = np.ascontiguousarray(x[:, :cols])
+    if block:
+        signs = rng.choice([-1.0, 1.0], size=block).astype(np.float32)
+        values = po.rotate(values, block, signs)
+        pvq.rotate_roundtrip(x_dev, block, torch.from_numpy(signs).cuda(), N, K, b, table, edges, levels, out=out[:, :cols])
+    else:
+        pvq.roundtrip(x_dev, N, K, b, table, edges, levels, out=out[:, :cols])
+    want = po.decode(*po.encode(values, N, K, b, e_np, W=pvq.code_words(N, K)), N, K, b, l_np)[0]
+    assert np.array_equal(bf16_bits(out[:, :cols].contiguous()), want)
+    assert bool((out[:, cols:] == 7.0).all())

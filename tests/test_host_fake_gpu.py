@@ -10,8 +10,11 @@ import threading
 
 import pytest
 
+from oracle import pvq_pyref as pr
 from paper_2410_16926_b200 import build as lib_build
 from paper_2410_16926_b200 import pvq
+
+import test_long_decode
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 P = 1 << 20  # an address, aligned; nothing is read there
@@ -196,6 +199,21 @@ def test_few_rows_still_fill_the_gpu(fake, N, K, rows, G, lanes):
     assert "encode_lanes" in fake.fake_launch_name(i).decode()
     threads = fake.fake_launch_grid(i) * fake.fake_launch_block(i)
     assert threads >= 0.75 * min(rows * G * lanes, 148 * 768)
+
+
+@pytest.mark.parametrize("N,K", test_long_decode.SETTINGS)
+def test_decoding_launches_that_rewrite_the_buckets(fake, N, K):
+    """The sizes that test_long_decode.py decodes take the kernels for launches of several rounds, with the table of the last
+    four positions where N = 32 has it; launches half as long do not."""
+    rows, quads = test_long_decode.long_rows(N, K, 64, 148), 0
+    for n, long_launch in ((rows, True), (int(rows / 2.1), False)):
+        assert decode(fake, N, K, rows=n, G=64) == 0
+        i = fake.fake_launches() - 1
+        name = fake.fake_launch_name(i).decode()
+        assert "decode_search" in name and ("ELb1EE" in name) == long_launch and ("ELb0EE" in name) != long_launch
+        tables = fake.fake_launch_shared(i) - 2 * (N + 4) * fake.fake_launch_block(i)  # (slots of two groups a thread)
+        quads = tables if long_launch else quads - tables
+    assert quads in (0, 4 * pr.count_table(4, 16)[4][16]) and (quads != 0 or (N, K) != (32, 22))
 
 
 @pytest.mark.parametrize("K,G,bf16,amp_mode,bufs", [(50, 4096, 1, 0, 2), (50, 4096, 1, 1, 2), (63, 4096, 1, 0, 2), (63, 128, 1, 1, 1), (50, 128, 0, 0, 1)])

@@ -60,14 +60,41 @@ def test_rewritten_entries(N, K):
         assert left_open > 0           # these codes do reach the case
 
 
+def long_rows(N, K, G, sms):
+    """Rows of G groups for rounds enough of two tiles of 32 groups for each of 32 warps an SM that the buckets are rewritten
+    (launch_search_g; that these sizes do it is tested in test_host_fake_gpu.py)."""
+    sec = bs.section(pr.count_table(N, K), N, K, pvq.code_words(N, K), 0)
+    rounds = 1.02 * max(3.0, (sec["t_off"] - sec["b_off"]) / 4 / (80 * N))
+    return int(rounds * 2 * sms * 32 * 32 / G) + 1
+
+
+@pytest.mark.gpu
+def test_last_four_positions():
+    """Every q of the table of the last four positions: behind 6 pulses and 27 zeros every point of four positions with 16, and
+    some with 17, whose q are partly beyond the table."""
+    N, K, G, b = 32, 22, 64, 16
+    W = pvq.code_words(N, K)
+    count = pr.count_table(N, K)
+    first = pr.enumerate_point([K - 16] + [0] * 27 + [0, 0, 0, 16], K)   # the lowest code of them
+    assert first + count[4][16] - 1 == pr.enumerate_point([K - 16] + [0] * 27 + [-16, 0, 0, 0], K)
+    some = list(range(first, first + count[4][16]))
+    some += [pr.enumerate_point([K - 17] + [0] * 27 + p, K) for p in ([17, 0, 0, 0], [-9, 8, 0, 0], [0, 0, 0, 17], [0, 0, 0, -17], [0, -1, 16, 0])]
+    rows = long_rows(N, K, G, torch.cuda.get_device_properties(0).multi_processor_count)
+    base = np.array([po.int_to_code(c, W) for c in some], dtype=np.uint32)
+    codes = np.resize(base, (rows * G, W)).reshape(rows, G, W)
+    sidx = np.random.default_rng(1).integers(0, 120, size=(rows, int(pvq.scale_row_stride(G, b))), dtype=np.uint8)  # finite binary16 amplitudes
+    rnorm = np.ones(rows, dtype=np.float32)
+    want, _ = po.decode(codes, sidx, rnorm, N, K, b, None)
+    got = pvq.decode(torch.from_numpy(codes.view(np.int32)).cuda(), torch.from_numpy(sidx).cuda(), torch.from_numpy(rnorm).cuda(), N, K, b,
+                     pvq.build_count_table(N, K), None)
+    assert np.array_equal(got.view(torch.int16).cpu().numpy().view(np.uint16), want)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("N,K", SETTINGS)
 def test_long_launch(N, K):
-    # enough rounds of two tiles of 32 groups for each of 32 warps an SM that the buckets are rewritten (launch_search_g)
-    sec = bs.section(pr.count_table(N, K), N, K, pvq.code_words(N, K), 0)
-    rounds = 1.02 * max(3.0, (sec["t_off"] - sec["b_off"]) / 4 / (80 * N))
     G, b = 64, 8
-    rows = int(rounds * 2 * torch.cuda.get_device_properties(0).multi_processor_count * 32 * 32 / G) + 1
+    rows = long_rows(N, K, G, torch.cuda.get_device_properties(0).multi_processor_count)
     W = pvq.code_words(N, K)
     rng = np.random.default_rng(3 * N + K)
     total = pr.count_table(N, K)[N][K]
