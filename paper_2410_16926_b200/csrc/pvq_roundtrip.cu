@@ -193,9 +193,12 @@ __global__ void __launch_bounds__(kRoundThreadsMax, 2) roundtrip_kernel(const __
     // quantised, not after the barrier: 16384 x 4096 72.8 -> 72.0 us, at N = 128 94.5 -> 92.8.  (Rotated: 23.0 -> 23.2, so not there.)
     const bool in_warp = a.C <= 32 && (a.C & (a.C - 1)) == 0, whole = !ROT && !in_warp && (a.C & 31) == 0;
     const int parts = whole ? a.gp * L / 32 : a.gp, used = whole ? a.C / 32 : a.G;
-    if (parts != used)  // the zero padding of the rows' trees
-        for (int j = tid; j < 2 * a.rpt * parts; j += T)
-            if ((j & (parts - 1)) >= used) reinterpret_cast<float*>(smem + a.ss_off)[j / (a.rpt * parts) * a.rpt * a.gp + j % (a.rpt * parts)] = 0.0f;
+    if (parts != used)  // the zero padding of the rows' trees, for both tiles at work
+        for (int j = tid; j < a.rpt * parts; j += T)
+            if ((j & (parts - 1)) >= used) {
+                float* p = reinterpret_cast<float*>(smem + a.ss_off) + j;
+                p[0] = p[a.rpt * a.gp] = 0.0f;
+            }
     const uint32_t lane_off = a.ring_off + static_cast<uint32_t>(tid) * (E * 2);  // rows of a tile follow one another
     int buf = 0, parity = 0;
     for (int i = 0;; ++i) {
