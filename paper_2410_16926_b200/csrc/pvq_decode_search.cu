@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kSearchThreads / (GP > 2 ? 2 : 1), 1)
 }
 
 template <int N, int W, int GP, int PLANE, bool LONG>
-int launch_search_t(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
+int launch_search_t(BatchArgs& a, const SearchLayout& S, const DeviceInfo& di, cudaStream_t stream) {
     constexpr int YS = N + 4;
     constexpr int kMaxThreads = kSearchThreads / (GP > 2 ? 2 : 1);
     const unsigned tiles = a.total_tiles;
@@ -193,9 +193,6 @@ int launch_search_t(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
     a.srch_t_off = S.t_off;
     a.srch_t_before_e = S.e_off - S.t_off;
     size_t staged = S.total - (S.e_off - S.t_off);
-    DeviceInfo di;
-    int st = device_info(&di);
-    if (st != PVQ_OK) return st;
     // (the table of the last four positions where it takes no threads away)
     a.srch_quads = LONG && staged + sizeof(QuadTable) + static_cast<size_t>(kMaxThreads) * YS * GP <= static_cast<size_t>(di.smem_max) ? sizeof(QuadTable) : 0u;
     staged += a.srch_quads;
@@ -225,7 +222,8 @@ int launch_search_t(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
     }
     if (threads == 0) return PVQ_ERR_UNSUPPORTED;
     int per_sm = 0;
-    if ((st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm)) != PVQ_OK) return st;
+    const int st = prepare_kernel(reinterpret_cast<const void*>(kern), threads, smem, &per_sm);
+    if (st != PVQ_OK) return st;
     if (per_sm < 1) return PVQ_ERR_UNSUPPORTED;
     const unsigned warps_per_block = threads / 32;
     const unsigned blocks_needed = (tiles + warps_per_block * GP - 1) / (warps_per_block * GP);
@@ -255,9 +253,9 @@ int launch_search_g(BatchArgs& a, const SearchLayout& S, cudaStream_t stream) {
     const double rounds = tiles / (2.0 * di.sms * (kSearchThreads / 32)), buckets = (S.t_off - S.b_off) / 4.0;
     const bool is_long = rounds > 3.0 && rounds * N * 80.0 > buckets;
     switch (S.plane) {  // entries per word plane of the section's rows
-        case 64: return is_long ? launch_search_t<N, W, 2, 64, true>(a, S, stream) : launch_search_t<N, W, 2, 64, false>(a, S, stream);
-        case 128: return is_long ? launch_search_t<N, W, 2, 128, true>(a, S, stream) : launch_search_t<N, W, 2, 128, false>(a, S, stream);
-        case 256: return is_long ? launch_search_t<N, W, 2, 256, true>(a, S, stream) : launch_search_t<N, W, 2, 256, false>(a, S, stream);
+        case 64: return is_long ? launch_search_t<N, W, 2, 64, true>(a, S, di, stream) : launch_search_t<N, W, 2, 64, false>(a, S, di, stream);
+        case 128: return is_long ? launch_search_t<N, W, 2, 128, true>(a, S, di, stream) : launch_search_t<N, W, 2, 128, false>(a, S, di, stream);
+        case 256: return is_long ? launch_search_t<N, W, 2, 256, true>(a, S, di, stream) : launch_search_t<N, W, 2, 256, false>(a, S, di, stream);
         default: return PVQ_ERR_UNSUPPORTED;
     }
 }
